@@ -103,13 +103,15 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 // work on at the same time -- then form a compact block of about BAND x (SMs / BAND) tiles that
 // shares its operand panels in L2, instead of a strip that spans every column of X.
 constexpr int BAND = 16;
+// One block per band, one thread per tile column: the tiles before the band (two tile rows 2h, 2h + 1 have h + 1 tiles
+// each, so r0 = 2h rows have h (h + 1)) and before the column have closed forms.  (One thread writing the whole list took
+// 13 us at 8192 features, 50 us at 18432.)
 __global__ void hessian_tile_order_kernel(int tiles_m, int2* __restrict__ tiles) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  int t = 0;
-  for (int r0 = 0; r0 < tiles_m; r0 += BAND) {
-    const int r1 = min(tiles_m, r0 + BAND);
-    for (int tn = 0; tn <= (r1 - 1) / 2; ++tn)
-      for (int tm = max(r0, 2 * tn); tm < r1; ++tm) tiles[t++] = make_int2(tm, tn);
+  const int r0 = blockIdx.x * BAND, r1 = min(tiles_m, r0 + BAND), h = r0 / 2;
+  for (int tn = threadIdx.x; tn <= (r1 - 1) / 2; tn += blockDim.x) {
+    int t = h * (h + 1) + min(tn, h) * (r1 - r0);
+    if (tn > h) t += (tn - h) * r1 - (tn * (tn - 1) - h * (h - 1));
+    for (int tm = max(r0, 2 * tn); tm < r1; ++tm) tiles[t++] = make_int2(tm, tn);
   }
 }
 
@@ -276,20 +278,69 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
   }
 }
 
-// Sum the K-split partials of every tile in ascending split order, add the previous H when
-// accumulating, and write the lower-triangle entry together with its mirror image.
+// Sum the K-split partials of every tile in ascending split order, add the previous H when accumulating, and write the
+// lower-triangle entries together with their mirror image.  A memory-bound pass: 4 bytes read per split and entry, 8
+// written.  One block per 64 x 64 piece of a tile, which it turns round through shared memory, so that the mirror image
+// is written along its rows too (written down the columns, one 4-byte sector per entry, the pass took 400 us at 8192
+// features and 2 ms at 18432).  VEC: rows of H start on 16-byte boundaries.
+constexpr int RP = 64;
+template <bool VEC>
 __global__ void __launch_bounds__(256) hessian_reduce_kernel(Params p, int accumulate, float* __restrict__ H) {
+  __shared__ float piece[RP][RP + 1];
   const int t = blockIdx.x;
-  const int tm = p.tiles[t].x, tn = p.tiles[t].y;
   const long long d = p.d_in;
-  for (int idx = threadIdx.x; idx < TILE_ELEMS; idx += blockDim.x) {
-    const long long r = (long long)tm * BM + idx / BN, c = (long long)tn * BN + idx % BN;
-    if (r >= d || c > r) continue;
-    float v = 0.f;
-    for (int s = 0; s < p.splits; ++s) v += p.partials[((size_t)s * p.ntiles + t) * TILE_ELEMS + idx];
-    if (accumulate) v += H[r * d + c];
-    H[r * d + c] = v;
-    if (c != r) H[c * d + r] = v;
+  const int pr = (int)blockIdx.y / (BN / RP) * RP, pc = (int)blockIdx.y % (BN / RP) * RP;   // the piece inside the tile
+  const long long r0 = (long long)p.tiles[t].x * BM + pr, c0 = (long long)p.tiles[t].y * BN + pc;
+  if (r0 >= d || c0 >= d || c0 > r0) return;   // outside, or above the diagonal (r0 and c0 are multiples of RP)
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const long long c = c0 + 4 * tx;
+#pragma unroll
+  for (int i = 0; i < RP / 16; ++i) {
+    const int rr = ty + 16 * i;
+    const long long r = r0 + rr;
+    const float* src = p.partials + (size_t)t * TILE_ELEMS + (size_t)(pr + rr) * BN + pc + 4 * tx;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < p.splits; ++s) {
+      const float4 w = *reinterpret_cast<const float4*>(src + (size_t)s * p.ntiles * TILE_ELEMS);
+      v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    }
+    float x[4] = {v.x, v.y, v.z, v.w};
+    float* dst = H + r * d + c;
+    if (r < d) {
+      if (VEC && c + 3 <= r) {   // (c + 3 <= r < d)
+        if (accumulate) {
+          const float4 o = *reinterpret_cast<const float4*>(dst);
+          x[0] += o.x; x[1] += o.y; x[2] += o.z; x[3] += o.w;
+        }
+        *reinterpret_cast<float4*>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (c + e <= r) {
+            if (accumulate) x[e] += dst[e];
+            dst[e] = x[e];
+          }
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) piece[rr][4 * tx + e] = x[e];
+  }
+  __syncthreads();
+  // the mirror image: row c of H, columns r
+#pragma unroll
+  for (int i = 0; i < RP / 16; ++i) {
+    const int cc = ty + 16 * i;
+    const long long mr = c0 + cc, mc = r0 + 4 * tx;
+    if (mr >= d) continue;
+    const float y[4] = {piece[4 * tx][cc], piece[4 * tx + 1][cc], piece[4 * tx + 2][cc], piece[4 * tx + 3][cc]};
+    float* dst = H + mr * d + mc;
+    if (VEC && mc > mr && mc + 3 < d) {
+      *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (mc + e > mr && mc + e < d) dst[e] = y[e];
+    }
   }
 }
 
@@ -363,7 +414,7 @@ cudaError_t launch_hessian_tc(const void* X, long long n, long long d_in, long l
   p.partials = (float*)ws;
   int2* tiles = (int2*)((char*)ws + align_up((size_t)pl.splits * pl.ntiles * TILE_ELEMS * sizeof(float)));
   p.tiles = tiles;
-  { hessian_tile_order_kernel<<<1, 32, 0, st>>>(pl.tiles_m, tiles); count_launch(); }
+  { hessian_tile_order_kernel<<<(pl.tiles_m + BAND - 1) / BAND, 128, 0, st>>>(pl.tiles_m, tiles); count_launch(); }
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;
   int dev = 0, sms = 0;
@@ -376,7 +427,9 @@ cudaError_t launch_hessian_tc(const void* X, long long n, long long d_in, long l
   { hessian_tc_kernel<<<grid, NUM_THREADS, SMEM_BYTES, st>>>(tmap, p); count_launch(); }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  { hessian_reduce_kernel<<<pl.ntiles, 256, 0, st>>>(p, accumulate, H); count_launch(); }
+  const dim3 pieces((unsigned)pl.ntiles, (BM / RP) * (BN / RP));
+  if (d_in % 4 == 0) { hessian_reduce_kernel<true><<<pieces, 256, 0, st>>>(p, accumulate, H); count_launch(); }
+  else { hessian_reduce_kernel<false><<<pieces, 256, 0, st>>>(p, accumulate, H); count_launch(); }
   return cudaGetLastError();
 }
 
