@@ -56,77 +56,97 @@ cudaError_t launch_hessian_verify(const void* X, cdq_dtype xt, long long n, long
 }
 
 // ---- tiled SIMT kernel -----------------------------------------------------
-constexpr int HT = 64;   // output tile edge
+// T x T tiles of the lower triangle, (T / M)^2 threads with M x M entries each, fp64 fused multiply-adds in ascending
+// order of the rows, whatever the tile.  Bound by the fp64 pipe (64 per clock and SM): the operands are widened once,
+// when a stage is stored to shared memory (widening them at every use kept the conversion pipe busy twice as long as the
+// fp64 pipe: 1.2 ms at 4099 rows by 1350 features), and the next stage's loads are issued before the present stage is used.
+// T = 64 for layers whose tiles fill the SMs; smaller tiles for narrow ones, where a 64-tile list leaves most SMs idle
+// (256 features: 10 tiles, 140 us at 1024 rows).
 constexpr int HK = 16;   // rows of X per stage
 
-template <typename T>
-__global__ void __launch_bounds__(256) hessian_simt_kernel(const T* __restrict__ X, long long n, long long d_in,
-                                                           long long ldx, int accumulate, float* __restrict__ H) {
+template <typename TX, int T, int M>
+__global__ void __launch_bounds__((T / M) * (T / M)) hessian_simt_kernel(const TX* __restrict__ X, long long n, long long d_in,
+                                                                         long long ldx, int accumulate, float* __restrict__ H) {
   // Only tiles on or below the diagonal are computed; the mirror image is written too.
   const int tp = blockIdx.y, tr = blockIdx.x;
   if (tr > tp) return;
-  __shared__ float sa[HK][HT + 4];
-  __shared__ float sb[HK][HT + 4];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const long long p0 = (long long)tp * HT, r0 = (long long)tr * HT;
-  double acc[4][4];
+  constexpr int TT = T / M, NTH = TT * TT, LD = HK * T / NTH;
+  __shared__ __align__(16) double sa[HK][T + 2];
+  __shared__ __align__(16) double sb[HK][T + 2];
+  const int tx = threadIdx.x % TT, ty = threadIdx.x / TT;
+  const long long p0 = (long long)tp * T, r0 = (long long)tr * T;
+  double acc[M][M];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < M; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-  for (long long k0 = 0; k0 < n; k0 += HK) {
-    for (int e = threadIdx.x; e < HK * HT; e += 256) {
-      const int kk = e / HT, cc = e % HT;
+    for (int b = 0; b < M; ++b) acc[a][b] = 0.0;
+  TX xa[LD], xb[LD];
+  auto fetch = [&](long long k0) {
+#pragma unroll
+    for (int e = 0; e < LD; ++e) {
+      const int idx = threadIdx.x + e * NTH, kk = idx / T, cc = idx % T;
       const long long k = k0 + kk;
-      float va = 0.f, vb = 0.f;
-      if (k < n) {
-        if (p0 + cc < d_in) va = (float)ld_as_double(X, k * ldx + p0 + cc);
-        if (r0 + cc < d_in) vb = (float)ld_as_double(X, k * ldx + r0 + cc);
-      }
-      sa[kk][cc] = va;
-      sb[kk][cc] = vb;
+      xa[e] = (k < n && p0 + cc < d_in) ? X[k * ldx + p0 + cc] : TX(0.f);
+      xb[e] = (k < n && r0 + cc < d_in) ? X[k * ldx + r0 + cc] : TX(0.f);
+    }
+  };
+  fetch(0);
+  for (long long k0 = 0; k0 < n; k0 += HK) {
+#pragma unroll
+    for (int e = 0; e < LD; ++e) {
+      const int idx = threadIdx.x + e * NTH, kk = idx / T, cc = idx % T;
+      sa[kk][cc] = (double)(float)xa[e];
+      sb[kk][cc] = (double)(float)xb[e];
     }
     __syncthreads();
+    if (k0 + HK < n) fetch(k0 + HK);
 #pragma unroll
     for (int kk = 0; kk < HK; ++kk) {
-      double a[4], b[4];
+      double a[M], b[M];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { a[u] = (double)sa[kk][ty * 4 + u]; b[u] = (double)sb[kk][tx * 4 + u]; }
+      for (int u = 0; u < M; u += 2) {
+        // (a thread's entries are pairs of neighbours, so that the 16-byte loads of neighbouring threads are contiguous)
+        const double2 va = *reinterpret_cast<const double2*>(&sa[kk][u * TT + 2 * ty]);
+        const double2 vb = *reinterpret_cast<const double2*>(&sb[kk][u * TT + 2 * tx]);
+        a[u] = va.x; a[u + 1] = va.y; b[u] = vb.x; b[u + 1] = vb.y;
+      }
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < M; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+        for (int v = 0; v < M; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
+  for (int u = 0; u < M; ++u)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const long long p = p0 + ty * 4 + u, r = r0 + tx * 4 + v;
+    for (int v = 0; v < M; ++v) {
+      const long long p = p0 + (u & ~1) * TT + 2 * ty + (u & 1), r = r0 + (v & ~1) * TT + 2 * tx + (v & 1);
       if (p < d_in && r < d_in) {
-        if (tp == tr) {
-          // diagonal tile: every entry is computed directly, no mirroring
-          const float prev = accumulate ? H[p * d_in + r] : 0.f;
-          H[p * d_in + r] = (float)((double)prev + acc[u][v]);
-        } else {
-          const float prev = accumulate ? H[p * d_in + r] : 0.f;
-          const float val = (float)((double)prev + acc[u][v]);
-          H[p * d_in + r] = val;
-          H[r * d_in + p] = val;
-        }
+        const float prev = accumulate ? H[p * d_in + r] : 0.f;
+        const float val = (float)((double)prev + acc[u][v]);
+        H[p * d_in + r] = val;
+        if (tp != tr) H[r * d_in + p] = val;   // (a diagonal tile computes every entry directly)
       }
     }
 }
 
+template <int T, int M>
+static void run_hessian_simt(const void* X, cdq_dtype xt, long long n, long long d_in, long long ldx, int accumulate,
+                             float* H, cudaStream_t st) {
+  const unsigned t = (unsigned)((d_in + T - 1) / T);
+  dim3 grid(t, t), block((T / M) * (T / M));
+  if (xt == CDQ_BF16)
+    { hessian_simt_kernel<__nv_bfloat16, T, M><<<grid, block, 0, st>>>((const __nv_bfloat16*)X, n, d_in, ldx, accumulate, H); count_launch(); }
+  else
+    { hessian_simt_kernel<float, T, M><<<grid, block, 0, st>>>((const float*)X, n, d_in, ldx, accumulate, H); count_launch(); }
+}
+
 cudaError_t launch_hessian_simt(const void* X, cdq_dtype xt, long long n, long long d_in, long long ldx,
                                 int accumulate, float* H, cudaStream_t st) {
-  const unsigned t = (unsigned)((d_in + HT - 1) / HT);
-  dim3 grid(t, t), block(256);
-  if (xt == CDQ_BF16)
-    { hessian_simt_kernel<__nv_bfloat16><<<grid, block, 0, st>>>((const __nv_bfloat16*)X, n, d_in, ldx, accumulate, H); count_launch(); }
-  else
-    { hessian_simt_kernel<float><<<grid, block, 0, st>>>((const float*)X, n, d_in, ldx, accumulate, H); count_launch(); }
+  if (d_in <= 512) run_hessian_simt<16, 2>(X, xt, n, d_in, ldx, accumulate, H, st);
+  else if (d_in <= 1024) run_hessian_simt<32, 2>(X, xt, n, d_in, ldx, accumulate, H, st);
+  else run_hessian_simt<64, 4>(X, xt, n, d_in, ldx, accumulate, H, st);
   return cudaGetLastError();
 }
 
