@@ -64,6 +64,7 @@ size_t init_rtn_workspace(long long d_in, long long d_out, long long g, int n_cl
 cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* scale, float* zero,
                             unsigned char* Q, float* gamma_out, cdq_mode mode, void* ws, cudaStream_t st);
 
+long long minmax_chunks(long long g);   // partial minima per group and column that launch_group_minmax needs room for
 cudaError_t launch_group_minmax(const Layer& ly, float* pmn, float* pmx, float* mn, float* mx, cudaStream_t st);
 
 // owc_cd.cu : greedy descent over per-group clipping strengths (paper: Algorithm 3)

@@ -8,29 +8,63 @@
 
 namespace cdq {
 
-constexpr int kChunkRows = 256;  // rows of one min/max partial
+constexpr int kChunkRows = 128;  // rows of one min/max partial
 
-__global__ void minmax_partial_kernel(const void* __restrict__ W, cdq_dtype wt, long long d_in, long long d_out,
+// V neighbouring weights of one row as floats (V = 4: one 8- or 16-byte load).
+template <int V, bool BF16>
+__device__ __forceinline__ void load_weights(const void* __restrict__ W, long long idx, float (&w)[V]) {
+  if constexpr (V == 4 && BF16) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>((const __nv_bfloat16*)W + idx));
+    w[0] = __uint_as_float(u.x << 16); w[1] = __uint_as_float(u.x & 0xFFFF0000u);
+    w[2] = __uint_as_float(u.y << 16); w[3] = __uint_as_float(u.y & 0xFFFF0000u);
+  } else if constexpr (V == 4) {
+    const float4 f = __ldg(reinterpret_cast<const float4*>((const float*)W + idx));
+    w[0] = f.x; w[1] = f.y; w[2] = f.z; w[3] = f.w;
+  } else if constexpr (BF16) {
+    w[0] = __bfloat162float(((const __nv_bfloat16*)W)[idx]);
+  } else {
+    w[0] = ((const float*)W)[idx];
+  }
+}
+// Four columns per thread: rows of W, and of what is d_out wide, have to start on the vector's boundaries.
+static bool four_columns(const Layer& ly) {
+  const size_t esz = ly.wt == CDQ_BF16 ? 2 : 4;
+  return ly.d_out % 4 == 0 && ly.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(ly.W) % (4 * esz) == 0;
+}
+
+template <int V, bool BF16>
+__global__ void minmax_partial_kernel(const void* __restrict__ W, long long d_out,
                                       long long ldw, long long g, long long cpg, float* __restrict__ pmn,
                                       float* __restrict__ pmx) {
-  const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long j = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
   const long long chunk = blockIdx.y;  // global chunk id = t * cpg + c
   if (j >= d_out) return;
   const long long t = chunk / cpg, c = chunk % cpg;
   const long long i0 = t * g + c * kChunkRows;
   long long i1 = i0 + kChunkRows;
   if (i1 > (t + 1) * g) i1 = (t + 1) * g;
-  float mn = 0.f, mx = 0.f;
-  bool first = true;
-  for (long long i = i0; i < i1; ++i) {
-    float w;
-    if (wt == CDQ_BF16) w = __bfloat162float(((const __nv_bfloat16*)W)[i * ldw + j]);
-    else w = ((const float*)W)[i * ldw + j];
-    if (first) { mn = mx = w; first = false; }
-    else { mn = fminf(mn, w); mx = fmaxf(mx, w); }
+  float mn[V], mx[V];
+  load_weights<V, BF16>(W, i0 * ldw + j, mn);
+#pragma unroll
+  for (int v = 0; v < V; ++v) mx[v] = mn[v];
+#pragma unroll 16
+  for (long long i = i0 + 1; i < i1; ++i) {
+    float w[V];
+    load_weights<V, BF16>(W, i * ldw + j, w);
+#pragma unroll
+    for (int v = 0; v < V; ++v) { mn[v] = fminf(mn[v], w[v]); mx[v] = fmaxf(mx[v], w[v]); }
   }
-  pmn[chunk * d_out + j] = mn;
-  pmx[chunk * d_out + j] = mx;
+#pragma unroll
+  for (int v = 0; v < V; ++v) { pmn[chunk * d_out + j + v] = mn[v]; pmx[chunk * d_out + j + v] = mx[v]; }
+}
+static void run_minmax_partial(const Layer& ly, long long cpg, float* pmn, float* pmx, cudaStream_t st) {
+  // (narrow layers: a column per thread, or there are too few threads to hide the latency of the loads)
+  const int v = four_columns(ly) && ly.d_out * ly.ng * cpg >= (1 << 18) ? 4 : 1;
+  const dim3 grid((unsigned)((ly.d_out + 128 * v - 1) / (128 * v)), (unsigned)(ly.ng * cpg));
+  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(ly.W, ly.d_out, ly.ldw, ly.g, cpg, pmn, pmx); };
+  if (ly.wt == CDQ_BF16) run(v == 4 ? minmax_partial_kernel<4, true> : minmax_partial_kernel<1, true>);
+  else run(v == 4 ? minmax_partial_kernel<4, false> : minmax_partial_kernel<1, false>);
+  count_launch();
 }
 
 __global__ void minmax_final_kernel(const float* __restrict__ pmn, const float* __restrict__ pmx, long long ng,
@@ -62,23 +96,50 @@ __global__ void scale_zero_kernel(const float* __restrict__ mn, const float* __r
   zero[t * d_out + j] = (float)lo;
 }
 
-__global__ void rtn_codes_kernel(const void* __restrict__ W, cdq_dtype wt, long long d_in, long long d_out,
-                                 long long ldw, long long g, int L, const float* __restrict__ scale,
-                                 const float* __restrict__ zero, unsigned char* __restrict__ Q) {
-  const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long i = blockIdx.y;
-  if (j >= d_out) return;
-  const float a32 = scale[(i / g) * d_out + j];
-  unsigned char q = 0;
-  if (a32 > 0.f) {
-    const double a = (double)a32, b = (double)zero[(i / g) * d_out + j];
-    const double w = load_w(W, wt, i * ldw + j);
-    double r = rint(__ddiv_rn(__dadd_rn(w, -b), a));
-    r = r < 0.0 ? 0.0 : r;
-    r = r > (double)L ? (double)L : r;
-    q = (unsigned char)r;
+// Codes of kCodeRows rows of one group by V columns per thread.  The code is the fp64 rounding of (w - b) / a.  The fp32
+// quotient is off by at most 3 * 2^-24 of itself, 5e-5 where it is within 256 levels, so unless it lies within 2e-4 of
+// the middle between two levels both round to the same level; the one in 2500 that does is decided in fp64.  (Memory-bound that way: 14336 x 16384 bf16 weights took 1180 us with an fp64 division and one byte per thread.)
+constexpr int kCodeRows = 16;
+__device__ __forceinline__ unsigned rtn_code(float w, float a, float inv_a, float b, float top) {
+  constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer, to the even one in the middle
+  const float t = (w - b) * inv_a;
+  const float c = fminf(fmaxf(t, 0.f), top);
+  const float m = c + kMagic;
+  if (!(fabsf(c - (m - kMagic)) < 0.4998f) || t != t) {
+    double q = rint(__ddiv_rn(__dadd_rn((double)w, -(double)b), (double)a));
+    q = q < 0.0 ? 0.0 : q;
+    q = q > (double)top ? (double)top : q;
+    return (unsigned)(unsigned char)q;
   }
-  Q[i * d_out + j] = q;
+  return __float_as_uint(m) & 255u;
+}
+template <int V, bool BF16>
+__global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__ W, long long d_out,
+                                                        long long ldw, long long g, int blocks_per_group, int L,
+                                                        const float* __restrict__ scale, const float* __restrict__ zero,
+                                                        unsigned char* __restrict__ Q) {
+  const long long j = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
+  if (j >= d_out) return;
+  const long long t = blockIdx.y / blocks_per_group, i0 = t * g + (blockIdx.y % blocks_per_group) * (long long)kCodeRows;
+  const long long i1 = min(i0 + kCodeRows, (t + 1) * g);
+  float a[V], b[V], inv[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    a[v] = scale[t * d_out + j + v];
+    b[v] = zero[t * d_out + j + v];
+    inv[v] = 1.0f / a[v];
+    if (!(inv[v] <= 3.4e38f)) inv[v] = __int_as_float(0x7FFFFFFF);   // a subnormal scale: decided in fp64
+  }
+#pragma unroll 4
+  for (long long i = i0; i < i1; ++i) {
+    float w[V];
+    load_weights<V, BF16>(W, i * ldw + j, w);
+    unsigned q = 0u;
+#pragma unroll
+    for (int v = 0; v < V; ++v) q |= (a[v] > 0.f ? rtn_code(w[v], a[v], inv[v], b[v], (float)L) : 0u) << (8 * v);
+    if constexpr (V == 4) *reinterpret_cast<unsigned*>(Q + i * d_out + j) = q;
+    else Q[i * d_out + j] = (unsigned char)q;
+  }
 }
 
 // Residual E[i][j] = (a q + b) - w in fp64, either from stored codes or, for the OWC search,
@@ -229,12 +290,13 @@ __global__ void fill_gamma_kernel(float* gamma_out, long long d_out) {
   if (j < d_out) gamma_out[j] = 1.0f;
 }
 
-// Group minima and maxima of every column: mn, mx [ng, d_out]; pmn, pmx [ng * ceil(g / 256), d_out] scratch.
+long long minmax_chunks(long long g) { return (g + kChunkRows - 1) / kChunkRows; }
+
+// Group minima and maxima of every column: mn, mx [ng, d_out]; pmn, pmx [ng * minmax_chunks(g), d_out] scratch.
 cudaError_t launch_group_minmax(const Layer& ly, float* pmn, float* pmx, float* mn, float* mx, cudaStream_t st) {
-  const long long cpg = (ly.g + kChunkRows - 1) / kChunkRows;
+  const long long cpg = minmax_chunks(ly.g);
   const unsigned bx = (unsigned)((ly.d_out + 127) / 128);
-  { minmax_partial_kernel<<<dim3(bx, (unsigned)(ly.ng * cpg)), 128, 0, st>>>(ly.W, ly.wt, ly.d_in, ly.d_out, ly.ldw, ly.g,
-                                                                            cpg, pmn, pmx); count_launch(); }
+  run_minmax_partial(ly, cpg, pmn, pmx, st);
   { minmax_final_kernel<<<dim3(bx, (unsigned)ly.ng), 128, 0, st>>>(pmn, pmx, ly.ng, ly.d_out, cpg, mn, mx); count_launch(); }
   return cudaGetLastError();
 }
@@ -254,7 +316,7 @@ struct InitWs {
 static InitWs init_ws_layout(long long d_in, long long d_out, long long g, int n_clip, cdq_mode mode) {
   InitWs w{};
   const long long ng = d_in / g;
-  const long long cpg = (g + kChunkRows - 1) / kChunkRows;
+  const long long cpg = minmax_chunks(g);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   w.pmn = take(sizeof(float) * ng * cpg * d_out);
@@ -302,7 +364,7 @@ size_t init_rtn_workspace(long long d_in, long long d_out, long long g, int n_cl
 cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* scale, float* zero,
                             unsigned char* Q, float* gamma_out, cdq_mode mode, void* ws, cudaStream_t st) {
   const long long d_in = ly.d_in, d_out = ly.d_out, g = ly.g, ng = ly.ng;
-  const long long cpg = (g + kChunkRows - 1) / kChunkRows;
+  const long long cpg = minmax_chunks(g);
   const int n_clip = grid.n_clip > 1 ? grid.n_clip : 1;
   const InitWs L = init_ws_layout(d_in, d_out, g, n_clip, mode);
   char* base = (char*)ws;
@@ -312,8 +374,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
   float* mx = (float*)(base + L.mx);
   const unsigned bx = (unsigned)((d_out + 127) / 128);
 
-  { minmax_partial_kernel<<<dim3(bx, (unsigned)(ng * cpg)), 128, 0, st>>>(ly.W, ly.wt, d_in, d_out, ly.ldw, g, cpg,
-                                                                         pmn, pmx); count_launch(); }
+  run_minmax_partial(ly, cpg, pmn, pmx, st);
   { minmax_final_kernel<<<dim3(bx, (unsigned)ng), 128, 0, st>>>(pmn, pmx, ng, d_out, cpg, mn, mx); count_launch(); }
 
   const double* gam_col = nullptr;
@@ -408,7 +469,12 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
     { fill_gamma_kernel<<<bx, 128, 0, st>>>(gamma_out, d_out); count_launch(); }
   }
   { scale_zero_kernel<<<dim3(bx, (unsigned)ng), 128, 0, st>>>(mn, mx, ng, d_out, ly.L, gam_col, scale, zero); count_launch(); }
-  { rtn_codes_kernel<<<dim3(bx, (unsigned)d_in), 128, 0, st>>>(ly.W, ly.wt, d_in, d_out, ly.ldw, g, ly.L, scale, zero, Q); count_launch(); }
+  const int bpg = (int)((g + kCodeRows - 1) / kCodeRows);
+  const bool four = four_columns(ly) && reinterpret_cast<uintptr_t>(Q) % 4 == 0 && d_out * ng * bpg >= (1 << 18);
+  const dim3 grid_q((unsigned)(four ? (d_out + 511) / 512 : bx), (unsigned)(ng * bpg));
+  auto run = [&](auto kern) { kern<<<grid_q, 128, 0, st>>>(ly.W, d_out, ly.ldw, g, bpg, ly.L, scale, zero, Q); count_launch(); };
+  if (ly.wt == CDQ_BF16) run(four ? rtn_codes_kernel<4, true> : rtn_codes_kernel<1, true>);
+  else run(four ? rtn_codes_kernel<4, false> : rtn_codes_kernel<1, false>);
   return cudaGetLastError();
 }
 

@@ -371,7 +371,7 @@ struct OwcWs {
 static OwcWs owc_ws_layout(long long d_in, long long d_out, long long g, int nk, cdq_mode mode) {
   OwcWs w{};
   const long long ng = d_in / g;
-  w.cpg = (g + 255) / 256;
+  w.cpg = minmax_chunks(g);
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   w.pmn = take(sizeof(float) * ng * w.cpg * d_out);
