@@ -92,7 +92,9 @@ SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool wit
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   w.ldg = (d_in + 3) / 4 * 4;
   w.d_pad = cd_fast_pad(d_in);
-  w.tc = mode == CDQ_MODE_FAST && gemm_tc_supported(d_in, d_out);
+  // On small layers (256 x 256: 2 tiles) the int8 product's 27 slice pairs are one long chain on a few SMs: 177 us and 30 us
+  // for the slices, against 47 us for the fp64 product; the two meet between 5e8 and 1e9 multiplications.
+  w.tc = mode == CDQ_MODE_FAST && gemm_tc_supported(d_in, d_out) && d_in * d_in * d_out >= 400000000ll;
   // the loss of a descended solution is a sum with heavy cancellation (the descent tunes e against the
   // large entries of H): it takes the same slice depth as the gradient; the shallower setting serves
   // the OWC search, whose residuals are plain rounding errors
