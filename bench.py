@@ -50,7 +50,9 @@ NCU_TRAFFIC_PER_MOVE: dict = {
 def descent_kernel_name(cfg, block: int) -> str:
     if block == 2:
         return "bcd2_kernel"
-    return "cd_tma_kernel" if cfg.d_in > 1536 and cfg.d_in % 4 == 0 else "cd_fast_kernel"
+    if cfg.d_in > 8192:
+        return "cd_ahead_kernel"
+    return "cd_tma_kernel" if cfg.d_in > 1536 else "cd_fast_kernel"
 
 
 def load_peaks():

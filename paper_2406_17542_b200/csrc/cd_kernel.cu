@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
   const int lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
   const long long d_in = p.d_in;
   const int nchunks = (int)((d_in + 3) >> 2);
-  const bool vec = EXACT || (d_in & 3) == 0;
   const float top = kMagic + (float)p.L;
 
   auto group_of = [&](unsigned i) -> unsigned { return p.g == 1 ? i : __umulhi(i, p.gmagic); };
@@ -215,16 +214,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
         if (EXACT) row[k] = ld_row4(rp + (long long)chunk * 4);
         else {
           row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (chunk < nchunks) {
-            if (vec) row[k] = ld_row4(rp + (long long)chunk * 4);
-            else {
-              const long long i0 = (long long)chunk * 4;
-              row[k].x = rp[i0];
-              if (i0 + 1 < d_in) row[k].y = rp[i0 + 1];
-              if (i0 + 2 < d_in) row[k].z = rp[i0 + 2];
-              if (i0 + 3 < d_in) row[k].w = rp[i0 + 3];
-            }
-          }
+          if (chunk < nchunks) row[k] = ld_row4(rp + (long long)chunk * 4);
         }
       }
       SweepBest sb;
@@ -275,7 +265,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
       float astar = 1.f;
       if (SMODE != kPerChannel) astar = ag_s[group_of((unsigned)istar)].x;
       c2 = 2.0 * ((double)astar * (double)dri);
-      rp = p.H + (long long)istar * d_in;
+      rp = p.H + (long long)istar * p.ldh;
       if (tid == 0) col_dsum += (double)__uint_as_float(~m);
       ++step;
     }
@@ -386,11 +376,22 @@ cudaError_t launch_round_rows_bf16(const float* H, long long d_in, __nv_bfloat16
   return cudaGetLastError();
 }
 
-cudaError_t launch_cd_fast(const Layer& ly, const __nv_bfloat16* H16, double* G, long long ldg, unsigned char* Qt,
+// Rows of H on 16-byte boundaries: a copy with the row stride ldh, a multiple of 4, and zeros past d_in.
+__global__ void pad_rows_kernel(const float* __restrict__ H, long long d_in, long long ldh, float* __restrict__ out) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x, r = blockIdx.y;
+  if (c < ldh) out[r * ldh + c] = c < d_in ? H[r * d_in + c] : 0.f;
+}
+
+cudaError_t launch_pad_rows(const float* H, long long d_in, long long ldh, float* out, cudaStream_t st) {
+  { pad_rows_kernel<<<dim3((unsigned)((ldh + 255) / 256), (unsigned)d_in), 256, 0, st>>>(H, d_in, ldh, out); count_launch(); }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, const __nv_bfloat16* H16, double* G, long long ldg, unsigned char* Qt,
                            long long ldq, const float* hdiag, const float* hs, long long steps_per_col,
                            CdCounters* ctr, cudaStream_t st) {
   CdParams p{};
-  p.H = ly.H; p.H16 = H16; p.d_in = ly.d_in; p.d_out = ly.d_out; p.G = G; p.ldg = ldg; p.Qt = Qt; p.ldq = ldq; p.scale = ly.scale;
+  p.H = rows; p.ldh = ldh; p.H16 = H16; p.d_in = ly.d_in; p.d_out = ly.d_out; p.G = G; p.ldg = ldg; p.Qt = Qt; p.ldq = ldq; p.scale = ly.scale;
   p.hdiag = hdiag; p.hs = hs; p.g = ly.g; p.ng = ly.ng; p.L = ly.L; p.T = steps_per_col; p.ctr = ctr;
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;
@@ -398,18 +399,14 @@ cudaError_t launch_cd_fast(const Layer& ly, const __nv_bfloat16* H16, double* G,
   const long long d = ly.d_in;
   if (steps_per_col <= 0) return cudaSuccess;   // nothing to do: the counters stay zero, the codes untouched
   // short rows are quickest as plain loads into registers, longer ones as bulk copies into shared memory
-  // (measured crossover: 1536 entries 2.0 against 2.5 ms, 1792 entries 11.5 against 10.8, 2048 entries 52.0 against 45.3)
-  if (d > 1536) {
-    const cudaError_t e = launch_cd_tma(p, st);
-    if (e != cudaErrorNotSupported) return e;
-  }
+  // (measured crossover: 1536 entries 2.0 against 2.5 ms, 1792 entries 11.5 against 10.8, 2048 entries 52.0 against 45.3);
+  // from 8192 entries on, where one team fills an SM, the next row travels during the sweep (see cd_kernel_ahead.cu)
+  if (d > 8192) return launch_cd_ahead(p, st);
+  if (d > 1536) return launch_cd_tma(p, st);
   if (H16) return cudaErrorNotSupported;
   auto team = [&](int ept) { return (int)(((d + ept - 1) / ept + 31) / 32 * 32); };
   if (d <= 512) return launch_cd_shape<2, 64, 8>(p, team(8), st);
-  if (d <= 4096) return launch_cd_shape<4, 256, 3>(p, team(16), st);
-  if (d <= 8192) return launch_cd_shape<8, 256, 2>(p, team(32), st);
-  if (d <= 14336) return launch_cd_shape<8, 448, 1>(p, team(32), st);
-  return launch_cd_shape<8, 576, 1>(p, team(32), st);
+  return launch_cd_shape<4, 256, 3>(p, team(16), st);
 }
 
 // ---------------------------------------------------------------------------

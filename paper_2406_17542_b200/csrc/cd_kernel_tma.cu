@@ -1,6 +1,5 @@
 // Greedy coordinate descent (paper: the loop of Algorithm 1; Algorithm 4 for sub-channel
-// grids), the variant for rows of H that have to come from HBM (large d_in) and are 16-byte
-// aligned (d_in % 4 == 0).
+// grids), the variant for rows of H of 1537 to 8192 entries, on 16-byte boundaries (longer rows: cd_kernel_ahead.cu).
 //
 // Same step as cd_kernel.cu -- score, argmin, read row i*, update the gradient -- but the row
 // H[i*, :] is fetched by one bulk asynchronous copy (cp.async.bulk, no multicast) into shared
@@ -35,7 +34,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_tma_kernel(CdParams p) {
 
   const int tid = threadIdx.x, NT = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
-  const int nchs = (int)(p.d_in >> 2);         // chunks of a row
+  const int nchs = (int)((p.d_in + 3) >> 2);         // chunks of a row
   const bool exact = nchs == NT * NCH;
   const float top = kMagic + (float)p.L;
 
@@ -43,7 +42,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_tma_kernel(CdParams p) {
   // H_ii and 0.5 / H_ii of the team's chunk slots sit in shared memory too: they are the same for every column and
   // every sweep reads them (8 d_in bytes); from L1 they cost more latency, and beside the row buffer of the longest
   // rows the L1 does not hold them.  (148 to 1184 columns, before -> after: 2048 entries 12.4 -> 10.6 ms, 6144
-  // 23.4 -> 19.4, 8192 42.1 -> 36.8, 14336 163.7 -> 160.1, 18432 67.5 -> 60.4.)
+  // 23.4 -> 19.4, 8192 42.1 -> 36.8.)
   unsigned char* row_s = dyn_smem;                                      // [NCH * NT] chunks
   float4* hd_s = reinterpret_cast<float4*>(row_s + (size_t)NCH * NT * CHB);   // [NCH * NT] H_ii
   float4* hs_s = hd_s + NCH * NT;                                             // [NCH * NT] 0.5 / H_ii
@@ -131,13 +130,13 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_tma_kernel(CdParams p) {
     double c2 = 0.0;       // twice the step being applied (code units when per-channel)
     double col_dsum = 0.0;
     bool done = frozen;
-    // Requests row `off / d_in` of H.  Called when every thread is past its reads of the previous row (behind the
+    // Requests row `off` of H.  Called when every thread is past its reads of the previous row (behind the
     // barrier of the argmin, or of the column prologue), and as early as the row is known: what follows the argmin
     // overlaps with the copy.
     auto request_row = [&](long long off) {
       if (tid == 0) {
-        const unsigned char* src = ROW16 ? reinterpret_cast<const unsigned char*>(p.H16 + off)
-                                         : reinterpret_cast<const unsigned char*>(p.H + off);
+        const unsigned char* src = ROW16 ? reinterpret_cast<const unsigned char*>(p.H16 + off * p.d_in)
+                                         : reinterpret_cast<const unsigned char*>(p.H + off * p.ldh);
         mbar_expect_tx(smem_u32(&s_bar), row_bytes);
         bulk_load(smem_u32(row_s), src, row_bytes, smem_u32(&s_bar));
       }
@@ -209,7 +208,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_tma_kernel(CdParams p) {
         if (tid == 0) atomicExch(p.status, (int)kFlagBadIndex);
         istar = 0;
       }
-      request_row((long long)istar * p.d_in);
+      request_row(istar);
       if constexpr (ROW16) { fix_diag = tid == tstar; kprev = kstar; vprev = vstar; }
       if (tid == tstar) {
         const unsigned dq = (unsigned)dri << (8 * vstar);
@@ -310,32 +309,14 @@ cudaError_t launch_mode(const CdParams& p, int nt, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_cd_tma(const CdParams& p, cudaStream_t st) {
-  if (p.d_in & 3) return cudaErrorNotSupported;
+  if (p.ldh & 3) return cudaErrorNotSupported;
   if ((reinterpret_cast<uintptr_t>(p.H) & 15) != 0) return cudaErrorNotSupported;
   if (p.H16 && ((p.d_in & 7) != 0 || (reinterpret_cast<uintptr_t>(p.H16) & 15) != 0)) return cudaErrorNotSupported;
-  const long long ch = p.d_in >> 2;
+  const long long ch = (p.d_in + 3) >> 2;
   auto team = [&](long long chunks, int nch) { return (int)((chunks + nch - 1) / nch + 31) / 32 * 32; };
   // (called for rows of more than 1536 entries)  Rows up to 8192 entries: several teams per SM.
   if (ch <= 1024) return launch_mode<8, 128, 4>(p, team(ch, 8), st);
   if (ch <= 2048) return launch_mode<8, 256, 2>(p, team(ch, 8), st);
-  // Longer rows: one team per SM.  Few threads with many chunks each beat many threads with few (no spills, a
-  // cheaper argmin exchange, fixed costs per thread spread over more state), and a team of full warps in equal
-  // numbers per scheduler beats a ragged one.  With H_ii and 0.5 / H_ii in shared memory eight warps hide the
-  // latencies that are left, so rows up to 14336 entries take 256 threads with 9 to 14 chunks each; beyond that the
-  // registers of a 256-thread team run out (15 and 16 chunks measured 3 % slower, 18 chunks 15 %) and the team is the
-  // smallest of 10..12 x 384 and 8 x 512 chunk slots that holds the row.  Cycles per move and SM against the
-  // 4 x 896 / 6 x 768 teams of an earlier version, which also read the tables through L1: d_in 10240 4049 (4813),
-  // 11008 4038 (5079), 14336 4892 (5903), 15360 5531 (7482), 16384 5879 (8022), 18432 6416 (8418).
-  if (ch <= 2304) return launch_mode<9, 256, 1>(p, team(ch, 9), st);
-  if (ch <= 2560) return launch_mode<10, 256, 1>(p, team(ch, 10), st);
-  if (ch <= 2816) return launch_mode<11, 256, 1>(p, team(ch, 11), st);
-  if (ch <= 3072) return launch_mode<12, 256, 1>(p, team(ch, 12), st);
-  if (ch <= 3328) return launch_mode<13, 256, 1>(p, team(ch, 13), st);
-  if (ch <= 3584) return launch_mode<14, 256, 1>(p, team(ch, 14), st);
-  if (ch <= 3840) return launch_mode<10, 384, 1>(p, team(ch, 10), st);
-  if (ch <= 4096) return launch_mode<8, 512, 1>(p, team(ch, 8), st);
-  if (ch <= 4224) return launch_mode<11, 384, 1>(p, team(ch, 11), st);
-  if (ch <= 4608) return launch_mode<12, 384, 1>(p, team(ch, 12), st);
   return cudaErrorNotSupported;
 }
 

@@ -7,6 +7,7 @@ namespace cdq {
 
 struct CdParams {
   const float* H;
+  long long ldh;              // row stride of H, a multiple of 4 (the entries past d_in are zero)
   const __nv_bfloat16* H16;   // bf16 copy of H for the rows of the update (NULL: fp32 rows)
   long long d_in, d_out;
   double* G;            // [d_out, ldg]
@@ -49,5 +50,7 @@ inline int cd_scale_mode(const CdParams& p, int nt) {
 // cudaErrorNotSupported when the shape has no such configuration (the caller then uses the
 // plain kernel).
 cudaError_t launch_cd_tma(const CdParams& p, cudaStream_t st);
+// cd_kernel_ahead.cu: the same for rows of more than 8192 entries, with the next row in flight during the sweep.
+cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st);
 
 }  // namespace cdq

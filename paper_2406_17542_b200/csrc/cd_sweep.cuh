@@ -20,31 +20,39 @@ struct SweepBest {
   __device__ __forceinline__ int dr() const { const int ipk = (int)bpk; return ipk - (((ipk + 512) >> 10) << 10); }
 };
 
-// Applies g += c2 * h to the 4 coordinates of chunk slot k and folds their best moves into the
-// thread's running best.  qpk: the 4 codes, packed; hd4: H_ii; hs4: 0.5 / H_ii; a, ia: scale of
-// the chunk and its reciprocal (grouped modes; per-channel columns run in code units, a == 1);
-// top = kMagic + L.
-template <int SMODE>
-__device__ __forceinline__ void sweep_chunk(double (&gk)[4], const float4 rv, const float4 hd4, const float4 hs4,
-                                            unsigned qpk, double c2, float a, float ia, float top, int k,
-                                            SweepBest& sb) {
-  const float hv[4] = {rv.x, rv.y, rv.z, rv.w};
+// Folds the best moves of the 4 coordinates of chunk slot k, whose gradients are gk, into the thread's running best.
+// qpk: the 4 codes, packed; hd4: H_ii; hs4: 0.5 / H_ii; a, ia: scale of the chunk and its reciprocal (grouped grids;
+// per-channel columns run in code units, a == 1); top = kMagic + L.
+template <bool GROUPED>
+__device__ __forceinline__ void score_chunk(const double (&gk)[4], const float4 hd4, const float4 hs4, unsigned qpk, float a,
+                                            float ia, float top, int k, SweepBest& sb) {
   const float hdv[4] = {hd4.x, hd4.y, hd4.z, hd4.w};
   const float hsv[4] = {hs4.x, hs4.y, hs4.z, hs4.w};
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    gk[v] = fma(c2, (double)hv[v], gk[v]);
     const float gf = (float)gk[v];
     // kMagic + q: a float whose unit in the last place is 1, so the fused multiply-add below
     // rounds the vertex to a level
     const float qmf = __uint_as_float(__byte_perm(qpk, kMagicBits, 0x7650 | v));
-    float t = fmaf(-gf, SMODE == kPerChannel ? hsv[v] : ia * hsv[v], qmf);
+    float t = fmaf(-gf, GROUPED ? ia * hsv[v] : hsv[v], qmf);
     t = fminf(fmaxf(t, kMagic), top);                    // clamped to the grid
     const float dr = t - qmf;
-    const float d = SMODE == kPerChannel ? dr : a * dr;
+    const float d = GROUPED ? a * dr : dr;
     const float dl = fmaf(d, hdv[v], gf) * d;            // change of the loss
     if (dl < sb.best) { sb.best = dl; sb.bpk = dr + (float)((4 * k + v) * 1024); }
   }
+}
+
+// Applies g += c2 * h to the 4 coordinates of chunk slot k, then scores them.
+template <int SMODE>
+__device__ __forceinline__ void sweep_chunk(double (&gk)[4], const float4 rv, const float4 hd4, const float4 hs4,
+                                            unsigned qpk, double c2, float a, float ia, float top, int k,
+                                            SweepBest& sb) {
+  gk[0] = fma(c2, (double)rv.x, gk[0]);
+  gk[1] = fma(c2, (double)rv.y, gk[1]);
+  gk[2] = fma(c2, (double)rv.z, gk[2]);
+  gk[3] = fma(c2, (double)rv.w, gk[3]);
+  score_chunk<SMODE != kPerChannel>(gk, hd4, hs4, qpk, a, ia, top, k, sb);
 }
 
 // The thread's candidate for the team-wide argmin: key orders by decrease (the complement of a

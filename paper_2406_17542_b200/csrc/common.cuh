@@ -130,8 +130,10 @@ cudaError_t launch_diag(const float* H, long long d_in, long long d_pad, float* 
 // col_loss[j] = 1/2 sum_i E[i][j] G[j][i] (E [d_in, d_out], G [d_out, ldg]): e^T H e from the gradient g = 2 H e.
 cudaError_t launch_loss_from_gradient(const double* E, const double* G, long long ldg, long long d_in, long long d_out,
                                       double* col_loss, cudaStream_t st);
-// H16 (may be NULL): bf16 copy of H for the rows of the update; cudaErrorNotSupported if the shape has no such kernel
-cudaError_t launch_cd_fast(const Layer& ly, const __nv_bfloat16* H16, double* G, long long ldg, unsigned char* Qt,
+// rows: H with the row stride ldh, a multiple of 4 (zeros past d_in); when d_in is not one, the entries of G and Qt past
+// d_in are zero too.  H16 (may be NULL): bf16 copy of H for the rows of the update; cudaErrorNotSupported if the shape has no such kernel
+cudaError_t launch_pad_rows(const float* H, long long d_in, long long ldh, float* out, cudaStream_t st);
+cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, const __nv_bfloat16* H16, double* G, long long ldg, unsigned char* Qt,
                            long long ldq, const float* hdiag, const float* hs, long long steps_per_col,
                            CdCounters* ctr, cudaStream_t st);
 bool cd_rows16_supported(long long d_in, long long g);   // shapes whose descent can read bf16 rows

@@ -1,0 +1,128 @@
+"""Kernels at the edges of their tiles, teams and dispatch rules: odd row lengths, rows that need a padded copy, tiny
+budgets, one-bit and eight-bit grids, weights in the middle between two levels."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2406_17542_b200 import binding as B
+from paper_2406_17542_b200 import inputs
+from tests.util import compare_with_oracle, grid_of
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _layer_h(cfg, rows):
+    X = inputs.make_x(cfg.scaled(n=rows), device=DEV).double()
+    H = X.T @ X
+    H.diagonal().add_(1e-2 * H.diagonal().mean())
+    return H.float()
+
+
+# (d_in, d_out, bits, group, steps): rows just past 8192 entries, odd ones, one level of room, 256 levels, many small
+# groups, a full and a ragged team of every width; budgets long enough for thresholds to be drawn anew many times
+@pytest.mark.parametrize("d_in,d_out,bits,g,steps", [
+    (8196, 5, 1, 0, 400), (8193, 4, 3, 0, 300), (8200, 4, 8, 40, 60), (9216, 4, 2, 4, 400), (8960, 5, 2, 128, 700),
+    (14336, 4, 4, 0, 900), (15362, 3, 3, 0, 200), (18432, 3, 3, 128, 500), (8704, 4, 4, 0, 1), (8704, 4, 4, 0, 2),
+    # shorter rows that are not a multiple of four: the padded copy, for both of their kernels
+    (1023, 9, 3, 0, 900), (1350, 9, 4, 0, 900), (1537, 9, 2, 0, 900), (2050, 9, 3, 0, 900), (5001, 5, 3, 0, 400),
+])
+def test_descent_at_the_edges(d_in, d_out, bits, g, steps):
+    cfg = inputs.CONFIGS["C1"].scaled(d_in=d_in, d_out=d_out, bits=bits, group_size=g, x_dtype="bf16", w_dtype="f32",
+                                      seed=700 + d_in % 89)
+    H = _layer_h(cfg, 768)
+    W = inputs.make_w(cfg, device=DEV)
+    W[:, 1] = 0.0123                        # a column without room anywhere
+    H[7, :] = 0.0
+    H[:, 7] = 0.0                           # a dead feature
+    grid = grid_of(cfg)
+    scale, zero, Q0, gamma = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    stats, loss, per = B.cdq_cd_solve_with_loss(H, W, grid, scale, zero, Q, steps, per_col=True)
+    assert B.load().cdq_last_device_status() == 0
+    assert stats["steps"] == steps * d_out and stats["committed"] <= steps * (d_out - 1)
+    assert torch.equal(Q[:, 1], Q0[:, 1]) and torch.equal(Q[7], Q0[7])
+    keep = np.array([c for c in range(d_out) if c != 1])     # (the oracle's audit needs columns that can move)
+    compare_with_oracle(cfg, H.cpu().numpy(), H, W, keep, grid, scale, zero, Q0, Q, gamma, per, steps,
+                        label=f"d_in={d_in} bits={bits} g={g} steps={steps}")
+
+
+def test_descent_result_does_not_depend_on_the_other_columns():
+    """Columns share a team one after the other, thresholds and watched coordinates included: any subset of the
+    columns gives the codes of the whole."""
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=8320, d_out=301, bits=3, group_size=64, seed=41)
+    H = _layer_h(cfg, 768)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q0, _ = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    B.cdq_cd_solve(H, W, grid, scale, zero, Q, 0, steps_per_col=600)
+    some = torch.arange(3, 301, 13, device=DEV)
+    Qs = Q0[:, some].contiguous()
+    B.cdq_cd_solve(H, W[:, some].contiguous(), grid, scale[:, some].contiguous(), zero[:, some].contiguous(), Qs, 0,
+                   steps_per_col=600)
+    assert torch.equal(Qs, Q[:, some])
+
+
+@pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
+def test_hessian_pieces_and_mirror(d_in, width):
+    """bf16 rows with a stride longer than d_in through the tensor-core kernel: every entry against fp64 (3e-5 of
+    sqrt(H_ii H_jj), the bar of the tensor-core path for up to 4096 rows), symmetric bit for bit, accumulated too."""
+    g = torch.Generator(device=DEV).manual_seed(d_in)
+    X = torch.randn((1536, width), generator=g, device=DEV).bfloat16()
+    Xv = X[:, :d_in]
+    H = B.cdq_hessian(Xv)
+    D = Xv.double()
+    want = D.T @ D
+    norm = torch.sqrt(torch.outer(want.diagonal(), want.diagonal()))
+    assert float(((H.double() - want).abs() / norm).max()) <= 3e-5
+    assert torch.equal(H, H.T.contiguous())
+    H2 = B.cdq_hessian(Xv, accumulate=True, out=H.clone())
+    assert torch.equal(H2, 2 * H)           # the second sum is the same, and doubling is exact
+
+
+@pytest.mark.parametrize("d_in", [1, 15, 16, 17, 33, 255, 511, 512, 513, 577, 1023, 1024, 1025, 1091])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_hessian_on_the_cuda_cores(d_in, dtype):
+    """Every tile size with odd edges, rows not a multiple of a stage, accumulated: fp64 sums rounded once to fp32,
+    so within half a unit in the last place (6e-8) of the exact sum plus the fp64 sum's own 2e-13."""
+    g = torch.Generator(device=DEV).manual_seed(d_in)
+    X = torch.randn((203, d_in + 3), generator=g, device=DEV).to(dtype)[:, :d_in]
+    H = B.cdq_hessian(X)
+    D = X.double()
+    want = D.T @ D
+    norm = torch.sqrt(torch.outer(want.diagonal(), want.diagonal()))
+    assert float(((H.double() - want).abs() / norm).max()) <= 6.1e-8
+    assert torch.equal(H, H.T.contiguous())
+    H2 = B.cdq_hessian(X, accumulate=True, out=H.clone())
+    assert float(((H2.double() - 2 * want).abs() / norm).max()) <= 2.5e-7
+
+
+@pytest.mark.parametrize("d_in,d_out,bits,g,dtype", [
+    (64, 8, 8, 16, "f32"), (48, 5, 3, 0, "f32"), (520, 1028, 4, 130, "bf16"), (1024, 1024, 8, 0, "f32"), (1000, 516, 2, 8, "f32"),
+])
+def test_codes_of_weights_between_two_levels(d_in, d_out, bits, g, dtype):
+    """Weights in the middle between two levels and one fp32 neighbour to either side: bit for bit the oracle's codes,
+    in the one-column and the four-column kernel."""
+    rng = np.random.default_rng(d_in + bits)
+    gg = g or d_in
+    L = 2 ** bits - 1
+    W = rng.standard_normal((d_in, d_out)).astype(np.float32) * 0.02
+    for t in range(d_in // gg):
+        blk = W[t * gg:(t + 1) * gg]
+        lo, hi = blk.min(0).astype(np.float64), blk.max(0).astype(np.float64)
+        a = (hi - lo) / L
+        k = rng.integers(0, L, blk.shape)
+        mid = (lo + a * (k + 0.5)).astype(np.float32)
+        mid = np.where(rng.random(blk.shape) < 0.3, np.nextafter(mid, np.float32(1)), mid)
+        mid = np.where(rng.random(blk.shape) < 0.3, np.nextafter(mid, np.float32(-1)), mid)
+        keep = (blk == blk.min(0)) | (blk == blk.max(0))
+        W[t * gg:(t + 1) * gg] = np.where(keep, blk, mid)
+    Wt = torch.from_numpy(W)
+    if dtype == "bf16":
+        Wt = Wt.bfloat16()
+    want = oracle.init_rtn(Wt, bits, g, 1, 1.0, 1.0)
+    scale, zero, Q, _ = B.cdq_init_rtn(Wt.to(DEV), B.Grid(bits, g))
+    assert np.array_equal(scale.cpu().numpy(), want["scale"]) and np.array_equal(zero.cpu().numpy(), want["zero"])
+    assert np.array_equal(Q.cpu().numpy(), want["Q"])
