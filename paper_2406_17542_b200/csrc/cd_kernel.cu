@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
   const int tid = threadIdx.x, NT = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
   const long long d_in = p.d_in;
-  const int nchunks = (int)((d_in + 3) >> 2);
+  const int nchunks = (int)(d_in >> 2);
   const float top = kMagic + (float)p.L;
 
   auto group_of = [&](unsigned i) -> unsigned { return p.g == 1 ? i : __umulhi(i, p.gmagic); };
@@ -188,12 +188,6 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
           g0 = *reinterpret_cast<const double2*>(gcol + (long long)chunk * 4);
           g1 = *reinterpret_cast<const double2*>(gcol + (long long)chunk * 4 + 2);
           qp[k] = *reinterpret_cast<const unsigned*>(qcol + (long long)chunk * 4);
-        }
-        if (!EXACT) {  // coordinates past d_in inside the last chunk: padding of the rows of G and Qt
-          const long long i0 = (long long)chunk * 4;
-          if (i0 + 1 >= d_in) { g0.y = 0.0; qp[k] &= 0x000000FFu; }
-          if (i0 + 2 >= d_in) { g1.x = 0.0; qp[k] &= 0x0000FFFFu; }
-          if (i0 + 3 >= d_in) { g1.y = 0.0; qp[k] &= 0x00FFFFFFu; }
         }
         g[4 * k] = g0.x * gscale; g[4 * k + 1] = g0.y * gscale; g[4 * k + 2] = g1.x * gscale; g[4 * k + 3] = g1.y * gscale;
       }
@@ -265,7 +259,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
       float astar = 1.f;
       if (SMODE != kPerChannel) astar = ag_s[group_of((unsigned)istar)].x;
       c2 = 2.0 * ((double)astar * (double)dri);
-      rp = p.H + (long long)istar * p.ldh;
+      rp = p.H + (long long)istar * d_in;
       if (tid == 0) col_dsum += (double)__uint_as_float(~m);
       ++step;
     }
@@ -391,12 +385,12 @@ cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, co
                            long long ldq, const float* hdiag, const float* hs, long long steps_per_col,
                            CdCounters* ctr, cudaStream_t st) {
   CdParams p{};
-  p.H = rows; p.ldh = ldh; p.H16 = H16; p.d_in = ly.d_in; p.d_out = ly.d_out; p.G = G; p.ldg = ldg; p.Qt = Qt; p.ldq = ldq; p.scale = ly.scale;
+  p.H = rows; p.H16 = H16; p.d_in = ldh; p.d_out = ly.d_out; p.G = G; p.ldg = ldg; p.Qt = Qt; p.ldq = ldq; p.scale = ly.scale;
   p.hdiag = hdiag; p.hs = hs; p.g = ly.g; p.ng = ly.ng; p.L = ly.L; p.T = steps_per_col; p.ctr = ctr;
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;
   p.gmagic = ly.g > 1 ? (unsigned)(((1ull << 32) + (unsigned long long)ly.g - 1) / (unsigned long long)ly.g) : 0u;
-  const long long d = ly.d_in;
+  const long long d = ldh;
   if (steps_per_col <= 0) return cudaSuccess;   // nothing to do: the counters stay zero, the codes untouched
   // short rows are quickest as plain loads into registers, longer ones as bulk copies into shared memory
   // (measured crossover: 1536 entries 2.0 against 2.5 ms, 1792 entries 11.5 against 10.8, 2048 entries 52.0 against 45.3);

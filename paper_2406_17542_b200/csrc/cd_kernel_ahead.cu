@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
   const int tid = threadIdx.x, NT = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
   const unsigned below = (1u << lane) - 1u;    // lanes before this one
-  const int nchs = (int)((p.d_in + 3) >> 2);         // chunks of a row
+  const int nchs = (int)(p.d_in >> 2);         // chunks of a row
   const bool exact = nchs == NT * NCH;
   const float top_q = (float)p.L, top = kMagic + top_q;
 
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       }
       if (tid == 0) {
         const unsigned char* src = ROW16 ? reinterpret_cast<const unsigned char*>(p.H16 + (long long)istar * p.d_in)
-                                         : reinterpret_cast<const unsigned char*>(p.H + (long long)istar * p.ldh);
+                                         : reinterpret_cast<const unsigned char*>(p.H + (long long)istar * p.d_in);
         mbar_expect_tx(smem_u32(&s_bar[b]), row_bytes);
         bulk_load(smem_u32(row_s + b * row_span), src, row_bytes, smem_u32(&s_bar[b]));
       }
@@ -589,13 +589,13 @@ cudaError_t launch_mode(const CdParams& p, int nt, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st) {
-  if (p.ldh & 3) return cudaErrorNotSupported;
+  if (p.d_in & 3) return cudaErrorNotSupported;
   if ((reinterpret_cast<uintptr_t>(p.H) & 15) != 0) return cudaErrorNotSupported;
   if (p.H16 && ((p.d_in & 7) != 0 || (reinterpret_cast<uintptr_t>(p.H16) & 15) != 0)) return cudaErrorNotSupported;
   // Few threads with many chunks each: no spills, a cheaper argmin exchange, fixed costs per thread spread over more
   // state; full warps in equal numbers per scheduler.  256 threads hold up to 14 chunks each in registers; beyond that the
   // team is the smallest of 10..12 x 384 and 8 x 512 chunk slots that holds the row.
-  const long long ch = (p.d_in + 3) >> 2;
+  const long long ch = p.d_in >> 2;
   auto team = [&](long long chunks, int nch) { return (int)((chunks + nch - 1) / nch + 31) / 32 * 32; };
   if (ch <= 2304) return launch_mode<9, 256, 1>(p, team(ch, 9), st);
   if (ch <= 2560) return launch_mode<10, 256, 1>(p, team(ch, 10), st);

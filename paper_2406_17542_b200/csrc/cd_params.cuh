@@ -7,9 +7,8 @@ namespace cdq {
 
 struct CdParams {
   const float* H;
-  long long ldh;              // row stride of H, a multiple of 4 (the entries past d_in are zero)
   const __nv_bfloat16* H16;   // bf16 copy of H for the rows of the update (NULL: fp32 rows)
-  long long d_in, d_out;
+  long long d_in, d_out;      // d_in: entries of a row, a multiple of 4 (zeros pad odd layers: H_ii = 0, so nothing moves there)
   double* G;            // [d_out, ldg]
   long long ldg;
   unsigned char* Qt;    // [d_out, ldq] (transposed codes, ldq a multiple of 4)
