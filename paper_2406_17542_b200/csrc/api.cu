@@ -388,10 +388,10 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
   CdCounters* ctr = (CdCounters*)(base + L.scalars + 64);
 
   // G0 = 2 H (W_hat - W) and the loss at entry
-  CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
+  if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
     CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, base + L.hbuf, st));
-    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, E, d_in, d_out, L.ne, L.smax, 2.0, G, L.ldg, col_loss, base + L.ebuf, st));
+    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 2.0, G, L.ldg, col_loss, base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, G, L.ldg, col_loss, part, st));
   } else {
@@ -526,10 +526,10 @@ cdq_status cdq_layer_loss(const float* H, const void* W, cdq_dtype wt, long long
   double* part = (double*)(base + L.part);
   double* col_loss = per_col ? per_col : (double*)(base + L.col_loss);
   double* loss_sum = (double*)(base + L.scalars);
-  CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
+  if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
     CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, base + L.hbuf, st));
-    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), L.ldg, col_loss,
+    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), L.ldg, col_loss,
                          base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, st));

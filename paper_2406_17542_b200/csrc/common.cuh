@@ -81,11 +81,14 @@ struct ResidualSrc {
   const float* mn; const float* mx; double gamma; int L; int use_gamma;  // OWC path
   long long g, d_out;      // d_out: columns of the layer (the width of W's companions scale, zero, Q, mn, mx)
   const int* col_idx;      // NULL: E has a column for every layer column; else E column c is layer column col_idx[c] ...
-  long long n_cols;        // ... and E is [d_in, n_cols]
+  long long n_cols;        // (not 0) E is [d_in, n_cols]; without col_idx its column c is layer column c % d_out under ...
   const int* col_gamma;    // OWC path, with col_idx: E column c takes the clipping strength gammas[col_gamma[c]] ...
-  const double* gammas;    // ... instead of `gamma` (NULL: `gamma` for every column)
+  const double* gammas;    // ... instead of `gamma`
+  int k0;                  // ... the strength gammas[k0 + c / d_out]
 };
-cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st);
+// colmax (may be NULL, zeroed by the caller): largest |E| per column as ordered bit patterns.
+cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st,
+                                unsigned long long* colmax = nullptr);
 
 // gemm_f64.cu : C = H * E in fp64.
 // G (may be NULL): [d_out, ldg] doubles, G[j][p] = 2 * C[p][j].
@@ -101,12 +104,12 @@ cudaError_t launch_gemm_he_verify(const float* H, long long d_in, long long d_ou
 
 // gemm_i8.cu : C[j, p] = scale * sum_k E[k, j] H[p, k] on the int8 tensor cores from 7-bit slices of
 // both operands (nh slices of H, ne of E, slice pairs up to i + j = smax); C is [d_out, ldc].
-// col_loss (may be NULL): [d_out], e_j^T H e_j.
+// col_loss (may be NULL): [d_out], e_j^T H e_j.  gemm_tc_run forms the residual E [d_in, d_out] from its source first.
 bool gemm_tc_supported(long long d_in, long long d_out);
 size_t gemm_tc_h_bytes(long long d_in, int nh);
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne);
 cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, void* hbuf, cudaStream_t st);
-cudaError_t gemm_tc_run(const void* hbuf, int nh, const double* E, long long d_in, long long d_out, int ne, int smax,
+cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
                         double scale, double* C, long long ldc, double* col_loss, void* ebuf, cudaStream_t st);
 // Slice counts: the gradient and the loss of a descended solution need ~1e-9 of a_j H_pp (see
 // gemm_i8.cu); the losses of the OWC search (round-to-nearest residuals) need ~1e-7 relative.

@@ -62,17 +62,7 @@ __global__ void row_exp_f32_kernel(const float* __restrict__ x, long long rows, 
   }
 }
 
-// Column maxima of a row-major fp64 matrix [rows, cols] -> exponent per column (two steps:
-// partial maxima over row blocks as ordered bit patterns, then the exponent).
-__global__ void col_max_f64_kernel(const double* __restrict__ x, long long rows, long long cols,
-                                   unsigned long long* __restrict__ colmax_bits) {
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  const long long r0 = (long long)blockIdx.y * 256, r1 = min(rows, r0 + 256);
-  double m = 0.0;
-  for (long long r = r0; r < r1; ++r) m = fmax(m, fabs(x[r * cols + c]));
-  if (isfinite(m)) atomicMax(&colmax_bits[c], (unsigned long long)__double_as_longlong(m));  // m >= 0: bits order like values
-}
+// Column maxima (ordered bit patterns) -> exponent per column.
 __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bits, long long cols, int* __restrict__ exps) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= cols) return;
@@ -82,48 +72,85 @@ __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bit
   exps[c] = e;
 }
 
-// The ns slices of one value already scaled into (-1, 1).
-__device__ __forceinline__ void slice_value(double r, int ns, signed char (&out)[MAX_SLICES]) {
+// |x| 2^-e 128^ns, truncated, as an integer (x 2^-e in (-1, 1), ns <= 6): slice i of x is its 7-bit digit number ns - i from
+// below with the sign of x, which is what truncating, subtracting and scaling up digit by digit gives.  The addition of
+// 2^52 towards zero leaves the integer in the mantissa; scale = 2^(7 ns - e), a normal number for every exponent of H and E.
+__device__ __forceinline__ unsigned long long slice_bits(double x, double scale) {
+  return (unsigned long long)__double_as_longlong(__dadd_rz(fabs(x) * scale, 4503599627370496.0)) & 0xFFFFFFFFFFFFFull;
+}
+// Digit i (from 1) of four neighbours, negated where `neg` has the byte's bits set, as four bytes.
+__device__ __forceinline__ unsigned slice_bytes(const unsigned long long (&v)[4], int shift, unsigned neg) {
+  unsigned d = 0u;
 #pragma unroll
-  for (int i = 0; i < MAX_SLICES; ++i) {
-    if (i < ns) {
-      r *= 128.0;
-      const double s = trunc(r);
-      r -= s;
-      out[i] = (signed char)(int)s;
-    }
-  }
+  for (int k = 0; k < 4; ++k) d |= ((unsigned)(v[k] >> shift) & 127u) << (8 * k);
+  return __vsub4(d ^ neg, neg);
 }
 
-// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p]; columns >= d zero).
+// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p]; columns >= d zero), four columns per thread.
+// Memory-bound: 4 bytes read and ns written per entry.  (One column per thread, with the digits taken off one after
+// the other in fp64: 1.46 ms for 14336^2 and six slices.)
 __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ exps,
                                int ns, signed char* __restrict__ out) {
   const long long p = blockIdx.y;
-  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long k = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
   if (k >= kp) return;
-  signed char s[MAX_SLICES] = {0, 0, 0, 0, 0, 0};
-  if (k < d) slice_value(ldexp((double)H[p * d + k], -exps[p]), ns, s);
-  for (int i = 0; i < ns; ++i) out[((size_t)i * d + p) * kp + k] = s[i];
+  const double scale = ldexp(1.0, 7 * ns - exps[p]);
+  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  if ((d & 3) == 0) {
+    if (k < d) {
+      const float4 f = *reinterpret_cast<const float4*>(H + p * d + k);
+      x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      if (k + v < d) x[v] = H[p * d + k + v];
+  }
+  unsigned long long b[4];
+  unsigned neg = 0u;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    b[v] = slice_bits((double)x[v], scale);
+    if (x[v] < 0.f) neg |= 0xFFu << (8 * v);
+  }
+  for (int i = 0; i < ns; ++i)
+    *reinterpret_cast<unsigned*>(out + ((size_t)i * d + p) * kp + k) = slice_bytes(b, 7 * (ns - 1 - i), neg);
 }
 
-// E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j]),
-// 32 x 32 tiles through shared memory so that both the reads and the writes are contiguous.
-__global__ void slice_et_kernel(const double* __restrict__ E, long long d_in, long long d_out, long long kp,
-                                const int* __restrict__ exps, int ns, signed char* __restrict__ out) {
-  __shared__ double tile[32][33];
-  const long long k0 = (long long)blockIdx.x * 32, j0 = (long long)blockIdx.y * 32;
-  for (int rr = threadIdx.y; rr < 32; rr += blockDim.y) {
-    const long long k = k0 + rr, j = j0 + threadIdx.x;
-    tile[rr][threadIdx.x] = (k < d_in && j < d_out) ? E[k * d_out + j] : 0.0;
+// E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j]), 128 x 32 tiles turned round
+// in shared memory so that reads and writes are contiguous, four rows of E per thread.  Memory-bound: 8 bytes read and ns
+// written per entry.  (32 x 32 tiles, single bytes, digits one after the other in fp64: 0.74 ms for 4096 x 32768 and
+// two slices.)
+constexpr int SK = 128, SJ = 32;
+__global__ void __launch_bounds__(256) slice_et_kernel(const double* __restrict__ E, long long d_in, long long d_out, long long kp,
+                                                       const int* __restrict__ exps, int ns, signed char* __restrict__ out) {
+  // entry (k, j) at [j][k ^ 2 (j & 15)]: the stores down a column spread over the banks, pairs of k stay together
+  __shared__ __align__(16) double tile[SJ][SK];
+  const long long k0 = (long long)blockIdx.x * SK, j0 = (long long)blockIdx.y * SJ;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int r = ty; r < SK; r += 8) {
+    const long long k = k0 + r, j = j0 + tx;
+    tile[tx][r ^ (2 * (tx & 15))] = (k < d_in && j < d_out) ? E[k * d_out + j] : 0.0;
   }
   __syncthreads();
-  for (int jj = threadIdx.y; jj < 32; jj += blockDim.y) {
-    const long long j = j0 + jj, k = k0 + threadIdx.x;
-    if (j < d_out && k < kp) {
-      signed char s[MAX_SLICES] = {0, 0, 0, 0, 0, 0};
-      slice_value(ldexp(tile[threadIdx.x][jj], -exps[j]), ns, s);
-      for (int i = 0; i < ns; ++i) out[((size_t)i * d_out + j) * kp + k] = s[i];
+#pragma unroll
+  for (int jj = ty; jj < SJ; jj += 8) {
+    const long long j = j0 + jj, k = k0 + 4 * tx;
+    if (j >= d_out) continue;   // (k < kp: kp is a multiple of SK)
+    const double scale = ldexp(1.0, 7 * ns - exps[j]);
+    const double2 x01 = *reinterpret_cast<const double2*>(&tile[jj][(4 * tx) ^ (2 * (jj & 15))]);
+    const double2 x23 = *reinterpret_cast<const double2*>(&tile[jj][(4 * tx + 2) ^ (2 * (jj & 15))]);
+    const double x[4] = {x01.x, x01.y, x23.x, x23.y};
+    unsigned long long b[4];
+    unsigned neg = 0u;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      b[v] = slice_bits(x[v], scale);
+      if (x[v] < 0.0) neg |= 0xFFu << (8 * v);
     }
+    for (int i = 0; i < ns; ++i)
+      *reinterpret_cast<unsigned*>(out + ((size_t)i * d_out + j) * kp + k) = slice_bytes(b, 7 * (ns - 1 - i), neg);
   }
 }
 
@@ -428,8 +455,8 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, void* hbuf
   signed char* slices = (signed char*)hbuf;
   int* hexp = (int*)((char*)hbuf + align_up((size_t)nh * d_in * kp));
   { i8::row_exp_f32_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, hexp); count_launch(); }
-  dim3 grid((unsigned)((kp + 255) / 256), (unsigned)d_in);
-  { i8::slice_h_kernel<<<grid, 256, 0, st>>>(H, d_in, kp, hexp, nh, slices); count_launch(); }
+  dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
+  { i8::slice_h_kernel<<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices); count_launch(); }
   return cudaGetLastError();
 }
 
@@ -456,10 +483,10 @@ static cudaError_t encode_map3(CUtensorMap* map, const void* base, long long kp,
   return cr == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// C[j, p] = scale * sum_k E[k, j] H[p, k]  for j < d_out, p < d_in, to the precision of
+// E = the residual of `src`, then C[j, p] = scale * sum_k E[k, j] H[p, k]  for j < d_out, p < d_in, to the precision of
 // (ne, nh, smax); optionally col_loss[j] = sum_p E[p, j] C[j, p] / scale.
 // hbuf: from gemm_tc_prepare_h with the same nh.  ebuf: gemm_tc_e_bytes of scratch.
-cudaError_t gemm_tc_run(const void* hbuf, int nh, const double* E, long long d_in, long long d_out, int ne, int smax,
+cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
                         double scale, double* C, long long ldc, double* col_loss, void* ebuf, cudaStream_t st) {
   using namespace i8;
   if (nh < 1 || nh > MAX_SLICES || ne < 1 || ne > MAX_SLICES || smax < 2) return cudaErrorInvalidValue;
@@ -473,13 +500,11 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const double* E, long long d_i
 
   cudaError_t e = cudaMemsetAsync(colmax, 0, sizeof(unsigned long long) * (size_t)d_out, st);
   if (e != cudaSuccess) return e;
-  {
-    dim3 grid((unsigned)((d_out + 255) / 256), (unsigned)((d_in + 255) / 256));
-    { col_max_f64_kernel<<<grid, 256, 0, st>>>(E, d_in, d_out, colmax); count_launch(); }
-    { col_exp_kernel<<<(unsigned)((d_out + 255) / 256), 256, 0, st>>>(colmax, d_out, eexp); count_launch(); }
-    dim3 g2((unsigned)((kp + 31) / 32), (unsigned)((d_out + 31) / 32)), b2(32, 8);
-    { slice_et_kernel<<<g2, b2, 0, st>>>(E, d_in, d_out, kp, eexp, ne, esl); count_launch(); }
-  }
+  e = launch_residual_f64(src, d_in, E, st, colmax);
+  if (e != cudaSuccess) return e;
+  { col_exp_kernel<<<(unsigned)((d_out + 255) / 256), 256, 0, st>>>(colmax, d_out, eexp); count_launch(); }
+  const dim3 slices((unsigned)(kp / SK), (unsigned)((d_out + SJ - 1) / SJ));
+  { slice_et_kernel<<<slices, 256, 0, st>>>(E, d_in, d_out, kp, eexp, ne, esl); count_launch(); }
   Params p{};
   p.M = (int)d_out; p.N = (int)d_in; p.kblocks = (int)(kp / BKB);
   p.tiles_m = (int)((d_out + BM - 1) / BM); p.tiles_n = (int)((d_in + BN - 1) / BN);

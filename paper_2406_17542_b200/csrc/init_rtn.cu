@@ -5,6 +5,7 @@
 //   q = clamp(round_half_even((w - b) / a), 0, L)      (decided in fp64)
 //   OWC: loss_k[j] = e_k^T H e_k for every gamma_k, argmin over k per column.
 #include "common.cuh"
+#include "rtn_code.cuh"
 
 namespace cdq {
 
@@ -96,23 +97,9 @@ __global__ void scale_zero_kernel(const float* __restrict__ mn, const float* __r
   zero[t * d_out + j] = (float)lo;
 }
 
-// Codes of kCodeRows rows of one group by V columns per thread.  The code is the fp64 rounding of (w - b) / a.  The fp32
-// quotient is off by at most 3 * 2^-24 of itself, 5e-5 where it is within 256 levels, so unless it lies within 2e-4 of
-// the middle between two levels both round to the same level; the one in 2500 that does is decided in fp64.  (Memory-bound that way: 14336 x 16384 bf16 weights took 1180 us with an fp64 division and one byte per thread.)
+// Codes of kCodeRows rows of one group by V columns per thread (see rtn_code).  Memory-bound: 14336 x 16384 bf16 weights
+// took 1180 us with an fp64 division and one byte per thread.
 constexpr int kCodeRows = 16;
-__device__ __forceinline__ unsigned rtn_code(float w, float a, float inv_a, float b, float top) {
-  constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer, to the even one in the middle
-  const float t = (w - b) * inv_a;
-  const float c = fminf(fmaxf(t, 0.f), top);
-  const float m = c + kMagic;
-  if (!(fabsf(c - (m - kMagic)) < 0.4998f) || t != t) {
-    double q = rint(__ddiv_rn(__dadd_rn((double)w, -(double)b), (double)a));
-    q = q < 0.0 ? 0.0 : q;
-    q = q > (double)top ? (double)top : q;
-    return (unsigned)(unsigned char)q;
-  }
-  return __float_as_uint(m) & 255u;
-}
 template <int V, bool BF16>
 __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__ W, long long d_out,
                                                         long long ldw, long long g, int blocks_per_group, int L,
@@ -127,56 +114,110 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
   for (int v = 0; v < V; ++v) {
     a[v] = scale[t * d_out + j + v];
     b[v] = zero[t * d_out + j + v];
-    inv[v] = 1.0f / a[v];
-    if (!(inv[v] <= 3.4e38f)) inv[v] = __int_as_float(0x7FFFFFFF);   // a subnormal scale: decided in fp64
+    inv[v] = rtn_inverse(a[v]);
   }
-#pragma unroll 4
-  for (long long i = i0; i < i1; ++i) {
-    float w[V];
-    load_weights<V, BF16>(W, i * ldw + j, w);
-    unsigned q = 0u;
+  constexpr int R = 8;   // rows whose loads are in flight together (the compiler moves no load past the branch of rtn_code)
+  for (long long i = i0; i < i1; i += R) {
+    float w[R][V];
 #pragma unroll
-    for (int v = 0; v < V; ++v) q |= (a[v] > 0.f ? rtn_code(w[v], a[v], inv[v], b[v], (float)L) : 0u) << (8 * v);
-    if constexpr (V == 4) *reinterpret_cast<unsigned*>(Q + i * d_out + j) = q;
-    else Q[i * d_out + j] = (unsigned char)q;
-  }
-}
-
-// Residual E[i][j] = (a q + b) - w in fp64, either from stored codes or, for the OWC search,
-// from min/max and a clipping strength (codes formed on the fly, never stored).
-__global__ void residual_kernel(ResidualSrc s, long long d_in, double* __restrict__ E) {
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;   // column of E
-  const long long i = blockIdx.y;
-  const long long width = s.col_idx ? s.n_cols : s.d_out;
-  if (c >= width) return;
-  const long long j = s.col_idx ? (long long)s.col_idx[c] : c;            // column of the layer
-  const long long t = i / s.g;
-  const double w = load_w(s.W, s.wt, i * s.ldw + j);
-  double a, b, q;
-  if (s.use_gamma) {
-    const double lo = (double)s.mn[t * s.d_out + j], hi = (double)s.mx[t * s.d_out + j];
-    const double gamma = s.col_gamma ? s.gammas[s.col_gamma[c]] : s.gamma;
-    const float a32 = (float)__ddiv_rn(__dmul_rn(gamma, __dadd_rn(hi, -lo)), (double)s.L);
-    a = (double)a32;
-    b = lo;
-    q = 0.0;
-    if (a32 > 0.f) {
-      q = rint(__ddiv_rn(__dadd_rn(w, -b), a));
-      q = q < 0.0 ? 0.0 : q;
-      q = q > (double)s.L ? (double)s.L : q;
+    for (int r = 0; r < R; ++r) load_weights<V, BF16>(W, min(i + r, i1 - 1) * ldw + j, w[r]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (i + r >= i1) break;
+      unsigned q = 0u;
+#pragma unroll
+      for (int v = 0; v < V; ++v) q |= (a[v] > 0.f ? rtn_code(w[r][v], a[v], inv[v], b[v], (float)L) : 0u) << (8 * v);
+      if constexpr (V == 4) *reinterpret_cast<unsigned*>(Q + (i + r) * d_out + j) = q;
+      else Q[(i + r) * d_out + j] = (unsigned char)q;
     }
-  } else {
-    a = (double)s.scale[t * s.d_out + j];
-    b = (double)s.zero[t * s.d_out + j];
-    q = (double)s.Q[i * s.d_out + j];
   }
-  E[i * width + c] = __dadd_rn(__dadd_rn(__dmul_rn(a, q), b), -w);
 }
 
-cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st) {
-  const long long width = src.col_idx ? src.n_cols : src.d_out;
-  dim3 block(128), grid((unsigned)((width + 127) / 128), (unsigned)d_in);
-  { residual_kernel<<<grid, block, 0, st>>>(src, d_in, E); count_launch(); }
+// Residual E[i][c] = (a q + b) - w in fp64, either from stored codes or, for the OWC search, from min/max and a clipping
+// strength (codes formed on the fly, never stored).  With colmax it also leaves the largest |E| of every column there (as
+// ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  Memory-bound: 8 bytes written
+// per entry.  (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
+// strengths of a 4096 x 4096 layer, 0.16 ms of them the maxima.)
+constexpr int kResRows = 32;   // rows per block, all of one group
+template <int V, bool BF16>
+__global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int blocks_per_group, double* __restrict__ E,
+                                                       unsigned long long* __restrict__ colmax) {
+  const long long c = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x);   // column of E
+  const long long width = s.n_cols ? s.n_cols : s.d_out;
+  if (c >= width) return;
+  const long long j = s.col_idx ? (long long)s.col_idx[c] : c % s.d_out;        // column of the layer
+  const long long t = blockIdx.y / blocks_per_group, i0 = t * s.g + (blockIdx.y % blocks_per_group) * (long long)kResRows;
+  const long long i1 = min(i0 + kResRows, (t + 1) * s.g);
+  float a[V], b[V], inv[V];
+  double m[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    m[v] = 0.0;
+    if (s.use_gamma) {
+      const double lo = (double)s.mn[t * s.d_out + j + v], hi = (double)s.mx[t * s.d_out + j + v];
+      const double gamma = s.col_gamma ? s.gammas[s.col_gamma[c + v]] : s.n_cols ? s.gammas[s.k0 + c / s.d_out] : s.gamma;
+      a[v] = (float)__ddiv_rn(__dmul_rn(gamma, __dadd_rn(hi, -lo)), (double)s.L);
+      b[v] = (float)lo;
+      inv[v] = rtn_inverse(a[v]);
+    } else {
+      a[v] = s.scale[t * s.d_out + j + v];
+      b[v] = s.zero[t * s.d_out + j + v];
+    }
+  }
+  constexpr int R = 4;   // rows whose loads are in flight together (the compiler moves no load past the branch of rtn_code)
+  for (long long i = i0; i < i1; i += R) {
+    float w[R][V];
+    unsigned q4[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const long long row = min(i + r, i1 - 1);
+      load_weights<V, BF16>(s.W, row * s.ldw + j, w[r]);
+      q4[r] = 0u;
+      if (!s.use_gamma) {
+        if constexpr (V == 4) q4[r] = *reinterpret_cast<const unsigned*>(s.Q + row * s.d_out + j);
+        else q4[r] = s.Q[row * s.d_out + j];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (i + r >= i1) break;
+      double e[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        unsigned q = (q4[r] >> (8 * v)) & 255u;
+        if (s.use_gamma) q = a[v] > 0.f ? rtn_code(w[r][v], a[v], inv[v], b[v], (float)s.L) : 0u;
+        // 2^52 + q: its lower word is q
+        const double qd = __hiloint2double(0x43300000, (int)q) - 4503599627370496.0;
+        e[v] = __dadd_rn(__dadd_rn(__dmul_rn((double)a[v], qd), (double)b[v]), -(double)w[r][v]);
+        m[v] = fmax(m[v], fabs(e[v]));
+      }
+      double* dst = E + (i + r) * width + c;
+      if constexpr (V == 4) {
+        *reinterpret_cast<double2*>(dst) = make_double2(e[0], e[1]);
+        *reinterpret_cast<double2*>(dst + 2) = make_double2(e[2], e[3]);
+      } else {
+        dst[0] = e[0];
+      }
+    }
+  }
+  if (colmax) {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      if (isfinite(m[v])) atomicMax(&colmax[c + v], (unsigned long long)__double_as_longlong(m[v]));   // >= 0: bits order like values
+  }
+}
+
+cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st, unsigned long long* colmax) {
+  const long long width = src.n_cols ? src.n_cols : src.d_out;
+  const int bpg = (int)((src.g + kResRows - 1) / kResRows);
+  const size_t esz = src.wt == CDQ_BF16 ? 2 : 4;
+  // four columns per thread: rows of W, Q and E on the vectors' boundaries, four neighbouring columns of one strength
+  const bool four = !src.col_idx && src.d_out % 4 == 0 && src.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(src.W) % (4 * esz) == 0 &&
+                    reinterpret_cast<uintptr_t>(src.Q) % 4 == 0 && width * (d_in / src.g) * bpg >= (1 << 17);
+  const dim3 grid((unsigned)((width + (four ? 511 : 127)) / (four ? 512 : 128)), (unsigned)(d_in / src.g * bpg));
+  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, bpg, E, colmax); count_launch(); };
+  if (src.wt == CDQ_BF16) run(four ? residual_kernel<4, true> : residual_kernel<1, true>);
+  else run(four ? residual_kernel<4, false> : residual_kernel<1, false>);
   return cudaGetLastError();
 }
 
@@ -268,15 +309,6 @@ __global__ void owc_concat_kernel(const int* __restrict__ idx, long long d_out, 
   while (k + 1 < n_clip && offs.off[k + 1] <= cc) ++k;
   cj[c] = idx[(long long)k * (d_out + 128) + (cc - offs.off[k])];
   ck[c] = k;
-}
-
-// Columns of a screening product over several strengths at once: column c is layer column c % d_out under strength
-// k0 + c / d_out.
-__global__ void owc_iota_kernel(long long d_out, int k0, long long width, int* __restrict__ cj, int* __restrict__ ck) {
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (c >= width) return;
-  cj[c] = (int)(c % d_out);
-  ck[c] = k0 + (int)(c / d_out);
 }
 
 __global__ void owc_scatter_kernel(const double* __restrict__ loss_c, const int* __restrict__ cj, const int* __restrict__ ck,
@@ -409,13 +441,8 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.W = ly.W; src.wt = ly.wt; src.ldw = ly.ldw;
         src.mn = mn; src.mx = mx; src.gamma = hg[k0]; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out;
-        if (gb > 1) {
-          { owc_iota_kernel<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(d_out, k0, width, cj, ck); count_launch(); }
-          src.col_idx = cj; src.n_cols = width; src.col_gamma = ck; src.gammas = gammas;
-        }
-        e = launch_residual_f64(src, d_in, E, st);
-        if (e != cudaSuccess) return e;
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
+        if (gb > 1) { src.n_cols = width; src.k0 = k0; src.gammas = gammas; }   // column c: layer column c % d_out
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
                         (double*)(base + L.C), L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
       }
@@ -439,9 +466,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.mn = mn; src.mx = mx; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out; src.col_idx = cj + b0; src.n_cols = width;
         src.col_gamma = ck + b0; src.gammas = gammas;
-        e = launch_residual_f64(src, d_in, E, st);
-        if (e != cudaSuccess) return e;
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
                         loss_c, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
         { owc_scatter_kernel<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(loss_c, cj + b0, ck + b0, width, d_out, table); count_launch(); }
@@ -452,15 +477,17 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
       src.W = ly.W; src.wt = ly.wt; src.ldw = ly.ldw;
       src.mn = mn; src.mx = mx; src.gamma = hg[k]; src.L = ly.L; src.use_gamma = 1;
       src.g = g; src.d_out = d_out;
-      e = launch_residual_f64(src, d_in, E, st);
-      if (e != cudaSuccess) return e;
-      if (L.tc)
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+      if (L.tc) {
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
                         table + (long long)k * d_out, base + L.ebuf, st);
-      else if (mode == CDQ_MODE_FAST)
-        e = launch_gemm_he(ly.H, d_in, d_out, E, nullptr, 0, table + (long long)k * d_out, part, st);
-      else
-        e = launch_gemm_he_verify(ly.H, d_in, d_out, E, part, nullptr, 0, table + (long long)k * d_out, st);
+      } else {
+        e = launch_residual_f64(src, d_in, E, st);
+        if (e != cudaSuccess) return e;
+        if (mode == CDQ_MODE_FAST)
+          e = launch_gemm_he(ly.H, d_in, d_out, E, nullptr, 0, table + (long long)k * d_out, part, st);
+        else
+          e = launch_gemm_he_verify(ly.H, d_in, d_out, E, part, nullptr, 0, table + (long long)k * d_out, st);
+      }
       if (e != cudaSuccess) return e;
     }
     { owc_argmin_kernel<<<bx, 128, 0, st>>>(table, n_clip, d_out, gammas, gcol, gamma_out); count_launch(); }
