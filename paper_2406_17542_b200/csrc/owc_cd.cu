@@ -19,6 +19,7 @@
 //           dot products of length g:  delta^T H_tt delta = r_k.M_k - 2 r_k.M_c + r_c.M_c;
 //           one warp per dot product, lanes across the group.
 #include "common.cuh"
+#include "rtn_code.cuh"
 
 namespace cdq {
 namespace owc {
@@ -356,6 +357,271 @@ __global__ void __launch_bounds__(NT, 2) owc_cd_kernel(Params p) {
   if (tid == 0 && my_moves) atomicAdd(&p.ctr->moves, my_moves);
 }
 
+// Production kernel for up to kCodesNk strengths and groups of up to kCodesG coordinates, on the codes of the strengths
+// instead of their residuals.
+//
+// What bounds it is the update: g rows of H per move, 2 MB at 4096 features in groups of 128, which come from L2 as long
+// as H stays there.  The tables of the general kernel (residuals and their products with H, 16 nk d_in bytes per
+// column in flight: 388 MB for 296 columns) drove H out of L2 and were themselves read from HBM at every step; here a
+// column has its codes (nk d_in bytes) and, per group, the products r_k^T H_tt r_l of every pair of strengths (8 nk^2 ng
+// bytes): 55 MB for the same columns.  Within a group r_k - r_l = a_k q_k - a_l q_l (weights and zeros cancel), so with
+// S_k = sum_i q_k,i G_i the change of a candidate k of a group that holds c is
+//     K_kk - 2 K_kc + K_cc + a_k S_k - a_c S_c.
+// 4096 x 1024, groups of 128, 20 strengths: 26.0 ms with the general kernel.
+constexpr int kCodesNk = 32, kCodesG = 512;
+constexpr size_t kCodesSmem = 100 * 1024;   // two CTAs per SM
+inline size_t codes_smem(long long g, long long ng, int nk) {   // quad, S, residuals and products of one group, delta; scales
+  return sizeof(double) * (2 * (size_t)(ng * nk) + 2 * (size_t)nk * g + g) + sizeof(float) * (size_t)(ng * nk);
+}
+// per CTA: G, e0, the products K [ng, nk, nk], the codes [nk, d_in]
+inline size_t codes_scratch(long long d_in, long long ng, int nk) {
+  return sizeof(double) * (2 * (size_t)d_in + (size_t)ng * nk * nk) + ((size_t)nk * d_in + 255) / 256 * 256;
+}
+inline bool codes_supported(long long g, long long ng, int nk) {
+  return nk <= kCodesNk && g <= kCodesG && codes_smem(g, ng, nk) <= kCodesSmem;
+}
+__device__ __forceinline__ double byte_to_double(unsigned q) {   // exact, on the fp64 pipe instead of the conversion pipe
+  return __hiloint2double(0x43300000, (int)q) - 4503599627370496.0;
+}
+
+__global__ void __launch_bounds__(NT, 2) owc_cd_codes_kernel(Params p) {
+  __shared__ int s_col;
+  __shared__ double s_val[NT / 32];
+  __shared__ int s_idx[NT / 32];
+  extern __shared__ double dyn[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int nwarps = NT / 32;
+  const int d_in = (int)p.d_in, g = (int)p.g, ng = (int)p.ng, nk = p.nk;
+  const long long d_out = p.d_out;
+  const int ntask = ng * nk;
+  double* quad = dyn;                    // [ng, nk] change without its linear part
+  double* sum = quad + ntask;            // [ng, nk] a_k S_k
+  double* rg = sum + ntask;              // [nk, g] residuals of one group
+  double* mg = rg + nk * g;              // [nk, g] H_tt r_k
+  double* delta = mg + nk * g;           // [g]
+  float* as = reinterpret_cast<float*>(delta + g);   // [ng, nk] scales
+  unsigned char* scratch = reinterpret_cast<unsigned char*>(p.scratch) + (size_t)blockIdx.x * p.scratch_per_cta * sizeof(double);
+  double* Gown = reinterpret_cast<double*>(scratch);                                   // [d_in]
+  double* e0 = Gown + d_in;                                                            // [d_in]
+  double* K = e0 + d_in;                                                               // [ng, nk, nk]
+  unsigned char* code = reinterpret_cast<unsigned char*>(K + (size_t)ng * nk * nk);    // [nk, d_in]
+  int* cur = p.cur + (size_t)blockIdx.x * ng;
+  const bool by4 = (d_in & 3) == 0 && (g & 3) == 0;
+  unsigned long long my_moves = 0;
+
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_col = atomicAdd(&p.ctr->next_col, 1);
+    __syncthreads();
+    const long long j = s_col;
+    if (j >= d_out) break;
+
+    // ---- scales and codes of every strength ----
+    for (int task = tid; task < ntask; task += NT) {
+      const int t = task / nk, k = task - t * nk;
+      resid(0.0, (double)p.mn[t * d_out + j], (double)p.mx[t * d_out + j], p.gammas[k], p.L, &as[task], nullptr);
+    }
+    for (int t = tid; t < ng; t += NT) cur[t] = nk - 1;
+    __syncthreads();
+    for (int i = tid; i < d_in; i += NT) {
+      const int t = i / g;
+      const double w = load_w(p.W, p.wt, (long long)i * p.ldw + j);
+      const float lo = p.mn[t * d_out + j];
+      for (int k = 0; k < nk; ++k) {
+        const float a = as[t * nk + k];
+        const unsigned q = a > 0.f ? rtn_code((float)w, a, rtn_inverse(a), lo, (float)p.L) : 0u;
+        code[(size_t)k * d_in + i] = (unsigned char)q;
+        if (k == nk - 1) e0[i] = __dadd_rn(__dadd_rn(__dmul_rn((double)a, (double)q), (double)lo), -w);
+      }
+    }
+    __syncthreads();
+
+    // ---- G = 2 H e and the starting loss ----
+    double* G = p.Gext ? p.Gext + j * p.ldg : Gown;
+    double loss;
+    if (p.Gext) {
+      loss = p.col_before[j];
+    } else {
+      double part = 0.0;
+      for (int pp = warp; pp < d_in; pp += nwarps) {
+        const float* row = p.H + (long long)pp * d_in;
+        double a0 = 0.0, a1 = 0.0;
+        int k = lane;
+        for (; k + 32 < d_in; k += 64) {
+          a0 = fma((double)row[k], e0[k], a0);
+          a1 = fma((double)row[k + 32], e0[k + 32], a1);
+        }
+        if (k < d_in) a0 = fma((double)row[k], e0[k], a0);
+        const double acc = warp_sum(a0 + a1);
+        if (lane == 0) { G[pp] = 2.0 * acc; part = fma(e0[pp], acc, part); }
+      }
+      if (lane == 0) s_val[warp] = part;
+      __syncthreads();
+      loss = 0.0;
+      for (int w = 0; w < nwarps; ++w) loss += s_val[w];
+      __syncthreads();
+      if (tid == 0) p.col_before[j] = loss;
+    }
+
+    // ---- K(t)[k, l] = r_k^T H_tt r_l ----
+    for (int t = 0; t < ng; ++t) {
+      const int t0 = t * g;
+      for (int idx = tid; idx < nk * g; idx += NT) {
+        const int k = idx / g, i = idx - k * g;
+        const double a = (double)as[t * nk + k], q = (double)code[(size_t)k * d_in + t0 + i];
+        // the residual of strength k from that of the last one: the weight is read once per coordinate
+        const double al = (double)as[t * nk + nk - 1], ql = (double)code[(size_t)(nk - 1) * d_in + t0 + i];
+        rg[idx] = e0[t0 + i] + (a * q - al * ql);
+      }
+      __syncthreads();
+      // M(k)[i] = sum_q H[t0 + q][t0 + i] r_k[q] (H is symmetric: neighbouring threads read neighbouring addresses), KC
+      // strengths per value of H
+      const int npass = (nk + KC - 1) / KC;
+      for (int idx = tid; idx < npass * g; idx += NT) {
+        const int ps = idx / g, i = idx - ps * g;
+        const float* col = p.H + (long long)t0 * d_in + t0 + i;
+        const double* r = rg + ps * KC * g;
+        const int kc = min(KC, nk - ps * KC);
+        double acc[KC];
+#pragma unroll
+        for (int c = 0; c < KC; ++c) acc[c] = 0.0;
+#pragma unroll 4
+        for (int q = 0; q < g; ++q) {
+          const double h = (double)col[(long long)q * d_in];
+#pragma unroll
+          for (int c = 0; c < KC; ++c)
+            if (c < kc) acc[c] = fma(h, r[c * g + q], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < KC; ++c)
+          if (c < kc) mg[(ps * KC + c) * g + i] = acc[c];
+      }
+      __syncthreads();
+      for (int pair = warp; pair < nk * nk; pair += nwarps) {
+        const int k = pair / nk, l = pair - k * nk;
+        if (l < k) continue;
+        double v = 0.0;
+        for (int i = lane; i < g; i += 32) v = fma(rg[k * g + i], mg[l * g + i], v);
+        v = warp_sum(v);
+        if (lane == 0) { K[((size_t)t * nk + k) * nk + l] = v; K[((size_t)t * nk + l) * nk + k] = v; }
+      }
+      __syncthreads();
+    }
+    auto refresh_quad = [&](int t, int k) {   // of candidate k of group t
+      const double* kt = K + (size_t)t * nk * nk;
+      const int c = cur[t];
+      quad[t * nk + k] = kt[k * nk + k] - 2.0 * kt[k * nk + c] + kt[c * nk + c];
+    };
+    for (int task = tid; task < ntask; task += NT) refresh_quad(task / nk, task % nk);
+    __syncthreads();
+
+    // ---- descent over the strengths (the loop of Algorithm 3) ----
+    long long nmoves = 0;
+    for (long long step = 0; step < p.steps; ++step) {
+      // a_k sum_i q_k,i G_i: one warp per group and four strengths
+      const int kq = (nk + 3) / 4;
+      for (int wt = warp; wt < ng * kq; wt += nwarps) {
+        const int t = wt / kq, k0 = (wt - t * kq) * 4, t0 = t * g;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        if (by4) {
+          for (int i = 4 * lane; i < g; i += 128) {
+            const double2 g0 = *reinterpret_cast<const double2*>(G + t0 + i), g1 = *reinterpret_cast<const double2*>(G + t0 + i + 2);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (k0 + u < nk) {
+                const unsigned q = *reinterpret_cast<const unsigned*>(code + (size_t)(k0 + u) * d_in + t0 + i);
+                acc[u] = fma(byte_to_double(q & 255u), g0.x, acc[u]);
+                acc[u] = fma(byte_to_double((q >> 8) & 255u), g0.y, acc[u]);
+                acc[u] = fma(byte_to_double((q >> 16) & 255u), g1.x, acc[u]);
+                acc[u] = fma(byte_to_double(q >> 24), g1.y, acc[u]);
+              }
+          }
+        } else {
+          for (int i = lane; i < g; i += 32) {
+            const double gv = G[t0 + i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (k0 + u < nk) acc[u] = fma(byte_to_double(code[(size_t)(k0 + u) * d_in + t0 + i]), gv, acc[u]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double v = warp_sum(acc[u]);
+          if (lane == 0 && k0 + u < nk) sum[t * nk + k0 + u] = (double)as[t * nk + k0 + u] * v;
+        }
+      }
+      __syncthreads();
+      // argmin: lowest (group, grid index) among equal scores; the current strength scores 0 and is never taken
+      double bv = 0.0;
+      int bi = 0x7FFFFFFF;
+      for (int task = tid; task < ntask; task += NT) {
+        const int t = task / nk, k = task - t * nk, c = cur[t];
+        const double v = k == c ? 0.0 : quad[task] + (sum[task] - sum[t * nk + c]);
+        if (v < bv) { bv = v; bi = task; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+        if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+      }
+      if (lane == 0) { s_val[warp] = bv; s_idx[warp] = bi; }
+      __syncthreads();
+      for (int w = 0; w < nwarps; ++w) {
+        const double ov = s_val[w];
+        const int oi = s_idx[w];
+        if (ov < bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+      }
+      if (bi == 0x7FFFFFFF) break;   // (the same in every thread)
+      const int ts = bi / nk, ks = bi - ts * nk, cs = cur[ts];
+      const double ak = (double)as[ts * nk + ks], ac = (double)as[ts * nk + cs];
+      for (int r = tid; r < g; r += NT)
+        delta[r] = ak * (double)code[(size_t)ks * d_in + ts * g + r] - ac * (double)code[(size_t)cs * d_in + ts * g + r];
+      __syncthreads();
+      // G += 2 H[:, group] delta: H is symmetric, so the g rows of the group are read along i
+      const float* rows = p.H + (long long)ts * g * d_in;
+      if ((d_in & 3) == 0) {
+        for (int i = 4 * tid; i < d_in; i += 4 * NT) {
+          double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+#pragma unroll 8
+          for (int r = 0; r < g; ++r) {
+            const float4 h = __ldg(reinterpret_cast<const float4*>(rows + (long long)r * d_in + i));
+            const double dl = delta[r];
+            a0 = fma((double)h.x, dl, a0);
+            a1 = fma((double)h.y, dl, a1);
+            a2 = fma((double)h.z, dl, a2);
+            a3 = fma((double)h.w, dl, a3);
+          }
+          G[i] += 2.0 * a0; G[i + 1] += 2.0 * a1; G[i + 2] += 2.0 * a2; G[i + 3] += 2.0 * a3;
+        }
+      } else {
+        for (int i = tid; i < d_in; i += NT) {
+          double a0 = 0.0;
+          for (int r = 0; r < g; ++r) a0 = fma((double)rows[(long long)r * d_in + i], delta[r], a0);
+          G[i] += 2.0 * a0;
+        }
+      }
+      if (tid == 0) cur[ts] = ks;
+      loss = __dadd_rn(loss, bv);
+      ++nmoves;
+      __syncthreads();
+      if (tid < nk) refresh_quad(ts, tid);
+      // (the sums of the next step are separated from the next use of quad by a barrier)
+    }
+    if (tid == 0) { p.col_after[j] = loss; my_moves += (unsigned long long)nmoves; }
+    __syncthreads();
+
+    // ---- emit grid, codes and strengths of the chosen points ----
+    for (int t = tid; t < ng; t += NT) {
+      p.scale[t * d_out + j] = as[t * nk + cur[t]];
+      p.zero[t * d_out + j] = p.mn[t * d_out + j];
+      if (p.gamma_out) p.gamma_out[t * d_out + j] = (float)p.gammas[cur[t]];
+    }
+    for (int i = tid; i < d_in; i += NT) p.Q[i * d_out + j] = code[(size_t)cur[i / g] * d_in + i];
+  }
+  if (tid == 0 && my_moves) atomicAdd(&p.ctr->moves, my_moves);
+}
+
 }  // namespace owc
 
 // ---------------------------------------------------------------------------------------------
@@ -363,6 +629,7 @@ constexpr int kOwcMaxCtas = 296;
 
 struct OwcWs {
   size_t pmn, pmx, mn, mx, gammas, scratch, cur, col_before, col_after, sums, ctr, E, G, hbuf, ebuf, total;
+  bool codes;         // the kernel on codes (see owc_cd_codes_kernel)
   bool tc;            // starting gradient by the int8 tensor-core GEMM (production mode, large enough layers)
   long long ldg;
   size_t scratch_per_cta;   // doubles
@@ -380,7 +647,9 @@ static OwcWs owc_ws_layout(long long d_in, long long d_out, long long g, int nk,
   w.mx = take(sizeof(float) * ng * d_out);
   w.gammas = take(sizeof(double) * nk);
   const size_t tail = (size_t)(ng * nk > g ? ng * nk : g);
-  w.scratch_per_cta = (2 * (size_t)nk * d_in + (size_t)d_in + tail + 31) / 32 * 32;
+  w.codes = mode == CDQ_MODE_FAST && owc::codes_supported(g, ng, nk);
+  w.scratch_per_cta = w.codes ? (owc::codes_scratch(d_in, ng, nk) / sizeof(double) + 31) / 32 * 32
+                              : (2 * (size_t)nk * d_in + (size_t)d_in + tail + 31) / 32 * 32;
   const long long ctas = d_out < kOwcMaxCtas ? d_out : kOwcMaxCtas;
   w.scratch = take(sizeof(double) * w.scratch_per_cta * ctas);
   w.cur = take(sizeof(int) * ng * ctas);
@@ -448,7 +717,12 @@ cudaError_t launch_owc_cd(const Layer& ly, const cdq_grid_desc& grid, long long 
   // the production kernel keeps two tables of ng * n_clip doubles in shared memory; grids too fine for
   // that run the fixed-order kernel (slower, same result)
   const size_t smem = 2 * sizeof(double) * (size_t)ng * nk;
-  if (mode == CDQ_MODE_FP64_VERIFY || smem > 160 * 1024) {
+  if (L.codes) {
+    const size_t csmem = owc::codes_smem(g, ng, nk);
+    e = cudaFuncSetAttribute(owc::owc_cd_codes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem);
+    if (e != cudaSuccess) return e;
+    { owc::owc_cd_codes_kernel<<<ctas, owc::NT, csmem, st>>>(p); count_launch(); }
+  } else if (mode == CDQ_MODE_FP64_VERIFY || smem > 160 * 1024) {
     p.Gext = nullptr;
     { owc::owc_cd_kernel<true><<<ctas, owc::NT, 0, st>>>(p); count_launch(); }
   } else {
