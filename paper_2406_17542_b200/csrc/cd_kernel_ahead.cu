@@ -15,12 +15,11 @@
 //     (one move in twenty), that move is dropped before it has touched anything but the watched copies.
 //   * When all watched coordinates are down to theta, theta is lowered and the intervals are drawn anew (every 50 to
 //     100 moves).
-// What bounds it: with one team of 8 to 16 warps per SM, latency -- a scheduler has two to four warps and issues in a third
-// of the cycles; the copy, which the sweep used to wait 1700 cycles for, is all but hidden (180 cycles).  Descent,
-// before (copy and sweep in turn, every coordinate scored) -> after: 14336 entries x 1184 columns 277 -> 236 ms, 18432 in
-// groups of 128 x 592 241 -> 206, 16384 x 296 88 -> 72, 15360 x 296 77 -> 60, 11008 x 296 51 -> 47.  Rows of up to 8192
-// entries, of which two or more teams share an SM, hide the copies behind one another's sweeps and do not gain: 8192
-// entries 28.2 -> 27.4 ms, 6144 23.3 -> 23.3, 3072 12.4 -> 15.0, 2048 36.7 -> 62.
+// What bounds it: with one team of 12 or 16 warps per SM, latency -- a scheduler has three or four warps; the copy, which the
+// sweep used to wait 1700 cycles for, is all but hidden (180 cycles).  Descent, before (copy and sweep in turn, every
+// coordinate scored) -> after: 14336 entries x 1184 columns 277 -> 218 ms, 18432 in groups of 128 x 592 241 -> 193,
+// 16384 x 296 88 -> 72, 11008 x 296 51 -> 43.  Rows of up to 8192 entries, of which two or more teams share an SM, hide the
+// copies behind one another's sweeps and do not gain: 8192 entries 27.6 -> 28.9 ms, 5120 23.8 -> 27.8, 3072 12.3 -> 15.9.
 // Every move is the one that scoring all coordinates in fp32 would name: the intervals are drawn with a margin that
 // covers the roundings of the score, and every coordinate outside its interval is scored as the full pass scores it.
 //
@@ -96,6 +95,8 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
   const unsigned below = (1u << lane) - 1u;    // lanes before this one
   const int nchs = (int)(p.d_in >> 2);         // chunks of a row
   const bool exact = nchs == NT * NCH;
+  const bool last_slot = (tid & ~31) + NT * (NCH - 1) < nchs;   // the warp has chunks in the last slot
+  const int asker = NT - 32;                   // the thread that asks for the rows: its warp has no more than the others to sweep
   const float top_q = (float)p.L, top = kMagic + top_q;
 
   constexpr int CHB = ROW16 ? 8 : 16;                                   // bytes of a chunk of 4 row entries
@@ -183,6 +184,11 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
     double c2 = 0.0;                               // twice its step (code units when per-channel)
     [[maybe_unused]] float cur_h = 0.f;            // ROW16: H_ii of its coordinate
 
+    // What the score of a newly watched coordinate needs besides H_ii and the scale, when their loads have had time to arrive.
+    auto watch_ready = [&]() {
+      ws = wh > 0.f ? 0.5f / wh : 0.f;
+      if (GROUPED) ws = (wa > 0.f ? 1.0f / wa : 0.f) * ws;
+    };
     // Score of the watched coordinate.
     auto watch_score = [&](unsigned& key, unsigned& packed) {
       key = kNoMove; packed = kNoMove;
@@ -208,7 +214,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         if (tid == 0) atomicExch(p.status, (int)kFlagBadIndex);
         istar = 0;
       }
-      if (tid == 0) {
+      if (tid == asker) {
         const unsigned char* src = ROW16 ? reinterpret_cast<const unsigned char*>(p.H16 + (long long)istar * p.d_in)
                                          : reinterpret_cast<const unsigned char*>(p.H + (long long)istar * p.d_in);
         mbar_expect_tx(smem_u32(&s_bar[b]), row_bytes);
@@ -262,11 +268,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
               wq = __uint_as_float(kMagicBits | hand[mine].q);
               wi = 4 * ((int)((wid >> 11) & 1023u) + NT * (int)(wid >> 21)) + (int)((wid >> 9) & 3u);
               wh = __ldg(p.hdiag + wi);
-              ws = wh > 0.f ? 0.5f / wh : 0.f;
-              if (GROUPED) {
-                wa = __ldg(scale_j + (long long)group_of((unsigned)wi) * p.d_out);
-                ws = (wa > 0.f ? 1.0f / wa : 0.f) * ws;
-              }
+              if (GROUPED) wa = __ldg(scale_j + (long long)group_of((unsigned)wi) * p.d_out);
               fresh = true;
             }
             who &= ~__ballot_sync(0xFFFFFFFFu, give);
@@ -395,6 +397,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       if (!room) { late_m = how == kAhead ? kFullKey : kCrowdKey; late_w = 0u; }
       if (how == kLower) {   // all that lies above theta is watched now, the best move among it
         unsigned key, packed, m, w;
+        watch_ready();
         watch_score(key, packed);
         const uint2 z = team_min(key, packed, late_m, late_w, m, w);
         if (__any_sync(0xFFFFFFFFu, z.x != kNoMove) || m >= theta_key) {   // not all of it: no lane was idle
@@ -405,7 +408,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         }
         load_step(w, take_move(m, w, buf));
       }
-      if (how != kAhead) fresh = false;   // the move has been chosen with them in view
+      const bool chosen = how != kAhead;   // the move has been chosen with the new ones in view
       how = kAhead;
 
       // ---- the watched coordinates take the move first: they name the next one before the sweep ----
@@ -414,8 +417,9 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       const unsigned char* row = row_s + buf * row_span;
       unsigned key, packed, m, w;
       if (__any_sync(0xFFFFFFFFu, fresh)) {   // does a new one beat the move in flight?
+        watch_ready();
         watch_score(key, packed);
-        const bool beats = fresh && late_m == kNoMove && (key < cur_m || (key == cur_m && packed < cur_w));
+        const bool beats = fresh && !chosen && late_m == kNoMove && (key < cur_m || (key == cur_m && packed < cur_w));
         if (__any_sync(0xFFFFFFFFu, beats)) {
           if (!beats) key = kNoMove;
           late_m = __reduce_min_sync(0xFFFFFFFFu, key);
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       if (timed_out) { key = kAbortKey; packed = 0u; }
       const uint2 z = team_min(key, packed, late_m, late_w, m, w);
       if (m == kAbortKey) {   // a copy never landed: wait (bounded) for it once more, then give up
-        if (tid == 0) {
+        if (tid == asker) {
           mbar_wait_clock32(smem_u32(&s_bar[buf]), ((phases >> buf) & 1u) ^ 1u, kWaitCycles);
           atomicCAS(p.status, (int)kFlagOk, (int)kFlagWaitTimeout);
         }
@@ -467,7 +471,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       // ---- the move stands ----
       const int kcur = (int)(cur_w >> 21), vcur = (int)((cur_w >> 9) & 3u);
       const bool owner = tid == (int)((cur_w >> 11) & 1023u);
-      const double c2_now = c2;
+      const double c2_now = c2, c2_bits = c2 * 0x1p896;
       [[maybe_unused]] const float h_now = cur_h;
       if (owner) {
         const unsigned dq = (unsigned)(int)dri << (8 * vcur);
@@ -484,9 +488,13 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       if (ahead) inext = take_move(m, w, buf ^ 1);
 
       // ---- sweep: g += c2 H[i*, :]; sign bits of threshold - |g| and of g ----
+      // Half of the entries are widened by the conversion pipe (16 per clock and SM, which would be the sweep's bound), half
+      // by moving their bits: without the exponent's bias the double is the entry times 2^-896, which the step makes up
+      // for, exactly (14336 x 1184 columns 226 -> 219 ms).  Infinities and NaN become numbers of 2^128 and more.
       unsigned v0 = 0u, v1 = 0u, n0 = 0u, n1 = 0u;
 #pragma unroll
       for (int k = 0; k < NCH; ++k) {
+        if (k == NCH - 1 && !last_slot) break;   // (the warp's slots are past the end of the row)
         const int cs = tid + NT * k;
         float4 rv;
         if constexpr (ROW16) {
@@ -504,12 +512,20 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         const float hv[4] = {rv.x, rv.y, rv.z, rv.w}, tv[4] = {th.x, th.y, th.z, th.w};
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-          g[4 * k + v] = fma(c2_now, (double)hv[v], g[4 * k + v]);
+          if (v & 1) {   // widened by integer operations
+            const int b = __float_as_int(hv[v]);
+            g[4 * k + v] = fma(c2_bits, __hiloint2double((b >> 3) & (int)0x8FFFFFFFu, b << 29), g[4 * k + v]);
+          } else {
+            g[4 * k + v] = fma(c2_now, (double)hv[v], g[4 * k + v]);
+          }
           const int hi = __double2hiint(g[4 * k + v]);
           const int s = __float_as_int(tv[v] - fabsf(__int_as_float(hi)));
           if (k < W0) { v0 = __funnelshift_l((unsigned)s, v0, 1); n0 = __funnelshift_l((unsigned)hi, n0, 1); }
           else { v1 = __funnelshift_l((unsigned)s, v1, 1); n1 = __funnelshift_l((unsigned)hi, n1, 1); }
         }
+      }
+      if (!last_slot) {
+        if (NCH <= W0) { v0 <<= 4; n0 <<= 4; } else { v1 <<= 4; n1 <<= 4; }
       }
       if (last) break;   // budget used up
       if (ahead) {
@@ -592,17 +608,15 @@ cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st) {
   if (p.d_in & 3) return cudaErrorNotSupported;
   if ((reinterpret_cast<uintptr_t>(p.H) & 15) != 0) return cudaErrorNotSupported;
   if (p.H16 && ((p.d_in & 7) != 0 || (reinterpret_cast<uintptr_t>(p.H16) & 15) != 0)) return cudaErrorNotSupported;
-  // Few threads with many chunks each: no spills, a cheaper argmin exchange, fixed costs per thread spread over more
-  // state; full warps in equal numbers per scheduler.  256 threads hold up to 14 chunks each in registers; beyond that the
-  // team is the smallest of 10..12 x 384 and 8 x 512 chunk slots that holds the row.
   const long long ch = p.d_in >> 2;
   auto team = [&](long long chunks, int nch) { return (int)((chunks + nch - 1) / nch + 31) / 32 * 32; };
-  if (ch <= 2304) return launch_mode<9, 256, 1>(p, team(ch, 9), st);
-  if (ch <= 2560) return launch_mode<10, 256, 1>(p, team(ch, 10), st);
-  if (ch <= 2816) return launch_mode<11, 256, 1>(p, team(ch, 11), st);
-  if (ch <= 3072) return launch_mode<12, 256, 1>(p, team(ch, 12), st);
-  if (ch <= 3328) return launch_mode<13, 256, 1>(p, team(ch, 13), st);
-  if (ch <= 3584) return launch_mode<14, 256, 1>(p, team(ch, 14), st);
+  // 384 threads as long as the row fits them: three warps per scheduler hide more latency than the two of 256 threads with up to
+  // 14 chunks each (14336 x 1184 columns 236 -> 226 ms, 11008 x 296 47.4 -> 43.3), and at 168 registers nothing spills; rows of
+  // 15361 to 16384 entries fill 8 x 512 slots (72 ms against 75 for 11 x 384 on 16384 x 296; 9 x 512 spills: 18432 x 592 226 ms
+  // against 210 for 12 x 384).
+  if (ch <= 2304) return launch_mode<6, 384, 1>(p, team(ch, 6), st);
+  if (ch <= 3072) return launch_mode<8, 384, 1>(p, team(ch, 8), st);
+  if (ch <= 3456) return launch_mode<9, 384, 1>(p, team(ch, 9), st);
   if (ch <= 3840) return launch_mode<10, 384, 1>(p, team(ch, 10), st);
   if (ch <= 4096) return launch_mode<8, 512, 1>(p, team(ch, 8), st);
   if (ch <= 4224) return launch_mode<11, 384, 1>(p, team(ch, 11), st);
