@@ -166,6 +166,7 @@ struct Params {
   int group_s[MAX_GROUPS];            // i + j of the group (slices numbered from 1)
   signed char pair_e[MAX_SLICES * MAX_SLICES], pair_h[MAX_SLICES * MAX_SLICES];  // slice indices (from 0)
   double* C;                // [M, ldc] fp64
+  int keep_c;               // C is wanted (else only the column dots are, and C holds the running sums in between)
   long long ldc;
   const int* eexp;          // [M]
   const int* hexp;          // [N]
@@ -213,6 +214,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+
+// Exact, and on the fp64 pipe instead of the conversion pipe.
+__device__ __forceinline__ double int_to_double(uint32_t r) {
+  return __hiloint2double(0x43300000, (int)(r ^ 0x80000000u)) - 4503601774854144.0;   // 2^52 + 2^31
+}
+// 2^e for the exponents of normal numbers (those of products of fp32 data are).
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 // Tiles are handed out in bands of 8 tile rows, column by column inside a band, so that the
 // tiles in flight at one time share their operand panels in L2.
@@ -330,10 +338,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
     }
   } else {
     // ---------------- epilogue: TMEM -> fp64 running sum in C ----------------
-    // Two warps per TMEM lane quarter; they take the 16-column chunks of the tile in turn.
+    // Two warps per TMEM lane quarter; they take the 16-column chunks of the tile in turn.  A product of two groups (the
+    // screen of the clipping search) waits for both accumulators and needs no running sum.
     const int q = warp & 3;                 // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;       // which of the two warps of the quarter
     const int row = q * 32 + lane;          // row of the tile
+    const bool both = p.ngroups == 2;
     int buf = 0;
     uint32_t tphase = 0;
     bool ok = true;
@@ -346,60 +356,72 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
       double* crow = p.C + (row_ok ? j : 0) * p.ldc;
       const int ej = row_ok ? p.eexp[j] : 0;
       double dot = 0.0;
-      for (int g = 0; g < p.ngroups && ok; ++g) {
-        if (!mbar_wait(tfull_bar(buf), tphase, abort_flag)) { ok = false; break; }
+      for (int g = both ? 1 : 0; g < p.ngroups && ok; ++g) {
+        if (both && !mbar_wait(tfull_bar(buf ^ 1), tphase, abort_flag)) { ok = false; break; }
+        if (both) buf ^= 1;   // (buf: the accumulator of group g; groups 0 and 1 lie in buffers 0 and 1)
+        if (!mbar_wait(tfull_bar(both ? 0 : buf), tphase, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const double w = ldexp(1.0, -7 * p.group_s[g]);
+        const double w = pow2(-7 * p.group_s[g]), w0 = pow2(-7 * p.group_s[0]);
         const bool first = g == 0, last = g == p.ngroups - 1;
 #pragma unroll 1
         for (int c = half; c < BN / 16; c += 2) {
-          uint32_t r[16];
+          uint32_t r[16], r0[16];
           tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 16), r);
+          if (both) tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), r0);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (row_ok) {
-            const long long pc0 = p0 + c * 16;
-            if (pc0 + 16 <= p.N) {
-              // whole chunk inside the matrix: 16-byte accesses (ldc is a multiple of 4, pc0 of 16)
-              double2* cp = reinterpret_cast<double2*>(crow + pc0);
+          if (!row_ok) continue;
+          const long long pc0 = p0 + c * 16;
+          if (pc0 + 16 <= p.N) {
+            // whole chunk inside the matrix: 16-byte accesses (ldc is a multiple of 4, pc0 of 16)
+            double2* cp = reinterpret_cast<double2*>(crow + pc0);
+            double x[16];
+#pragma unroll
+            for (int v = 0; v < 16; ++v) x[v] = w * int_to_double(r[v]);
+            if (both) {
+#pragma unroll
+              for (int v = 0; v < 16; ++v) x[v] += w0 * int_to_double(r0[v]);
+            } else if (!first) {
               double2 old[8];
-              if (!first) {
 #pragma unroll
-                for (int v = 0; v < 8; ++v) old[v] = cp[v];
+              for (int v = 0; v < 8; ++v) old[v] = cp[v];
+#pragma unroll
+              for (int v = 0; v < 8; ++v) { x[2 * v] += old[v].x; x[2 * v + 1] += old[v].y; }
+            }
+            if (last) {
+#pragma unroll
+              for (int v = 0; v < 16; ++v) x[v] = x[v] * p.final_scale * pow2(ej + p.hexp[pc0 + v]);
+              if (p.dot_part) {
+#pragma unroll
+                for (int v = 0; v < 16; ++v) dot = fma(p.E[(pc0 + v) * p.lde + j], x[v], dot);
               }
+            }
+            if (!last || p.keep_c) {
 #pragma unroll
-              for (int v = 0; v < 8; ++v) {
-                double x0 = w * (double)(int)r[2 * v], x1 = w * (double)(int)r[2 * v + 1];
-                if (!first) { x0 += old[v].x; x1 += old[v].y; }
+              for (int v = 0; v < 8; ++v) cp[v] = make_double2(x[2 * v], x[2 * v + 1]);
+            }
+          } else {
+#pragma unroll
+            for (int v = 0; v < 16; ++v) {
+              const long long pc = pc0 + v;
+              if (pc < p.N) {
+                double x = w * int_to_double(r[v]);
+                if (both) x += w0 * int_to_double(r0[v]);
+                else if (!first) x += crow[pc];
                 if (last) {
-                  x0 = ldexp(x0 * p.final_scale, ej + p.hexp[pc0 + 2 * v]);
-                  x1 = ldexp(x1 * p.final_scale, ej + p.hexp[pc0 + 2 * v + 1]);
-                  if (p.dot_part) {
-                    dot = fma(p.E[(pc0 + 2 * v) * p.lde + j], x0, dot);
-                    dot = fma(p.E[(pc0 + 2 * v + 1) * p.lde + j], x1, dot);
-                  }
+                  x = x * p.final_scale * pow2(ej + p.hexp[pc]);
+                  if (p.dot_part) dot = fma(p.E[pc * p.lde + j], x, dot);
                 }
-                cp[v] = make_double2(x0, x1);
-              }
-            } else {
-#pragma unroll
-              for (int v = 0; v < 16; ++v) {
-                const long long pc = pc0 + v;
-                if (pc < p.N) {
-                  double x = w * (double)(int)r[v];
-                  if (!first) x += crow[pc];
-                  if (last) {
-                    x = ldexp(x * p.final_scale, ej + p.hexp[pc]);
-                    if (p.dot_part) dot = fma(p.E[pc * p.lde + j], x, dot);
-                  }
-                  crow[pc] = x;
-                }
+                if (!last || p.keep_c) crow[pc] = x;
               }
             }
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(tempty_bar(buf));
+        if (lane == 0) {
+          if (both) mbar_arrive(tempty_bar(0));
+          mbar_arrive(tempty_bar(buf));
+        }
         if (++buf == 2) { buf = 0; tphase ^= 1u; }
       }
       if (p.dot_part && row_ok && ok) p.dot_part[(size_t)(2 * tn + half) * p.M + j] = dot;
@@ -487,7 +509,7 @@ static cudaError_t encode_map3(CUtensorMap* map, const void* base, long long kp,
 // (ne, nh, smax); optionally col_loss[j] = sum_p E[p, j] C[j, p] / scale.
 // hbuf: from gemm_tc_prepare_h with the same nh.  ebuf: gemm_tc_e_bytes of scratch.
 cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
-                        double scale, double* C, long long ldc, double* col_loss, void* ebuf, cudaStream_t st) {
+                        double scale, double* C, bool keep_c, long long ldc, double* col_loss, void* ebuf, cudaStream_t st) {
   using namespace i8;
   if (nh < 1 || nh > MAX_SLICES || ne < 1 || ne > MAX_SLICES || smax < 2) return cudaErrorInvalidValue;
   const long long kp = tc_kpad(d_in);
@@ -524,7 +546,7 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double
   if (ng == 0) return cudaErrorInvalidValue;
   p.group_first[ng] = npairs;
   p.ngroups = ng;
-  p.C = C; p.ldc = ldc; p.eexp = eexp; p.hexp = hexp; p.final_scale = scale;
+  p.C = C; p.keep_c = keep_c ? 1 : 0; p.ldc = ldc; p.eexp = eexp; p.hexp = hexp; p.final_scale = scale;
   p.E = E; p.lde = d_out; p.dot_part = col_loss ? dot_part : nullptr;
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;

@@ -443,7 +443,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.g = g; src.d_out = d_out;
         if (gb > 1) { src.n_cols = width; src.k0 = k0; src.gammas = gammas; }   // column c: layer column c % d_out
         e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
-                        (double*)(base + L.C), L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
+                        (double*)(base + L.C), false, L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
       }
       { owc_candidates_kernel<<<bx, 128, 0, st>>>(screen, n_clip, d_out, mask, table); count_launch(); }
@@ -466,7 +466,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.mn = mn; src.mx = mx; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out; src.col_idx = cj + b0; src.n_cols = width;
         src.col_gamma = ck + b0; src.gammas = gammas;
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), false, L.ldc,
                         loss_c, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
         { owc_scatter_kernel<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(loss_c, cj + b0, ck + b0, width, d_out, table); count_launch(); }
@@ -478,7 +478,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
       src.mn = mn; src.mx = mx; src.gamma = hg[k]; src.L = ly.L; src.use_gamma = 1;
       src.g = g; src.d_out = d_out;
       if (L.tc) {
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), false, L.ldc,
                         table + (long long)k * d_out, base + L.ebuf, st);
       } else {
         e = launch_residual_f64(src, d_in, E, st);

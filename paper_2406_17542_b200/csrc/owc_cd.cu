@@ -709,7 +709,7 @@ cudaError_t launch_owc_cd(const Layer& ly, const cdq_grid_desc& grid, long long 
     e = gemm_tc_prepare_h(ly.H, d_in, kTcGradNH, base + L.hbuf, st);
     if (e != cudaSuccess) return e;
     p.Gext = (double*)(base + L.G); p.ldg = L.ldg;
-    e = gemm_tc_run(base + L.hbuf, kTcGradNH, src, E, d_in, d_out, kTcGradNE, kTcGradSmax, 2.0, p.Gext, p.ldg, p.col_before,
+    e = gemm_tc_run(base + L.hbuf, kTcGradNH, src, E, d_in, d_out, kTcGradNE, kTcGradSmax, 2.0, p.Gext, true, p.ldg, p.col_before,
                     base + L.ebuf, st);
     if (e != cudaSuccess) return e;
   }
