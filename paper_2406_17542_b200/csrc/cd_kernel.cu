@@ -205,10 +205,14 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
 #pragma unroll
       for (int k = 0; k < NCH; ++k) {
         const int chunk = tid + NT * k;
-        if (EXACT) row[k] = ld_row4(rp + (long long)chunk * 4);
+        // the rows of the shortest layers (1 MB at 512 entries) may stay in L1, longer ones would only pass through it
+        auto load = [&]() {
+          return NCH <= 2 ? __ldg(reinterpret_cast<const float4*>(rp) + chunk) : ld_row4(rp + (long long)chunk * 4);
+        };
+        if (EXACT) row[k] = load();
         else {
           row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (chunk < nchunks) row[k] = ld_row4(rp + (long long)chunk * 4);
+          if (chunk < nchunks) row[k] = load();
         }
       }
       SweepBest sb;
@@ -400,7 +404,9 @@ cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, co
   if (H16) return cudaErrorNotSupported;
   auto team = [&](int ept) { return (int)(((d + ept - 1) / ept + 31) / 32 * 32); };
   if (d <= 512) return launch_cd_shape<2, 64, 8>(p, team(8), st);
-  return launch_cd_shape<4, 256, 3>(p, team(16), st);
+  // three chunks per thread: more warps per column than four hide more of a step's latency (768 x 8192 2.00 -> 1.64 ms, 1152 x
+  // 8192 6.7 -> 5.4, 1350 x 677 1.56 -> 1.44), and two cost more in the exchange (1350 x 677 1.78)
+  return launch_cd_shape<3, 128, 6>(p, team(12), st);
 }
 
 // ---------------------------------------------------------------------------

@@ -14,8 +14,84 @@ constexpr int GM = 128;  // tile of p (rows of H)
 constexpr int GN = 64;   // tile of j (columns of the layer)
 constexpr int GK = 16;
 
+constexpr int GS = 32;   // tile of the small kernel, both ways
+
+// Layers with fewer than 74 tiles of 128 x 64 leave more than half of the SMs idle: they take tiles of 32 x 32 (256 x 256:
+// 47 us in 8 tiles).
+static bool small_tiles(long long d_in, long long d_out) {
+  return ((d_in + GM - 1) / GM) * ((d_out + GN - 1) / GN) < 74;
+}
+static long long row_tiles(long long d_in, long long d_out) {
+  const int m = small_tiles(d_in, d_out) ? GS : GM;
+  return (d_in + m - 1) / m;
+}
 size_t gemm_partials_elems(long long d_in, long long d_out) {
-  return (size_t)((d_in + GM - 1) / GM) * (size_t)d_out;
+  return (size_t)row_tiles(d_in, d_out) * (size_t)d_out;
+}
+
+// The product of gemm_he_kernel in tiles of 32 x 32, two by two entries per thread; the next stage's loads are in flight while
+// the present one is used.
+__global__ void __launch_bounds__(256) gemm_he_small_kernel(const float* __restrict__ H, long long d_in, long long d_out,
+                                                            const double* __restrict__ E, double* __restrict__ G,
+                                                            long long ldg, double* __restrict__ part) {
+  constexpr int KS = 32, LD = KS * GS / 256;
+  __shared__ __align__(16) double sA[KS][GS + 2];   // sA[k][p]
+  __shared__ __align__(16) double sB[KS][GS + 2];   // sB[k][j]
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const long long p0 = (long long)blockIdx.y * GS, j0 = (long long)blockIdx.x * GS;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  float a[LD];
+  double b[LD];
+  auto fetch = [&](long long k0) {
+#pragma unroll
+    for (int e = 0; e < LD; ++e) {
+      const int r = (tid >> 5) + 8 * e, c = tid & 31;
+      a[e] = (p0 + r < d_in && k0 + c < d_in) ? H[(p0 + r) * d_in + k0 + c] : 0.f;        // row p0 + r, along k
+      b[e] = (k0 + r < d_in && j0 + c < d_out) ? E[(k0 + r) * d_out + j0 + c] : 0.0;      // row k0 + r, along j
+    }
+  };
+  fetch(0);
+  for (long long k0 = 0; k0 < d_in; k0 += KS) {
+#pragma unroll
+    for (int e = 0; e < LD; ++e) {
+      const int r = (tid >> 5) + 8 * e, c = tid & 31;
+      sA[c][r] = (double)a[e];
+      sB[r][c] = b[e];
+    }
+    __syncthreads();
+    if (k0 + KS < d_in) fetch(k0 + KS);
+#pragma unroll
+    for (int kk = 0; kk < KS; ++kk) {
+      const double2 x = *reinterpret_cast<const double2*>(&sA[kk][2 * ty]), y = *reinterpret_cast<const double2*>(&sB[kk][2 * tx]);
+      acc[0][0] = fma(x.x, y.x, acc[0][0]);
+      acc[0][1] = fma(x.x, y.y, acc[0][1]);
+      acc[1][0] = fma(x.y, y.x, acc[1][0]);
+      acc[1][1] = fma(x.y, y.y, acc[1][1]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const long long j = j0 + 2 * tx + v;
+    double t = 0.0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const long long p = p0 + 2 * ty + u;
+      if (p >= d_in || j >= d_out) continue;
+      if (G) G[j * ldg + p] = 2.0 * acc[u][v];
+      if (part) t = fma(E[p * d_out + j], acc[u][v], t);
+    }
+    sA[ty][2 * tx + v] = t;
+  }
+  if (part) {
+    __syncthreads();
+    if (tid < GS && j0 + tid < d_out) {
+      double t = 0.0;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) t += sA[r][tid];
+      part[(long long)blockIdx.y * d_out + j0 + tid] = t;
+    }
+  }
 }
 
 __global__ void __launch_bounds__(256) gemm_he_kernel(const float* __restrict__ H, long long d_in, long long d_out,
@@ -147,10 +223,16 @@ __global__ void partials_reduce_kernel(const double* __restrict__ part, long lon
 
 cudaError_t launch_gemm_he(const float* H, long long d_in, long long d_out, const double* E, double* G,
                            long long ldg, double* col_loss, double* part, cudaStream_t st) {
-  dim3 grid((unsigned)((d_out + GN - 1) / GN), (unsigned)((d_in + GM - 1) / GM));
-  { gemm_he_kernel<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); }
+  const long long tiles = row_tiles(d_in, d_out);
+  if (small_tiles(d_in, d_out)) {
+    const dim3 grid((unsigned)((d_out + GS - 1) / GS), (unsigned)tiles);
+    { gemm_he_small_kernel<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); }
+  } else {
+    const dim3 grid((unsigned)((d_out + GN - 1) / GN), (unsigned)tiles);
+    { gemm_he_kernel<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); }
+  }
   if (col_loss)
-    { partials_reduce_kernel<<<(unsigned)((d_out + 127) / 128), 128, 0, st>>>(part, (d_in + GM - 1) / GM, d_out, col_loss); count_launch(); }
+    { partials_reduce_kernel<<<(unsigned)((d_out + 127) / 128), 128, 0, st>>>(part, tiles, d_out, col_loss); count_launch(); }
   return cudaGetLastError();
 }
 

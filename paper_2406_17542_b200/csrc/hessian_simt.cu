@@ -56,97 +56,122 @@ cudaError_t launch_hessian_verify(const void* X, cdq_dtype xt, long long n, long
 }
 
 // ---- tiled SIMT kernel -----------------------------------------------------
-// T x T tiles of the lower triangle, (T / M)^2 threads with M x M entries each, fp64 fused multiply-adds in ascending
-// order of the rows, whatever the tile.  Bound by the fp64 pipe (64 per clock and SM): the operands are widened once,
-// when a stage is stored to shared memory (widening them at every use kept the conversion pipe busy twice as long as the
-// fp64 pipe: 1.2 ms at 4099 rows by 1350 features), and the next stage's loads are issued before the present stage is used.
-// T = 64 for layers whose tiles fill the SMs; smaller tiles for narrow ones, where a 64-tile list leaves most SMs idle
-// (256 features: 10 tiles, 140 us at 1024 rows).
-constexpr int HK = 16;   // rows of X per stage
-
-template <typename TX, int T, int M>
-__global__ void __launch_bounds__((T / M) * (T / M)) hessian_simt_kernel(const TX* __restrict__ X, long long n, long long d_in,
-                                                                         long long ldx, int accumulate, float* __restrict__ H) {
-  // Only tiles on or below the diagonal are computed; the mirror image is written too.
-  const int tp = blockIdx.y, tr = blockIdx.x;
-  if (tr > tp) return;
-  constexpr int TT = T / M, NTH = TT * TT, LD = HK * T / NTH;
-  __shared__ __align__(16) double sa[HK][T + 2];
-  __shared__ __align__(16) double sb[HK][T + 2];
-  const int tx = threadIdx.x % TT, ty = threadIdx.x / TT;
-  const long long p0 = (long long)tp * T, r0 = (long long)tr * T;
-  double acc[M][M];
+// TP x TR tiles that reach the lower triangle, MP x MR entries per thread, fp64 fused multiply-adds.  The operands are
+// widened once, when a stage is stored to shared memory (widening them at every use kept the conversion pipe busy twice as
+// long as the fp64 pipe), and the next stage's loads are issued before the present stage is used.  What bounds the wide
+// tile is shared memory: MP / 2 + MR / 2 loads of 16 bytes per MP MR multiply-adds, so it takes 8 x 4 per thread; 1350 features
+// by 4099 rows: 1.2 ms with floats in shared memory, 0.8 with 4 x 4.  Narrow layers, which have few tiles, are bound by the chain of
+// multiply-adds behind an entry: they take smaller tiles, and KS groups of threads take every KS-th row of a stage, their sums
+// added in a fixed order (256 features by 1024 rows: 140 us with 64 x 64 tiles, 33 with 16 x 16 and one group).
+template <typename TX, int TP, int TR, int MP, int MR, int HK, int KS>
+__global__ void __launch_bounds__((TP / MP) * (TR / MR) * KS) hessian_simt_kernel(const TX* __restrict__ X, long long n,
+                                                                                  long long d_in, long long ldx, int accumulate,
+                                                                                  float* __restrict__ H) {
+  const long long p0 = (long long)blockIdx.y * TP, r0 = (long long)blockIdx.x * TR;
+  if (r0 > p0 + TP - 1) return;   // above the diagonal: the mirror image is written from below it
+  constexpr int NP = TP / MP, NR = TR / MR, NTH = NP * NR * KS, LP = HK * TP / NTH, LR = HK * TR / NTH;
+  static_assert(HK * TP % NTH == 0 && HK * TR % NTH == 0 && HK % KS == 0 && MP % 2 == 0 && MR % 2 == 0, "whole loads");
+  __shared__ __align__(16) double sa[HK][TP + 2];
+  __shared__ __align__(16) double sb[HK][TR + 2];
+  __shared__ double red[KS > 1 ? (KS - 1) * TP * TR : 1];
+  const int ks = threadIdx.x / (NP * NR), tx = threadIdx.x % NR, ty = threadIdx.x / NR % NP;
+  double acc[MP][MR];
 #pragma unroll
-  for (int a = 0; a < M; ++a)
+  for (int a = 0; a < MP; ++a)
 #pragma unroll
-    for (int b = 0; b < M; ++b) acc[a][b] = 0.0;
-  TX xa[LD], xb[LD];
+    for (int b = 0; b < MR; ++b) acc[a][b] = 0.0;
+  TX xa[LP], xb[LR];
   auto fetch = [&](long long k0) {
 #pragma unroll
-    for (int e = 0; e < LD; ++e) {
-      const int idx = threadIdx.x + e * NTH, kk = idx / T, cc = idx % T;
-      const long long k = k0 + kk;
-      xa[e] = (k < n && p0 + cc < d_in) ? X[k * ldx + p0 + cc] : TX(0.f);
-      xb[e] = (k < n && r0 + cc < d_in) ? X[k * ldx + r0 + cc] : TX(0.f);
+    for (int e = 0; e < LP; ++e) {
+      const int idx = threadIdx.x + e * NTH, kk = idx / TP, cc = idx % TP;
+      xa[e] = (k0 + kk < n && p0 + cc < d_in) ? X[(k0 + kk) * ldx + p0 + cc] : TX(0.f);
+    }
+#pragma unroll
+    for (int e = 0; e < LR; ++e) {
+      const int idx = threadIdx.x + e * NTH, kk = idx / TR, cc = idx % TR;
+      xb[e] = (k0 + kk < n && r0 + cc < d_in) ? X[(k0 + kk) * ldx + r0 + cc] : TX(0.f);
     }
   };
   fetch(0);
   for (long long k0 = 0; k0 < n; k0 += HK) {
 #pragma unroll
-    for (int e = 0; e < LD; ++e) {
-      const int idx = threadIdx.x + e * NTH, kk = idx / T, cc = idx % T;
-      sa[kk][cc] = (double)(float)xa[e];
-      sb[kk][cc] = (double)(float)xb[e];
+    for (int e = 0; e < LP; ++e) {
+      const int idx = threadIdx.x + e * NTH;
+      sa[idx / TP][idx % TP] = (double)(float)xa[e];
+    }
+#pragma unroll
+    for (int e = 0; e < LR; ++e) {
+      const int idx = threadIdx.x + e * NTH;
+      sb[idx / TR][idx % TR] = (double)(float)xb[e];
     }
     __syncthreads();
     if (k0 + HK < n) fetch(k0 + HK);
 #pragma unroll
-    for (int kk = 0; kk < HK; ++kk) {
-      double a[M], b[M];
+    for (int k = 0; k < HK / KS; ++k) {
+      const int kk = k * KS + ks;
+      double a[MP], b[MR];
+      // (a thread's entries are pairs of neighbours, so that the 16-byte loads of neighbouring threads are contiguous)
 #pragma unroll
-      for (int u = 0; u < M; u += 2) {
-        // (a thread's entries are pairs of neighbours, so that the 16-byte loads of neighbouring threads are contiguous)
-        const double2 va = *reinterpret_cast<const double2*>(&sa[kk][u * TT + 2 * ty]);
-        const double2 vb = *reinterpret_cast<const double2*>(&sb[kk][u * TT + 2 * tx]);
-        a[u] = va.x; a[u + 1] = va.y; b[u] = vb.x; b[u + 1] = vb.y;
+      for (int u = 0; u < MP; u += 2) {
+        const double2 va = *reinterpret_cast<const double2*>(&sa[kk][u * NP + 2 * ty]);
+        a[u] = va.x; a[u + 1] = va.y;
       }
 #pragma unroll
-      for (int u = 0; u < M; ++u)
+      for (int u = 0; u < MR; u += 2) {
+        const double2 vb = *reinterpret_cast<const double2*>(&sb[kk][u * NR + 2 * tx]);
+        b[u] = vb.x; b[u + 1] = vb.y;
+      }
 #pragma unroll
-        for (int v = 0; v < M; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+      for (int u = 0; u < MP; ++u)
+#pragma unroll
+        for (int v = 0; v < MR; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
     }
     __syncthreads();
   }
+  if constexpr (KS > 1) {
+    const int t = threadIdx.x % (NP * NR);
 #pragma unroll
-  for (int u = 0; u < M; ++u)
+    for (int u = 0; u < MP; ++u)
 #pragma unroll
-    for (int v = 0; v < M; ++v) {
-      const long long p = p0 + (u & ~1) * TT + 2 * ty + (u & 1), r = r0 + (v & ~1) * TT + 2 * tx + (v & 1);
-      if (p < d_in && r < d_in) {
+      for (int v = 0; v < MR; ++v)
+        if (ks > 0) red[((ks - 1) * MP * MR + u * MR + v) * NP * NR + t] = acc[u][v];
+    __syncthreads();
+    if (ks > 0) return;
+    for (int s = 0; s < KS - 1; ++s)
+#pragma unroll
+      for (int u = 0; u < MP; ++u)
+#pragma unroll
+        for (int v = 0; v < MR; ++v) acc[u][v] += red[(s * MP * MR + u * MR + v) * NP * NR + t];
+  }
+#pragma unroll
+  for (int u = 0; u < MP; ++u)
+#pragma unroll
+    for (int v = 0; v < MR; ++v) {
+      const long long p = p0 + (u & ~1) * NP + 2 * ty + (u & 1), r = r0 + (v & ~1) * NR + 2 * tx + (v & 1);
+      if (p < d_in && r <= p) {
         const float prev = accumulate ? H[p * d_in + r] : 0.f;
         const float val = (float)((double)prev + acc[u][v]);
         H[p * d_in + r] = val;
-        if (tp != tr) H[r * d_in + p] = val;   // (a diagonal tile computes every entry directly)
+        if (r < p) H[r * d_in + p] = val;
       }
     }
 }
 
-template <int T, int M>
+template <int TP, int TR, int MP, int MR, int HK, int KS>
 static void run_hessian_simt(const void* X, cdq_dtype xt, long long n, long long d_in, long long ldx, int accumulate,
                              float* H, cudaStream_t st) {
-  const unsigned t = (unsigned)((d_in + T - 1) / T);
-  dim3 grid(t, t), block((T / M) * (T / M));
+  const dim3 grid((unsigned)((d_in + TR - 1) / TR), (unsigned)((d_in + TP - 1) / TP)), block((TP / MP) * (TR / MR) * KS);
   if (xt == CDQ_BF16)
-    { hessian_simt_kernel<__nv_bfloat16, T, M><<<grid, block, 0, st>>>((const __nv_bfloat16*)X, n, d_in, ldx, accumulate, H); count_launch(); }
+    { hessian_simt_kernel<__nv_bfloat16, TP, TR, MP, MR, HK, KS><<<grid, block, 0, st>>>((const __nv_bfloat16*)X, n, d_in, ldx, accumulate, H); count_launch(); }
   else
-    { hessian_simt_kernel<float, T, M><<<grid, block, 0, st>>>((const float*)X, n, d_in, ldx, accumulate, H); count_launch(); }
+    { hessian_simt_kernel<float, TP, TR, MP, MR, HK, KS><<<grid, block, 0, st>>>((const float*)X, n, d_in, ldx, accumulate, H); count_launch(); }
 }
 
 cudaError_t launch_hessian_simt(const void* X, cdq_dtype xt, long long n, long long d_in, long long ldx,
                                 int accumulate, float* H, cudaStream_t st) {
-  if (d_in <= 512) run_hessian_simt<16, 2>(X, xt, n, d_in, ldx, accumulate, H, st);
-  else if (d_in <= 1024) run_hessian_simt<32, 2>(X, xt, n, d_in, ldx, accumulate, H, st);
-  else run_hessian_simt<64, 4>(X, xt, n, d_in, ldx, accumulate, H, st);
+  if (d_in <= 512) run_hessian_simt<16, 16, 2, 2, 64, 4>(X, xt, n, d_in, ldx, accumulate, H, st);
+  else run_hessian_simt<64, 32, 4, 4, 32, 2>(X, xt, n, d_in, ldx, accumulate, H, st);
   return cudaGetLastError();
 }
 

@@ -138,16 +138,15 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
 // ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  Memory-bound: 8 bytes written
 // per entry.  (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
 // strengths of a 4096 x 4096 layer, 0.16 ms of them the maxima.)
-constexpr int kResRows = 32;   // rows per block, all of one group
 template <int V, bool BF16>
-__global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int blocks_per_group, double* __restrict__ E,
+__global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_per_block, int blocks_per_group, double* __restrict__ E,
                                                        unsigned long long* __restrict__ colmax) {
   const long long c = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x);   // column of E
   const long long width = s.n_cols ? s.n_cols : s.d_out;
   if (c >= width) return;
   const long long j = s.col_idx ? (long long)s.col_idx[c] : c % s.d_out;        // column of the layer
-  const long long t = blockIdx.y / blocks_per_group, i0 = t * s.g + (blockIdx.y % blocks_per_group) * (long long)kResRows;
-  const long long i1 = min(i0 + kResRows, (t + 1) * s.g);
+  const long long t = blockIdx.y / blocks_per_group, i0 = t * s.g + (blockIdx.y % blocks_per_group) * (long long)rows_per_block;
+  const long long i1 = min(i0 + rows_per_block, (t + 1) * s.g);
   float a[V], b[V], inv[V];
   double m[V];
 #pragma unroll
@@ -209,13 +208,14 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int blocks
 
 cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st, unsigned long long* colmax) {
   const long long width = src.n_cols ? src.n_cols : src.d_out;
-  const int bpg = (int)((src.g + kResRows - 1) / kResRows);
+  // rows per block, all of one group: few on small layers, which have no more blocks to offer
+  const int rows = width * d_in >= (1ll << 22) ? 32 : 4, bpg = (int)((src.g + rows - 1) / rows);
   const size_t esz = src.wt == CDQ_BF16 ? 2 : 4;
   // four columns per thread: rows of W, Q and E on the vectors' boundaries, four neighbouring columns of one strength
   const bool four = !src.col_idx && src.d_out % 4 == 0 && src.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(src.W) % (4 * esz) == 0 &&
                     reinterpret_cast<uintptr_t>(src.Q) % 4 == 0 && width * (d_in / src.g) * bpg >= (1 << 17);
   const dim3 grid((unsigned)((width + (four ? 511 : 127)) / (four ? 512 : 128)), (unsigned)(d_in / src.g * bpg));
-  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, bpg, E, colmax); count_launch(); };
+  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, rows, bpg, E, colmax); count_launch(); };
   if (src.wt == CDQ_BF16) run(four ? residual_kernel<4, true> : residual_kernel<1, true>);
   else run(four ? residual_kernel<4, false> : residual_kernel<1, false>);
   return cudaGetLastError();
