@@ -65,6 +65,22 @@ def test_descent_result_does_not_depend_on_the_other_columns():
     assert torch.equal(Qs, Q[:, some])
 
 
+@pytest.mark.parametrize("d_in,at", [(8704, 4096), (8704, 4097), (8704, 8703), (9001, 9000), (4096, 33)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_a_feature_that_is_not_a_number_shows_in_the_loss(d_in, at, value):
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=150, bits=3, seed=43)
+    H = _layer_h(cfg, 512)
+    H[at, :] = value
+    H[:, at] = value
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q0, _ = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    stats, loss, per = B.cdq_cd_solve_with_loss(H, W, grid, scale, zero, Q, 40, per_col=True)
+    assert B.load().cdq_last_device_status() == 0
+    assert not np.isfinite(loss) and not bool(torch.isfinite(per).any())
+
+
 @pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
 def test_hessian_pieces_and_mirror(d_in, width):
     """bf16 rows with a stride longer than d_in through the tensor-core kernel: every entry against fp64 (3e-5 of
