@@ -1,5 +1,6 @@
 // extern "C" entry points declared in include/cdq.h: argument validation, workspace
 // carving and kernel sequencing.  No device memory is allocated here.
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -438,18 +439,25 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
     double* col_after = per_col_out ? per_col_out : col_loss;   // col_loss has been summed into loss_sum[0] by now
     CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
     CDQ_CUDA(launch_loss_from_gradient(E, G, L.ldg, d_in, d_out, col_after, st));
-    if (loss_out) {
-      CDQ_CUDA(launch_sum_f64_tree(col_after, d_out, loss_sum + 1, st));
-      CDQ_CUDA(cudaMemcpyAsync(loss_out, loss_sum + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
-      if (!stats) CDQ_CUDA(cudaStreamSynchronize(st));
+    if (loss_out) CDQ_CUDA(launch_sum_f64_tree(col_after, d_out, loss_sum + 1, st));
+  }
+  // What the host wants lies side by side and comes in one copy: a copy to pageable memory waits for itself, 10 us each.
+  struct { double before, after; char pad[48]; CdCounters ctr; } host;
+  static_assert(offsetof(decltype(host), ctr) == 64, "the layout of the workspace's scalars");
+  int flag = kFlagOk;
+  if (stats || (loss_from_g && loss_out)) {
+    CDQ_CUDA(cudaMemcpyAsync(&host, loss_sum, sizeof(host), cudaMemcpyDeviceToHost, st));
+    if (stats) {
+      const int* status = device_status_word();
+      if (!status) return CDQ_ERR_CUDA;
+      CDQ_CUDA(cudaMemcpyAsync(&flag, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     }
+    CDQ_CUDA(cudaStreamSynchronize(st));
+    if (loss_from_g && loss_out) *loss_out = host.after;
   }
   if (stats) {
-    CdCounters hc;
-    double lb = 0.0;
-    CDQ_CUDA(cudaMemcpyAsync(&hc, ctr, sizeof(CdCounters), cudaMemcpyDeviceToHost, st));
-    CDQ_CUDA(cudaMemcpyAsync(&lb, loss_sum, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CDQ_CUDA(cudaStreamSynchronize(st));
+    const CdCounters& hc = host.ctr;
+    const double lb = host.before;
     stats->steps = (unsigned long long)steps_per_col * (unsigned long long)d_out;
     stats->committed = hc.committed;
     stats->columns_converged = hc.converged;
@@ -458,8 +466,10 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
     float ms = 0.f;
     CDQ_CUDA(cudaEventElapsedTime(&ms, ev0, ev1));
     stats->kernel_ms = (double)ms;
-    const cdq_status ds = read_device_status_after_sync();
-    if (ds != CDQ_OK) return ds;
+    if (flag != kFlagOk) {
+      const cdq_status ds = read_device_status_after_sync();
+      if (ds != CDQ_OK) return ds;
+    }
   }
   if (want_loss && !loss_from_g)
     return cdq_layer_loss(H, W, wt, d_in, d_out, ldw, grid, scale, zero, Q, loss_out, per_col_out, mode, ws, ws_bytes, stream);
