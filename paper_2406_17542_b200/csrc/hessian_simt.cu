@@ -58,11 +58,12 @@ cudaError_t launch_hessian_verify(const void* X, cdq_dtype xt, long long n, long
 // ---- tiled SIMT kernel -----------------------------------------------------
 // TP x TR tiles that reach the lower triangle, MP x MR entries per thread, fp64 fused multiply-adds.  The operands are
 // widened once, when a stage is stored to shared memory (widening them at every use kept the conversion pipe busy twice as
-// long as the fp64 pipe), and the next stage's loads are issued before the present stage is used.  What bounds the wide
-// tile is shared memory: MP / 2 + MR / 2 loads of 16 bytes per MP MR multiply-adds, so it takes 8 x 4 per thread; 1350 features
-// by 4099 rows: 1.2 ms with floats in shared memory, 0.8 with 4 x 4.  Narrow layers, which have few tiles, are bound by the chain of
-// multiply-adds behind an entry: they take smaller tiles, and KS groups of threads take every KS-th row of a stage, their sums
-// added in a fixed order (256 features by 1024 rows: 140 us with 64 x 64 tiles, 33 with 16 x 16 and one group).
+// long as the fp64 pipe), and the next stage's loads are issued before the present stage is used.  What bounds it is shared
+// memory (MP / 2 + MR / 2 loads of 16 bytes per MP MR multiply-adds) and idle SMs: 1350 features by 4099 rows took 1.2 ms with
+// floats in shared memory, 0.9 in 128 x 64 tiles with 8 x 4, 0.8 in 64 x 64 with 4 x 4, 0.7 in 64 x 32 tiles with two groups of
+// threads that take every other row of a stage (KS groups, their sums added in a fixed order).  Narrow layers are bound by the
+// chain of multiply-adds behind an entry: 16 x 16 tiles and four groups (256 features by 1024 rows: 140 us with 64 x 64 tiles,
+// 33 with 16 x 16 and one group, 21 with four).
 template <typename TX, int TP, int TR, int MP, int MR, int HK, int KS>
 __global__ void __launch_bounds__((TP / MP) * (TR / MR) * KS) hessian_simt_kernel(const TX* __restrict__ X, long long n,
                                                                                   long long d_in, long long ldx, int accumulate,
