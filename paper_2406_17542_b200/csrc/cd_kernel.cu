@@ -41,6 +41,20 @@ cudaError_t launch_diag(const float* H, long long d_in, long long d_pad, float* 
   return cudaGetLastError();
 }
 
+// A feature whose calibration inputs held an infinity or a NaN has no gradient, in any column, and so the loss is none: the
+// descent of the long rows widens every second entry of a row by its bits and would make such values finite.
+__global__ void mark_features_kernel(const float* __restrict__ H, long long d_in, long long d_out, double* __restrict__ G,
+                                     long long ldg) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (i >= d_in || fabsf(H[i * d_in + i]) <= 3.402823466e38f) return;
+  for (long long j = 0; j < d_out; ++j) G[j * ldg + i] = __longlong_as_double(0x7FF8000000000000ll);
+}
+
+cudaError_t launch_mark_features(const float* H, long long d_in, long long d_out, double* G, long long ldg, cudaStream_t st) {
+  { mark_features_kernel<<<(unsigned)((d_in + 127) / 128), 128, 0, st>>>(H, d_in, d_out, G, ldg); count_launch(); }
+  return cudaGetLastError();
+}
+
 // dst[c][r] = src[r][c] for byte matrices with leading dimensions, 32x32 tiles through shared memory.
 __global__ void transpose_u8_kernel(const unsigned char* __restrict__ src, long long rows, long long cols,
                                     long long ld_src, unsigned char* __restrict__ dst, long long ld_dst) {
@@ -399,7 +413,7 @@ cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, co
   // short rows are quickest as plain loads into registers, longer ones as bulk copies into shared memory
   // (measured crossover: 1536 entries 2.0 against 2.5 ms, 1792 entries 11.5 against 10.8, 2048 entries 52.0 against 45.3);
   // from 8192 entries on, where one team fills an SM, the next row travels during the sweep (see cd_kernel_ahead.cu)
-  if (d > 8192) return launch_cd_ahead(p, st);
+  if (cd_long_rows(d)) return launch_cd_ahead(p, st);
   if (d > 1536) return launch_cd_tma(p, st);
   if (H16) return cudaErrorNotSupported;
   auto team = [&](int ept) { return (int)(((d + ept - 1) / ept + 31) / 32 * 32); };

@@ -160,13 +160,6 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         }
         g[4 * k] = g0.x * gscale; g[4 * k + 1] = g0.y * gscale; g[4 * k + 2] = g1.x * gscale; g[4 * k + 3] = g1.y * gscale;
       }
-      // A feature whose calibration inputs held an infinity or a NaN: its gradient is none, and so is the loss (the sweep widens
-      // every second entry of a row without looking for such values).
-#pragma unroll
-      for (int e = 0; e < 4 * NCH; ++e) {
-        const long long i = 4ll * (tid + NT * (e >> 2)) + (e & 3);
-        if (i < p.d_in && !(fabsf(p.H[i * (p.d_in + 1)]) <= 3.402823466e38f)) g[e] = __longlong_as_double(0x7FF8000000000000ll);
-      }
     }
 
     // ---- descent ----
@@ -498,7 +491,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       // Half of the entries are widened by the conversion pipe (16 per clock and SM, which would be the sweep's bound), half
       // by moving their bits: without the exponent's bias the double is the entry times 2^-896, which the step makes up
       // for, exactly (14336 x 1184 columns 226 -> 219 ms).  (Infinities and NaN
-      // would become numbers of 2^128 and more: see the column's prologue.)
+      // would become numbers of 2^128 and more: see mark_features_kernel.)
       unsigned v0 = 0u, v1 = 0u, n0 = 0u, n1 = 0u;
 #pragma unroll
       for (int k = 0; k < NCH; ++k) {

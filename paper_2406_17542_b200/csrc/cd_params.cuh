@@ -6,7 +6,7 @@
 namespace cdq {
 
 struct CdParams {
-  const float* H;
+  const float* H;             // as many rows as the layer has inputs: the padding of d_in below has none
   const __nv_bfloat16* H16;   // bf16 copy of H for the rows of the update (NULL: fp32 rows)
   long long d_in, d_out;      // d_in: entries of a row, a multiple of 4 (zeros pad odd layers: H_ii = 0, so nothing moves there)
   double* G;            // [d_out, ldg]

@@ -81,6 +81,39 @@ def test_a_feature_that_is_not_a_number_shows_in_the_loss(d_in, at, value):
     assert not np.isfinite(loss) and not bool(torch.isfinite(per).any())
 
 
+class _ExactWorkspace:
+    """A workspace of exactly the bytes asked for, between bytes of 0xFF (NaN as floats and doubles) that the library has
+    no business with."""
+    GUARD = 1 << 20      # rows of padding are at most 3 x 18432 floats
+
+    def get(self, nbytes, device):
+        self.need = nbytes
+        self.buf = torch.full((nbytes + 2 * self.GUARD,), 0xFF, dtype=torch.uint8, device=device)
+        return self.buf.data_ptr() + self.GUARD, nbytes
+
+    def guards_intact(self):
+        return bool((self.buf[:self.GUARD] == 0xFF).all()) and bool((self.buf[self.GUARD + self.need:] == 0xFF).all())
+
+
+@pytest.mark.parametrize("d_in", [1029, 5001, 8193, 8194, 8195, 9001, 18431])
+def test_padding_of_odd_rows_takes_nothing_from_behind_the_workspace(d_in):
+    """The padding coordinates of an odd layer have no row in H.  Their gradients lie in the workspace (behind the residual,
+    [columns, d_in rounded up to 4] doubles) and stay zero whatever follows the workspace in memory."""
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=3, bits=3, seed=44)
+    H = _layer_h(cfg, 256)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
+    ws = _ExactWorkspace()
+    _, loss, per = B.cdq_cd_solve_with_loss(H, W, grid, scale, zero, Q, 30, per_col=True, ws=ws)
+    assert B.load().cdq_last_device_status() == 0
+    assert np.isfinite(loss) and bool(torch.isfinite(per).all()) and ws.guards_intact()
+    ldg = (d_in + 3) // 4 * 4
+    off = ws.GUARD + (8 * d_in * 3 + 255) // 256 * 256
+    G = ws.buf[off:off + 8 * 3 * ldg].view(torch.float64).view(3, ldg)
+    assert bool((G[:, d_in:] == 0).all()) and bool(torch.isfinite(G).all())
+
+
 @pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
 def test_hessian_pieces_and_mirror(d_in, width):
     """bf16 rows with a stride longer than d_in through the tensor-core kernel: every entry against fp64 (3e-5 of
