@@ -86,8 +86,9 @@ struct SolveWs {
   bool tc;        // H E on the int8 tensor cores
   int nh, ne, smax;
 };
-SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool with_cd, long long bcd_steps = 0,
-                        bool rows16 = false) {
+// pad_rows: the greedy descent runs on a copy of H with rows on 16-byte boundaries (see descent_pads_rows).
+SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool with_cd, bool pad_rows = false,
+                        long long bcd_steps = 0, bool rows16 = false) {
   SolveWs w{};
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
@@ -119,9 +120,19 @@ SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool wit
     w.h16 = take(sizeof(__nv_bfloat16) * (size_t)d_in * d_in);
     w.hr = take(sizeof(float) * (size_t)d_in * d_in);
   }
-  if (with_cd && mode == CDQ_MODE_FAST && d_in % 4) w.hpad = take(sizeof(float) * (size_t)d_in * w.ldg);
+  if (pad_rows) {   // the slices of H and the residual are done with when the descent begins: the copy takes their place if it fits
+    const size_t bytes = sizeof(float) * (size_t)d_in * w.ldg;
+    if (w.tc) w.hpad = w.hbuf;   // six bytes per entry of rows of at least ldg
+    else w.hpad = bytes <= sizeof(double) * (size_t)d_in * d_out ? w.E : take(bytes);
+  }
   w.total = off;
   return w;
+}
+
+// Greedy descents whose rows of H do not lie on 16-byte boundaries and that run in the fast kernels.
+bool descent_pads_rows(long long d_in, const cdq_grid_desc* grid, cdq_mode mode) {
+  const long long g = grid && grid->group_size > 0 ? grid->group_size : d_in;
+  return mode == CDQ_MODE_FAST && d_in % 4 != 0 && cd_fast_supported(d_in, g);
 }
 
 ResidualSrc codes_src(const Layer& ly, const unsigned char* Q) {
@@ -258,16 +269,19 @@ size_t cdq_workspace_bytes(cdq_call which, long long n, long long d_in, long lon
     }
     case CDQ_CALL_CD_SOLVE:
       if (d_out < 1) return 0;
-      return solve_ws_layout(d_in, d_out, mode, true).total;
-    case CDQ_CALL_BCD_SOLVE:  // n: steps per column
+      return solve_ws_layout(d_in, d_out, mode, true, descent_pads_rows(d_in, grid, mode)).total;
+    case CDQ_CALL_BCD_SOLVE: {  // n: steps per column; the block size is not known here: the larger of the two
       if (d_out < 1 || n < 0) return 0;
-      return solve_ws_layout(d_in, d_out, mode, true, n).total;
+      const size_t greedy = solve_ws_layout(d_in, d_out, mode, true, descent_pads_rows(d_in, grid, mode)).total;
+      const size_t pairs = d_in % 2 ? 0 : solve_ws_layout(d_in, d_out, mode, true, false, n).total;
+      return greedy > pairs ? greedy : pairs;
+    }
     case CDQ_CALL_LAYER_LOSS:
       if (d_out < 1) return 0;
       return solve_ws_layout(d_in, d_out, mode, false).total;
     case CDQ_CALL_CD_SOLVE_ROWS16:
       if (d_out < 1) return 0;
-      return solve_ws_layout(d_in, d_out, mode, true, 0, true).total;
+      return solve_ws_layout(d_in, d_out, mode, true, false, 0, true).total;
   }
   return 0;
 }
@@ -366,7 +380,8 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
     const long long g = grid->group_size > 0 ? grid->group_size : d_in;
     if (mode != CDQ_MODE_FAST || block != 1 || !cd_rows16_supported(d_in, g)) return CDQ_ERR_UNSUPPORTED;
   }
-  const SolveWs L = solve_ws_layout(d_in, d_out, mode, true, block > 1 ? steps_per_col : 0, rows16);
+  const bool pad_rows = block == 1 && descent_pads_rows(d_in, grid, mode);
+  const SolveWs L = solve_ws_layout(d_in, d_out, mode, true, pad_rows, block > 1 ? steps_per_col : 0, rows16);
   s = check_ws(ws, ws_bytes, L.total);
   if (s != CDQ_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
@@ -417,7 +432,7 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
     CDQ_CUDA(launch_diag(H, d_in, L.d_pad, hdiag, half_inv, st));
     if (cd_long_rows(L.ldg)) CDQ_CUDA(launch_mark_features(H, d_in, d_out, G, L.ldg, st));
     const float* rows = H;
-    if (d_in % 4) {   // odd rows of H on 16-byte boundaries (1350 entries: 5 us for the copy, and the descent 0.6 of its time)
+    if (pad_rows) {   // odd rows of H on 16-byte boundaries (1350 entries: 5 us for the copy, and the descent 0.6 of its time)
       float* hpad = (float*)(base + L.hpad);
       CDQ_CUDA(launch_pad_rows(H, d_in, L.ldg, hpad, st));
       CDQ_CUDA(cudaMemset2DAsync(G + d_in, sizeof(double) * L.ldg, 0, sizeof(double) * (L.ldg - d_in), d_out, st));

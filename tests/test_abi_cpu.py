@@ -60,6 +60,21 @@ def test_workspace_sizes(lib):
     assert owc_cd > 2 * 20 * 4096 * 8
 
 
+def test_padded_rows_of_odd_layers_cost_workspace_only_where_nothing_else_lies_idle(lib):
+    """The descent's copy of H with rows on 16-byte boundaries (4 bytes per entry) takes the place of the residual or of the
+    slices of H; only narrow layers, which have neither, get room for it, and calls that never build it get none."""
+    need = lambda which, d_in, d_out, g=0, n=0, mode="fast": B.workspace_bytes(which, n, d_in, d_out, B.Grid(3, g), mode)
+    for d_in, d_out in [(8193, 150), (18431, 256), (1350, 677), (301, 200), (255, 255), (129, 70)]:
+        up = (d_in + 3) // 4 * 4
+        assert need(B.CALL_CD_SOLVE, d_in, d_out) <= need(B.CALL_CD_SOLVE, up, d_out)
+    assert need(B.CALL_CD_SOLVE, 8193, 3) >= 4 * 8193 * 8196
+    # the fixed-order kernel: rows past the fast kernels' range, groups that are not a multiple of four, the verification mode
+    for d_in, d_out, g, mode in [(20001, 8, 0, "fast"), (8190, 8, 10, "fast"), (8193, 8, 0, "verify")]:
+        assert need(B.CALL_CD_SOLVE, d_in, d_out, g, mode=mode) < 4 * d_in * d_in
+    # pairs with 4 d_in steps need more for their table than the copy would take
+    assert need(B.CALL_BCD_SOLVE, 1026, 8, n=4104) < need(B.CALL_BCD_SOLVE, 1028, 8, n=4104) + 4096
+
+
 def test_bad_arguments_are_rejected_before_any_launch(lib):
     gd = B.Grid(bits=3).c()
     dummy = ctypes.c_void_p(256)  # never dereferenced: validation fails first

@@ -95,11 +95,13 @@ class _ExactWorkspace:
         return bool((self.buf[:self.GUARD] == 0xFF).all()) and bool((self.buf[self.GUARD + self.need:] == 0xFF).all())
 
 
-@pytest.mark.parametrize("d_in", [1029, 5001, 8193, 8194, 8195, 9001, 18431])
-def test_padding_of_odd_rows_takes_nothing_from_behind_the_workspace(d_in):
+# (few columns: the padded copy of H is the last block; 200 columns of 301: in the place of the residual; the rest: of the slices)
+@pytest.mark.parametrize("d_in,d_out", [(1029, 3), (5001, 3), (8193, 3), (8194, 3), (8195, 3), (9001, 3), (18431, 3), (301, 200),
+                                        (1351, 300), (8202, 130)])
+def test_padding_of_odd_rows_takes_nothing_from_behind_the_workspace(d_in, d_out):
     """The padding coordinates of an odd layer have no row in H.  Their gradients lie in the workspace (behind the residual,
     [columns, d_in rounded up to 4] doubles) and stay zero whatever follows the workspace in memory."""
-    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=3, bits=3, seed=44)
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=d_out, bits=3, seed=44)
     H = _layer_h(cfg, 256)
     W = inputs.make_w(cfg, device=DEV)
     grid = grid_of(cfg)
@@ -109,9 +111,30 @@ def test_padding_of_odd_rows_takes_nothing_from_behind_the_workspace(d_in):
     assert B.load().cdq_last_device_status() == 0
     assert np.isfinite(loss) and bool(torch.isfinite(per).all()) and ws.guards_intact()
     ldg = (d_in + 3) // 4 * 4
-    off = ws.GUARD + (8 * d_in * 3 + 255) // 256 * 256
-    G = ws.buf[off:off + 8 * 3 * ldg].view(torch.float64).view(3, ldg)
+    off = ws.GUARD + (8 * d_in * d_out + 255) // 256 * 256
+    G = ws.buf[off:off + 8 * d_out * ldg].view(torch.float64).view(d_out, ldg)
     assert bool((G[:, d_in:] == 0).all()) and bool(torch.isfinite(G).all())
+    want, cols = B.cdq_layer_loss(H, W, grid, scale, zero, Q, per_col=True)
+    assert abs(loss - want) <= 1e-9 * want and bool(((per - cols).abs() <= 1e-9 * cols).all())
+
+
+def test_pairs_need_no_room_for_padded_rows():
+    """Pairs read H as it is: a workspace for the descent without the padded copy is enough (1026 entries: 4.2 MB)."""
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=1026, d_out=8, bits=3, seed=45)
+    H = _layer_h(cfg, 1100)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
+    Q2 = Q.clone()
+    want = B.cdq_bcd_solve(H, W, grid, scale, zero, Q, 2, 16, seed=3)
+
+    class Smaller(_ExactWorkspace):   # less the padded copy, plus the pairs of 16 steps (16 bytes each)
+        def get(self, nbytes, device):
+            return super().get(nbytes - (4 * 1026 * 1028) // 256 * 256 + 16 * 16 * 1026, device)
+
+    ws = Smaller()
+    got = B.cdq_bcd_solve(H, W, grid, scale, zero, Q2, 2, 16, seed=3, ws=ws)
+    assert torch.equal(Q, Q2) and got["committed"] == want["committed"] and ws.guards_intact()
 
 
 @pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
