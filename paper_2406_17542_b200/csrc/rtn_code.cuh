@@ -1,8 +1,9 @@
 // The round-to-nearest code of one weight (paper: Eq. 2).
 //
 // The code is the fp64 rounding of (w - b) / a, half to even, clamped to the grid.  The fp32 quotient is off by at most
-// 3 * 2^-24 of itself, 5e-5 where it is within 256 levels, so unless it lies within 2e-4 of the middle between two
-// levels both round to the same level; the one in 2500 that does is decided in fp64.
+// 3 * 2^-24 of itself (6 * 2^-24 where the inverse of the scale is subnormal), 1e-4 where it is within 256 levels, so
+// unless it lies within 2e-4 of the middle between two levels both round to the same level; the one in 2500 that does is
+// decided in fp64, and so is a quotient that is none or overflows (groups that span more than 3.4e38).
 #pragma once
 
 #include "common.cuh"
@@ -27,7 +28,7 @@ __device__ __forceinline__ unsigned rtn_code(float w, float a, float inv_a, floa
   const float t = (w - b) * inv_a;
   const float c = fminf(fmaxf(t, 0.f), top);
   const float m = c + kMagic;
-  if (!(fabsf(c - (m - kMagic)) < 0.4998f) || t != t) return rtn_code_f64(w, a, b, top);
+  if (!(fabsf(c - (m - kMagic)) < 0.4998f) || !(fabsf(t) <= 3.402823466e38f)) return rtn_code_f64(w, a, b, top);
   return __float_as_uint(m) & 255u;
 }
 

@@ -198,3 +198,28 @@ def test_codes_of_weights_between_two_levels(d_in, d_out, bits, g, dtype):
     scale, zero, Q, _ = B.cdq_init_rtn(Wt.to(DEV), B.Grid(bits, g))
     assert np.array_equal(scale.cpu().numpy(), want["scale"]) and np.array_equal(zero.cpu().numpy(), want["zero"])
     assert np.array_equal(Q.cpu().numpy(), want["Q"])
+
+
+@pytest.mark.parametrize("d_in,d_out,bits,g,dtype", [
+    (64, 32, 2, 0, "f32"), (64, 32, 3, 16, "f32"), (96, 33, 8, 0, "bf16"), (4096, 1024, 4, 0, "f32"),
+])
+def test_codes_of_groups_that_span_more_than_the_largest_float(d_in, d_out, bits, g, dtype):
+    """w - b overflows in fp32 (the scale does not, from two bits on): the oracle's codes all the same, in the codes and in the
+    residuals of the clipping search."""
+    rng = np.random.default_rng(bits)
+    Wt = torch.from_numpy((3e38 * (2 * rng.random((d_in, d_out)) - 1)).astype(np.float32))
+    if dtype == "bf16":
+        Wt = Wt.bfloat16()
+    want = oracle.init_rtn(Wt, bits, g, 1, 1.0, 1.0)
+    scale, zero, Q, _ = B.cdq_init_rtn(Wt.to(DEV), B.Grid(bits, g))
+    assert np.array_equal(scale.cpu().numpy(), want["scale"]) and np.array_equal(zero.cpu().numpy(), want["zero"])
+    assert np.array_equal(Q.cpu().numpy(), want["Q"])
+    if d_in > 96:
+        return
+    X = torch.from_numpy(rng.standard_normal((4 * d_in, d_in)).astype(np.float32))
+    H = (X.double().T @ X.double()).float()
+    # (strengths from 0.5: the library takes the ends of the grid as floats, the oracle as doubles, and 0.6 is another number as each)
+    want = oracle.init_rtn(Wt, bits, g, 5, 0.5, 1.0, H=H.numpy())
+    scale, zero, Q, gamma = B.cdq_init_rtn(Wt.to(DEV), B.Grid(bits, g, 5, 0.5, 1.0), H=H.to(DEV))
+    assert np.array_equal(gamma.cpu().numpy(), oracle.gamma_grid(5, 0.5, 1.0).astype(np.float32)[want["gamma_idx"]])
+    assert np.array_equal(scale.cpu().numpy(), want["scale"]) and np.array_equal(Q.cpu().numpy(), want["Q"])
