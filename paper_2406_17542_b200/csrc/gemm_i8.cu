@@ -75,8 +75,11 @@ __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bit
 // |x| 2^-e 128^ns, truncated, as an integer (x 2^-e in (-1, 1), ns <= 6): slice i of x is its 7-bit digit number ns - i from
 // below with the sign of x, which is what truncating, subtracting and scaling up digit by digit gives.  The addition of
 // 2^52 towards zero leaves the integer in the mantissa; scale = 2^(7 ns - e), a normal number for every exponent of H and E.
+// A NaN counts as zero, whatever its payload (that of CUDA's float NaN would pass for digits): a product leaves out the
+// entry and keeps the rest of its row.
 __device__ __forceinline__ unsigned long long slice_bits(double x, double scale) {
-  return (unsigned long long)__double_as_longlong(__dadd_rz(fabs(x) * scale, 4503599627370496.0)) & 0xFFFFFFFFFFFFFull;
+  const double s = __dadd_rz(fabs(x) * scale, 4503599627370496.0);
+  return s != s ? 0ull : (unsigned long long)__double_as_longlong(s) & 0xFFFFFFFFFFFFFull;
 }
 // Digit i (from 1) of four neighbours, negated where `neg` has the byte's bits set, as four bytes.
 __device__ __forceinline__ unsigned slice_bytes(const unsigned long long (&v)[4], int shift, unsigned neg) {

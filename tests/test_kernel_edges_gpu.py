@@ -137,6 +137,45 @@ def test_pairs_need_no_room_for_padded_rows():
     assert torch.equal(Q, Q2) and got["committed"] == want["committed"] and ws.guards_intact()
 
 
+def _float_of_bits(bits):
+    return torch.from_numpy(np.array([bits], dtype=np.uint32).view(np.int32)).to(DEV).view(torch.float32)
+
+
+# (layers whose gradient comes from the int8 product, for each of the descent's kernels)
+@pytest.mark.parametrize("d_in,d_out", [(512, 1600), (1024, 600), (2048, 128), (8704, 128)])
+@pytest.mark.parametrize("bits", [0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF, 0x7F800001])
+def test_a_nan_is_left_out_of_the_gradient_whatever_its_payload(d_in, d_out, bits):
+    """0x7FFFFFFF is the NaN that CUDA's arithmetic makes, 0x7FC00000 that of a Python literal.  A NaN weight takes code 0 and
+    leaves its column as one with the zero of the grid there, a NaN feature of H its layer as one without the feature; the
+    losses show both."""
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=d_out, bits=3, seed=46)
+    H = _layer_h(cfg, 768)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    T = min(d_in, 600)
+    nan = _float_of_bits(bits)
+
+    def solve(Hs, Ws):
+        scale, zero, Q, _ = B.cdq_init_rtn(Ws, grid)
+        _, loss, per = B.cdq_cd_solve_with_loss(Hs, Ws, grid, scale, zero, Q, T, per_col=True)
+        assert B.load().cdq_last_device_status() == 0
+        return Q, per
+
+    Wn, Wz = W.clone(), W.clone()
+    Wn[5, 3:4] = nan
+    Wz[5, 3] = torch.cat([W[:5, 3], W[6:, 3]]).min()
+    Q, per = solve(H, Wn)
+    Qz, perz = solve(H, Wz)
+    assert torch.equal(Q, Qz)
+    assert bool(per[3].isnan()) and torch.equal(per[:3], perz[:3]) and torch.equal(per[4:], perz[4:])
+    Hn, Hz = H.clone(), H.clone()
+    Hn[7, :], Hn[:, 7] = nan.expand(d_in), nan.expand(d_in)
+    Hz[7, :], Hz[:, 7] = 0.0, 0.0
+    Q, per = solve(Hn, W)
+    Qz, _ = solve(Hz, W)
+    assert torch.equal(Q, Qz) and bool(per.isnan().all())
+
+
 @pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
 def test_hessian_pieces_and_mirror(d_in, width):
     """bf16 rows with a stride longer than d_in through the tensor-core kernel: every entry against fp64 (3e-5 of
