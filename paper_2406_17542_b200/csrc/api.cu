@@ -409,7 +409,7 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
     CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, base + L.hbuf, st));
     CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 2.0, G, true, L.ldg, col_loss, base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
-    CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, G, L.ldg, col_loss, part, st));
+    CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, G, L.ldg, col_loss, part, gemm_tc_supported(d_in, d_out), st));
   } else {
     CDQ_CUDA(launch_gemm_he_verify(H, d_in, d_out, E, part, G, L.ldg, col_loss, st));
   }
@@ -558,7 +558,7 @@ cdq_status cdq_layer_loss(const float* H, const void* W, cdq_dtype wt, long long
     CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), false, L.ldg, col_loss,
                          base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
-    CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, st));
+    CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, gemm_tc_supported(d_in, d_out), st));
   } else {
     CDQ_CUDA(launch_gemm_he_verify(H, d_in, d_out, E, part, nullptr, 0, col_loss, st));
   }

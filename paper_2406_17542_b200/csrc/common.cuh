@@ -93,10 +93,10 @@ cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* 
 // gemm_f64.cu : C = H * E in fp64.
 // G (may be NULL): [d_out, ldg] doubles, G[j][p] = 2 * C[p][j].
 // col_loss (may be NULL): [d_out] doubles, e_j^T H e_j = sum_p E[p][j] C[p][j]; needs the
-// scratch `part` of gemm_partials_elems(d_in, d_out) doubles.
+// scratch `part` of gemm_partials_elems(d_in, d_out) doubles.  leave_nan_out: NaN operands of the product count as zero.
 size_t gemm_partials_elems(long long d_in, long long d_out);
 cudaError_t launch_gemm_he(const float* H, long long d_in, long long d_out, const double* E,
-                           double* G, long long ldg, double* col_loss, double* part, cudaStream_t st);
+                           double* G, long long ldg, double* col_loss, double* part, bool leave_nan_out, cudaStream_t st);
 // fixed-order version (ascending k, no fused multiply-add)
 // C: scratch of d_in * d_out doubles.
 cudaError_t launch_gemm_he_verify(const float* H, long long d_in, long long d_out, const double* E, double* C,

@@ -29,8 +29,16 @@ size_t gemm_partials_elems(long long d_in, long long d_out) {
   return (size_t)row_tiles(d_in, d_out) * (size_t)d_out;
 }
 
+// LEAVE_NAN_OUT: a NaN in an operand counts as zero, as it does in the int8 product, so that a layer on either side of the line
+// between the two keeps the rest of a column with a NaN weight, and of a layer with a NaN feature.  (The column dots take E as it is.)
+template <bool LEAVE_NAN_OUT, typename T>
+__device__ __forceinline__ double operand(T x) {
+  return LEAVE_NAN_OUT && x != x ? 0.0 : (double)x;
+}
+
 // The product of gemm_he_kernel in tiles of 32 x 32, two by two entries per thread; the next stage's loads are in flight while
 // the present one is used.
+template <bool LEAVE_NAN_OUT>
 __global__ void __launch_bounds__(256) gemm_he_small_kernel(const float* __restrict__ H, long long d_in, long long d_out,
                                                             const double* __restrict__ E, double* __restrict__ G,
                                                             long long ldg, double* __restrict__ part) {
@@ -55,8 +63,8 @@ __global__ void __launch_bounds__(256) gemm_he_small_kernel(const float* __restr
 #pragma unroll
     for (int e = 0; e < LD; ++e) {
       const int r = (tid >> 5) + 8 * e, c = tid & 31;
-      sA[c][r] = (double)a[e];
-      sB[r][c] = b[e];
+      sA[c][r] = operand<LEAVE_NAN_OUT>(a[e]);
+      sB[r][c] = operand<LEAVE_NAN_OUT>(b[e]);
     }
     __syncthreads();
     if (k0 + KS < d_in) fetch(k0 + KS);
@@ -94,6 +102,7 @@ __global__ void __launch_bounds__(256) gemm_he_small_kernel(const float* __restr
   }
 }
 
+template <bool LEAVE_NAN_OUT>
 __global__ void __launch_bounds__(256) gemm_he_kernel(const float* __restrict__ H, long long d_in, long long d_out,
                                                       const double* __restrict__ E, double* __restrict__ G,
                                                       long long ldg, double* __restrict__ part) {
@@ -131,7 +140,7 @@ __global__ void __launch_bounds__(256) gemm_he_kernel(const float* __restrict__ 
         }
       }
 #pragma unroll
-      for (int e = 0; e < 8; ++e) sA[a_k + e][a_p] = (double)a[e];
+      for (int e = 0; e < 8; ++e) sA[a_k + e][a_p] = operand<LEAVE_NAN_OUT>(a[e]);
     }
     {  // B tile
       const long long k = k0 + b_k;
@@ -148,7 +157,7 @@ __global__ void __launch_bounds__(256) gemm_he_kernel(const float* __restrict__ 
         }
       }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) sB[b_k][b_j + e] = b[e];
+      for (int e = 0; e < 4; ++e) sB[b_k][b_j + e] = operand<LEAVE_NAN_OUT>(b[e]);
     }
     __syncthreads();
 #pragma unroll
@@ -222,15 +231,13 @@ __global__ void partials_reduce_kernel(const double* __restrict__ part, long lon
 }
 
 cudaError_t launch_gemm_he(const float* H, long long d_in, long long d_out, const double* E, double* G,
-                           long long ldg, double* col_loss, double* part, cudaStream_t st) {
+                           long long ldg, double* col_loss, double* part, bool leave_nan_out, cudaStream_t st) {
   const long long tiles = row_tiles(d_in, d_out);
-  if (small_tiles(d_in, d_out)) {
-    const dim3 grid((unsigned)((d_out + GS - 1) / GS), (unsigned)tiles);
-    { gemm_he_small_kernel<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); }
-  } else {
-    const dim3 grid((unsigned)((d_out + GN - 1) / GN), (unsigned)tiles);
-    { gemm_he_kernel<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); }
-  }
+  const bool small = small_tiles(d_in, d_out);
+  const dim3 grid((unsigned)((d_out + (small ? GS : GN) - 1) / (small ? GS : GN)), (unsigned)tiles);
+  auto run = [&](auto kern) { kern<<<grid, 256, 0, st>>>(H, d_in, d_out, E, G, ldg, col_loss ? part : nullptr); count_launch(); };
+  if (small) run(leave_nan_out ? gemm_he_small_kernel<true> : gemm_he_small_kernel<false>);
+  else run(leave_nan_out ? gemm_he_kernel<true> : gemm_he_kernel<false>);
   if (col_loss)
     { partials_reduce_kernel<<<(unsigned)((d_out + 127) / 128), 128, 0, st>>>(part, tiles, d_out, col_loss); count_launch(); }
   return cudaGetLastError();

@@ -86,7 +86,7 @@ extern "C" cdq_status cdq_layer_loss_static(const float* H, const void* W, cdq_d
   src.d_out = d_out;
   // every scratch region is fully overwritten before it is read, so nothing needs clearing
   if ((e = launch_residual_f64(src, d_in, E, st)) != cudaSuccess ||
-      (e = launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, st)) != cudaSuccess) {
+      (e = launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, false, st)) != cudaSuccess) {
     set_error_detail(cudaGetErrorString(e));
     return CDQ_ERR_CUDA;
   }

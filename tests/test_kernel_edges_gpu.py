@@ -141,13 +141,13 @@ def _float_of_bits(bits):
     return torch.from_numpy(np.array([bits], dtype=np.uint32).view(np.int32)).to(DEV).view(torch.float32)
 
 
-# (layers whose gradient comes from the int8 product, for each of the descent's kernels)
-@pytest.mark.parametrize("d_in,d_out", [(512, 1600), (1024, 600), (2048, 128), (8704, 128)])
+# (layers whose gradient comes from the int8 product, for each of the descent's kernels, and from both fp64 products)
+@pytest.mark.parametrize("d_in,d_out", [(512, 1600), (1024, 600), (2048, 128), (8704, 128), (256, 128), (301, 400), (256, 6000)])
 @pytest.mark.parametrize("bits", [0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF, 0x7F800001])
 def test_a_nan_is_left_out_of_the_gradient_whatever_its_payload(d_in, d_out, bits):
     """0x7FFFFFFF is the NaN that CUDA's arithmetic makes, 0x7FC00000 that of a Python literal.  A NaN weight takes code 0 and
     leaves its column as one with the zero of the grid there, a NaN feature of H its layer as one without the feature; the
-    losses show both."""
+    losses of the descent show both."""
     cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=d_out, bits=3, seed=46)
     H = _layer_h(cfg, 768)
     W = inputs.make_w(cfg, device=DEV)
@@ -174,6 +174,9 @@ def test_a_nan_is_left_out_of_the_gradient_whatever_its_payload(d_in, d_out, bit
     Q, per = solve(Hn, W)
     Qz, _ = solve(Hz, W)
     assert torch.equal(Q, Qz) and bool(per.isnan().all())
+    scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
+    loss, lossz = (B.cdq_layer_loss(Hs, W, grid, scale, zero, Q) for Hs in (Hn, Hz))
+    assert loss == lossz and np.isfinite(loss)
 
 
 @pytest.mark.parametrize("d_in,width", [(256, 256), (257, 264), (319, 320), (384, 392), (641, 648), (1158, 1160), (1283, 1288)])
