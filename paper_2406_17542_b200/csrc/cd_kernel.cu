@@ -41,17 +41,35 @@ cudaError_t launch_diag(const float* H, long long d_in, long long d_pad, float* 
   return cudaGetLastError();
 }
 
-// A feature whose calibration inputs held an infinity or a NaN has no gradient, in any column, and so the loss is none: the
-// descent of the long rows widens every second entry of a row by its bits and would make such values finite.
-__global__ void mark_features_kernel(const float* __restrict__ H, long long d_in, long long d_out, double* __restrict__ G,
-                                     long long ldg) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= d_in || fabsf(H[i * d_in + i]) <= 3.402823466e38f) return;
-  for (long long j = 0; j < d_out; ++j) G[j * ldg + i] = __longlong_as_double(0x7FF8000000000000ll);
+// Features whose gradient is none, in any column, so that the loss is none either: those whose calibration inputs held an
+// infinity or a NaN (H_ii is not finite), and both ends of any other entry of H that is not finite.  The descent of the long rows
+// widens every second entry of a row by its bits and would make such values finite.  One block per row of H: memory-bound, one read
+// of H.
+__global__ void __launch_bounds__(256) mark_features_kernel(const float* __restrict__ H, long long d_in, long long d_out,
+                                                            double* __restrict__ G, long long ldg) {
+  constexpr float kMax = 3.402823466e38f;
+  const long long i = blockIdx.x;
+  const float* row = H + i * d_in;
+  bool bad = !(fabsf(row[i]) <= kMax);
+  if (!bad) {   // (an entry at a feature that is marked for its own H_kk says nothing about this one)
+    auto look = [&](long long k, float h) {
+      if (!(fabsf(h) <= kMax) && fabsf(H[k * d_in + k]) <= kMax) bad = true;
+    };
+    if ((d_in & 3) == 0) {
+      for (long long k = 4 * threadIdx.x; k < d_in; k += 4 * blockDim.x) {
+        const float4 h = __ldg(reinterpret_cast<const float4*>(row + k));
+        look(k, h.x); look(k + 1, h.y); look(k + 2, h.z); look(k + 3, h.w);
+      }
+    } else {
+      for (long long k = threadIdx.x; k < d_in; k += blockDim.x) look(k, row[k]);
+    }
+  }
+  if (!__syncthreads_or(bad)) return;
+  for (long long j = threadIdx.x; j < d_out; j += blockDim.x) G[j * ldg + i] = __longlong_as_double(0x7FF8000000000000ll);
 }
 
 cudaError_t launch_mark_features(const float* H, long long d_in, long long d_out, double* G, long long ldg, cudaStream_t st) {
-  { mark_features_kernel<<<(unsigned)((d_in + 127) / 128), 128, 0, st>>>(H, d_in, d_out, G, ldg); count_launch(); }
+  { mark_features_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_out, G, ldg); count_launch(); }
   return cudaGetLastError();
 }
 

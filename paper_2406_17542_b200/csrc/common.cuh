@@ -131,7 +131,7 @@ long long cd_fast_pad(long long d_in);      // padded length of hdiag / hs
 bool cd_fast_supported(long long d_in, long long g);
 // hdiag = H_ii, hs = 0.5 / H_ii
 cudaError_t launch_diag(const float* H, long long d_in, long long d_pad, float* hdiag, float* hs, cudaStream_t st);
-// G[j][i] = NaN in every column for the features whose H_ii is not finite; the descent of the long rows wants it.
+// G[j][i] = NaN in every column for the features with entries of H that are not finite; the descent of the long rows wants it.
 cudaError_t launch_mark_features(const float* H, long long d_in, long long d_out, double* G, long long ldg, cudaStream_t st);
 inline bool cd_long_rows(long long ldh) { return ldh > 8192; }   // rows of this stride: cd_kernel_ahead.cu
 // col_loss[j] = 1/2 sum_i E[i][j] G[j][i] (E [d_in, d_out], G [d_out, ldg]): e^T H e from the gradient g = 2 H e.

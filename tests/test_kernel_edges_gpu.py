@@ -137,6 +137,24 @@ def test_pairs_need_no_room_for_padded_rows():
     assert torch.equal(Q, Q2) and got["committed"] == want["committed"] and ws.guards_intact()
 
 
+@pytest.mark.parametrize("d_in", [8704, 8705])
+@pytest.mark.parametrize("i,k", [(4096, 17), (4097, 33), (8703, 8702), (6, 5)])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+def test_an_entry_off_the_diagonal_that_is_not_a_number_shows_in_the_loss(d_in, i, k, value):
+    """At even and odd places of a row; only the two features at its ends are kept from moving."""
+    cfg = inputs.CONFIGS["C3"].scaled(d_in=d_in, d_out=40, bits=3, seed=47)
+    H = _layer_h(cfg, 512)
+    H[i, k] = H[k, i] = value
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q0, _ = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    _, loss, per = B.cdq_cd_solve_with_loss(H, W, grid, scale, zero, Q, 40, per_col=True)
+    assert B.load().cdq_last_device_status() == 0
+    assert not np.isfinite(loss) and not bool(torch.isfinite(per).any())
+    assert torch.equal(Q[i], Q0[i]) and torch.equal(Q[k], Q0[k])
+
+
 def _float_of_bits(bits):
     return torch.from_numpy(np.array([bits], dtype=np.uint32).view(np.int32)).to(DEV).view(torch.float32)
 
