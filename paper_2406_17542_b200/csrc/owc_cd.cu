@@ -357,8 +357,8 @@ __global__ void __launch_bounds__(NT, 2) owc_cd_kernel(Params p) {
   if (tid == 0 && my_moves) atomicAdd(&p.ctr->moves, my_moves);
 }
 
-// Production kernel for up to kCodesNk strengths and groups of up to kCodesG coordinates, on the codes of the strengths
-// instead of their residuals.
+// Production kernel for groups of 40 to kCodesG coordinates and up to kCodesNk strengths (see codes_supported), on the codes of
+// the strengths instead of their residuals.
 //
 // What bounds it is the update: g rows of H per move, 2 MB at 4096 features in groups of 128, which come from L2 as long
 // as H stays there.  The tables of the general kernel (residuals and their products with H, 16 nk d_in bytes per
@@ -377,8 +377,13 @@ inline size_t codes_smem(long long g, long long ng, int nk) {   // quad, S, resi
 inline size_t codes_scratch(long long d_in, long long ng, int nk) {
   return sizeof(double) * (2 * (size_t)d_in + (size_t)ng * nk * nk) + ((size_t)nk * d_in + 255) / 256 * 256;
 }
+// Groups of at least 40 coordinates and some two per strength: what a group costs beside its coordinates (three barriers and
+// nk^2 / 2 products of a warp when a column begins, a warp's reduction per four strengths and step) does not shrink with it.
+// General kernel -> this one: 1920 x 512 columns with 20 strengths in groups of 32 6.5 -> 7.4 ms, 40 6.3 -> 5.7, 64 4.4 -> 3.6; with
+// 32 strengths in groups of 48 7.8 -> 7.9, 60 6.7 -> 6.3; 960 x 200 with 20 strengths in groups of 32 1.39 -> 1.53, 40 1.35 -> 1.29, with
+// 32 in groups of 48 1.59 -> 1.78, 60 1.50 -> 1.52; 2048 x 512 in groups of 16 19.2 -> 23.2, 256 x 2000 in pairs 0.77 -> 1.92.
 inline bool codes_supported(long long g, long long ng, int nk) {
-  return nk <= kCodesNk && g <= kCodesG && codes_smem(g, ng, nk) <= kCodesSmem;
+  return nk <= kCodesNk && g >= 40 && 15 * nk <= 8 * g && g <= kCodesG && codes_smem(g, ng, nk) <= kCodesSmem;
 }
 __device__ __forceinline__ double byte_to_double(unsigned q) {   // exact, on the fp64 pipe instead of the conversion pipe
   return __hiloint2double(0x43300000, (int)q) - 4503599627370496.0;

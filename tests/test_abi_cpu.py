@@ -75,6 +75,17 @@ def test_padded_rows_of_odd_layers_cost_workspace_only_where_nothing_else_lies_i
     assert need(B.CALL_BCD_SOLVE, 1026, 8, n=4104) < need(B.CALL_BCD_SOLVE, 1028, 8, n=4104) + 4096
 
 
+def test_small_groups_keep_the_tables_of_the_general_owc_cd_kernel(lib):
+    """The kernel on codes takes a fraction of the general kernel's tables (16 bytes per strength and coordinate for each of up to 296
+    columns); on small groups it is the slower one."""
+    tables = lambda d_in, d_out, nk: 16 * nk * d_in * min(d_out, 296)
+    ws = lambda d_in, d_out, g, nk: B.workspace_bytes(B.CALL_INIT_OWC_CD, 0, d_in, d_out, B.Grid(2, g, nk, 0.5, 1.0))
+    for d_in, d_out, g, nk in [(2048, 512, 16, 20), (256, 2000, 2, 4), (256, 2000, 1, 2), (768, 300, 24, 32), (4096, 512, 32, 20)]:
+        assert ws(d_in, d_out, g, nk) >= tables(d_in, d_out, nk)
+    for d_in, d_out, g, nk in [(4096, 1024, 128, 20), (1920, 512, 64, 32)]:
+        assert ws(d_in, d_out, g, nk) - ws(d_in, d_out, g, 2) < tables(d_in, d_out, nk) / 2
+
+
 def test_bad_arguments_are_rejected_before_any_launch(lib):
     gd = B.Grid(bits=3).c()
     dummy = ctypes.c_void_p(256)  # never dereferenced: validation fails first

@@ -61,6 +61,16 @@ def test_owc_cd_matches_oracle(d_in, d_out, n, bits, g, n_clip, steps, mode):
     assert stats["loss_after"] <= stats["loss_before"]
 
 
+@pytest.mark.parametrize("d_in,d_out,n,bits,g,n_clip,steps", [
+    # production kernels on either side of their limits: groups of 40 and 512 coordinates, two per strength; odd ones, whose codes and
+    # gradients lie off the vectors' boundaries; 32 and 33 strengths; two strengths; eight bits
+    (120, 9, 500, 3, 40, 21, 0), (120, 9, 500, 3, 40, 22, 0), (117, 9, 500, 3, 39, 6, 0), (205, 11, 700, 2, 41, 5, 0),
+    (512, 5, 900, 3, 512, 6, 3), (130, 7, 600, 4, 65, 32, 0), (130, 7, 600, 4, 65, 33, 0), (342, 6, 900, 8, 57, 2, 0),
+])
+def test_owc_cd_matches_oracle_at_the_limits_of_its_kernels(d_in, d_out, n, bits, g, n_clip, steps):
+    test_owc_cd_matches_oracle(d_in, d_out, n, bits, g, n_clip, steps, "fast")
+
+
 def test_owc_cd_then_descent_never_worse_than_owc_then_descent_start():
     """Per-group strengths start the descent at or below the loss of the one-strength-per-column search."""
     cfg = inputs.CONFIGS["C2"].scaled(d_in=512, d_out=160, n=2048, seed=9)
