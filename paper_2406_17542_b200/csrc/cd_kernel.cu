@@ -159,6 +159,10 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
   const long long d_in = p.d_in;
   const int nchunks = (int)(d_in >> 2);
   const float top = kMagic + (float)p.L;
+  // How the slots past the end of a row are kept from reading past it: by a branch, behind which the compiler serialises the loads of
+  // some variants (960 x 148 columns in groups of 64, four chunks: 1.36 ms against 0.98; x 888 in groups of 20 1.59 against 1.29), or
+  // by reading the last chunk again (slower per channel, 1.22 against 0.83, and with three chunks in groups of 20, 0.88 against 0.71).
+  constexpr bool kClamp = !EXACT && ((NCH >= 3 && SMODE == kGroupFast) || (NCH >= 4 && SMODE == kGroupAny));
 
   auto group_of = [&](unsigned i) -> unsigned { return p.g == 1 ? i : __umulhi(i, p.gmagic); };
   float2* ag_s = reinterpret_cast<float2*>(dyn_smem);  // [ag_count] (a, 1/a), grouped modes
@@ -238,13 +242,16 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_fast_kernel(CdParams p) {
       for (int k = 0; k < NCH; ++k) {
         const int chunk = tid + NT * k;
         // the rows of the shortest layers (1 MB at 512 entries) may stay in L1, longer ones would only pass through it
-        auto load = [&]() {
-          return NCH <= 2 ? __ldg(reinterpret_cast<const float4*>(rp) + chunk) : ld_row4(rp + (long long)chunk * 4);
+        auto load = [&](int c) {
+          return NCH <= 2 ? __ldg(reinterpret_cast<const float4*>(rp) + c) : ld_row4(rp + (long long)c * 4);
         };
-        if (EXACT) row[k] = load();
+        // Slots past the end of the row: zeros, or, where kClamp, the row's last chunk (their gradients go nowhere: H_ii is zero
+        // there, so they never move).
+        if (EXACT) row[k] = load(chunk);
+        else if (kClamp) row[k] = load(min(chunk, nchunks - 1));
         else {
           row[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (chunk < nchunks) row[k] = load();
+          if (chunk < nchunks) row[k] = load(chunk);
         }
       }
       SweepBest sb;
@@ -360,15 +367,17 @@ static cudaError_t launch_cd_cfg(CdParams p, int nt, cudaStream_t st) {
 // Picks the scale mode and whether the team covers d_in exactly.
 template <int NCH, int MAXNT, int MINB>
 static cudaError_t launch_cd_shape(const CdParams& p, int nt, cudaStream_t st) {
+  // (with three and four chunks the variant for rows that fill the team is the slower one, by its schedule: 1152 x 148 columns 1.02
+  // against 0.73 ms)
   const bool exact = p.d_in == 4ll * nt * NCH;
   const int smode = cd_scale_mode(p, nt);
   if (smode < 0) return cudaErrorNotSupported;
-  if (smode == kPerChannel)
-    return exact ? launch_cd_cfg<NCH, MAXNT, MINB, kPerChannel, true>(p, nt, st)
-                 : launch_cd_cfg<NCH, MAXNT, MINB, kPerChannel, false>(p, nt, st);
-  if (smode == kGroupFast)
-    return exact ? launch_cd_cfg<NCH, MAXNT, MINB, kGroupFast, true>(p, nt, st)
-                 : launch_cd_cfg<NCH, MAXNT, MINB, kGroupFast, false>(p, nt, st);
+  if constexpr (NCH <= 2) {
+    if (exact && smode == kPerChannel) return launch_cd_cfg<NCH, MAXNT, MINB, kPerChannel, true>(p, nt, st);
+    if (exact && smode == kGroupFast) return launch_cd_cfg<NCH, MAXNT, MINB, kGroupFast, true>(p, nt, st);
+  }
+  if (smode == kPerChannel) return launch_cd_cfg<NCH, MAXNT, MINB, kPerChannel, false>(p, nt, st);
+  if (smode == kGroupFast) return launch_cd_cfg<NCH, MAXNT, MINB, kGroupFast, false>(p, nt, st);
   return launch_cd_cfg<NCH, MAXNT, MINB, kGroupAny, false>(p, nt, st);
 }
 
@@ -436,8 +445,23 @@ cudaError_t launch_cd_fast(const Layer& ly, const float* rows, long long ldh, co
   if (H16) return cudaErrorNotSupported;
   auto team = [&](int ept) { return (int)(((d + ept - 1) / ept + 31) / 32 * 32); };
   if (d <= 512) return launch_cd_shape<2, 64, 8>(p, team(8), st);
-  // three chunks per thread: more warps per column than four hide more of a step's latency (768 x 8192 2.00 -> 1.64 ms, 1152 x
-  // 8192 6.7 -> 5.4, 1350 x 677 1.56 -> 1.44), and two cost more in the exchange (1350 x 677 1.78)
+  // Three chunks per thread: more warps per column than four hide more of a step's latency (1350 x 677 1.56 -> 1.44 ms, 1152 x 8192
+  // 6.7 -> 5.4), and two cost more in the exchange (1350 x 677 1.78).  Rows of 769 to 1024 entries take three warps that way instead
+  // of two: with more than five columns per SM four chunks are quicker (960 entries, columns per SM, three against four chunks: 4
+  // 0.80 / 0.90 ms, 6 1.11 / 1.00, 12 1.93 / 1.69, 26 3.93 / 3.37; in groups of 64 4 0.81 / 1.03, 6 1.16 / 1.10, 26 4.12 / 3.84).
+  // Longer rows take four warps instead of three, six columns per SM instead of eight: eight are one round of four-chunk teams and
+  // two of the others (per channel, 1280 entries 2.32 / 2.36, 1536 2.79 / 2.88; 9 2.76 / 2.46, 16 4.59 / 4.25; in groups never).
+  // On grouped grids a team whose threads meet the group scales at a fixed stride goes before that (groups of 12, three chunks,
+  // which do not, against four: 1536 entries, 20 columns per SM 7.3 / 6.7 ms, 1440 entries, 7 2.83 / 2.66).
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long per_sm = sms > 0 ? (ly.d_out + sms - 1) / sms : 0;
+  const bool any3 = cd_scale_mode(p, team(12)) == kGroupAny, any4 = cd_scale_mode(p, team(16)) == kGroupAny;
+  bool four = false;
+  if (d > 768 && d <= 1024) four = per_sm > 5 && (any3 || !any4);
+  else if (d > 1152) four = ly.ng == 1 ? per_sm == 8 : per_sm > 5 && any3 && !any4;
+  if (four) return launch_cd_shape<4, 256, 3>(p, team(16), st);
   return launch_cd_shape<3, 128, 6>(p, team(12), st);
 }
 

@@ -65,6 +65,31 @@ def test_descent_result_does_not_depend_on_the_other_columns():
     assert torch.equal(Qs, Q[:, some])
 
 
+# (d_in, columns per SM, bits, g): teams of three and of four chunks per thread on either side of their rules, per channel, with group
+# scales at a fixed stride (4, 64; 12 on three-chunk teams of 960 and four-chunk teams of 1440 entries) and without one (20)
+@pytest.mark.parametrize("d_in,per_sm,bits,g", [
+    (769, 6, 3, 0), (1021, 6, 3, 0), (1024, 6, 4, 64), (1024, 5, 3, 0), (772, 6, 3, 4), (960, 6, 3, 12), (960, 6, 2, 20), (840, 6, 8, 24),
+    (1153, 8, 3, 0), (1536, 8, 3, 0), (1440, 6, 3, 12), (1440, 6, 3, 20), (1536, 7, 3, 64),
+])
+def test_descent_of_short_rows_with_many_columns(d_in, per_sm, bits, g):
+    d_out = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = inputs.CONFIGS["C1"].scaled(d_in=d_in, d_out=d_out, bits=bits, group_size=g, w_dtype="f32", seed=800 + d_in % 89)
+    H = _layer_h(cfg, 1600)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q0, gamma = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    _, loss, per = B.cdq_cd_solve_with_loss(H, W, grid, scale, zero, Q, 500, per_col=True)
+    assert B.load().cdq_last_device_status() == 0
+    some = torch.arange(1, d_out, 37, device=DEV)           # the same columns in a layer of few
+    Qs = Q0[:, some].contiguous()
+    B.cdq_cd_solve(H, W[:, some].contiguous(), grid, scale[:, some].contiguous(), zero[:, some].contiguous(), Qs, 0,
+                   steps_per_col=500)
+    assert torch.equal(Qs, Q[:, some])
+    compare_with_oracle(cfg, H.cpu().numpy(), H, W, np.array([0, d_out // 2, d_out - 1]), grid, scale, zero, Q0, Q, gamma, per, 500,
+                        label=f"d_in={d_in} x {d_out} bits={bits} g={g}")
+
+
 @pytest.mark.parametrize("d_in,at", [(8704, 4096), (8704, 4097), (8704, 8703), (9001, 9000), (4096, 33)])
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 def test_a_feature_that_is_not_a_number_shows_in_the_loss(d_in, at, value):
