@@ -533,35 +533,65 @@ bool bcd_supported(long long d_in, int block) {
   return block == 2 && d_in >= 2 && (d_in & 1) == 0 && d_in <= 32768;
 }
 
+// A kernel for a layer: threads per column, what lies in shared memory, columns per SM.
+struct BcdFit {
+  int nt, per_sm, g_in_smem, a_in_smem;
+  size_t smem;
+};
+
 template <int PPT, int MAXNT, int MINB>
-static cudaError_t launch_bcd_cfg(const CdParams& p, const uint4* tab, int nt, cudaStream_t st) {
+static cudaError_t fit_bcd(const CdParams& p, int nt, BcdFit& f) {
   auto kern = bcd2_kernel<PPT, MAXNT, MINB>;
-  int dev = 0, sms = 0, smem_max = 0;
+  int dev = 0, smem_max = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const size_t q_bytes = (size_t)((p.ldg + 15) / 16 * 16), a_bytes = sizeof(float2) * (size_t)p.ng;
   const size_t budget = (size_t)smem_max - 2048;  // the kernel's static shared memory and the runtime's share
-  const int a_in_smem = q_bytes + a_bytes <= budget / 2 ? 1 : 0;
-  size_t smem = q_bytes + (a_in_smem ? a_bytes : 0);
-  if (smem > budget) return cudaErrorNotSupported;
+  f.nt = nt;
+  f.a_in_smem = q_bytes + a_bytes <= budget / 2 ? 1 : 0;
+  f.smem = q_bytes + (f.a_in_smem ? a_bytes : 0);
+  if (f.smem > budget) return cudaErrorNotSupported;
   // CDQ_BCD_G=global in the environment keeps the gradient in global memory at every size
   static const bool force_global = [] { const char* e = getenv("CDQ_BCD_G"); return e && e[0] == 'g'; }();
-  const int g_in_smem = !force_global && smem + sizeof(double) * (size_t)p.ldg <= budget ? 1 : 0;
-  if (g_in_smem) smem += sizeof(double) * (size_t)p.ldg;
+  f.g_in_smem = !force_global && f.smem + sizeof(double) * (size_t)p.ldg <= budget ? 1 : 0;
+  if (f.g_in_smem) f.smem += sizeof(double) * (size_t)p.ldg;
   cudaError_t e;
-  if (smem > 32 * 1024) {   // the 48 KB that need no opt-in include the kernel's static shared memory
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (f.smem > 32 * 1024) {   // the 48 KB that need no opt-in include the kernel's static shared memory
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem);
     if (e != cudaSuccess) return e;
   }
-  int per_sm = 1;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.per_sm, kern, nt, f.smem);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  long long blocks = (long long)sms * per_sm;
+  return f.per_sm < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
+static int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms > 0 ? sms : 1;
+}
+
+template <int PPT, int MAXNT, int MINB>
+static cudaError_t launch_bcd_cfg(const CdParams& p, const uint4* tab, int nt, cudaStream_t st) {
+  BcdFit f{};
+  cudaError_t e = fit_bcd<PPT, MAXNT, MINB>(p, nt, f);
+  if (e != cudaSuccess) return e;
+  long long blocks = (long long)sm_count() * f.per_sm;
   if (blocks > p.d_out) blocks = p.d_out;
-  { kern<<<(unsigned)blocks, nt, smem, st>>>(p, tab, g_in_smem, a_in_smem); count_launch(); }
+  { bcd2_kernel<PPT, MAXNT, MINB><<<(unsigned)blocks, nt, f.smem, st>>>(p, tab, f.g_in_smem, f.a_in_smem); count_launch(); }
   return cudaGetLastError();
+}
+
+// Time of a layer's columns in rounds of per_sm per SM: a column alone on its SM takes `alone`, every further one beside it a
+// fifth of what a column with four pairs per thread takes alone.  Measured on rows of 2052 to 4096 entries, 256 steps from
+// round-to-nearest codes (one, two, ... per SM; four pairs per thread, then eight): 2052 1.47 1.70 2.03, 2.11 2.29 2.49 2.75 - 3.43; 3072 1.68 2.04, 2.66
+// 2.88 3.18 3.42 3.98; 4096 1.84 2.36, 2.80 3.08 3.46 4.01 ms.
+static double bcd_rounds(const BcdFit& f, long long d_out, int sms, double alone) {
+  const long long at_once = (long long)sms * f.per_sm, rest = d_out % at_once;
+  double t = (double)(d_out / at_once) * (alone + 0.2 * (f.per_sm - 1));
+  if (rest) t += alone + 0.2 * (double)((rest + sms - 1) / sms - 1);
+  return t;
 }
 
 size_t bcd_table_bytes(long long d_in, long long steps_per_col) {
@@ -592,10 +622,21 @@ cudaError_t launch_bcd(const Layer& ly, double* G, long long ldg, unsigned char*
   }
   auto team = [&](int ppt) { return (int)(((nb + ppt - 1) / ppt + 31) / 32 * 32); };
   if (nb <= 256) return launch_bcd_cfg<1, 256, 2>(p, tab, team(1), st);
-  // up to 2048 entries four pairs per thread, up to 4096 eight: twice as many columns per SM hide the steps' latencies there
-  // (3072 x 4096 34.6 -> 30.4 ms, 4096 x 2048 31.8 -> 30.3), on shorter rows they do not pay (1024 x 4096 3.9 -> 4.8 ms)
   if (nb <= 1024) return launch_bcd_cfg<4, 256, 4>(p, tab, team(4), st);
-  if (nb <= 2048) return launch_bcd_cfg<8, 256, 4>(p, tab, team(8), st);
+  if (nb <= 2048) {
+    // Rows of 2049 to 4096 entries: eight pairs per thread put twice as many columns on an SM, which hide the steps' latencies
+    // (3072 x 4096 34.6 -> 30.4 ms, 4096 x 2048 31.8 -> 30.3), but a column alone takes half as long again (4096 x 148 1.8 -> 2.8).
+    BcdFit four{}, eight{};
+    cudaError_t e = fit_bcd<4, 512, 2>(p, team(4), four);
+    if (e == cudaSuccess) e = fit_bcd<8, 256, 4>(p, team(8), eight);
+    if (e != cudaSuccess) return e;
+    // (up to three columns per SM four pairs are the better choice after a greedy descent whatever the rounds say: 3584 x 400 2.38
+    // against 2.71 ms, from round-to-nearest codes 3.62 against 3.27)
+    const int sms = sm_count();
+    if (p.d_out <= 3ll * sms || bcd_rounds(four, p.d_out, sms, 1.0) < bcd_rounds(eight, p.d_out, sms, 1.5))
+      return launch_bcd_cfg<4, 512, 2>(p, tab, team(4), st);
+    return launch_bcd_cfg<8, 256, 4>(p, tab, team(8), st);
+  }
   if (nb <= 7168) return launch_bcd_cfg<8, 896, 1>(p, tab, team(8), st);
   if (nb <= 8192) return launch_bcd_cfg<8, 1024, 1>(p, tab, team(8), st);
   if (nb <= 9216) return launch_bcd_cfg<12, 768, 1>(p, tab, team(12), st);

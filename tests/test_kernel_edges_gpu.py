@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2406_17542_b200 import binding as B
 from paper_2406_17542_b200 import inputs
-from tests.util import compare_with_oracle, grid_of
+from tests.util import compare_pairs_with_oracle, compare_with_oracle, grid_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -88,6 +88,29 @@ def test_descent_of_short_rows_with_many_columns(d_in, per_sm, bits, g):
     assert torch.equal(Qs, Q[:, some])
     compare_with_oracle(cfg, H.cpu().numpy(), H, W, np.array([0, d_out // 2, d_out - 1]), grid, scale, zero, Q0, Q, gamma, per, 500,
                         label=f"d_in={d_in} x {d_out} bits={bits} g={g}")
+
+
+@pytest.mark.parametrize("d_in,per_sm,bits,g", [(2050, 4, 2, 0), (2050, 3, 2, 0), (2304, 6, 2, 128), (3072, 4, 3, 0), (4096, 4, 2, 64), (4094, 2, 3, 0)])
+def test_pairs_on_either_side_of_the_rule_for_their_teams(d_in, per_sm, bits, g):
+    """Four pairs per thread for few columns, eight for many, from round-to-nearest codes (where every step moves): the oracle's
+    codes, and the same ones from a layer of few columns."""
+    d_out = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = inputs.CONFIGS["C2"].scaled(d_in=d_in, d_out=d_out, bits=bits, group_size=g, n_clip=1, clip_lo=1.0, clip_hi=1.0,
+                                      passes=0, seed=820 + d_in % 89)
+    H = _layer_h(cfg, 2 * d_in)
+    W = inputs.make_w(cfg, device=DEV)
+    grid = grid_of(cfg)
+    scale, zero, Q0, _ = B.cdq_init_rtn(W, grid)
+    Q = Q0.clone()
+    B.cdq_bcd_solve(H, W, grid, scale, zero, Q, 2, 40, seed=5)
+    _, per = B.cdq_layer_loss(H, W, grid, scale, zero, Q, per_col=True)
+    some = torch.arange(2, d_out, 41, device=DEV)
+    Qs = Q0[:, some].contiguous()
+    B.cdq_bcd_solve(H, W[:, some].contiguous(), grid, scale[:, some].contiguous(), zero[:, some].contiguous(), Qs, 2, 40, seed=5)
+    assert B.load().cdq_last_device_status() == 0
+    assert torch.equal(Qs, Q[:, some])
+    compare_pairs_with_oracle(cfg, H.cpu().numpy(), H, W, np.array([0, 1, d_out - 1]), grid, scale, zero, Q0, Q, per, 40, 5,
+                              label=f"d_in={d_in} x {d_out}")
 
 
 @pytest.mark.parametrize("d_in,at", [(8704, 4096), (8704, 4097), (8704, 8703), (9001, 9000), (4096, 33)])
