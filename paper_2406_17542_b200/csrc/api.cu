@@ -430,7 +430,7 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
                         st));
   } else if (fast_cd) {
     CDQ_CUDA(launch_diag(H, d_in, L.d_pad, hdiag, half_inv, st));
-    if (cd_long_rows(L.ldg)) CDQ_CUDA(launch_mark_features(H, d_in, d_out, G, L.ldg, st));
+    if (cd_ahead_takes(L.ldg, rows16)) CDQ_CUDA(launch_mark_features(H, d_in, d_out, G, L.ldg, st));
     const float* rows = H;
     if (pad_rows) {   // odd rows of H on 16-byte boundaries (1350 entries: 5 us for the copy, and the descent 0.6 of its time)
       float* hpad = (float*)(base + L.hpad);

@@ -1,5 +1,6 @@
 // Greedy coordinate descent (paper: the loop of Algorithm 1; Algorithm 4 for sub-channel
-// grids), the variant for rows of H of 1537 to 8192 entries, on 16-byte boundaries (longer rows: cd_kernel_ahead.cu).
+// grids), the variant for rows of H of 1537 to 8192 entries (bf16 rows: to 10240), on 16-byte boundaries (longer rows:
+// cd_kernel_ahead.cu).
 //
 // Same step as cd_kernel.cu -- score, argmin, read row i*, update the gradient -- but the row
 // H[i*, :] is fetched by one bulk asynchronous copy (cp.async.bulk, no multicast) into shared
@@ -306,6 +307,16 @@ cudaError_t launch_mode(const CdParams& p, int nt, cudaStream_t st) {
   return cudaErrorNotSupported;
 }
 
+// The same for bf16 rows alone.
+template <int NCH, int MAXNT, int MINB>
+cudaError_t launch_mode_rows16(const CdParams& p, int nt, cudaStream_t st) {
+  const int smode = cd_scale_mode(p, nt);
+  if (smode == kPerChannel) return launch_cfg<NCH, MAXNT, MINB, kPerChannel, true>(p, nt, st);
+  if (smode == kGroupFast) return launch_cfg<NCH, MAXNT, MINB, kGroupFast, true>(p, nt, st);
+  if (smode == kGroupAny) return launch_cfg<NCH, MAXNT, MINB, kGroupAny, true>(p, nt, st);
+  return cudaErrorNotSupported;
+}
+
 }  // namespace
 
 cudaError_t launch_cd_tma(const CdParams& p, cudaStream_t st) {
@@ -317,6 +328,9 @@ cudaError_t launch_cd_tma(const CdParams& p, cudaStream_t st) {
   // (called for rows of more than 1536 entries)  Rows up to 8192 entries: several teams per SM.
   if (ch <= 1024) return launch_mode<8, 128, 4>(p, team(ch, 8), st);
   if (ch <= 2048) return launch_mode<8, 256, 2>(p, team(ch, 8), st);
+  // Longer ones, as bf16: one team per SM (see cd_ahead_takes).
+  if (p.H16 && ch <= 2304) return launch_mode_rows16<9, 256, 1>(p, team(ch, 9), st);
+  if (p.H16 && ch <= 2560) return launch_mode_rows16<10, 256, 1>(p, team(ch, 10), st);
   return cudaErrorNotSupported;
 }
 

@@ -45,9 +45,9 @@ inline int cd_scale_mode(const CdParams& p, int nt) {
   return nt % (int)(p.g >> 2) == 0 ? kGroupFast : kGroupAny;
 }
 
-// cd_kernel_tma.cu: rows of 1537 to 8192 entries, staged through shared memory by bulk copies.
+// cd_kernel_tma.cu: rows of more than 1536 entries, staged through shared memory by bulk copies.
 cudaError_t launch_cd_tma(const CdParams& p, cudaStream_t st);
-// cd_kernel_ahead.cu: the same for rows of more than 8192 entries, with the next row in flight during the sweep.
+// cd_kernel_ahead.cu: the same for the longest rows (cd_ahead_takes), with the next row in flight during the sweep.
 cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st);
 
 }  // namespace cdq

@@ -133,7 +133,10 @@ bool cd_fast_supported(long long d_in, long long g);
 cudaError_t launch_diag(const float* H, long long d_in, long long d_pad, float* hdiag, float* hs, cudaStream_t st);
 // G[j][i] = NaN in every column for the features with entries of H that are not finite; the descent of the long rows wants it.
 cudaError_t launch_mark_features(const float* H, long long d_in, long long d_out, double* G, long long ldg, cudaStream_t st);
-inline bool cd_long_rows(long long ldh) { return ldh > 8192; }   // rows of this stride: cd_kernel_ahead.cu
+// Rows of this stride run in cd_kernel_ahead.cu: those of which one team fills an SM, unless a row of bf16 is so short that its copy
+// takes no longer than what that kernel spends to hide it (296 columns, that kernel against cd_kernel_tma.cu, per channel and in groups
+// of 128: 8704 entries 27.6 / 27.4, 29.7 / 28.5 ms, 10240 36.9 / 35.5, 38.8 / 36.8, 11264 40.7 / 42.0, 43.2 / 45.2).
+inline bool cd_ahead_takes(long long ldh, bool rows16) { return ldh > (rows16 ? 10240 : 8192); }
 // col_loss[j] = 1/2 sum_i E[i][j] G[j][i] (E [d_in, d_out], G [d_out, ldg]): e^T H e from the gradient g = 2 H e.
 cudaError_t launch_loss_from_gradient(const double* E, const double* G, long long ldg, long long d_in, long long d_out,
                                       double* col_loss, cudaStream_t st);

@@ -32,7 +32,7 @@ def _h_from_rows(cfg, rows, ridge=1e-3):
     ("C3", 4608, 64, 0, 4, 4096, 64),          # two 256-thread teams per SM
     ("C3", 6144, 148, 0, 3, 4096, 32),
     ("C3", 11008, 148, 0, 4, 4096, 16),        # ragged: the last chunk slots reach past the row
-    ("C3", 14336, 296, 0, 4, 8192, 24),        # the C3 team (256 threads x 14 chunks)
+    ("C3", 14336, 296, 0, 4, 8192, 24),        # the C3 team (384 threads x 10 chunks)
     ("C4", 18432, 148, 128, 3, 4096, 12),      # the C4 team (384 threads x 12 chunks), groups of 128
 ])
 def test_bf16_rows_against_the_oracle_on_the_rounded_matrix(name, d_in, d_out, g, bits, rows, n_sample):
@@ -61,6 +61,11 @@ def test_bf16_rows_against_the_oracle_on_the_rounded_matrix(name, d_in, d_out, g
     print(f"rows16 {d_in}x{d_out}: loss on H after the descent: fp32 rows {l32:.6g}, bf16 rows {l16:.6g} "
           f"(ratio {l16 / l32:.5f}); round-to-nearest start {l0:.6g}")
     assert l16 <= 1.02 * l32 and l16 < l0
+
+
+@pytest.mark.parametrize("d_in,g,bits", [(8200, 0, 3), (9216, 128, 3), (9224, 0, 8), (10240, 20, 2), (10248, 0, 3)])
+def test_bf16_rows_on_either_side_of_the_kernels_that_take_them(d_in, g, bits):
+    test_bf16_rows_against_the_oracle_on_the_rounded_matrix("C3", d_in, 8, g, bits, 2048, 4)
 
 
 def test_shapes_without_a_bf16_row_kernel_are_refused():
