@@ -94,9 +94,11 @@ SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool wit
   auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
   w.ldg = (d_in + 3) / 4 * 4;
   w.d_pad = cd_fast_pad(d_in);
-  // On small layers (256 x 256: 2 tiles) the int8 product's 27 slice pairs are one long chain on a few SMs: 177 us and 30 us
-  // for the slices, against 47 us for the fp64 product; the two meet between 5e8 and 1e9 multiplications.
-  w.tc = mode == CDQ_MODE_FAST && gemm_tc_supported(d_in, d_out) && d_in * d_in * d_out >= 400000000ll;
+  // On small layers the int8 product's 27 slice pairs are one long chain on a few SMs, and the slices come on top.  Loss of given
+  // codes, int8 against fp64 product (device time in us): 2.7e8 multiplications 229 / 98 (256 x 4096), 258 / 131 (1024 x 256), 280 / 161
+  // (1448 x 128); 5.4e8 237 / 139 (256 x 8192), 266 / 181 (1024 x 512), 312 / 215 (2048 x 128); 8.4e8 244 / 280 (724 x 1600); 1.07e9
+  // 250 / 224 (256 x 16384), 294 / 293 (1448 x 512), 330 / 307 (2048 x 256); 2.1e9 263 / 367 (512 x 8192), 300 / 519 (1448 x 1024).
+  w.tc = mode == CDQ_MODE_FAST && gemm_tc_supported(d_in, d_out) && d_in * d_in * d_out >= 800000000ll;
   // the loss of a descended solution is a sum with heavy cancellation (the descent tunes e against the
   // large entries of H): it takes the same slice depth as the gradient; the shallower setting serves
   // the OWC search, whose residuals are plain rounding errors
