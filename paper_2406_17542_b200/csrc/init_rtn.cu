@@ -59,7 +59,8 @@ __global__ void minmax_partial_kernel(const void* __restrict__ W, long long d_ou
   for (int v = 0; v < V; ++v) { pmn[chunk * d_out + j + v] = mn[v]; pmx[chunk * d_out + j + v] = mx[v]; }
 }
 static void run_minmax_partial(const Layer& ly, long long cpg, float* pmn, float* pmx, cudaStream_t st) {
-  // (narrow layers: a column per thread, or there are too few threads to hide the latency of the loads)
+  // (narrow layers: a column per thread, or there are too few threads to hide the latency of the loads: 4096 x 2048 weights in groups of 64,
+  // 2^17 columns and chunks, 14.5 us against 16.9 with four columns, 4096 x 4096 20.6 / 26.4; 4096 x 4096 in groups of 16, 2^20, 35 / 14)
   const int v = four_columns(ly) && ly.d_out * ly.ng * cpg >= (1 << 18) ? 4 : 1;
   const dim3 grid((unsigned)((ly.d_out + 128 * v - 1) / (128 * v)), (unsigned)(ly.ng * cpg));
   auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(ly.W, ly.d_out, ly.ldw, ly.g, cpg, pmn, pmx); };
@@ -208,12 +209,14 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
 
 cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st, unsigned long long* colmax) {
   const long long width = src.n_cols ? src.n_cols : src.d_out;
-  // rows per block, all of one group: few on small layers, which have no more blocks to offer
+  // rows per block, all of one group: few on small layers, which have no more blocks to offer (1024 x 1024 entries with 32 rows 17 us)
   const int rows = width * d_in >= (1ll << 22) ? 32 : 4, bpg = (int)((src.g + rows - 1) / rows);
   const size_t esz = src.wt == CDQ_BF16 ? 2 : 4;
-  // four columns per thread: rows of W, Q and E on the vectors' boundaries, four neighbouring columns of one strength
-  const bool four = !src.col_idx && src.d_out % 4 == 0 && src.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(src.W) % (4 * esz) == 0 &&
-                    reinterpret_cast<uintptr_t>(src.Q) % 4 == 0 && width * (d_in / src.g) * bpg >= (1 << 17);
+  // four columns per thread: rows of W, Q and E on the vectors' boundaries, four neighbouring columns of one strength, and 32 rows per
+  // block (residual of codes with column maxima, one column against four, us: 1024 x 1024 entries with four rows per block 8.0 / 14.1, 2048 x
+  // 1024 11.6 / 25.5, 4096 x 256 14.0 / 43.2; 2048 x 2048 with 32 rows 21.0 / 15.8, 2048 x 4096 37.9 / 22.9, 4096 x 4096 60.5 / 49.7)
+  const bool four = rows == 32 && !src.col_idx && src.d_out % 4 == 0 && src.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(src.W) % (4 * esz) == 0 &&
+                    reinterpret_cast<uintptr_t>(src.Q) % 4 == 0;
   const dim3 grid((unsigned)((width + (four ? 511 : 127)) / (four ? 512 : 128)), (unsigned)(d_in / src.g * bpg));
   auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, rows, bpg, E, colmax); count_launch(); };
   if (src.wt == CDQ_BF16) run(four ? residual_kernel<4, true> : residual_kernel<1, true>);
@@ -497,6 +500,8 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
   }
   { scale_zero_kernel<<<dim3(bx, (unsigned)ng), 128, 0, st>>>(mn, mx, ng, d_out, ly.L, gam_col, scale, zero); count_launch(); }
   const int bpg = (int)((g + kCodeRows - 1) / kCodeRows);
+  // (as for the minima; bf16 weights, one column against four, us: 1024 x 2048, 2^17 columns and row blocks, 5.7 / 7.2, 2048 x 2048 9.5 / 7.6,
+  // 4096 x 4096 27 / 19)
   const bool four = four_columns(ly) && reinterpret_cast<uintptr_t>(Q) % 4 == 0 && d_out * ng * bpg >= (1 << 18);
   const dim3 grid_q((unsigned)(four ? (d_out + 511) / 512 : bx), (unsigned)(ng * bpg));
   auto run = [&](auto kern) { kern<<<grid_q, 128, 0, st>>>(ly.W, d_out, ly.ldw, g, bpg, ly.L, scale, zero, Q); count_launch(); };
