@@ -33,14 +33,17 @@
  *     exceeds its bound is reported as CDQ_ERR_TIMEOUT by the next call that
  *     synchronises (cdq_last_device_status reads it explicitly).
  *   - Two arithmetic modes.  CDQ_MODE_FAST is the production path: fp32 H, tensor cores for
- *     the Hessian (bf16) and for the products H (W_hat - W) (exact int8 slices, summed in fp64),
- *     the gradient of the descent kept in fp64 and the candidate scores in fp32.  Grouped grids
+ *     the Hessian (bf16) and for the products H (W_hat - W) (exact int8 slices, summed in fp64; small
+ *     layers take an fp64 product), the gradient of the descent kept in fp64 and the candidate scores in fp32.  Grouped grids
  *     whose group size is not a multiple of 4, and layers longer than 18432 inputs, run their
  *     descent with the fp64 kernel of the other mode.  CDQ_MODE_FP64_VERIFY runs plain fp64
  *     kernels that follow a fixed summation order (ascending index, no fused multiply-add) so
  *     that codes can be compared bit for bit with a CPU implementation of the same steps; it is
  *     meant for small layers.
- *   - H must be finite; the descent multiplies rows of H by a zero step in its first sweep.
+ *   - H must be finite; the descent multiplies rows of H by a zero step in its first sweep.  What FAST makes of
+ *     a H or W with entries that are not numbers: from 256 x 128 on the products leave a NaN out, so that the rest
+ *     of the layer, or of a column with a NaN weight, is solved without it; its feature stays where it was and the
+ *     loss of the descent is not finite.
  *   - H must be 16-byte aligned wherever it is passed (it is read with 16-byte vector loads and
  *     bulk copies); a misaligned H is CDQ_ERR_INVALID_ARG before anything is launched.
  *   - Environment (read once per process, for debugging only): CDQ_DEBUG_SYNC=1 synchronises the
@@ -147,7 +150,8 @@ cdq_status cdq_hessian_add_lambda(float* H, long long d_in, float lambda_rel, vo
  * strengths are first screened with three slice-pair products (six on grids of more than 4 bits); a strength
  * within 1 % of a column's smallest screened loss stays a candidate and gets the thirteen-pair loss (~1e-8
  * relative); the argmin is taken over the candidates.  The candidate counts go through the host: one synchronisation of `stream`.
- * The rounding decision is taken in fp64 in both modes.
+ * The codes are those of a rounding decision in fp64, in both modes (an fp32 quotient decides where it is clear of
+ * the middle between two levels).
  */
 cdq_status cdq_init_rtn(const void* W, cdq_dtype wt, long long d_in, long long d_out, long long ldw,
                         const float* H, const cdq_grid_desc* grid, float* scale, float* zero,
@@ -177,8 +181,9 @@ typedef struct {
  *   gamma_out  [d_in/g, d_out] fp32 out, chosen strengths; may be NULL.
  *   stats      host pointer, may be NULL (then the call does not synchronise).
  * fp64 in both modes; VERIFY sums in ascending order without fused multiply-add
- * (bit-reproducible against a CPU statement of the steps), FAST tabulates H_tt r per grid point
- * once per column so that a step costs dot products of length g.
+ * (bit-reproducible against a CPU statement of the steps), FAST tabulates once per column what a step needs of
+ * delta^T H_tt delta -- the products r_k^T H_tt r_l of a group's residuals, or H_tt r per grid point for small groups,
+ * groups of more than 512 and grids of more than 32 points -- so that a step costs dot products of length g.
  */
 cdq_status cdq_init_owc_cd(const void* W, cdq_dtype wt, long long d_in, long long d_out, long long ldw,
                            const float* H, const cdq_grid_desc* grid, long long steps, float* scale,
@@ -328,7 +333,8 @@ cdq_status cdq_layer_loss_static(const float* H, const void* W, cdq_dtype wt, lo
                                  const float* scale, const float* zero, const unsigned char* Q,
                                  double* loss, double* per_col, void* stream);
 
-/* Bytes of workspace `which` needs for these sizes (n is used by the Hessian only). */
+/* Bytes of workspace `which` needs for these sizes (n: rows of X for the Hessian, steps per column for
+ * CDQ_CALL_BCD_SOLVE, which covers either block size; otherwise not used). */
 size_t cdq_workspace_bytes(cdq_call which, long long n, long long d_in, long long d_out,
                            const cdq_grid_desc* grid, cdq_mode mode);
 

@@ -90,7 +90,8 @@ __device__ __forceinline__ unsigned slice_bytes(const unsigned long long (&v)[4]
 }
 
 // H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p]; columns >= d zero), four columns per thread.
-// Memory-bound: 4 bytes read and ns written per entry.  (One column per thread, with the digits taken off one after
+// 4 bytes read and ns written per entry; what bounds it is the integer operations of the digits (4096^2, six slices: 45 us, the ALU pipe
+// 63 % busy, 2.5 TB/s).  (One column per thread, with the digits taken off one after
 // the other in fp64: 1.46 ms for 14336^2 and six slices.)
 __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ exps,
                                int ns, signed char* __restrict__ out) {
@@ -121,8 +122,8 @@ __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long lo
 }
 
 // E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j]), 128 x 32 tiles turned round
-// in shared memory so that reads and writes are contiguous, four rows of E per thread.  Memory-bound: 8 bytes read and ns
-// written per entry.  (32 x 32 tiles, single bytes, digits one after the other in fp64: 0.74 ms for 4096 x 32768 and
+// in shared memory so that reads and writes are contiguous, four rows of E per thread.  8 bytes read and ns
+// written per entry; bound as slice_h_kernel (4096^2, five slices: 52 us, ALU pipe 63 %, 3.5 TB/s).  (32 x 32 tiles, single bytes, digits one after the other in fp64: 0.74 ms for 4096 x 32768 and
 // two slices.)
 constexpr int SK = 128, SJ = 32;
 __global__ void __launch_bounds__(256) slice_et_kernel(const double* __restrict__ E, long long d_in, long long d_out, long long kp,

@@ -98,7 +98,8 @@ __global__ void scale_zero_kernel(const float* __restrict__ mn, const float* __r
   zero[t * d_out + j] = (float)lo;
 }
 
-// Codes of kCodeRows rows of one group by V columns per thread (see rtn_code).  Memory-bound: 14336 x 16384 bf16 weights
+// Codes of kCodeRows rows of one group by V columns per thread (see rtn_code).  Bound by instructions (14336 x 16384 bf16 weights in
+// groups of 128: 231 us, 3.1 instructions per clock and SM, ALU pipe 51 %, 3.0 TB/s): these weights
 // took 1180 us with an fp64 division and one byte per thread.
 constexpr int kCodeRows = 16;
 template <int V, bool BF16>
@@ -136,8 +137,9 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
 
 // Residual E[i][c] = (a q + b) - w in fp64, either from stored codes or, for the OWC search, from min/max and a clipping
 // strength (codes formed on the fly, never stored).  With colmax it also leaves the largest |E| of every column there (as
-// ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  Memory-bound: 8 bytes written
-// per entry.  (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
+// ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  8 bytes written
+// per entry; bound by the latency of its loads (4096 x 4096 bf16 weights in groups: 46 us, 16 warps per SM at 86 registers, 2.8 TB/s).
+// (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
 // strengths of a 4096 x 4096 layer, 0.16 ms of them the maxima.)
 template <int V, bool BF16>
 __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_per_block, int blocks_per_group, double* __restrict__ E,

@@ -11,13 +11,15 @@
 // loss; the paper's box has the linear term with the opposite sign of its own definitions).
 // Ties go to the lowest group, then the lowest grid index; a change must strictly lower the loss.
 //
-// One CTA per column at a time (columns handed out by an atomic counter), fp64 throughout.  The
-// residual table r(., k) of the column is built once in a per-CTA scratch area.
-//   VERIFY: every sum in ascending index order without fused multiply-add, one thread per output,
-//           so that indices and codes can be compared bit for bit with a CPU statement of the steps.
-//   FAST:   M(k) = H_tt r(t, k) is tabulated once per column, after which a step needs only
-//           dot products of length g:  delta^T H_tt delta = r_k.M_k - 2 r_k.M_c + r_c.M_c;
-//           one warp per dot product, lanes across the group.
+// One CTA per column at a time (columns handed out by an atomic counter), fp64 throughout.
+//   owc_cd_kernel: the residual table r(., k) of the column is built once in a per-CTA scratch area.
+//     VERIFY: every sum in ascending index order without fused multiply-add, one thread per output,
+//             so that indices and codes can be compared bit for bit with a CPU statement of the steps.
+//     FAST:   M(k) = H_tt r(t, k) is tabulated once per column, after which a step needs only
+//             dot products of length g:  delta^T H_tt delta = r_k.M_k - 2 r_k.M_c + r_c.M_c;
+//             one warp per dot product, lanes across the group.
+//   owc_cd_codes_kernel (FAST, most grids: see codes_supported): the codes of every strength instead of the
+//     residuals, and the products r_k^T H_tt r_l instead of M.
 #include "common.cuh"
 #include "rtn_code.cuh"
 
