@@ -408,7 +408,7 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
   // G0 = 2 H (W_hat - W) and the loss at entry
   if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
-    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, base + L.hbuf, st));
+    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, false, base + L.hbuf, st));
     CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 2.0, G, true, L.ldg, col_loss, base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, G, L.ldg, col_loss, part, gemm_tc_supported(d_in, d_out), st));
@@ -556,7 +556,7 @@ cdq_status cdq_layer_loss(const float* H, const void* W, cdq_dtype wt, long long
   double* loss_sum = (double*)(base + L.scalars);
   if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
-    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, base + L.hbuf, st));
+    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, true, base + L.hbuf, st));
     CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), false, L.ldg, col_loss,
                          base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {

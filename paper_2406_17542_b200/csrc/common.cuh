@@ -109,7 +109,7 @@ cudaError_t launch_gemm_he_verify(const float* H, long long d_in, long long d_ou
 bool gemm_tc_supported(long long d_in, long long d_out);
 size_t gemm_tc_h_bytes(long long d_in, int nh);
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne);
-cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, void* hbuf, cudaStream_t st);
+cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, bool losses, void* hbuf, cudaStream_t st);
 cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
                         double scale, double* C, bool keep_c, long long ldc, double* col_loss, void* ebuf, cudaStream_t st);
 // Slice counts: the gradient and the loss of a descended solution need ~1e-9 of a_j H_pp (see

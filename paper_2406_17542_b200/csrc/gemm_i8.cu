@@ -20,6 +20,15 @@
 // K-major operands in 128-byte swizzled tiles loaded by TMA, tcgen05.mma kind::i8 with the
 // int32 accumulators in TMEM (two of them, so the epilogue of one group overlaps the MMAs of
 // the next), the same warp roles as the Hessian kernel.  Every mbarrier wait is bounded.
+//
+// Losses alone take half of the product.  H is symmetric, so with its rows and columns in blocks of 256, a column's loss is
+//     e^T H e = 2 sum_P e_P^T (T_P e_P + sum_{K in half(P)} H_PK e_K),
+// where half(P) holds one of the blocks (P, K), (K, P) of every pair: the nb / 2 blocks that follow P, in a circle, so that every tile
+// has the same work.  T_P is the lower triangle of the diagonal block with half of its diagonal; it has slices of its own, [ns][d][256].
+// What bounds the error is the digits of the small entries of H's rows; an entry's error, which the two halves of the whole product
+// would average with another one's, counts twice here, so the digits are rounded to nearest instead of truncated.  Column losses of given
+// codes against 64 bits (rms over columns and six layers each), whole -> half: 3072 x 512 5.2e-13 -> 5.2e-13 (solved codes 7.6e-12 ->
+// 6.2e-12), 4096 x 512 in groups 1.51e-12 -> 1.49e-12 (3.5e-10 -> 4.6e-11), 6144 x 256 in groups 3.4e-12 -> 3.1e-12 (9.1e-10 -> 6.0e-11).
 #include <cuda.h>
 
 #include "async_copy.cuh"
@@ -77,8 +86,11 @@ __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bit
 // 2^52 towards zero leaves the integer in the mantissa; scale = 2^(7 ns - e), a normal number for every exponent of H and E.
 // A NaN counts as zero, whatever its payload (that of CUDA's float NaN would pass for digits): a product leaves out the
 // entry and keeps the rest of its row.
-__device__ __forceinline__ unsigned long long slice_bits(double x, double scale) {
-  const double s = __dadd_rz(fabs(x) * scale, 4503599627370496.0);
+// NEAREST: rounded instead of truncated, half the error, up to `largest`, the largest number of ns digits.
+template <bool NEAREST>
+__device__ __forceinline__ unsigned long long slice_bits(double x, double scale, double largest = 0.0) {
+  const double f = fabs(x) * scale;
+  const double s = NEAREST ? __dadd_rn(f > largest ? largest : f, 4503599627370496.0) : __dadd_rz(f, 4503599627370496.0);
   return s != s ? 0ull : (unsigned long long)__double_as_longlong(s) & 0xFFFFFFFFFFFFFull;
 }
 // Digit i (from 1) of four neighbours, negated where `neg` has the byte's bits set, as four bytes.
@@ -93,12 +105,14 @@ __device__ __forceinline__ unsigned slice_bytes(const unsigned long long (&v)[4]
 // 4 bytes read and ns written per entry; what bounds it is the integer operations of the digits (4096^2, six slices: 45 us, the ALU pipe
 // 63 % busy, 2.5 TB/s).  (One column per thread, with the digits taken off one after
 // the other in fp64: 1.46 ms for 14336^2 and six slices.)
+// NEAREST: for half products.
+template <bool NEAREST>
 __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ exps,
                                int ns, signed char* __restrict__ out) {
   const long long p = blockIdx.y;
   const long long k = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
   if (k >= kp) return;
-  const double scale = ldexp(1.0, 7 * ns - exps[p]);
+  const double scale = ldexp(1.0, 7 * ns - exps[p]), largest = ldexp(1.0, 7 * ns) - 1.0;
   float x[4] = {0.f, 0.f, 0.f, 0.f};
   if ((d & 3) == 0) {
     if (k < d) {
@@ -114,11 +128,35 @@ __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long lo
   unsigned neg = 0u;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    b[v] = slice_bits((double)x[v], scale);
+    b[v] = slice_bits<NEAREST>((double)x[v], scale, largest);
     if (x[v] < 0.f) neg |= 0xFFu << (8 * v);
   }
   for (int i = 0; i < ns; ++i)
     *reinterpret_cast<unsigned*>(out + ((size_t)i * d + p) * kp + k) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+}
+
+// The lower triangles of the diagonal blocks of H, half of the diagonal -> slices [ns][d][256] int8 (row p scaled by 2^-exps[p]):
+// one row per warp, eight columns per thread.
+__global__ void __launch_bounds__(256) slice_diag_kernel(const float* __restrict__ H, long long d, const int* __restrict__ exps,
+                                                         int ns, signed char* __restrict__ out) {
+  const long long p = blockIdx.x * 8ll + (threadIdx.x >> 5);
+  if (p >= d) return;
+  const double scale = ldexp(1.0, 7 * ns - exps[p]), largest = ldexp(1.0, 7 * ns) - 1.0;
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    const int c = 4 * (threadIdx.x & 31) + 128 * part;
+    const long long k = p / BN * BN + c;
+    unsigned long long b[4];
+    unsigned neg = 0u;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const double x = k + v < p ? (double)H[p * d + k + v] : k + v == p ? 0.5 * (double)H[p * d + p] : 0.0;
+      b[v] = slice_bits<true>(x, scale, largest);
+      if (x < 0.0) neg |= 0xFFu << (8 * v);
+    }
+    for (int i = 0; i < ns; ++i)
+      *reinterpret_cast<unsigned*>(out + ((size_t)i * d + p) * BN + c) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+  }
 }
 
 // E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j]), 128 x 32 tiles turned round
@@ -150,7 +188,7 @@ __global__ void __launch_bounds__(256) slice_et_kernel(const double* __restrict_
     unsigned neg = 0u;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      b[v] = slice_bits(x[v], scale);
+      b[v] = slice_bits<false>(x[v], scale);
       if (x[v] < 0.0) neg |= 0xFFu << (8 * v);
     }
     for (int i = 0; i < ns; ++i)
@@ -171,6 +209,7 @@ struct Params {
   signed char pair_e[MAX_SLICES * MAX_SLICES], pair_h[MAX_SLICES * MAX_SLICES];  // slice indices (from 0)
   double* C;                // [M, ldc] fp64
   int keep_c;               // C is wanted (else only the column dots are, and C holds the running sums in between)
+  int half;                 // half of the product, the losses twice the dots
   long long ldc;
   const int* eexp;          // [M]
   const int* hexp;          // [N]
@@ -226,6 +265,8 @@ __device__ __forceinline__ double int_to_double(uint32_t r) {
 // 2^e for the exponents of normal numbers (those of products of fp32 data are).
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
+// Half of the product: how many blocks of 256 columns of H follow the diagonal one in tile column tn.
+__device__ __forceinline__ int blocks_after(int tn, int nb) { return (nb - 1) / 2 + ((nb & 1) == 0 && tn < nb / 2 ? 1 : 0); }
 // Tiles are handed out in bands of 8 tile rows, column by column inside a band, so that the
 // tiles in flight at one time share their operand panels in L2.
 __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tm, int& tn) {
@@ -237,7 +278,8 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 }
 
 __global__ void __launch_bounds__(NUM_THREADS, 1)
-gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_h, const Params p) {
+gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_h,
+               const __grid_constant__ CUtensorMap map_d, const Params p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;           // stage buffers, 1 KB aligned
@@ -285,12 +327,21 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
         for (int g = 0; g < p.ngroups && ok; ++g) {
           for (int pr = p.group_first[g]; pr < p.group_first[g + 1] && ok; ++pr) {
             const int se = p.pair_e[pr], sh = p.pair_h[pr];
-            for (int kb = 0; kb < p.kblocks; ++kb) {
+            const int steps = !p.half ? p.kblocks : 2 + 2 * blocks_after(tn, p.tiles_n);
+            for (int it = 0; it < steps; ++it) {
+              // K block of this step (half of the product: those of the diagonal block first; past the last column, zeros)
+              int kb = it;
+              if (p.half) {
+                const int block = tn + (it >> 1);
+                kb = 2 * (block < p.tiles_n ? block : block - p.tiles_n) + (it & 1);
+              }
+              const bool diag = p.half && it < 2;
               if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
               mbar_expect_tx(full_bar(stage), STAGE_BYTES);
               const uint32_t a_dst = tiles + (uint32_t)stage * STAGE_BYTES;
               tma_load_3d(a_dst, &map_e, kb * BKB, tm * BM, se, full_bar(stage));
-              tma_load_3d(a_dst + A_BYTES, &map_h, kb * BKB, tn * BN, sh, full_bar(stage));
+              if (diag) tma_load_3d(a_dst + A_BYTES, &map_d, it * BKB, tn * BN, sh, full_bar(stage));
+              else tma_load_3d(a_dst + A_BYTES, &map_h, kb * BKB, tn * BN, sh, full_bar(stage));
               ++issued;
               if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
@@ -318,11 +369,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
       uint32_t tphase = 0;
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+        int tm, tn;
+        tile_coords(t, p.tiles_m, p.tiles_n, tm, tn);
+        const int steps = !p.half ? p.kblocks : 2 + 2 * blocks_after(tn, p.tiles_n);
         for (int g = 0; g < p.ngroups && ok; ++g) {
           if (!mbar_wait(tempty_bar(buf), tphase ^ 1u, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t tmem_d = tmem_base + (uint32_t)buf * BN;
-          const int nsteps = (p.group_first[g + 1] - p.group_first[g]) * p.kblocks;
+          const int nsteps = (p.group_first[g + 1] - p.group_first[g]) * steps;
           for (int it = 0; it < nsteps; ++it) {
             if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -466,8 +520,15 @@ bool gemm_tc_supported(long long d_in, long long d_out) {
   return d_in >= 256 && d_out >= 128 && d_in <= 26000 && d_out < (1ll << 30);
 }
 
+// Losses by half of the product.  Short sums are bound by the slices and the epilogue: loss of given codes, whole / half (us):
+// 257 x 16384 388 / 406, 512 x 8192 273 / 276, 1350 x 677 291 / 283, 2048 x 2048 364 / 329, 3072 x 2048 775 / 657, 3072 x 130 407 / 371,
+// 4096 x 4096 1803 / 1290, 5376 x 300 640 / 499, 8192 x 1024 1719 / 1185; and with a few blocks only, halving costs precision
+// (257 x 16384 1.1e-13 -> 3.5e-13).
+static bool half_product(long long d_in) { return d_in >= 3072; }
+
 size_t gemm_tc_h_bytes(long long d_in, int nh) {
-  return align_up((size_t)nh * d_in * tc_kpad(d_in)) + align_up(sizeof(int) * (size_t)d_in);
+  return align_up((size_t)nh * d_in * tc_kpad(d_in)) + align_up(sizeof(int) * (size_t)d_in) +
+         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) : 0);   // the diagonal blocks
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -475,14 +536,22 @@ size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
          align_up(sizeof(unsigned long long) * (size_t)d_out);
 }
 
-// Slices of H (done once per call of the library; the OWC search reuses them for every gamma).
-cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, void* hbuf, cudaStream_t st) {
+// Slices of H (done once per call of the library; the OWC search reuses them for every gamma).  losses: for products without keep_c.
+cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, bool losses, void* hbuf, cudaStream_t st) {
   const long long kp = tc_kpad(d_in);
+  const bool half = losses && half_product(d_in);
   signed char* slices = (signed char*)hbuf;
   int* hexp = (int*)((char*)hbuf + align_up((size_t)nh * d_in * kp));
   { i8::row_exp_f32_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, hexp); count_launch(); }
   dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
-  { i8::slice_h_kernel<<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices); count_launch(); }
+  if (half) i8::slice_h_kernel<true><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices);
+  else i8::slice_h_kernel<false><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices);
+  count_launch();
+  if (half) {
+    signed char* diag = (signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
+    i8::slice_diag_kernel<<<(unsigned)((d_in + 7) / 8), 256, 0, st>>>(H, d_in, hexp, nh, diag);
+    count_launch();
+  }
   return cudaGetLastError();
 }
 
@@ -517,8 +586,10 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double
   using namespace i8;
   if (nh < 1 || nh > MAX_SLICES || ne < 1 || ne > MAX_SLICES || smax < 2) return cudaErrorInvalidValue;
   const long long kp = tc_kpad(d_in);
+  const bool half = !keep_c && half_product(d_in);
   const signed char* hsl = (const signed char*)hbuf;
   const int* hexp = (const int*)((const char*)hbuf + align_up((size_t)nh * d_in * kp));
+  const signed char* dsl = (const signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
   signed char* esl = (signed char*)ebuf;
   int* eexp = (int*)((char*)ebuf + align_up((size_t)ne * d_out * kp));
   unsigned long long* colmax = (unsigned long long*)((char*)eexp + align_up(sizeof(int) * (size_t)d_out));
@@ -550,15 +621,18 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double
   if (ng == 0) return cudaErrorInvalidValue;
   p.group_first[ng] = npairs;
   p.ngroups = ng;
-  p.C = C; p.keep_c = keep_c ? 1 : 0; p.ldc = ldc; p.eexp = eexp; p.hexp = hexp; p.final_scale = scale;
+  p.C = C; p.keep_c = keep_c ? 1 : 0; p.half = half ? 1 : 0; p.ldc = ldc; p.eexp = eexp; p.hexp = hexp; p.final_scale = scale;
   p.E = E; p.lde = d_out; p.dot_part = col_loss ? dot_part : nullptr;
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;
 
-  CUtensorMap map_e, map_h;
+  CUtensorMap map_e, map_h, map_d;
   e = encode_map3(&map_e, esl, kp, d_out, ne, BM);
   if (e != cudaSuccess) return e;
   e = encode_map3(&map_h, hsl, kp, d_in, nh, BN);
+  if (e != cudaSuccess) return e;
+  map_d = map_h;
+  if (half) e = encode_map3(&map_d, dsl, BN, d_in, nh, BN);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -566,11 +640,11 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double
   e = cudaFuncSetAttribute(gemm_i8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int ntiles = p.tiles_m * p.tiles_n;
-  { gemm_i8_kernel<<<ntiles < sms ? ntiles : sms, NUM_THREADS, SMEM_BYTES, st>>>(map_e, map_h, p); count_launch(); }
+  { gemm_i8_kernel<<<ntiles < sms ? ntiles : sms, NUM_THREADS, SMEM_BYTES, st>>>(map_e, map_h, map_d, p); count_launch(); }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (col_loss) {
-    { dot_reduce_kernel<<<(unsigned)((d_out + 255) / 256), 256, 0, st>>>(dot_part, 2 * p.tiles_n, d_out, 1.0 / scale, col_loss); count_launch(); }
+    { dot_reduce_kernel<<<(unsigned)((d_out + 255) / 256), 256, 0, st>>>(dot_part, 2 * p.tiles_n, d_out, (half ? 2.0 : 1.0) / scale, col_loss); count_launch(); }
     e = cudaGetLastError();
   }
   return e;

@@ -428,7 +428,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
     if (e != cudaSuccess) return e;
     // the host array must outlive the copy: pageable memcpy is staged before return
     if (L.tc) {   // the slices of H serve every clipping strength
-      e = gemm_tc_prepare_h(ly.H, d_in, kTcLossNH, base + L.hbuf, st);
+      e = gemm_tc_prepare_h(ly.H, d_in, kTcLossNH, true, base + L.hbuf, st);
       if (e != cudaSuccess) return e;
     }
     if (L.screened) {

@@ -1,0 +1,36 @@
+"""Losses by half of the product (rows of H from 3072 entries on): odd and even numbers of blocks of 256, a last block of fewer columns,
+few and many layer columns, against fp64 on the GPU."""
+import pytest
+import torch
+
+from paper_2406_17542_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d_in,d_out,group", [(3072, 130, 0), (3073, 128, 0), (3200, 300, 64), (3328, 257, 0), (3585, 1000, 0), (4100, 129, 4)])
+def test_losses_by_half_of_the_product(d_in, d_out, group):
+    dev = "cuda:0"
+    gen = torch.Generator(dev).manual_seed(d_in)
+    X = torch.randn(2000, d_in, generator=gen, device=dev) * torch.randn(d_in, generator=gen, device=dev).exp()
+    H = (X.double().T @ X.double()).float()
+    H = (torch.tril(H) + torch.tril(H, -1).T).contiguous()
+    W = torch.randn(d_in, d_out, generator=gen, device=dev) * 0.02
+    grid = B.Grid(3, group, 1, 1.0, 1.0)
+    scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
+    g = group or d_in
+    E = scale.double().repeat_interleave(g, 0) * Q.double() + zero.double().repeat_interleave(g, 0) - W.double()
+    want = ((H.double() @ E) * E).sum(0)
+    total, got = B.cdq_layer_loss(H, W, grid, scale, zero, Q, per_col=True)
+    # The digits of H end 42 bits below a row's power of two, those of a column of E 35 bits below its own, and slice pairs below
+    # 2^-63 of the two are left out: at most 2^-42 |e_p| |e_k| row_p + 2^-35 |e_p| |H_pk| col (both counted twice, rounding halves the
+    # first) + 12 K 2^-56 row_p col |e_p| (products of two digits of 7 bits).
+    row = torch.exp2(torch.frexp(H.abs().amax(1).double())[1].double())
+    col = torch.exp2(torch.frexp(E.abs().amax(0))[1].double())
+    a = E.abs()
+    bound = (2.0 ** -42 * (row @ a) * a.sum(0) + 2.0 ** -34 * (a * H.double().abs().sum(1, keepdim=True)).sum(0) * col
+             + 12 * d_in * 2.0 ** -56 * (row @ a) * col + 1e-13 * want.abs())
+    assert bool(((got - want).abs() <= bound).all())
+    # and far below that where the errors are as random as they are here
+    assert float(((got - want) / want).abs().max()) < 1e-9
+    assert abs(total - float(want.sum())) <= 1e-10 * float(want.sum())
