@@ -39,7 +39,7 @@ constexpr unsigned kAbortKey = 0u;    // a copy did not land
 constexpr unsigned kFullKey = 1u;     // drop the move in flight and score everything (a warp has no idle lane left)
 constexpr unsigned kCrowdKey = 2u;    // the move in flight stands, but score everything after it (same reason)
 constexpr unsigned kNever = 0x7F000000u;   // a threshold that no gradient reaches
-constexpr int kHand = 16;             // coordinates a warp hands over to its idle lanes at a time
+constexpr int kHand = 8;             // coordinates a warp hands over to its idle lanes at a time
 constexpr float kGap0 = 0.3f, kGapMin = 1.f / 256, kGapMax = 0.5f, kGapGrow = 1.25f;
 
 // A coordinate that a lane is to watch, handed over by the thread that owns its chunk.
@@ -106,10 +106,20 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
   unsigned char* row_s = dyn_smem;                                      // [2][NCH * NT] chunks
   float4* thr_s = reinterpret_cast<float4*>(row_s + 2 * (size_t)row_span);    // [NCH * NT] thresholds of the column
   Handover* hand = reinterpret_cast<Handover*>(thr_s + NCH * NT) + kHand * warp;   // [warps][kHand]
+  // H_ii and the column's group scales, if they fit beside the rows.  A coordinate that has just left its interval is scored before the
+  // team can go on, and from memory they come behind the row that is on its way into the SM (18432 in groups of 128 x 296 96.1 -> 93.3 ms,
+  // 9004 in groups of 4 x 296 16.4 -> 15.5, 13312 in groups of 128 x 296 46.1 -> 45.4, 14336 x 592 111.9 -> 110.3).
+  unsigned char* more = reinterpret_cast<unsigned char*>(reinterpret_cast<Handover*>(thr_s + NCH * NT) + kHand * nwarps);
+  const bool hd_here = (p.tables & 1) != 0, ag_here = GROUPED && (p.tables & 2) != 0;
+  float* hd_s = reinterpret_cast<float*>(more);
+  float* ag_s = hd_s + (hd_here ? 4 * NCH * NT : 0);
+  const float* hd_t = hd_here ? hd_s : p.hdiag;
   auto group_of = [&](unsigned i) -> unsigned { return p.g == 1 ? i : __umulhi(i, p.gmagic); };
 
   // slots past the end of the row stay zero: no copy ever writes there
   for (int t = tid; t < 2 * NCH * NT * CHB / 8; t += NT) reinterpret_cast<uint2*>(row_s)[t] = make_uint2(0u, 0u);
+  if (hd_here)
+    for (int t = tid; t < NCH * NT; t += NT) reinterpret_cast<float4*>(hd_s)[t] = __ldg(reinterpret_cast<const float4*>(p.hdiag) + t);
   if (tid == 0) {
     mbar_init(smem_u32(&s_bar[0]), 1);
     mbar_init(smem_u32(&s_bar[1]), 1);
@@ -142,7 +152,12 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       frozen = !(a_col > 0.f);   // constant column: its grid has one point, nothing can move
       gscale = frozen ? 0.0 : 1.0 / (double)a_col;
     }
-    const float* scale_j = p.scale + j;   // GROUPED: scale of group t at scale_j[t * d_out]
+    const float* scale_j = ag_here ? ag_s : p.scale + j;   // GROUPED: scale of group t at scale_j[t * scale_step]
+    const long long scale_step = ag_here ? 1 : p.d_out;
+    if (ag_here) {
+      for (int t = tid; t < (int)p.ng; t += NT) ag_s[t] = p.scale[(long long)t * p.d_out + j];
+      __syncthreads();
+    }
     double g[4 * NCH];
     unsigned qp[NCH];
     {
@@ -225,9 +240,9 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
     // The step of move w, and what else its sweep needs (loads: they overlap with the copy).
     auto load_step = [&](unsigned w, int istar) {
       float a = 1.f;
-      if (GROUPED) a = __ldg(scale_j + (long long)group_of((unsigned)istar) * p.d_out);
+      if (GROUPED) a = scale_j[(long long)group_of((unsigned)istar) * scale_step];
       c2 = 2.0 * ((double)a * (double)((int)(w & 511u) - 256));
-      if constexpr (ROW16) cur_h = __ldg(p.hdiag + istar);
+      if constexpr (ROW16) cur_h = hd_t[istar];
     };
     // Hands the coordinates of the two words over to idle lanes of the warp; true in the lanes that got one.
     // room: whether there were enough.
@@ -267,8 +282,8 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
               wid = hand[mine].id;
               wq = __uint_as_float(kMagicBits | hand[mine].q);
               wi = 4 * ((int)((wid >> 11) & 1023u) + NT * (int)(wid >> 21)) + (int)((wid >> 9) & 3u);
-              wh = __ldg(p.hdiag + wi);
-              if (GROUPED) wa = __ldg(scale_j + (long long)group_of((unsigned)wi) * p.d_out);
+              wh = hd_t[wi];
+              if (GROUPED) wa = scale_j[(long long)group_of((unsigned)wi) * scale_step];
               fresh = true;
             }
             who &= ~__ballot_sync(0xFFFFFFFFu, give);
@@ -299,11 +314,11 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
 #pragma unroll 1
       for (int k = 0; k < NCH; ++k) {
         const int cs = tid + NT * k;
-        const float4 hd = __ldg(reinterpret_cast<const float4*>(p.hdiag) + cs);
+        const float4 hd = reinterpret_cast<const float4*>(hd_t)[cs];
         const float4 hs = __ldg(reinterpret_cast<const float4*>(p.hs) + cs);
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
-          a = cs < nchs ? __ldg(scale_j + (long long)group_of(4u * (unsigned)cs) * p.d_out) : 0.f;
+          a = cs < nchs ? scale_j[(long long)group_of(4u * (unsigned)cs) * scale_step] : 0.f;
           ia = a > 0.f ? 1.0f / a : 0.f;
         }
         double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -328,10 +343,10 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
 #pragma unroll 1
       for (int k = 0; k < NCH; ++k) {
         const int cs = tid + NT * k;
-        const float4 hd = __ldg(reinterpret_cast<const float4*>(p.hdiag) + cs);
+        const float4 hd = reinterpret_cast<const float4*>(hd_t)[cs];
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
-          a = cs < nchs ? __ldg(scale_j + (long long)group_of(4u * (unsigned)cs) * p.d_out) : 0.f;
+          a = cs < nchs ? scale_j[(long long)group_of(4u * (unsigned)cs) * scale_step] : 0.f;
           ia = a > 0.f ? 1.0f / a : 0.f;
         }
         double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -574,14 +589,26 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
 }
 
 template <int NCH, int MAXNT, int MINB, bool GROUPED, bool ROW16>
-cudaError_t launch_cfg(const CdParams& p, int nt, cudaStream_t st) {
+cudaError_t launch_cfg(CdParams p, int nt, cudaStream_t st) {
   auto kern = cd_ahead_kernel<NCH, MAXNT, MINB, GROUPED, ROW16>;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // two rows, the thresholds, the handovers
-  const size_t smem = (size_t)NCH * nt * (ROW16 ? 16 : 32) + (size_t)NCH * nt * 16 + sizeof(Handover) * kHand * (size_t)(nt / 32);
+  size_t smem = (size_t)NCH * nt * (ROW16 ? 16 : 32) + (size_t)NCH * nt * 16 + sizeof(Handover) * kHand * (size_t)(nt / 32);
   cudaError_t e;
+  {   // H_ii and the group scales beside them where they fit (fp32 rows: up to 14336 entries)
+    cudaFuncAttributes fa{};
+    int optin = 0;
+    e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    const size_t room = (size_t)optin - fa.sharedSizeBytes, hd = (size_t)NCH * nt * 16, ag = GROUPED ? ((size_t)p.ng * 4 + 15) / 16 * 16 : 0;
+    p.tables = 0;
+    if (smem + hd <= room) { p.tables |= 1; smem += hd; }
+    if (GROUPED && smem + ag <= room) { p.tables |= 2; smem += ag; }
+  }
   if (smem > 32 * 1024) {   // the 48 KB that need no opt-in include the kernel's static shared memory
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -612,12 +639,14 @@ cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st) {
   const long long ch = p.d_in >> 2;
   auto team = [&](long long chunks, int nch) { return (int)((chunks + nch - 1) / nch + 31) / 32 * 32; };
   // 384 threads as long as the row fits them: three warps per scheduler hide more latency than the two of 256 threads with up to
-  // 14 chunks each (14336 x 1184 columns 236 -> 226 ms, 11008 x 296 47.4 -> 43.3), and at 168 registers nothing spills; rows of
+  // 14 chunks each (14336 x 1184 columns 236 -> 226 ms, 11008 x 296 47.4 -> 43.3), and at 168 registers nothing spills; rows of 13825 to 14336 entries
+  // fill 8 x 448 slots, with room for the table of H_ii beside them; rows of
   // 15361 to 16384 entries fill 8 x 512 slots (72 ms against 75 for 11 x 384 on 16384 x 296; 9 x 512 spills: 18432 x 592 226 ms
   // against 210 for 12 x 384).
   if (ch <= 2304) return launch_mode<6, 384, 1>(p, team(ch, 6), st);
   if (ch <= 3072) return launch_mode<8, 384, 1>(p, team(ch, 8), st);
   if (ch <= 3456) return launch_mode<9, 384, 1>(p, team(ch, 9), st);
+  if (ch <= 3584) return launch_mode<8, 448, 1>(p, team(ch, 8), st);
   if (ch <= 3840) return launch_mode<10, 384, 1>(p, team(ch, 10), st);
   if (ch <= 4096) return launch_mode<8, 512, 1>(p, team(ch, 8), st);
   if (ch <= 4224) return launch_mode<11, 384, 1>(p, team(ch, 11), st);

@@ -23,6 +23,7 @@ struct CdParams {
   long long T;
   CdCounters* ctr;
   int* status;          // device status word
+  int tables;           // cd_kernel_ahead.cu: bit 0 H_ii, bit 1 the column's group scales lie in shared memory
 };
 
 constexpr float kMagic = 12582912.0f;       // 1.5 * 2^23: adding it rounds to an integer
