@@ -6,16 +6,16 @@
 // tensor core (d_in is the contiguous dimension), so one TMA tensor map serves both.
 //
 //   * tile 128 x 256 per CTA, one tcgen05.mma (kind::f16, bf16 in, fp32 accumulate in TMEM)
-//     per 16 rows of X; only tiles that touch the lower triangle are computed (SYRK), the
-//     mirror image is written by the reduction kernel;
+//     per 16 rows of X; only tiles that touch the lower triangle are computed (SYRK);
 //   * TMA boxes of 64 columns x 64 rows with the 128-byte swizzle land in shared memory in
 //     exactly the canonical MN-major layout: 64-column blocks LBO = 8 KB apart, groups of
 //     8 rows SBO = 1 KB apart;
 //   * 4-stage TMA ring (full/empty mbarriers), two 256-column TMEM accumulators so that the
 //     epilogue of one tile overlaps the MMAs of the next, persistent CTAs over a static
 //     round-robin list of (K-split, tile) units;
-//   * warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2-5 = epilogue;
-//   * split-K partial tiles go to the caller's workspace and are summed in a fixed order, so
+//   * warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, warps 2-9 = epilogue;
+//   * without K splits the epilogue itself adds the tile to H and writes its mirror image, behind the MMAs of the
+//     next tile; split-K partial tiles go to the caller's workspace and a reduction kernel sums them in a fixed order, so
 //     the result does not depend on scheduling.
 // Every mbarrier wait is bounded: on expiry the kernel records kFlagWaitTimeout in the
 // device status word, lets the other roles drain, frees its TMEM and returns.
@@ -40,7 +40,8 @@ constexpr int TILE_ELEMS = BM * BN;
 // low, with 262144 rows past the 1e-3 the Hessian is allowed.  256 blocks = 16384 rows per accumulator bound
 // that near 6e-5; the chunks of a tile are added up by the epilogue with round-to-nearest fp32 adds.
 constexpr int KCHUNK = 256;
-constexpr int NUM_THREADS = 192;
+constexpr int EPI_WARPS = 8;          // two per TMEM lane quarter
+constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr int TMEM_COLS = 512;
 constexpr uint32_t SPIN_LIMIT = 1u << 22;
 constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)STAGES * STAGE_BYTES + 256;
@@ -50,6 +51,8 @@ struct Params {
   int tiles_m, ntiles, splits, kblocks;
   float* partials;   // [splits][ntiles][BM*BN]
   const int2* tiles; // [ntiles] (tm, tn) in the order the tiles are handed out
+  float* H;          // without K splits: where the epilogue adds the tiles ...
+  int accumulate;    // ... to what is there
   int* status;
 };
 
@@ -115,6 +118,10 @@ __global__ void hessian_tile_order_kernel(int tiles_m, int2* __restrict__ tiles)
   }
 }
 
+// DIRECT: no K splits, the epilogue writes H (8 batches of 4096 x 8192: the pass over the partial tiles took 0.1 of 0.38 ms per batch,
+// 2.69 -> 2.27 ms in all; 4096 x 8192 4 batches 0.39 -> 0.32;
+// streaming loads and stores of H no faster, with four epilogue warps 5352 features x 2048 rows 0.69 -> 0.78 ms).
+template <bool DIRECT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
   extern __shared__ unsigned char smem_raw[];
@@ -133,7 +140,7 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 4); }
+    for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), EPI_WARPS); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -231,6 +238,7 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
   } else {
     // ---------------- epilogue: TMEM -> registers -> partial tile in global memory ----------------
     const int q = warp & 3;                 // TMEM lane quarter this warp may read
+    const int half = (warp - 2) >> 2;       // which of the two warps of the quarter: they take the chunks of 32 columns in turn
     const int row = q * 32 + lane;          // row of the tile
     int buf = 0;
     uint32_t tphase = 0;
@@ -243,8 +251,71 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
         if (!mbar_wait(tfull_bar(buf), tphase, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const bool first = kc0 == kb0;   // later chunks add to what this thread stored before (round-to-nearest adds)
+        if (DIRECT && kc0 + KCHUNK >= kb1) {
+          // ---- the tile is complete: its entries below the diagonal go to H, with their mirror image ----
+          const int2 tc = p.tiles[u];
+          const long long d = p.d_in, rw = (long long)tc.x * BM + q * 32, r = rw + lane, c0 = (long long)tc.y * BN;
+          const bool rows_in = rw + 31 < d && (d & 3) == 0;
+          float* hrow = p.H + r * d + c0;
+          float4 old[8];
+          // a chunk of 32 columns whose entries all lie below the diagonal, in rows on 16-byte boundaries
+          auto whole = [&](int c) { return rows_in && c0 + c * 32 + 31 < rw; };
+          auto fetch = [&](int c) {
+            if (p.accumulate && c < BN / 32 && whole(c)) {
+#pragma unroll
+              for (int v = 0; v < 8; ++v) old[v] = *reinterpret_cast<const float4*>(hrow + c * 32 + v * 4);
+            } else {
+#pragma unroll
+              for (int v = 0; v < 8; ++v) old[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          };
+          fetch(half);
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
+          for (int c = half; c < BN / 32; c += 2) {
+            const long long cb = c0 + c * 32;
+            if (rw >= d || cb >= d || cb > rw + 31) break;   // outside, or above the diagonal, like all chunks after it
+            uint32_t b[32];
+            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), b);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            float x[32];
+#pragma unroll
+            for (int v = 0; v < 32; ++v) x[v] = __uint_as_float(b[v]);
+            if (!first) {
+#pragma unroll
+              for (int v = 0; v < 8; ++v) {
+                const float4 y = *reinterpret_cast<const float4*>(out + c * 32 + v * 4);
+                x[4 * v] += y.x; x[4 * v + 1] += y.y; x[4 * v + 2] += y.z; x[4 * v + 3] += y.w;
+              }
+            }
+            if (whole(c)) {
+              if (p.accumulate) {
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                  x[4 * v] += old[v].x; x[4 * v + 1] += old[v].y; x[4 * v + 2] += old[v].z; x[4 * v + 3] += old[v].w;
+                }
+                fetch(c + 2);   // on its way while this chunk is written
+              }
+#pragma unroll
+              for (int v = 0; v < 8; ++v)
+                *reinterpret_cast<float4*>(hrow + c * 32 + v * 4) = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+              float* mirror = p.H + cb * d + r;   // one column of the tile after the other, 32 rows side by side
+#pragma unroll
+              for (int v = 0; v < 32; ++v) mirror[v * d] = x[v];
+            } else if (r < d) {
+#pragma unroll
+              for (int v = 0; v < 32; ++v) {
+                const long long cc = cb + v;
+                if (cc <= r) {
+                  if (p.accumulate) x[v] += p.H[r * d + cc];
+                  p.H[r * d + cc] = x[v];
+                  if (cc < r) p.H[cc * d + r] = x[v];
+                }
+              }
+            }
+          }
+        } else {
+#pragma unroll 1
+        for (int c = half; c < BN / 32; c += 2) {
           uint32_t r[32];
           tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), r);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -259,6 +330,7 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
             }
             *dst = x;
           }
+        }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -420,13 +492,16 @@ cudaError_t launch_hessian_tc(const void* X, long long n, long long d_in, long l
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e = cudaFuncSetAttribute(hessian_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+  const bool direct = pl.splits == 1;
+  p.H = H; p.accumulate = accumulate;
+  auto kern = direct ? hessian_tc_kernel<true> : hessian_tc_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int units = pl.ntiles * pl.splits;
   const int grid = units < sms ? units : sms;
-  { hessian_tc_kernel<<<grid, NUM_THREADS, SMEM_BYTES, st>>>(tmap, p); count_launch(); }
+  { kern<<<grid, NUM_THREADS, SMEM_BYTES, st>>>(tmap, p); count_launch(); }
   e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || direct) return e;
   const dim3 pieces((unsigned)pl.ntiles, (BM / RP) * (BN / RP));
   if (d_in % 4 == 0) { hessian_reduce_kernel<true><<<pieces, 256, 0, st>>>(p, accumulate, H); count_launch(); }
   else { hessian_reduce_kernel<false><<<pieces, 256, 0, st>>>(p, accumulate, H); count_launch(); }
