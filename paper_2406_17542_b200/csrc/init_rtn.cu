@@ -4,6 +4,8 @@
 //   min/max per (group, column)  ->  b = min, a = fp32(gamma (max-min) / L)
 //   q = clamp(round_half_even((w - b) / a), 0, L)      (decided in fp64)
 //   OWC: loss_k[j] = e_k^T H e_k for every gamma_k, argmin over k per column.
+#include <type_traits>
+
 #include "common.cuh"
 #include "rtn_code.cuh"
 
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
   for (int v = 0; v < V; ++v) {
     a[v] = scale[t * d_out + j + v];
     b[v] = zero[t * d_out + j + v];
-    inv[v] = rtn_inverse(a[v]);
+    inv[v] = rtn_inverse_or_zero(a[v]);
   }
   constexpr int R = 8;   // rows whose loads are in flight together (the compiler moves no load past the branch of rtn_code)
   for (long long i = i0; i < i1; i += R) {
@@ -126,12 +128,80 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (i + r >= i1) break;
-      unsigned q = 0u;
-#pragma unroll
-      for (int v = 0; v < V; ++v) q |= (a[v] > 0.f ? rtn_code(w[r][v], a[v], inv[v], b[v], (float)L) : 0u) << (8 * v);
-      if constexpr (V == 4) *reinterpret_cast<unsigned*>(Q + (i + r) * d_out + j) = q;
-      else Q[(i + r) * d_out + j] = (unsigned char)q;
+      if constexpr (V == 4) *reinterpret_cast<unsigned*>(Q + (i + r) * d_out + j) = rtn_code4(w[r], a, inv, b, (float)L);
+      else Q[(i + r) * d_out + j] = (unsigned char)(a[0] > 0.f ? rtn_code(w[r][0], a[0], inv[0], b[0], (float)L) : 0u);
     }
+  }
+}
+
+// Grid and codes of one group of at most 8 WARPS rows for 128 columns, without a clipping search: the weights are read once and stay in
+// registers, eight rows of four columns per thread, while the block's warps put their minima and maxima together.  14336 x 16384
+// weights in groups of 128, against three passes: bf16 336 -> 265 us (2.7 TB/s), fp32 399 -> 271 (4.3); bound by instructions and by the
+// divisions that a block waits for.
+template <int WARPS, bool BF16>
+__global__ void __launch_bounds__(32 * WARPS, 1024 / (32 * WARPS)) group_codes_kernel(const void* __restrict__ W, long long d_out, long long ldw, long long g, int L,
+                                                          float* __restrict__ scale, float* __restrict__ zero,
+                                                          unsigned char* __restrict__ Q) {
+  constexpr int ROWS = 8;
+  __shared__ __align__(16) float s_mn[WARPS][128], s_mx[WARPS][128], s_a[128], s_b[128], s_inv[128];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long j0 = blockIdx.x * 128ll, j = j0 + 4 * lane, t = blockIdx.y, i1 = (t + 1) * g, i0 = t * g + warp * ROWS;
+  const bool inside = j < d_out;   // (d_out is a multiple of four)
+  using Four = std::conditional_t<BF16, uint2, float4>;   // four weights as they lie in memory
+  Four w[ROWS];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r)
+    w[r] = __ldg(reinterpret_cast<const Four*>((const char*)W + (min(i0 + r, i1 - 1) * ldw + (inside ? j : 0)) * (BF16 ? 2 : 4)));
+  auto widen = [](const Four& f, float (&x)[4]) {
+    if constexpr (BF16) {
+      x[0] = __uint_as_float(f.x << 16); x[1] = __uint_as_float(f.x & 0xFFFF0000u);
+      x[2] = __uint_as_float(f.y << 16); x[3] = __uint_as_float(f.y & 0xFFFF0000u);
+    } else {
+      x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
+    }
+  };
+  float4 mn, mx;
+  if constexpr (BF16) {   // two at a time
+    uint2 lo = w[0], hi = w[0];
+#pragma unroll
+    for (int r = 1; r < ROWS; ++r) {
+      asm("min.bf16x2 %0, %0, %1;" : "+r"(lo.x) : "r"(w[r].x)); asm("min.bf16x2 %0, %0, %1;" : "+r"(lo.y) : "r"(w[r].y));
+      asm("max.bf16x2 %0, %0, %1;" : "+r"(hi.x) : "r"(w[r].x)); asm("max.bf16x2 %0, %0, %1;" : "+r"(hi.y) : "r"(w[r].y));
+    }
+    float x[4];
+    widen(lo, x); mn = make_float4(x[0], x[1], x[2], x[3]);
+    widen(hi, x); mx = make_float4(x[0], x[1], x[2], x[3]);
+  } else {
+    mn = mx = w[0];
+#pragma unroll
+    for (int r = 1; r < ROWS; ++r) {
+      mn.x = fminf(mn.x, w[r].x); mn.y = fminf(mn.y, w[r].y); mn.z = fminf(mn.z, w[r].z); mn.w = fminf(mn.w, w[r].w);
+      mx.x = fmaxf(mx.x, w[r].x); mx.y = fmaxf(mx.y, w[r].y); mx.z = fmaxf(mx.z, w[r].z); mx.w = fmaxf(mx.w, w[r].w);
+    }
+  }
+  *reinterpret_cast<float4*>(&s_mn[warp][4 * lane]) = mn;
+  *reinterpret_cast<float4*>(&s_mx[warp][4 * lane]) = mx;
+  __syncthreads();
+  if (threadIdx.x < 128) {
+    const int c = threadIdx.x;
+    float lo = s_mn[0][c], hi = s_mx[0][c];
+#pragma unroll
+    for (int k = 1; k < WARPS; ++k) { lo = fminf(lo, s_mn[k][c]); hi = fmaxf(hi, s_mx[k][c]); }
+    // as scale_zero_kernel with a clipping strength of one
+    const float a = (float)__ddiv_rn(__dadd_rn((double)hi, -(double)lo), (double)L);
+    s_a[c] = a; s_b[c] = lo; s_inv[c] = rtn_inverse_or_zero(a);
+    if (j0 + c < d_out) { scale[t * d_out + j0 + c] = a; zero[t * d_out + j0 + c] = lo; }
+  }
+  __syncthreads();
+  if (!inside) return;
+  const float4 a4 = *reinterpret_cast<const float4*>(&s_a[4 * lane]), b4 = *reinterpret_cast<const float4*>(&s_b[4 * lane]);
+  const float4 v4 = *reinterpret_cast<const float4*>(&s_inv[4 * lane]);
+  const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w}, inv[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+    float x[4];
+    widen(w[r], x);
+    if (i0 + r < i1) *reinterpret_cast<unsigned*>(Q + (i0 + r) * d_out + j) = rtn_code4(x, a, inv, b, (float)L);
   }
 }
 
@@ -160,7 +230,7 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
       const double gamma = s.col_gamma ? s.gammas[s.col_gamma[c + v]] : s.n_cols ? s.gammas[s.k0 + c / s.d_out] : s.gamma;
       a[v] = (float)__ddiv_rn(__dmul_rn(gamma, __dadd_rn(hi, -lo)), (double)s.L);
       b[v] = (float)lo;
-      inv[v] = rtn_inverse(a[v]);
+      inv[v] = rtn_inverse_or_zero(a[v]);
     } else {
       a[v] = s.scale[t * s.d_out + j + v];
       b[v] = s.zero[t * s.d_out + j + v];
@@ -184,10 +254,13 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
     for (int r = 0; r < R; ++r) {
       if (i + r >= i1) break;
       double e[V];
+      if (s.use_gamma) {
+        if constexpr (V == 4) q4[r] = rtn_code4(w[r], a, inv, b, (float)s.L);
+        else q4[r] = a[0] > 0.f ? rtn_code(w[r][0], a[0], inv[0], b[0], (float)s.L) : 0u;
+      }
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        unsigned q = (q4[r] >> (8 * v)) & 255u;
-        if (s.use_gamma) q = a[v] > 0.f ? rtn_code(w[r][v], a[v], inv[v], b[v], (float)s.L) : 0u;
+        const unsigned q = (q4[r] >> (8 * v)) & 255u;
         // 2^52 + q: its lower word is q
         const double qd = __hiloint2double(0x43300000, (int)q) - 4503599627370496.0;
         e[v] = __dadd_rn(__dadd_rn(__dmul_rn((double)a[v], qd), (double)b[v]), -(double)w[r][v]);
@@ -411,6 +484,18 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
   float* mx = (float*)(base + L.mx);
   const unsigned bx = (unsigned)((d_out + 127) / 128);
 
+  const bool fours = four_columns(ly) && reinterpret_cast<uintptr_t>(Q) % 4 == 0;
+  const dim3 grid_g(bx, (unsigned)ng);
+  // Groups that a block holds at once, and blocks enough to fill the SMs twice (three passes / this, us: 4096 x 4096 bf16 in groups
+  // of 128 50 / 37, 1536 x 4100 in groups of 4 46 / 30; with fewer blocks the two are equal, both launches: 512 x 700 38 / 38).
+  if (n_clip == 1 && fours && g <= 128 && (long long)bx * ng >= 592) {
+    if (gamma_out) { fill_gamma_kernel<<<bx, 128, 0, st>>>(gamma_out, d_out); count_launch(); }
+    const int warps = g <= 32 ? 4 : g <= 64 ? 8 : 16;
+    auto run = [&](auto kern) { kern<<<grid_g, 32 * warps, 0, st>>>(ly.W, d_out, ly.ldw, g, ly.L, scale, zero, Q); count_launch(); };
+    if (ly.wt == CDQ_BF16) run(warps == 4 ? group_codes_kernel<4, true> : warps == 8 ? group_codes_kernel<8, true> : group_codes_kernel<16, true>);
+    else run(warps == 4 ? group_codes_kernel<4, false> : warps == 8 ? group_codes_kernel<8, false> : group_codes_kernel<16, false>);
+    return cudaGetLastError();
+  }
   run_minmax_partial(ly, cpg, pmn, pmx, st);
   { minmax_final_kernel<<<dim3(bx, (unsigned)ng), 128, 0, st>>>(pmn, pmx, ng, d_out, cpg, mn, mx); count_launch(); }
 
@@ -504,7 +589,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
   const int bpg = (int)((g + kCodeRows - 1) / kCodeRows);
   // (as for the minima; bf16 weights, one column against four, us: 1024 x 2048, 2^17 columns and row blocks, 5.7 / 7.2, 2048 x 2048 9.5 / 7.6,
   // 4096 x 4096 27 / 19)
-  const bool four = four_columns(ly) && reinterpret_cast<uintptr_t>(Q) % 4 == 0 && d_out * ng * bpg >= (1 << 18);
+  const bool four = fours && d_out * ng * bpg >= (1 << 18);
   const dim3 grid_q((unsigned)(four ? (d_out + 511) / 512 : bx), (unsigned)(ng * bpg));
   auto run = [&](auto kern) { kern<<<grid_q, 128, 0, st>>>(ly.W, d_out, ly.ldw, g, bpg, ly.L, scale, zero, Q); count_launch(); };
   if (ly.wt == CDQ_BF16) run(four ? rtn_codes_kernel<4, true> : rtn_codes_kernel<1, true>);

@@ -31,5 +31,31 @@ __device__ __forceinline__ unsigned rtn_code(float w, float a, float inv_a, floa
   if (!(fabsf(c - (m - kMagic)) < 0.4998f) || !(fabsf(t) <= 3.402823466e38f)) return rtn_code_f64(w, a, b, top);
   return __float_as_uint(m) & 255u;
 }
+// Four neighbouring codes as bytes (a <= 0: code 0).  One branch for the four (with one for each, and the bytes put together by shifts, the
+// codes of 14336 x 16384 weights took a quarter longer;
+// min, max and a sum that keeps a NaN instead of a chain of conditions: 341 -> 287 us for grid and codes of them in groups of 128).
+__device__ __forceinline__ float rtn_inverse_or_zero(float a) { return a > 0.f ? rtn_inverse(a) : 0.f; }
+__device__ __forceinline__ unsigned rtn_code4(const float (&w)[4], const float (&a)[4], const float (&inv_a)[4], const float (&b)[4],
+                                              float top) {
+  constexpr float kMagic = 12582912.0f;
+  unsigned m[4];
+  float off = 0.f, not_finite = 0.f;   // the largest distance from a level; a NaN if a quotient is none or overflows
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const float t = (w[v] - b[v]) * inv_a[v];
+    const float c = fminf(fmaxf(t, 0.f), top);
+    const float r = c + kMagic;
+    off = fmaxf(off, fabsf(c - (r - kMagic)));
+    not_finite = fmaf(t, 0.f, not_finite);
+    m[v] = __float_as_uint(r);
+  }
+  if (!(off < 0.4998f && not_finite == 0.f)) {
+    unsigned q = 0u;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) q |= (a[v] > 0.f ? rtn_code(w[v], a[v], inv_a[v], b[v], top) : 0u) << (8 * v);
+    return q;
+  }
+  return __byte_perm(__byte_perm(m[0], m[1], 0x0040), __byte_perm(m[2], m[3], 0x0040), 0x5410);
+}
 
 }  // namespace cdq
