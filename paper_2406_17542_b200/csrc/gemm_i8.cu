@@ -208,7 +208,7 @@ struct Params {
   int group_s[MAX_GROUPS];            // i + j of the group (slices numbered from 1)
   signed char pair_e[MAX_SLICES * MAX_SLICES], pair_h[MAX_SLICES * MAX_SLICES];  // slice indices (from 0)
   double* C;                // [M, ldc] fp64
-  int keep_c;               // C is wanted (else only the column dots are, and C holds the running sums in between)
+  int keep_c;               // C is wanted, else only the column dots are
   int half;                 // half of the product, the losses twice the dots
   long long ldc;
   const int* eexp;          // [M]
@@ -396,12 +396,12 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
     }
   } else {
     // ---------------- epilogue: TMEM -> fp64 running sum in C ----------------
-    // Two warps per TMEM lane quarter; they take the 16-column chunks of the tile in turn.  A product of two groups (the
-    // screen of the clipping search) waits for both accumulators and needs no running sum.
+    // Two warps per TMEM lane quarter; they take the 16-column chunks of the tile in turn.  Where only the dots are wanted, every group
+    // gives its own, 128^-s E . acc, and there is no running sum
+    // (16 bytes per entry and group; loss of 4096 x 4096 codes 1290 -> 1001 us, 1350 x 677 291 -> 202, clipping search 4.3 -> 4.1 ms).
     const int q = warp & 3;                 // TMEM lane quarter this warp may read
     const int half = (warp - 2) >> 2;       // which of the two warps of the quarter
     const int row = q * 32 + lane;          // row of the tile
-    const bool both = p.ngroups == 2;
     int buf = 0;
     uint32_t tphase = 0;
     bool ok = true;
@@ -414,31 +414,36 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
       double* crow = p.C + (row_ok ? j : 0) * p.ldc;
       const int ej = row_ok ? p.eexp[j] : 0;
       double dot = 0.0;
-      for (int g = both ? 1 : 0; g < p.ngroups && ok; ++g) {
-        if (both && !mbar_wait(tfull_bar(buf ^ 1), tphase, abort_flag)) { ok = false; break; }
-        if (both) buf ^= 1;   // (buf: the accumulator of group g; groups 0 and 1 lie in buffers 0 and 1)
-        if (!mbar_wait(tfull_bar(both ? 0 : buf), tphase, abort_flag)) { ok = false; break; }
+      for (int g = 0; g < p.ngroups && ok; ++g) {
+        if (!mbar_wait(tfull_bar(buf), tphase, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const double w = pow2(-7 * p.group_s[g]), w0 = pow2(-7 * p.group_s[0]);
+        const double w = pow2(-7 * p.group_s[g]);
         const bool first = g == 0, last = g == p.ngroups - 1;
+        double part = 0.0;
 #pragma unroll 1
         for (int c = half; c < BN / 16; c += 2) {
-          uint32_t r[16], r0[16];
+          uint32_t r[16];
           tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 16), r);
-          if (both) tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), r0);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (!row_ok) continue;
           const long long pc0 = p0 + c * 16;
-          if (pc0 + 16 <= p.N) {
+          if (!p.keep_c) {
+            const double* e = p.E + pc0 * p.lde + j;
+            if (pc0 + 16 <= p.N) {
+#pragma unroll
+              for (int v = 0; v < 16; ++v) part = fma(e[v * p.lde], int_to_double(r[v]) * pow2(p.hexp[pc0 + v]), part);
+            } else {
+#pragma unroll
+              for (int v = 0; v < 16; ++v)
+                if (pc0 + v < p.N) part = fma(e[v * p.lde], int_to_double(r[v]) * pow2(p.hexp[pc0 + v]), part);
+            }
+          } else if (pc0 + 16 <= p.N) {
             // whole chunk inside the matrix: 16-byte accesses (ldc is a multiple of 4, pc0 of 16)
             double2* cp = reinterpret_cast<double2*>(crow + pc0);
             double x[16];
 #pragma unroll
             for (int v = 0; v < 16; ++v) x[v] = w * int_to_double(r[v]);
-            if (both) {
-#pragma unroll
-              for (int v = 0; v < 16; ++v) x[v] += w0 * int_to_double(r0[v]);
-            } else if (!first) {
+            if (!first) {
               double2 old[8];
 #pragma unroll
               for (int v = 0; v < 8; ++v) old[v] = cp[v];
@@ -453,36 +458,31 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
                 for (int v = 0; v < 16; ++v) dot = fma(p.E[(pc0 + v) * p.lde + j], x[v], dot);
               }
             }
-            if (!last || p.keep_c) {
 #pragma unroll
-              for (int v = 0; v < 8; ++v) cp[v] = make_double2(x[2 * v], x[2 * v + 1]);
-            }
+            for (int v = 0; v < 8; ++v) cp[v] = make_double2(x[2 * v], x[2 * v + 1]);
           } else {
 #pragma unroll
             for (int v = 0; v < 16; ++v) {
               const long long pc = pc0 + v;
               if (pc < p.N) {
                 double x = w * int_to_double(r[v]);
-                if (both) x += w0 * int_to_double(r0[v]);
-                else if (!first) x += crow[pc];
+                if (!first) x += crow[pc];
                 if (last) {
                   x = x * p.final_scale * pow2(ej + p.hexp[pc]);
                   if (p.dot_part) dot = fma(p.E[pc * p.lde + j], x, dot);
                 }
-                if (!last || p.keep_c) crow[pc] = x;
+                crow[pc] = x;
               }
             }
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
-        if (lane == 0) {
-          if (both) mbar_arrive(tempty_bar(0));
-          mbar_arrive(tempty_bar(buf));
-        }
+        if (lane == 0) mbar_arrive(tempty_bar(buf));
+        dot = fma(w, part, dot);   // (the smallest group comes first)
         if (++buf == 2) { buf = 0; tphase ^= 1u; }
       }
-      if (p.dot_part && row_ok && ok) p.dot_part[(size_t)(2 * tn + half) * p.M + j] = dot;
+      if (p.dot_part && row_ok && ok) p.dot_part[(size_t)(2 * tn + half) * p.M + j] = p.keep_c ? dot : dot * p.final_scale * pow2(ej);
     }
   }
 
@@ -520,9 +520,9 @@ bool gemm_tc_supported(long long d_in, long long d_out) {
   return d_in >= 256 && d_out >= 128 && d_in <= 26000 && d_out < (1ll << 30);
 }
 
-// Losses by half of the product.  Short sums are bound by the slices and the epilogue: loss of given codes, whole / half (us):
-// 257 x 16384 388 / 406, 512 x 8192 273 / 276, 1350 x 677 291 / 283, 2048 x 2048 364 / 329, 3072 x 2048 775 / 657, 3072 x 130 407 / 371,
-// 4096 x 4096 1803 / 1290, 5376 x 300 640 / 499, 8192 x 1024 1719 / 1185; and with a few blocks only, halving costs precision
+// Losses by half of the product.  Short sums are bound by the slices and the epilogue: loss of given codes, whole / half (us, both with a
+// running sum): 257 x 16384 388 / 406, 512 x 8192 273 / 276, 1350 x 677 291 / 283, 2048 x 2048 364 / 329, 3072 x 2048 775 / 657, 3072 x 130
+// 407 / 371, 4096 x 4096 1803 / 1290, 5376 x 300 640 / 499, 8192 x 1024 1719 / 1185; and with a few blocks only, it costs precision
 // (257 x 16384 1.1e-13 -> 3.5e-13).
 static bool half_product(long long d_in) { return d_in >= 3072; }
 
