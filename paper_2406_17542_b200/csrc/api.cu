@@ -408,8 +408,8 @@ static cdq_status cd_solve_impl(const float* H, const void* W, cdq_dtype wt, lon
   // G0 = 2 H (W_hat - W) and the loss at entry
   if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
-    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, false, base + L.hbuf, st));
-    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 2.0, G, true, L.ldg, col_loss, base + L.ebuf, st));
+    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, kTcProduct, base + L.hbuf, st));
+    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, kTcProduct, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 2.0, G, L.ldg, col_loss, base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, G, L.ldg, col_loss, part, gemm_tc_supported(d_in, d_out), st));
   } else {
@@ -556,8 +556,8 @@ cdq_status cdq_layer_loss(const float* H, const void* W, cdq_dtype wt, long long
   double* loss_sum = (double*)(base + L.scalars);
   if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
-    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, true, base + L.hbuf, st));
-    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), false, L.ldg, col_loss,
+    CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, kTcLoss, base + L.hbuf, st));
+    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, kTcLoss, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), L.ldg, col_loss,
                          base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, gemm_tc_supported(d_in, d_out), st));

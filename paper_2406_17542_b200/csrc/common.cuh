@@ -86,9 +86,9 @@ struct ResidualSrc {
   const double* gammas;    // ... instead of `gamma`
   int k0;                  // ... the strength gammas[k0 + c / d_out]
 };
-// colmax (may be NULL, zeroed by the caller): largest |E| per column as ordered bit patterns.
+// colmax (may be NULL, zeroed by the caller): largest |E| per column as ordered bit patterns, row i counted 2^row_exp[i] (may be NULL).
 cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st,
-                                unsigned long long* colmax = nullptr);
+                                unsigned long long* colmax = nullptr, const int* row_exp = nullptr);
 
 // gemm_f64.cu : C = H * E in fp64.
 // G (may be NULL): [d_out, ldg] doubles, G[j][p] = 2 * C[p][j].
@@ -105,13 +105,15 @@ cudaError_t launch_gemm_he_verify(const float* H, long long d_in, long long d_ou
 // gemm_i8.cu : C[j, p] = scale * sum_k E[k, j] H[p, k] on the int8 tensor cores from 7-bit slices of
 // both operands (nh slices of H, ne of E, slice pairs up to i + j = smax); C is [d_out, ldc].
 // col_loss (may be NULL): [d_out], e_j^T H e_j.  gemm_tc_run forms the residual E [d_in, d_out] from its source first;
-// without keep_c the caller wants col_loss only and C is scratch.
+// C is written by kTcProduct only; the other uses are for col_loss alone: the loss of codes, and the clipping search, whose few digits the
+// features are scaled for.
+enum TcUse { kTcProduct, kTcLoss, kTcSearch };
 bool gemm_tc_supported(long long d_in, long long d_out);
 size_t gemm_tc_h_bytes(long long d_in, int nh);
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne);
-cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, bool losses, void* hbuf, cudaStream_t st);
-cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
-                        double scale, double* C, bool keep_c, long long ldc, double* col_loss, void* ebuf, cudaStream_t st);
+cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use, void* hbuf, cudaStream_t st);
+cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
+                        double scale, double* C, long long ldc, double* col_loss, void* ebuf, cudaStream_t st);
 // Slice counts: the gradient and the loss of a descended solution need ~1e-9 of a_j H_pp (see
 // gemm_i8.cu); the losses of the OWC search (round-to-nearest residuals) need ~1e-7 relative.
 constexpr int kTcGradNH = 6, kTcGradNE = 5, kTcGradSmax = 9;

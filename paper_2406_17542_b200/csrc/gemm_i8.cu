@@ -25,11 +25,18 @@
 //     e^T H e = 2 sum_P e_P^T (T_P e_P + sum_{K in half(P)} H_PK e_K),
 // where half(P) holds one of the blocks (P, K), (K, P) of every pair: the nb / 2 blocks that follow P, in a circle, so that every tile
 // has the same work.  T_P is the lower triangle of the diagonal block with half of its diagonal; it has slices of its own, [ns][d][256].
-// What bounds the error is the digits of the small entries of H's rows; an entry's error, which the two halves of the whole product
-// would average with another one's, counts twice here, so the digits are rounded to nearest instead of truncated.  Column losses of given
-// codes against 64 bits (rms over columns and six layers each), whole -> half: 3072 x 512 5.2e-13 -> 5.2e-13 (solved codes 7.6e-12 ->
-// 6.2e-12), 4096 x 512 in groups 1.51e-12 -> 1.49e-12 (3.5e-10 -> 4.6e-11), 6144 x 256 in groups 3.4e-12 -> 3.1e-12 (9.1e-10 -> 6.0e-11).
+// The two halves of the whole product average an entry's slicing error with that of its mirror image; here it counts twice.  Two things
+// make up for that.  The digits are balanced (balanced_bits below).  And the clipping search, whose screen has two or three digits of
+// either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk), so the rows no
+// longer mix entries of many sizes, and what an entry of E weighs in the loss is its size.  The residuals of given codes are a few dozen
+// bits on one grid, which five digits hold exactly, and D would take them off it: cdq_layer_loss goes without (column losses of
+// 8192 x 300 codes against 64 bits, rms: with D 3.9e-13, without 1.1e-13; whole product 1.0e-13).  Errors against 64 bits, whole -> half:
+//   thirteen pairs (largest of five layers of 2 to 8 bits, heavy weights among them) 2.4e-7 -> 1e-8
+//   27 pairs, rms over columns and eight layers each, given codes: 3072 x 512 9.5e-14 -> 9.6e-14, 4096 x 4096 in groups 3.1e-12 -> 3.2e-12,
+//   6144 x 256 in groups 9.3e-13 -> 9.4e-13; solved codes 1.5e-12 -> 1.4e-12, 5.8e-10 -> 4.5e-11, 6.0e-11 -> 1.5e-11
 #include <cuda.h>
+
+#include <type_traits>
 
 #include "async_copy.cuh"
 #include "common.cuh"
@@ -51,34 +58,55 @@ constexpr int MAX_GROUPS = 12;
 // ---------------------------------------------------------------------------------------------
 // Slicing.  exps[r] = e with max_k |x[r,k]| 2^-e in [0.5, 1) (0 for an all-zero row).
 
-// Row maxima of a row-major fp32 matrix [rows, cols] -> exponent per row.
-__global__ void row_exp_f32_kernel(const float* __restrict__ x, long long rows, long long cols, int* __restrict__ exps) {
+// BALANCED: for balanced digits (below), whose top one is at most 127: max_k |x[r,k]| 2^-e at most 127.49 / 128.
+template <bool BALANCED>
+__device__ __forceinline__ int slice_exponent(double m) {
+  // (a normal number, as products of fp32 data are: its exponent field)
+  return m > 0.0 ? (__double2hiint(BALANCED ? 1.004 * m : m) >> 20) - 1022 : 0;
+}
+
+// 2^e for the exponents of normal numbers (those of products of fp32 data are).
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// feat[k] = s_k with 2^s_k near sqrt(H_kk); 0 for a diagonal entry that is no positive number.
+__global__ void feature_exp_kernel(const float* __restrict__ H, long long d, int* __restrict__ feat) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float h = H[k * d + k];
+  int e = 0;
+  if (h > 0.f && h < __int_as_float(0x7f800000)) frexpf(h, &e);
+  feat[k] = e >> 1;
+}
+
+// Row maxima of a row-major fp32 matrix [rows, cols] -> exponent per row.  feat (BALANCED; may be NULL): column k counts 2^-feat[k].
+template <bool BALANCED>
+__global__ void row_exp_f32_kernel(const float* __restrict__ x, long long rows, long long cols, const int* __restrict__ feat,
+                                   int* __restrict__ exps) {
+  using Real = std::conditional_t<BALANCED, double, float>;   // (scaled, an entry may leave the range of a float)
   const long long r = blockIdx.x;
-  float m = 0.f;
-  for (long long k = threadIdx.x; k < cols; k += blockDim.x) m = fmaxf(m, fabsf(x[r * cols + k]));
-  __shared__ float red[32];
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+  Real m = 0;
+  for (long long k = threadIdx.x; k < cols; k += blockDim.x) {
+    Real a = fabsf(x[r * cols + k]);
+    if constexpr (BALANCED) a *= feat ? pow2(-feat[k]) : 1.0;
+    m = a > m ? a : m;
+  }
+  __shared__ Real red[32];
+  for (int o = 16; o > 0; o >>= 1) { const Real a = __shfl_xor_sync(0xFFFFFFFFu, m, o); m = a > m ? a : m; }
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    if (threadIdx.x == 0) {
-      int e = 0;
-      if (m > 0.f && m < __int_as_float(0x7f800000)) frexpf(m, &e);
-      exps[r] = e;
-    }
+    m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : Real(0);
+    for (int o = 16; o > 0; o >>= 1) { const Real a = __shfl_xor_sync(0xFFFFFFFFu, m, o); m = a > m ? a : m; }
+    if (threadIdx.x == 0) exps[r] = isfinite(m) ? slice_exponent<BALANCED>((double)m) : 0;
   }
 }
 
 // Column maxima (ordered bit patterns) -> exponent per column.
+template <bool BALANCED>
 __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bits, long long cols, int* __restrict__ exps) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= cols) return;
-  const double m = __longlong_as_double((long long)colmax_bits[c]);
-  int e = 0;
-  if (m > 0.0) frexp(m, &e);
-  exps[c] = e;
+  exps[c] = slice_exponent<BALANCED>(__longlong_as_double((long long)colmax_bits[c]));
 }
 
 // |x| 2^-e 128^ns, truncated, as an integer (x 2^-e in (-1, 1), ns <= 6): slice i of x is its 7-bit digit number ns - i from
@@ -86,11 +114,8 @@ __global__ void col_exp_kernel(const unsigned long long* __restrict__ colmax_bit
 // 2^52 towards zero leaves the integer in the mantissa; scale = 2^(7 ns - e), a normal number for every exponent of H and E.
 // A NaN counts as zero, whatever its payload (that of CUDA's float NaN would pass for digits): a product leaves out the
 // entry and keeps the rest of its row.
-// NEAREST: rounded instead of truncated, half the error, up to `largest`, the largest number of ns digits.
-template <bool NEAREST>
-__device__ __forceinline__ unsigned long long slice_bits(double x, double scale, double largest = 0.0) {
-  const double f = fabs(x) * scale;
-  const double s = NEAREST ? __dadd_rn(f > largest ? largest : f, 4503599627370496.0) : __dadd_rz(f, 4503599627370496.0);
+__device__ __forceinline__ unsigned long long slice_bits(double x, double scale) {
+  const double s = __dadd_rz(fabs(x) * scale, 4503599627370496.0);
   return s != s ? 0ull : (unsigned long long)__double_as_longlong(s) & 0xFFFFFFFFFFFFFull;
 }
 // Digit i (from 1) of four neighbours, negated where `neg` has the byte's bits set, as four bytes.
@@ -100,72 +125,102 @@ __device__ __forceinline__ unsigned slice_bytes(const unsigned long long (&v)[4]
   for (int k = 0; k < 4; ++k) d |= ((unsigned)(v[k] >> shift) & 127u) << (8 * k);
   return __vsub4(d ^ neg, neg);
 }
+// Balanced digits, for half products: x 2^-e 128^ns rounded to the nearest integer, digits from -64 to 63 (the top one from -127 to 127),
+// so that every prefix of the digits is x to the nearest multiple of its last one.  A truncated prefix is off by up to a whole
+// unit, always towards zero: half of a product does not average that over an entry and its mirror image, and the two-digit screen of
+// the clipping search came out with 1.4 times the error of the whole product (see kScreenBand).
+// balanced_magic: 1.5 2^52, which leaves the integer in the mantissa, and 64 in each of the lower digits, which makes them non-negative
+// there.  What is no number or beyond the digits counts as zero.
+__device__ __forceinline__ double balanced_magic(int ns) {
+  return 6755399441055744.0 + (double)(64ll * (((1ll << (7 * (ns - 1))) - 1) / 127));
+}
+__device__ __forceinline__ unsigned long long balanced_bits(double x, double scale, double magic) {
+  const double s = x * scale + magic;
+  return (unsigned long long)__double_as_longlong(__double2hiint(s) >> 20 == 0x433 ? s : magic);   // (2^52 to 2^53)
+}
+__device__ __forceinline__ unsigned balanced_bytes(const unsigned long long (&v)[4], int shift, bool top) {
+  const unsigned d = __byte_perm(__byte_perm((unsigned)(v[0] >> shift), (unsigned)(v[1] >> shift), 0x0040),
+                                 __byte_perm((unsigned)(v[2] >> shift), (unsigned)(v[3] >> shift), 0x0040), 0x5410);
+  return top ? d : ((d | 0x80808080u) - 0x40404040u) ^ 0x80808080u;   // the lower seven bits, less 64, in every byte
+}
+// The ns slices of four neighbours x, the first at `out`, the next `step` bytes on.
+template <bool BALANCED>
+__device__ __forceinline__ void write_slices(const double (&x)[4], int ns, int e, signed char* out, size_t step) {
+  const double scale = pow2(7 * ns - e);
+  unsigned long long b[4];
+  if constexpr (BALANCED) {
+    const double magic = balanced_magic(ns);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) b[v] = balanced_bits(x[v], scale, magic);
+    for (int i = 0; i < ns; ++i) *reinterpret_cast<unsigned*>(out + i * step) = balanced_bytes(b, 7 * (ns - 1 - i), i == 0);
+  } else {
+    unsigned neg = 0u;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      b[v] = slice_bits(x[v], scale);
+      if (x[v] < 0.0) neg |= 0xFFu << (8 * v);
+    }
+    for (int i = 0; i < ns; ++i) *reinterpret_cast<unsigned*>(out + i * step) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+  }
+}
 
-// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p]; columns >= d zero), four columns per thread.
+// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p], BALANCED: column k by 2^-feat[k]; columns >= d zero), four
+// columns per thread.
 // 4 bytes read and ns written per entry; what bounds it is the integer operations of the digits (4096^2, six slices: 45 us, the ALU pipe
 // 63 % busy, 2.5 TB/s).  (One column per thread, with the digits taken off one after
 // the other in fp64: 1.46 ms for 14336^2 and six slices.)
-// NEAREST: for half products.
-template <bool NEAREST>
+template <bool BALANCED>
 __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ exps,
-                               int ns, signed char* __restrict__ out) {
+                               const int* __restrict__ feat, int ns, signed char* __restrict__ out) {
   const long long p = blockIdx.y;
   const long long k = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
   if (k >= kp) return;
-  const double scale = ldexp(1.0, 7 * ns - exps[p]), largest = ldexp(1.0, 7 * ns) - 1.0;
-  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  double x[4] = {0.0, 0.0, 0.0, 0.0};
   if ((d & 3) == 0) {
     if (k < d) {
       const float4 f = *reinterpret_cast<const float4*>(H + p * d + k);
-      x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
+      x[0] = (double)f.x; x[1] = (double)f.y; x[2] = (double)f.z; x[3] = (double)f.w;
     }
   } else {
 #pragma unroll
     for (int v = 0; v < 4; ++v)
-      if (k + v < d) x[v] = H[p * d + k + v];
+      if (k + v < d) x[v] = (double)H[p * d + k + v];
   }
-  unsigned long long b[4];
-  unsigned neg = 0u;
+  if (BALANCED && feat) {
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    b[v] = slice_bits<NEAREST>((double)x[v], scale, largest);
-    if (x[v] < 0.f) neg |= 0xFFu << (8 * v);
+    for (int v = 0; v < 4; ++v)
+      if (k + v < d) x[v] *= pow2(-feat[k + v]);
   }
-  for (int i = 0; i < ns; ++i)
-    *reinterpret_cast<unsigned*>(out + ((size_t)i * d + p) * kp + k) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+  write_slices<BALANCED>(x, ns, exps[p], out + (size_t)p * kp + k, (size_t)d * kp);
 }
 
-// The lower triangles of the diagonal blocks of H, half of the diagonal -> slices [ns][d][256] int8 (row p scaled by 2^-exps[p]):
+// The lower triangles of the diagonal blocks of H, half of the diagonal -> slices [ns][d][256] int8, scaled as those of H:
 // one row per warp, eight columns per thread.
 __global__ void __launch_bounds__(256) slice_diag_kernel(const float* __restrict__ H, long long d, const int* __restrict__ exps,
-                                                         int ns, signed char* __restrict__ out) {
+                                                         const int* __restrict__ feat, int ns, signed char* __restrict__ out) {
   const long long p = blockIdx.x * 8ll + (threadIdx.x >> 5);
   if (p >= d) return;
-  const double scale = ldexp(1.0, 7 * ns - exps[p]), largest = ldexp(1.0, 7 * ns) - 1.0;
 #pragma unroll
   for (int part = 0; part < 2; ++part) {
     const int c = 4 * (threadIdx.x & 31) + 128 * part;
     const long long k = p / BN * BN + c;
-    unsigned long long b[4];
-    unsigned neg = 0u;
+    double x[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const double x = k + v < p ? (double)H[p * d + k + v] : k + v == p ? 0.5 * (double)H[p * d + p] : 0.0;
-      b[v] = slice_bits<true>(x, scale, largest);
-      if (x < 0.0) neg |= 0xFFu << (8 * v);
-    }
-    for (int i = 0; i < ns; ++i)
-      *reinterpret_cast<unsigned*>(out + ((size_t)i * d + p) * BN + c) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+    for (int v = 0; v < 4; ++v)
+      x[v] = k + v > p ? 0.0 : (k + v == p ? 0.5 : 1.0) * (feat ? pow2(-feat[k + v]) : 1.0) * (double)H[p * d + k + v];
+    write_slices<true>(x, ns, exps[p], out + (size_t)p * BN + c, (size_t)d * BN);
   }
 }
 
-// E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j]), 128 x 32 tiles turned round
+// E [d_in, d_out] fp64 -> slices of E^T [ns][d_out][kp] int8 (column j scaled by 2^-exps[j], BALANCED: row k by 2^feat[k]), 128 x 32 tiles turned round
 // in shared memory so that reads and writes are contiguous, four rows of E per thread.  8 bytes read and ns
 // written per entry; bound as slice_h_kernel (4096^2, five slices: 52 us, ALU pipe 63 %, 3.5 TB/s).  (32 x 32 tiles, single bytes, digits one after the other in fp64: 0.74 ms for 4096 x 32768 and
 // two slices.)
 constexpr int SK = 128, SJ = 32;
+template <bool BALANCED>
 __global__ void __launch_bounds__(256) slice_et_kernel(const double* __restrict__ E, long long d_in, long long d_out, long long kp,
-                                                       const int* __restrict__ exps, int ns, signed char* __restrict__ out) {
+                                                       const int* __restrict__ exps, const int* __restrict__ feat, int ns,
+                                                       signed char* __restrict__ out) {
   // entry (k, j) at [j][k ^ 2 (j & 15)]: the stores down a column spread over the banks, pairs of k stay together
   __shared__ __align__(16) double tile[SJ][SK];
   const long long k0 = (long long)blockIdx.x * SK, j0 = (long long)blockIdx.y * SJ;
@@ -173,26 +228,19 @@ __global__ void __launch_bounds__(256) slice_et_kernel(const double* __restrict_
 #pragma unroll
   for (int r = ty; r < SK; r += 8) {
     const long long k = k0 + r, j = j0 + tx;
-    tile[tx][r ^ (2 * (tx & 15))] = (k < d_in && j < d_out) ? E[k * d_out + j] : 0.0;
+    double x = (k < d_in && j < d_out) ? E[k * d_out + j] : 0.0;
+    if (BALANCED && feat && k < d_in) x *= pow2(feat[k]);
+    tile[tx][r ^ (2 * (tx & 15))] = x;
   }
   __syncthreads();
 #pragma unroll
   for (int jj = ty; jj < SJ; jj += 8) {
     const long long j = j0 + jj, k = k0 + 4 * tx;
     if (j >= d_out) continue;   // (k < kp: kp is a multiple of SK)
-    const double scale = ldexp(1.0, 7 * ns - exps[j]);
     const double2 x01 = *reinterpret_cast<const double2*>(&tile[jj][(4 * tx) ^ (2 * (jj & 15))]);
     const double2 x23 = *reinterpret_cast<const double2*>(&tile[jj][(4 * tx + 2) ^ (2 * (jj & 15))]);
     const double x[4] = {x01.x, x01.y, x23.x, x23.y};
-    unsigned long long b[4];
-    unsigned neg = 0u;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      b[v] = slice_bits<false>(x[v], scale);
-      if (x[v] < 0.0) neg |= 0xFFu << (8 * v);
-    }
-    for (int i = 0; i < ns; ++i)
-      *reinterpret_cast<unsigned*>(out + ((size_t)i * d_out + j) * kp + k) = slice_bytes(b, 7 * (ns - 1 - i), neg);
+    write_slices<BALANCED>(x, ns, exps[j], out + (size_t)j * kp + k, (size_t)d_out * kp);
   }
 }
 
@@ -262,9 +310,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 __device__ __forceinline__ double int_to_double(uint32_t r) {
   return __hiloint2double(0x43300000, (int)(r ^ 0x80000000u)) - 4503601774854144.0;   // 2^52 + 2^31
 }
-// 2^e for the exponents of normal numbers (those of products of fp32 data are).
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-
 // Half of the product: how many blocks of 256 columns of H follow the diagonal one in tile column tn.
 __device__ __forceinline__ int blocks_after(int tn, int nb) { return (nb - 1) / 2 + ((nb & 1) == 0 && tn < nb / 2 ? 1 : 0); }
 // Tiles are handed out in bands of 8 tile rows, column by column inside a band, so that the
@@ -528,7 +573,7 @@ static bool half_product(long long d_in) { return d_in >= 3072; }
 
 size_t gemm_tc_h_bytes(long long d_in, int nh) {
   return align_up((size_t)nh * d_in * tc_kpad(d_in)) + align_up(sizeof(int) * (size_t)d_in) +
-         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) : 0);   // the diagonal blocks
+         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) + align_up(sizeof(int) * (size_t)d_in) : 0);   // diagonal blocks, D
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -536,21 +581,23 @@ size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
          align_up(sizeof(unsigned long long) * (size_t)d_out);
 }
 
-// Slices of H (done once per call of the library; the OWC search reuses them for every gamma).  losses: for products without keep_c.
-cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, bool losses, void* hbuf, cudaStream_t st) {
+// Slices of H (done once per call of the library; the OWC search reuses them for every gamma).
+cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use, void* hbuf, cudaStream_t st) {
   const long long kp = tc_kpad(d_in);
-  const bool half = losses && half_product(d_in);
+  const bool half = use != kTcProduct && half_product(d_in);
   signed char* slices = (signed char*)hbuf;
   int* hexp = (int*)((char*)hbuf + align_up((size_t)nh * d_in * kp));
-  { i8::row_exp_f32_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, hexp); count_launch(); }
-  dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
-  if (half) i8::slice_h_kernel<true><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices);
-  else i8::slice_h_kernel<false><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices);
-  count_launch();
+  const dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
   if (half) {
     signed char* diag = (signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
-    i8::slice_diag_kernel<<<(unsigned)((d_in + 7) / 8), 256, 0, st>>>(H, d_in, hexp, nh, diag);
-    count_launch();
+    int* feat = use == kTcSearch ? (int*)(diag + align_up((size_t)nh * d_in * i8::BN)) : nullptr;
+    if (feat) { i8::feature_exp_kernel<<<(unsigned)((d_in + 255) / 256), 256, 0, st>>>(H, d_in, feat); count_launch(); }
+    { i8::row_exp_f32_kernel<true><<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, feat, hexp); count_launch(); }
+    { i8::slice_h_kernel<true><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, feat, nh, slices); count_launch(); }
+    { i8::slice_diag_kernel<<<(unsigned)((d_in + 7) / 8), 256, 0, st>>>(H, d_in, hexp, feat, nh, diag); count_launch(); }
+  } else {
+    { i8::row_exp_f32_kernel<false><<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, nullptr, hexp); count_launch(); }
+    { i8::slice_h_kernel<false><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nullptr, nh, slices); count_launch(); }
   }
   return cudaGetLastError();
 }
@@ -580,16 +627,17 @@ static cudaError_t encode_map3(CUtensorMap* map, const void* base, long long kp,
 
 // E = the residual of `src`, then C[j, p] = scale * sum_k E[k, j] H[p, k]  for j < d_out, p < d_in, to the precision of
 // (ne, nh, smax); optionally col_loss[j] = sum_p E[p, j] C[j, p] / scale.
-// hbuf: from gemm_tc_prepare_h with the same nh.  ebuf: gemm_tc_e_bytes of scratch.
-cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
-                        double scale, double* C, bool keep_c, long long ldc, double* col_loss, void* ebuf, cudaStream_t st) {
+// hbuf: from gemm_tc_prepare_h with the same nh and use.  ebuf: gemm_tc_e_bytes of scratch.
+cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,
+                        double scale, double* C, long long ldc, double* col_loss, void* ebuf, cudaStream_t st) {
   using namespace i8;
   if (nh < 1 || nh > MAX_SLICES || ne < 1 || ne > MAX_SLICES || smax < 2) return cudaErrorInvalidValue;
   const long long kp = tc_kpad(d_in);
-  const bool half = !keep_c && half_product(d_in);
+  const bool keep_c = use == kTcProduct, half = !keep_c && half_product(d_in);
   const signed char* hsl = (const signed char*)hbuf;
   const int* hexp = (const int*)((const char*)hbuf + align_up((size_t)nh * d_in * kp));
   const signed char* dsl = (const signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
+  const int* feat = half && use == kTcSearch ? (const int*)(dsl + align_up((size_t)nh * d_in * BN)) : nullptr;
   signed char* esl = (signed char*)ebuf;
   int* eexp = (int*)((char*)ebuf + align_up((size_t)ne * d_out * kp));
   unsigned long long* colmax = (unsigned long long*)((char*)eexp + align_up(sizeof(int) * (size_t)d_out));
@@ -597,11 +645,16 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, const ResidualSrc& src, double
 
   cudaError_t e = cudaMemsetAsync(colmax, 0, sizeof(unsigned long long) * (size_t)d_out, st);
   if (e != cudaSuccess) return e;
-  e = launch_residual_f64(src, d_in, E, st, colmax);
+  e = launch_residual_f64(src, d_in, E, st, colmax, feat);
   if (e != cudaSuccess) return e;
-  { col_exp_kernel<<<(unsigned)((d_out + 255) / 256), 256, 0, st>>>(colmax, d_out, eexp); count_launch(); }
+  const unsigned cols = (unsigned)((d_out + 255) / 256);
+  if (half) col_exp_kernel<true><<<cols, 256, 0, st>>>(colmax, d_out, eexp);
+  else col_exp_kernel<false><<<cols, 256, 0, st>>>(colmax, d_out, eexp);
+  count_launch();
   const dim3 slices((unsigned)(kp / SK), (unsigned)((d_out + SJ - 1) / SJ));
-  { slice_et_kernel<<<slices, 256, 0, st>>>(E, d_in, d_out, kp, eexp, ne, esl); count_launch(); }
+  if (half) slice_et_kernel<true><<<slices, 256, 0, st>>>(E, d_in, d_out, kp, eexp, feat, ne, esl);
+  else slice_et_kernel<false><<<slices, 256, 0, st>>>(E, d_in, d_out, kp, eexp, nullptr, ne, esl);
+  count_launch();
   Params p{};
   p.M = (int)d_out; p.N = (int)d_in; p.kblocks = (int)(kp / BKB);
   p.tiles_m = (int)((d_out + BM - 1) / BM); p.tiles_n = (int)((d_in + BN - 1) / BN);

@@ -206,14 +206,14 @@ __global__ void __launch_bounds__(32 * WARPS, 1024 / (32 * WARPS)) group_codes_k
 }
 
 // Residual E[i][c] = (a q + b) - w in fp64, either from stored codes or, for the OWC search, from min/max and a clipping
-// strength (codes formed on the fly, never stored).  With colmax it also leaves the largest |E| of every column there (as
+// strength (codes formed on the fly, never stored).  With colmax it also leaves the largest |E| 2^row_exp of every column there (as
 // ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  8 bytes written
 // per entry; bound by the latency of its loads (4096 x 4096 bf16 weights in groups: 46 us, 16 warps per SM at 86 registers, 2.8 TB/s).
 // (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
 // strengths of a 4096 x 4096 layer, 0.16 ms of them the maxima.)
 template <int V, bool BF16>
 __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_per_block, int blocks_per_group, double* __restrict__ E,
-                                                       unsigned long long* __restrict__ colmax) {
+                                                       unsigned long long* __restrict__ colmax, const int* __restrict__ row_exp) {
   const long long c = V * (blockIdx.x * (long long)blockDim.x + threadIdx.x);   // column of E
   const long long width = s.n_cols ? s.n_cols : s.d_out;
   if (c >= width) return;
@@ -240,9 +240,11 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
   for (long long i = i0; i < i1; i += R) {
     float w[R][V];
     unsigned q4[R];
+    int weight[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const long long row = min(i + r, i1 - 1);
+      weight[r] = row_exp ? row_exp[row] : 0;
       load_weights<V, BF16>(s.W, row * s.ldw + j, w[r]);
       q4[r] = 0u;
       if (!s.use_gamma) {
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
         // 2^52 + q: its lower word is q
         const double qd = __hiloint2double(0x43300000, (int)q) - 4503599627370496.0;
         e[v] = __dadd_rn(__dadd_rn(__dmul_rn((double)a[v], qd), (double)b[v]), -(double)w[r][v]);
-        m[v] = fmax(m[v], fabs(e[v]));
+        m[v] = fmax(m[v], fabs(e[v]) * __hiloint2double((1023 + weight[r]) << 20, 0));
       }
       double* dst = E + (i + r) * width + c;
       if constexpr (V == 4) {
@@ -282,7 +284,8 @@ __global__ void __launch_bounds__(128) residual_kernel(ResidualSrc s, int rows_p
   }
 }
 
-cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st, unsigned long long* colmax) {
+cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* E, cudaStream_t st, unsigned long long* colmax,
+                                const int* row_exp) {
   const long long width = src.n_cols ? src.n_cols : src.d_out;
   // rows per block, all of one group: few on small layers, which have no more blocks to offer (1024 x 1024 entries with 32 rows 17 us)
   const int rows = width * d_in >= (1ll << 22) ? 32 : 4, bpg = (int)((src.g + rows - 1) / rows);
@@ -293,7 +296,7 @@ cudaError_t launch_residual_f64(const ResidualSrc& src, long long d_in, double* 
   const bool four = rows == 32 && !src.col_idx && src.d_out % 4 == 0 && src.ldw % 4 == 0 && reinterpret_cast<uintptr_t>(src.W) % (4 * esz) == 0 &&
                     reinterpret_cast<uintptr_t>(src.Q) % 4 == 0;
   const dim3 grid((unsigned)((width + (four ? 511 : 127)) / (four ? 512 : 128)), (unsigned)(d_in / src.g * bpg));
-  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, rows, bpg, E, colmax); count_launch(); };
+  auto run = [&](auto kern) { kern<<<grid, 128, 0, st>>>(src, rows, bpg, E, colmax, row_exp); count_launch(); };
   if (src.wt == CDQ_BF16) run(four ? residual_kernel<4, true> : residual_kernel<1, true>);
   else run(four ? residual_kernel<4, false> : residual_kernel<1, false>);
   return cudaGetLastError();
@@ -319,13 +322,15 @@ __global__ void owc_argmin_kernel(const double* __restrict__ table, int n_clip, 
 // The losses of all clipping strengths are first formed cheaply (three slice-pair products instead of thirteen);
 // a strength stays a candidate of a column if its screened loss is within kScreenBand of the column's smallest.
 // Only candidates get the thirteen-pair loss, and the argmin is taken over those: the same result as the full
-// table as long as the screening error stays inside the band.  The loss as a function of the strength is smooth
-// with one minimum, and the second-best strength of a column is typically percents away (median 2.5 % on 2-bit,
+// table as long as the screening errors of a column's strengths differ by less than the band.  The loss as a function of the strength is
+// smooth with one minimum, and the second-best strength of a column is typically percents away (median 2.5 % on 2-bit,
 // 5 % on 3-bit grouped layers), so a band of 1 % keeps 1.1 to 1.3 candidates per column.  The screen keeps two
-// 7-bit slices of the residual and of H on grids of up to 4 bits: the slicing truncates below 2^-14 of the column's
-// largest residual, and a clipped weight leaves a residual up to (1 - gamma) L times the typical rounding error
-// (7.5 times at 4 bits), which put the screened loss off by up to 6e-4 on a 3-bit layer -- a factor of 8 inside half
-// the band.  Finer grids (L up to 255) keep three slices and six products.
+// 7-bit slices of the residual and of H on grids of up to 4 bits: it cuts off 2^-14 of the column's largest residual, and a clipped
+// weight leaves a residual up to (1 - gamma) L times the typical rounding error (7.5 times at 4 bits).  Against 64 bits, on layers of 3072 and
+// 4096 rows with 2 to 4 bits, heavy weights among them, a screened loss is off by up to 4.2e-3 (3.4e-4 to 4.7e-4 rms), and the errors of a
+// column's strengths differ by up to 5.4e-3: half of the band.  (Below 3072 rows, by the whole product of truncated slices, up to 6.7e-3, 6e-4
+// to 9e-4 rms, and they differ by up to 7.9e-3.  By half of the product with truncated slices it was 1.0e-2, 1.3e-3 and 1.2e-2; rows of H that one
+// feature dominates lost strengths.)  Finer grids (L up to 255) keep three slices and six products: up to 3e-5.
 constexpr double kScreenBand = 1e-2;
 __host__ __device__ constexpr int screen_slices(int bits) { return bits <= 4 ? 2 : 3; }   // pairs up to i + j = slices + 1
 
@@ -513,7 +518,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
     if (e != cudaSuccess) return e;
     // the host array must outlive the copy: pageable memcpy is staged before return
     if (L.tc) {   // the slices of H serve every clipping strength
-      e = gemm_tc_prepare_h(ly.H, d_in, kTcLossNH, true, base + L.hbuf, st);
+      e = gemm_tc_prepare_h(ly.H, d_in, kTcLossNH, kTcSearch, base + L.hbuf, st);
       if (e != cudaSuccess) return e;
     }
     if (L.screened) {
@@ -532,8 +537,8 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.mn = mn; src.mx = mx; src.gamma = hg[k0]; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out;
         if (gb > 1) { src.n_cols = width; src.k0 = k0; src.gammas = gammas; }   // column c: layer column c % d_out
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
-                        (double*)(base + L.C), false, L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
+                        (double*)(base + L.C), L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
       }
       { owc_candidates_kernel<<<bx, 128, 0, st>>>(screen, n_clip, d_out, mask, table); count_launch(); }
@@ -556,7 +561,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.mn = mn; src.mx = mx; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out; src.col_idx = cj + b0; src.n_cols = width;
         src.col_gamma = ck + b0; src.gammas = gammas;
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), false, L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
                         loss_c, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
         { owc_scatter_kernel<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(loss_c, cj + b0, ck + b0, width, d_out, table); count_launch(); }
@@ -568,7 +573,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
       src.mn = mn; src.mx = mx; src.gamma = hg[k]; src.L = ly.L; src.use_gamma = 1;
       src.g = g; src.d_out = d_out;
       if (L.tc) {
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), false, L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
                         table + (long long)k * d_out, base + L.ebuf, st);
       } else {
         e = launch_residual_f64(src, d_in, E, st);

@@ -713,10 +713,10 @@ cudaError_t launch_owc_cd(const Layer& ly, const cdq_grid_desc& grid, long long 
     src.W = ly.W; src.wt = ly.wt; src.ldw = ly.ldw; src.mn = mn; src.mx = mx; src.gamma = hg[nk - 1]; src.L = ly.L;
     src.use_gamma = 1; src.g = g; src.d_out = d_out;
     double* E = (double*)(base + L.E);
-    e = gemm_tc_prepare_h(ly.H, d_in, kTcGradNH, false, base + L.hbuf, st);
+    e = gemm_tc_prepare_h(ly.H, d_in, kTcGradNH, kTcProduct, base + L.hbuf, st);
     if (e != cudaSuccess) return e;
     p.Gext = (double*)(base + L.G); p.ldg = L.ldg;
-    e = gemm_tc_run(base + L.hbuf, kTcGradNH, src, E, d_in, d_out, kTcGradNE, kTcGradSmax, 2.0, p.Gext, true, p.ldg, p.col_before,
+    e = gemm_tc_run(base + L.hbuf, kTcGradNH, kTcProduct, src, E, d_in, d_out, kTcGradNE, kTcGradSmax, 2.0, p.Gext, p.ldg, p.col_before,
                     base + L.ebuf, st);
     if (e != cudaSuccess) return e;
   }

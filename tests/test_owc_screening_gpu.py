@@ -22,6 +22,9 @@ TIE = 1e-7
     ("C4", 3, 128, 2048, 768),
     ("C2", 4, 0, 1536, 512),
     ("C2", 8, 256, 1024, 512),
+    ("C2", 2, 128, 3072, 384),      # from 3072 rows on by half of the product
+    ("C4", 4, 0, 3328, 300),
+    ("C2", 8, 256, 3072, 256),
 ])
 def test_screened_search_picks_the_oracles_strength(base, bits, group, d_in, d_out):
     dev = "cuda:0"
@@ -49,3 +52,33 @@ def test_screened_search_picks_the_oracles_strength(base, bits, group, d_in, d_o
     assert np.array_equal(Q.cpu().numpy()[:, same], init["Q"][:, same])
     assert np.array_equal(scale.cpu().numpy()[:, same], init["scale"][:, same])
     print(f"{bits}-bit g={group} {d_in}x{d_out}: strength differs on {len(differs)} of {d_out} columns (near-ties)")
+
+
+@pytest.mark.parametrize("bits,lo,hi,dominance", [(2, 0.5, 1.0, 500.0), (3, 0.7, 0.8, 80.0), (4, 0.8, 0.9, 200.0), (8, 0.8, 0.9, 2000.0)])
+def test_screen_of_rows_that_one_feature_dominates(bits, lo, hi, dominance):
+    """Every column against fp64 on the GPU.  One feature is far larger than the others, which all hang together with it, so that its entries
+    are the largest of every row of H, but its residual is zero: the loss lies in the small entries.  Strengths close to one another,
+    most of them within a few percent of a column's best.  The thirteen-pair losses are good to 1e-6 here."""
+    dev, d_in, d_out, n_clip = "cuda:0", 3072, 2048, 20
+    lo, hi = float(np.float32(lo)), float(np.float32(hi))   # as the library gets them
+    gen = torch.Generator(dev).manual_seed(3)
+    z = torch.randn(512, d_in, generator=gen, device=dev)
+    sign = torch.randint(0, 2, (d_in,), generator=gen, device=dev).float() * 2 - 1
+    X = z + 0.5 * sign * z[:, :1]
+    X[:, 0] = dominance * z[:, 0]
+    H = (X.double().T @ X.double()).float()
+    H = (torch.tril(H) + torch.tril(H, -1).T).contiguous()
+    W = torch.randn(d_in, d_out, generator=gen, device=dev) * 0.02
+    W[0] = W.amin(0) - 1e-3                       # the zero of the grid: code 0, no residual at any strength
+    gamma = B.cdq_init_rtn(W, B.Grid(bits, 0, n_clip, lo, hi), H=H)[3]
+    mn, mx, Wd, Hd = W.amin(0).double(), W.amax(0).double(), W.double(), H.double()
+    table = []
+    for g in oracle.gamma_grid(n_clip, lo, hi):
+        a = (float(g) * (mx - mn) / (2 ** bits - 1)).float().double()
+        E = a * ((Wd - mn) / a).round().clamp(0, 2 ** bits - 1) + mn - Wd
+        table.append(((Hd @ E) * E).sum(0))
+    table = torch.stack(table)
+    grid = torch.from_numpy(oracle.gamma_grid(n_clip, lo, hi).astype(np.float32)).to(dev)
+    chosen = (grid[:, None] == gamma[None, :]).double().argmax(0)
+    excess = table.gather(0, chosen[None])[0] / table.amin(0) - 1
+    assert float(excess.max()) <= 1e-6
