@@ -290,7 +290,8 @@ cdq_status cdq_cd_solve_rows16(const float* H, const void* W, cdq_dtype wt, long
 
 /*
  * Layer loss sum_j e_j^T H e_j with e = W_hat - W (paper: Eq. 1 written with
- * H = X^T X; the objective value the paper reports for a solution).
+ * H = X^T X; the objective value the paper reports for a solution).  The value is that of the H given, e_j^T H e_j with
+ * both triangles in it, also where they differ.
  *   loss     host pointer to one double, may be NULL.
  *   per_col  [d_out] fp64 device out, may be NULL.
  */

@@ -21,10 +21,12 @@
 // int32 accumulators in TMEM (two of them, so the epilogue of one group overlaps the MMAs of
 // the next), the same warp roles as the Hessian kernel.  Every mbarrier wait is bounded.
 //
-// Losses alone take half of the product.  H is symmetric, so with its rows and columns in blocks of 256, a column's loss is
-//     e^T H e = 2 sum_P e_P^T (T_P e_P + sum_{K in half(P)} H_PK e_K),
+// Losses alone take half of the product.  e^T H e is that of H's symmetric part S = (H + H^T) / 2, and with the rows and columns of S
+// in blocks of 256, a column's loss is
+//     e^T S e = 2 sum_P e_P^T (T_P e_P + sum_{K in half(P)} S_PK e_K),
 // where half(P) holds one of the blocks (P, K), (K, P) of every pair: the nb / 2 blocks that follow P, in a circle, so that every tile
-// has the same work.  T_P is the lower triangle of the diagonal block with half of its diagonal; it has slices of its own, [ns][d][256].
+// has the same work.  (S is formed where the slices are, so that an H which is symmetric only up to rounding, or not at all, has the loss
+// that the whole product gives it.)  T_P is the lower triangle of the diagonal block with half of its diagonal; it has slices of its own, [ns][d][256].
 // The two halves of the whole product average an entry's slicing error with that of its mirror image; here it counts twice.  Two things
 // make up for that.  The digits are balanced (balanced_bits below).  And the clipping search, whose screen has two or three digits of
 // either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk), so the rows no
@@ -35,8 +37,6 @@
 //   27 pairs, rms over columns and eight layers each, given codes: 3072 x 512 9.5e-14 -> 9.6e-14, 4096 x 4096 in groups 3.1e-12 -> 3.2e-12,
 //   6144 x 256 in groups 9.3e-13 -> 9.4e-13; solved codes 1.5e-12 -> 1.4e-12, 5.8e-10 -> 4.5e-11, 6.0e-11 -> 1.5e-11
 #include <cuda.h>
-
-#include <type_traits>
 
 #include "async_copy.cuh"
 #include "common.cuh"
@@ -68,36 +68,19 @@ __device__ __forceinline__ int slice_exponent(double m) {
 // 2^e for the exponents of normal numbers (those of products of fp32 data are).
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// feat[k] = s_k with 2^s_k near sqrt(H_kk); 0 for a diagonal entry that is no positive number.
-__global__ void feature_exp_kernel(const float* __restrict__ H, long long d, int* __restrict__ feat) {
-  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (k >= d) return;
-  const float h = H[k * d + k];
-  int e = 0;
-  if (h > 0.f && h < __int_as_float(0x7f800000)) frexpf(h, &e);
-  feat[k] = e >> 1;
-}
-
-// Row maxima of a row-major fp32 matrix [rows, cols] -> exponent per row.  feat (BALANCED; may be NULL): column k counts 2^-feat[k].
-template <bool BALANCED>
-__global__ void row_exp_f32_kernel(const float* __restrict__ x, long long rows, long long cols, const int* __restrict__ feat,
-                                   int* __restrict__ exps) {
-  using Real = std::conditional_t<BALANCED, double, float>;   // (scaled, an entry may leave the range of a float)
+// Row maxima of a row-major fp32 matrix [rows, cols] -> exponent per row.
+__global__ void row_exp_f32_kernel(const float* __restrict__ x, long long rows, long long cols, int* __restrict__ exps) {
   const long long r = blockIdx.x;
-  Real m = 0;
-  for (long long k = threadIdx.x; k < cols; k += blockDim.x) {
-    Real a = fabsf(x[r * cols + k]);
-    if constexpr (BALANCED) a *= feat ? pow2(-feat[k]) : 1.0;
-    m = a > m ? a : m;
-  }
-  __shared__ Real red[32];
-  for (int o = 16; o > 0; o >>= 1) { const Real a = __shfl_xor_sync(0xFFFFFFFFu, m, o); m = a > m ? a : m; }
+  float m = 0.f;
+  for (long long k = threadIdx.x; k < cols; k += blockDim.x) m = fmaxf(m, fabsf(x[r * cols + k]));
+  __shared__ float red[32];
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x < 32) {
-    m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : Real(0);
-    for (int o = 16; o > 0; o >>= 1) { const Real a = __shfl_xor_sync(0xFFFFFFFFu, m, o); m = a > m ? a : m; }
-    if (threadIdx.x == 0) exps[r] = isfinite(m) ? slice_exponent<BALANCED>((double)m) : 0;
+    m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    if (threadIdx.x == 0) exps[r] = m < __int_as_float(0x7f800000) ? slice_exponent<false>((double)m) : 0;
   }
 }
 
@@ -164,14 +147,12 @@ __device__ __forceinline__ void write_slices(const double (&x)[4], int ns, int e
   }
 }
 
-// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p], BALANCED: column k by 2^-feat[k]; columns >= d zero), four
-// columns per thread.
+// H [d, d] fp32 -> slices [ns][d][kp] int8 (row p scaled by 2^-exps[p]; columns >= d zero), four columns per thread.
 // 4 bytes read and ns written per entry; what bounds it is the integer operations of the digits (4096^2, six slices: 45 us, the ALU pipe
 // 63 % busy, 2.5 TB/s).  (One column per thread, with the digits taken off one after
 // the other in fp64: 1.46 ms for 14336^2 and six slices.)
-template <bool BALANCED>
 __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ exps,
-                               const int* __restrict__ feat, int ns, signed char* __restrict__ out) {
+                               int ns, signed char* __restrict__ out) {
   const long long p = blockIdx.y;
   const long long k = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
   if (k >= kp) return;
@@ -186,29 +167,122 @@ __global__ void slice_h_kernel(const float* __restrict__ H, long long d, long lo
     for (int v = 0; v < 4; ++v)
       if (k + v < d) x[v] = (double)H[p * d + k + v];
   }
-  if (BALANCED && feat) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-      if (k + v < d) x[v] *= pow2(-feat[k + v]);
-  }
-  write_slices<BALANCED>(x, ns, exps[p], out + (size_t)p * kp + k, (size_t)d * kp);
+  write_slices<false>(x, ns, exps[p], out + (size_t)p * kp + k, (size_t)d * kp);
 }
 
-// The lower triangles of the diagonal blocks of H, half of the diagonal -> slices [ns][d][256] int8, scaled as those of H:
-// one row per warp, eight columns per thread.
-__global__ void __launch_bounds__(256) slice_diag_kernel(const float* __restrict__ H, long long d, const int* __restrict__ exps,
-                                                         const int* __restrict__ feat, int ns, signed char* __restrict__ out) {
-  const long long p = blockIdx.x * 8ll + (threadIdx.x >> 5);
-  if (p >= d) return;
+// ---- half products ----
+// Half of the product: how many blocks of 256 columns of H follow the diagonal one in tile column tn.
+__device__ __forceinline__ int blocks_after(int tn, int nb) { return (nb - 1) / 2 + ((nb & 1) == 0 && tn < nb / 2 ? 1 : 0); }
+
+// feat[k] = s_k with 2^s_k near sqrt(H_kk); 0 for a diagonal entry that is no positive number.
+__global__ void feature_exp_kernel(const float* __restrict__ H, long long d, int* __restrict__ feat) {
+  const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (k >= d) return;
+  const float h = H[k * d + k];
+  int e = 0;
+  if (h > 0.f && h < __int_as_float(0x7f800000)) frexpf(h, &e);
+  feat[k] = e >> 1;
+}
+// Four neighbours of a row of H from column k on (zero from d on).  VEC: rows start on 16-byte boundaries.
+template <bool VEC>
+__device__ __forceinline__ float4 four_of_row(const float* __restrict__ H, long long d, long long row, long long k) {
+  const float* p = H + row * d + k;
+  if (VEC) return k < d ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return make_float4(k < d ? p[0] : 0.f, k + 1 < d ? p[1] : 0.f, k + 2 < d ? p[2] : 0.f, k + 3 < d ? p[3] : 0.f);
+}
+// An entry that is no finite number counts as zero.
+__device__ __forceinline__ float finite(float x) { return fabsf(x) <= 3.402823466e38f ? x : 0.f; }
+// rowmax[p]: the largest |H_pk| 2^-feat[k] and |H_kp| 2^-feat[k], rounded up, as a bit pattern; no entry of row p of S D^-1 is above it.  16
+// rows x 1024 columns per block, four columns per thread: one pass over H from memory (4096^2: 33 us, 2 TB/s, bound by
+// the latency of its loads).  feat may be NULL (D = 1).
+template <bool VEC>
+__global__ void __launch_bounds__(256) half_max_kernel(const float* __restrict__ H, long long d, const int* __restrict__ feat,
+                                                       unsigned* __restrict__ rowmax) {
+  constexpr int ROWS = 16;
+  __shared__ unsigned s_row[ROWS];
+  const long long c = 4 * (blockIdx.x * 256ll + threadIdx.x), r0 = (long long)blockIdx.y * ROWS;
+  if (threadIdx.x < ROWS) s_row[threadIdx.x] = 0u;
+  __syncthreads();
+  auto weight = [&](long long k) { return feat && k < d ? __int_as_float((127 - feat[k]) << 23) : 1.f; };   // (feat: -75 to 64)
+  float wc[4], col[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-  for (int part = 0; part < 2; ++part) {
-    const int c = 4 * (threadIdx.x & 31) + 128 * part;
-    const long long k = p / BN * BN + c;
+  for (int v = 0; v < 4; ++v) wc[v] = weight(c + v);
+#pragma unroll 8
+  for (int r = 0; r < ROWS; ++r) {
+    if (r0 + r >= d) break;
+    const float4 h4 = four_of_row<VEC>(H, d, r0 + r, c);
+    const float h[4] = {fabsf(h4.x), fabsf(h4.y), fabsf(h4.z), fabsf(h4.w)}, wr = weight(r0 + r);
+    float row = 0.f;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {   // (the maximum leaves a NaN out)
+      row = fmaxf(row, __fmul_ru(h[v], wc[v]));
+      col[v] = fmaxf(col[v], __fmul_ru(h[v], wr));
+    }
+    const unsigned most = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(row));
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_row[r], most);
+  }
+#pragma unroll
+  for (int v = 0; v < 4; ++v)
+    if (c + v < d) atomicMax(&rowmax[c + v], __float_as_uint(col[v]));
+  __syncthreads();
+  if (threadIdx.x < ROWS && r0 + threadIdx.x < d) atomicMax(&rowmax[r0 + threadIdx.x], s_row[threadIdx.x]);
+}
+// Slices of S D^-1 (rows scaled by 2^-exps): the blocks (P, K) of 256 with K in half(P) into `out`, [ns][d][kp] (nothing reads the others),
+// the triangles T_P into `diag`, [ns][d][256].  64 rows x 128 columns per block; the mirror image of the tile is turned round in
+// shared memory, so that both are read along their rows, once.  An entry that is no finite number is left out, its mirror image is not.
+// 4 bytes read and ns / 2 written per entry (4096^2, six slices: 39 us; all blocks of H, without its mirror image, and the triangles 53 us).
+template <bool VEC>
+__global__ void __launch_bounds__(256) half_slice_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ feat,
+                                                         const unsigned* __restrict__ rowmax, int ns, int* __restrict__ exps,
+                                                         signed char* __restrict__ out, signed char* __restrict__ diag) {
+  constexpr int TP = 64, TK = 128;
+  __shared__ __align__(16) float mirror[TP][TK];   // H[k][p] at [p][k ^ 4 (p / 4 % 8)]
+  const int nb = (int)((d + BN - 1) / BN), P = (int)blockIdx.z, m = (int)blockIdx.y;
+  if (m > blocks_after(P, nb)) return;
+  const int K = P + m < nb ? P + m : P + m - nb;
+  const long long p0 = (long long)P * BN + (blockIdx.x >> 1) * TP, k0 = (long long)K * BN + (blockIdx.x & 1) * TK;
+  if (p0 >= d || (m > 0 && k0 >= kp)) return;
+  const int kk = 4 * (threadIdx.x & 31);
+  float4 h[TP / 8];   // rows p0 + warp, 8 further on, ...: on their way beside the mirror image
+#pragma unroll
+  for (int i = 0; i < TP / 8; ++i) {
+    const long long p = p0 + 8 * i + (threadIdx.x >> 5);
+    h[i] = p < d ? four_of_row<VEC>(H, d, p, k0 + kk) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  {
+    const int t = 4 * (threadIdx.x & 15);
+#pragma unroll
+    for (int i = 0; i < TK / 16; ++i) {
+      const int k = 16 * i + (threadIdx.x >> 4);
+      const float4 g = k0 + k < d ? four_of_row<VEC>(H, d, k0 + k, p0 + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int at = k ^ (t & 28);
+      mirror[t][at] = g.x; mirror[t + 1][at] = g.y; mirror[t + 2][at] = g.z; mirror[t + 3][at] = g.w;
+    }
+  }
+  __syncthreads();
+  double w[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) w[v] = feat && k0 + kk + v < d ? 0.5 * pow2(-feat[k0 + kk + v]) : 0.5;
+#pragma unroll
+  for (int i = 0; i < TP / 8; ++i) {
+    const int pp = 8 * i + (threadIdx.x >> 5);
+    const long long p = p0 + pp;
+    if (p >= d) break;
+    const float4 g = *reinterpret_cast<const float4*>(&mirror[pp][kk ^ (pp & 28)]);
+    const unsigned top = rowmax[p];
+    const int e = top < 0x7f800000u ? slice_exponent<true>((double)__uint_as_float(top)) : 205;   // (2^128 2^75 and less)
+    const float a[4] = {h[i].x, h[i].y, h[i].z, h[i].w}, b[4] = {g.x, g.y, g.z, g.w};
     double x[4];
 #pragma unroll
-    for (int v = 0; v < 4; ++v)
-      x[v] = k + v > p ? 0.0 : (k + v == p ? 0.5 : 1.0) * (feat ? pow2(-feat[k + v]) : 1.0) * (double)H[p * d + k + v];
-    write_slices<true>(x, ns, exps[p], out + (size_t)p * BN + c, (size_t)d * BN);
+    for (int v = 0; v < 4; ++v) x[v] = w[v] * ((double)finite(a[v]) + (double)finite(b[v]));
+    if (m > 0) {
+      write_slices<true>(x, ns, e, out + (size_t)p * kp + k0 + kk, (size_t)d * kp);
+    } else {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) x[v] = k0 + kk + v > p ? 0.0 : k0 + kk + v == p ? 0.5 * x[v] : x[v];
+      write_slices<true>(x, ns, e, diag + (size_t)p * BN + (k0 - (long long)K * BN) + kk, (size_t)d * BN);
+      if ((blockIdx.x & 1) == 0 && (threadIdx.x & 31) == 0) exps[p] = e;
+    }
   }
 }
 
@@ -310,8 +384,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 __device__ __forceinline__ double int_to_double(uint32_t r) {
   return __hiloint2double(0x43300000, (int)(r ^ 0x80000000u)) - 4503601774854144.0;   // 2^52 + 2^31
 }
-// Half of the product: how many blocks of 256 columns of H follow the diagonal one in tile column tn.
-__device__ __forceinline__ int blocks_after(int tn, int nb) { return (nb - 1) / 2 + ((nb & 1) == 0 && tn < nb / 2 ? 1 : 0); }
 // Tiles are handed out in bands of 8 tile rows, column by column inside a band, so that the
 // tiles in flight at one time share their operand panels in L2.
 __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int& tm, int& tn) {
@@ -573,7 +645,7 @@ static bool half_product(long long d_in) { return d_in >= 3072; }
 
 size_t gemm_tc_h_bytes(long long d_in, int nh) {
   return align_up((size_t)nh * d_in * tc_kpad(d_in)) + align_up(sizeof(int) * (size_t)d_in) +
-         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) + align_up(sizeof(int) * (size_t)d_in) : 0);   // diagonal blocks, D
+         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) + 2 * align_up(sizeof(int) * (size_t)d_in) : 0);   // diagonal blocks, D, row maxima
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -587,17 +659,25 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use,
   const bool half = use != kTcProduct && half_product(d_in);
   signed char* slices = (signed char*)hbuf;
   int* hexp = (int*)((char*)hbuf + align_up((size_t)nh * d_in * kp));
-  const dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
   if (half) {
     signed char* diag = (signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
-    int* feat = use == kTcSearch ? (int*)(diag + align_up((size_t)nh * d_in * i8::BN)) : nullptr;
+    unsigned* rowmax = (unsigned*)(diag + align_up((size_t)nh * d_in * i8::BN));
+    int* feat = use == kTcSearch ? (int*)((char*)rowmax + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
+    const int nb = (int)((d_in + i8::BN - 1) / i8::BN);
+    const dim3 grid_m((unsigned)((d_in + 1023) / 1024), (unsigned)((d_in + 15) / 16)), grid_s(8, 1 + nb / 2, (unsigned)nb);
+    cudaError_t e = cudaMemsetAsync(rowmax, 0, sizeof(unsigned) * (size_t)d_in, st);
+    if (e != cudaSuccess) return e;
     if (feat) { i8::feature_exp_kernel<<<(unsigned)((d_in + 255) / 256), 256, 0, st>>>(H, d_in, feat); count_launch(); }
-    { i8::row_exp_f32_kernel<true><<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, feat, hexp); count_launch(); }
-    { i8::slice_h_kernel<true><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, feat, nh, slices); count_launch(); }
-    { i8::slice_diag_kernel<<<(unsigned)((d_in + 7) / 8), 256, 0, st>>>(H, d_in, hexp, feat, nh, diag); count_launch(); }
+    auto run = [&](auto max_kern, auto slice_kern) {
+      { max_kern<<<grid_m, 256, 0, st>>>(H, d_in, feat, rowmax); count_launch(); }
+      { slice_kern<<<grid_s, 256, 0, st>>>(H, d_in, kp, feat, rowmax, nh, hexp, slices, diag); count_launch(); }
+    };
+    if (d_in % 4 == 0) run(i8::half_max_kernel<true>, i8::half_slice_kernel<true>);
+    else run(i8::half_max_kernel<false>, i8::half_slice_kernel<false>);
   } else {
-    { i8::row_exp_f32_kernel<false><<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, nullptr, hexp); count_launch(); }
-    { i8::slice_h_kernel<false><<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nullptr, nh, slices); count_launch(); }
+    const dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
+    { i8::row_exp_f32_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, hexp); count_launch(); }
+    { i8::slice_h_kernel<<<grid, 128, 0, st>>>(H, d_in, kp, hexp, nh, slices); count_launch(); }
   }
   return cudaGetLastError();
 }
@@ -637,7 +717,7 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& 
   const signed char* hsl = (const signed char*)hbuf;
   const int* hexp = (const int*)((const char*)hbuf + align_up((size_t)nh * d_in * kp));
   const signed char* dsl = (const signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
-  const int* feat = half && use == kTcSearch ? (const int*)(dsl + align_up((size_t)nh * d_in * BN)) : nullptr;
+  const int* feat = half && use == kTcSearch ? (const int*)(dsl + align_up((size_t)nh * d_in * BN) + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
   signed char* esl = (signed char*)ebuf;
   int* eexp = (int*)((char*)ebuf + align_up((size_t)ne * d_out * kp));
   unsigned long long* colmax = (unsigned long long*)((char*)eexp + align_up(sizeof(int) * (size_t)d_out));

@@ -34,3 +34,31 @@ def test_losses_by_half_of_the_product(d_in, d_out, group):
     # and far below that where the errors are as random as they are here
     assert float(((got - want) / want).abs().max()) < 1e-9
     assert abs(total - float(want.sum())) <= 1e-10 * float(want.sum())
+
+
+@pytest.mark.parametrize("kind", ["rounding", "triangle", "one NaN"])
+@pytest.mark.parametrize("d_in,d_out", [(3072, 130), (3333, 300)])
+def test_hessians_that_are_not_symmetric_bit_for_bit(d_in, d_out, kind):
+    """The loss is e^T H e whatever the class of sizes: of an H whose triangles were rounded apart, of one with a single triangle, and of one with
+    a NaN whose mirror image is a number (the NaN is left out, the number counts)."""
+    dev = "cuda:0"
+    gen = torch.Generator(dev).manual_seed(d_in)
+    X = torch.randn(2 * d_in, d_in, generator=gen, device=dev) * torch.randn(d_in, generator=gen, device=dev).exp()
+    H = X.double().T @ X.double()
+    if kind == "rounding":
+        H *= 1 + 1e-6 * torch.randn(d_in, d_in, generator=gen, device=dev).double()
+    elif kind == "triangle":
+        H = torch.tril(H)
+    H = H.float().contiguous()
+    there = H.double()
+    if kind == "one NaN":
+        H[700, 2900] = float("nan")
+        there[700, 2900] = 0.0
+    W = torch.randn(d_in, d_out, generator=gen, device=dev) * 0.02
+    grid = B.Grid(3, 0, 1, 1.0, 1.0)
+    scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
+    E = scale.double() * Q.double() + zero.double() - W.double()
+    want = ((there @ E) * E).sum(0)
+    got = B.cdq_layer_loss(H, W, grid, scale, zero, Q, per_col=True)[1]
+    # far above the slicing errors (3e-12), far below what one triangle in the place of the other would give (4e-8 and more)
+    assert float(((got - want) / want).abs().max()) <= 1e-9
