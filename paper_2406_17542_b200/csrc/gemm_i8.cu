@@ -211,10 +211,10 @@ __global__ void __launch_bounds__(256) half_max_kernel(const float* __restrict__
   for (int r = 0; r < ROWS; ++r) {
     if (r0 + r >= d) break;
     const float4 h4 = four_of_row<VEC>(H, d, r0 + r, c);
-    const float h[4] = {fabsf(h4.x), fabsf(h4.y), fabsf(h4.z), fabsf(h4.w)}, wr = weight(r0 + r);
+    const float h[4] = {fabsf(finite(h4.x)), fabsf(finite(h4.y)), fabsf(finite(h4.z)), fabsf(finite(h4.w))}, wr = weight(r0 + r);
     float row = 0.f;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {   // (the maximum leaves a NaN out)
+    for (int v = 0; v < 4; ++v) {
       row = fmaxf(row, __fmul_ru(h[v], wc[v]));
       col[v] = fmaxf(col[v], __fmul_ru(h[v], wr));
     }

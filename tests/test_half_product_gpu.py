@@ -36,11 +36,11 @@ def test_losses_by_half_of_the_product(d_in, d_out, group):
     assert abs(total - float(want.sum())) <= 1e-10 * float(want.sum())
 
 
-@pytest.mark.parametrize("kind", ["rounding", "triangle", "one NaN"])
+@pytest.mark.parametrize("kind", ["rounding", "triangle", "one NaN", "infinity"])
 @pytest.mark.parametrize("d_in,d_out", [(3072, 130), (3333, 300)])
 def test_hessians_that_are_not_symmetric_bit_for_bit(d_in, d_out, kind):
-    """The loss is e^T H e whatever the class of sizes: of an H whose triangles were rounded apart, of one with a single triangle, and of one with
-    a NaN whose mirror image is a number (the NaN is left out, the number counts)."""
+    """The loss is e^T H e whatever the class of sizes: of an H whose triangles were rounded apart, of one with a single triangle, of one with
+    a NaN whose mirror image is a number (the NaN is left out, the number counts), and of one with infinite entries (left out, like a NaN)."""
     dev = "cuda:0"
     gen = torch.Generator(dev).manual_seed(d_in)
     X = torch.randn(2 * d_in, d_in, generator=gen, device=dev) * torch.randn(d_in, generator=gen, device=dev).exp()
@@ -54,6 +54,9 @@ def test_hessians_that_are_not_symmetric_bit_for_bit(d_in, d_out, kind):
     if kind == "one NaN":
         H[700, 2900] = float("nan")
         there[700, 2900] = 0.0
+    if kind == "infinity":
+        H[40, 41], H[41, 40], H[2000, 3000] = float("inf"), float("inf"), -float("inf")
+        there[40, 41] = there[41, 40] = there[2000, 3000] = 0.0
     W = torch.randn(d_in, d_out, generator=gen, device=dev) * 0.02
     grid = B.Grid(3, 0, 1, 1.0, 1.0)
     scale, zero, Q, _ = B.cdq_init_rtn(W, grid)
