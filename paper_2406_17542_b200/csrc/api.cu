@@ -104,9 +104,9 @@ SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool wit
   // the OWC search, whose residuals are plain rounding errors
   w.nh = kTcGradNH; w.ne = kTcGradNE; w.smax = kTcGradSmax;
   w.E = take(sizeof(double) * d_in * d_out);
-  if (with_cd || w.tc) w.G = take(sizeof(double) * d_out * w.ldg);
+  if (with_cd) w.G = take(sizeof(double) * d_out * w.ldg);
   if (w.tc) {
-    w.hbuf = take(gemm_tc_h_bytes(d_in, w.nh));
+    w.hbuf = take(gemm_tc_h_bytes(d_in, w.nh, with_cd ? kTcProduct : kTcLoss));
     w.ebuf = take(gemm_tc_e_bytes(d_in, d_out, w.ne));
   }
   if (with_cd) {
@@ -557,7 +557,7 @@ cdq_status cdq_layer_loss(const float* H, const void* W, cdq_dtype wt, long long
   if (!L.tc) CDQ_CUDA(launch_residual_f64(codes_src(ly, Q), d_in, E, st));
   if (L.tc) {
     CDQ_CUDA(gemm_tc_prepare_h(H, d_in, L.nh, kTcLoss, base + L.hbuf, st));
-    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, kTcLoss, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, (double*)(base + L.G), L.ldg, col_loss,
+    CDQ_CUDA(gemm_tc_run(base + L.hbuf, L.nh, kTcLoss, codes_src(ly, Q), E, d_in, d_out, L.ne, L.smax, 1.0, nullptr, 0, col_loss,
                          base + L.ebuf, st));
   } else if (mode == CDQ_MODE_FAST) {
     CDQ_CUDA(launch_gemm_he(H, d_in, d_out, E, nullptr, 0, col_loss, part, gemm_tc_supported(d_in, d_out), st));

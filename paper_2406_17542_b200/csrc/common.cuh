@@ -105,11 +105,11 @@ cudaError_t launch_gemm_he_verify(const float* H, long long d_in, long long d_ou
 // gemm_i8.cu : C[j, p] = scale * sum_k E[k, j] H[p, k] on the int8 tensor cores from 7-bit slices of
 // both operands (nh slices of H, ne of E, slice pairs up to i + j = smax); C is [d_out, ldc].
 // col_loss (may be NULL): [d_out], e_j^T H e_j.  gemm_tc_run forms the residual E [d_in, d_out] from its source first;
-// C is written by kTcProduct only; the other uses are for col_loss alone: the loss of codes, and the clipping search, whose few digits the
+// C belongs to kTcProduct; the other uses are for col_loss alone (C may be NULL): the loss of codes, and the clipping search, whose few digits the
 // features are scaled for.
 enum TcUse { kTcProduct, kTcLoss, kTcSearch };
 bool gemm_tc_supported(long long d_in, long long d_out);
-size_t gemm_tc_h_bytes(long long d_in, int nh);
+size_t gemm_tc_h_bytes(long long d_in, int nh, TcUse use);
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne);
 cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use, void* hbuf, cudaStream_t st);
 cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& src, double* E, long long d_in, long long d_out, int ne, int smax,

@@ -26,7 +26,7 @@
 //     e^T S e = 2 sum_P e_P^T (T_P e_P + sum_{K in half(P)} S_PK e_K),
 // where half(P) holds one of the blocks (P, K), (K, P) of every pair: the nb / 2 blocks that follow P, in a circle, so that every tile
 // has the same work.  (S is formed where the slices are, so that an H which is symmetric only up to rounding, or not at all, has the loss
-// that the whole product gives it.)  T_P is the lower triangle of the diagonal block with half of its diagonal; it has slices of its own, [ns][d][256].
+// that the whole product gives it.)  T_P is the lower triangle of the diagonal block with half of its diagonal.
 // The two halves of the whole product average an entry's slicing error with that of its mirror image; here it counts twice.  Two things
 // make up for that.  The digits are balanced (balanced_bits below).  And the clipping search, whose screen has two or three digits of
 // either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk), so the rows no
@@ -227,21 +227,21 @@ __global__ void __launch_bounds__(256) half_max_kernel(const float* __restrict__
   __syncthreads();
   if (threadIdx.x < ROWS && r0 + threadIdx.x < d) atomicMax(&rowmax[r0 + threadIdx.x], s_row[threadIdx.x]);
 }
-// Slices of S D^-1 (rows scaled by 2^-exps): the blocks (P, K) of 256 with K in half(P) into `out`, [ns][d][kp] (nothing reads the others),
-// the triangles T_P into `diag`, [ns][d][256].  64 rows x 128 columns per block; the mirror image of the tile is turned round in
+// Slices of S D^-1 (rows scaled by 2^-exps) into `out`, [ns][d][kp]: the blocks (P, K) of 256 with K in half(P) and, in the place of the
+// diagonal blocks, the triangles T_P; nothing reads the other blocks.  64 rows x 128 columns per block; the mirror image of the tile is turned round in
 // shared memory, so that both are read along their rows, once.  An entry that is no finite number is left out, its mirror image is not.
 // 4 bytes read and ns / 2 written per entry (4096^2, six slices: 39 us; all blocks of H, without its mirror image, and the triangles 53 us).
 template <bool VEC>
 __global__ void __launch_bounds__(256) half_slice_kernel(const float* __restrict__ H, long long d, long long kp, const int* __restrict__ feat,
                                                          const unsigned* __restrict__ rowmax, int ns, int* __restrict__ exps,
-                                                         signed char* __restrict__ out, signed char* __restrict__ diag) {
+                                                         signed char* __restrict__ out) {
   constexpr int TP = 64, TK = 128;
   __shared__ __align__(16) float mirror[TP][TK];   // H[k][p] at [p][k ^ 4 (p / 4 % 8)]
   const int nb = (int)((d + BN - 1) / BN), P = (int)blockIdx.z, m = (int)blockIdx.y;
   if (m > blocks_after(P, nb)) return;
   const int K = P + m < nb ? P + m : P + m - nb;
   const long long p0 = (long long)P * BN + (blockIdx.x >> 1) * TP, k0 = (long long)K * BN + (blockIdx.x & 1) * TK;
-  if (p0 >= d || (m > 0 && k0 >= kp)) return;
+  if (p0 >= d || k0 >= kp) return;
   const int kk = 4 * (threadIdx.x & 31);
   float4 h[TP / 8];   // rows p0 + warp, 8 further on, ...: on their way beside the mirror image
 #pragma unroll
@@ -275,14 +275,12 @@ __global__ void __launch_bounds__(256) half_slice_kernel(const float* __restrict
     double x[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) x[v] = w[v] * ((double)finite(a[v]) + (double)finite(b[v]));
-    if (m > 0) {
-      write_slices<true>(x, ns, e, out + (size_t)p * kp + k0 + kk, (size_t)d * kp);
-    } else {
+    if (m == 0) {
 #pragma unroll
       for (int v = 0; v < 4; ++v) x[v] = k0 + kk + v > p ? 0.0 : k0 + kk + v == p ? 0.5 * x[v] : x[v];
-      write_slices<true>(x, ns, e, diag + (size_t)p * BN + (k0 - (long long)K * BN) + kk, (size_t)d * BN);
       if ((blockIdx.x & 1) == 0 && (threadIdx.x & 31) == 0) exps[p] = e;
     }
+    write_slices<true>(x, ns, e, out + (size_t)p * kp + k0 + kk, (size_t)d * kp);
   }
 }
 
@@ -395,8 +393,7 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 }
 
 __global__ void __launch_bounds__(NUM_THREADS, 1)
-gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_h,
-               const __grid_constant__ CUtensorMap map_d, const Params p) {
+gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant__ CUtensorMap map_h, const Params p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;           // stage buffers, 1 KB aligned
@@ -452,13 +449,11 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
                 const int block = tn + (it >> 1);
                 kb = 2 * (block < p.tiles_n ? block : block - p.tiles_n) + (it & 1);
               }
-              const bool diag = p.half && it < 2;
               if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
               mbar_expect_tx(full_bar(stage), STAGE_BYTES);
               const uint32_t a_dst = tiles + (uint32_t)stage * STAGE_BYTES;
               tma_load_3d(a_dst, &map_e, kb * BKB, tm * BM, se, full_bar(stage));
-              if (diag) tma_load_3d(a_dst + A_BYTES, &map_d, it * BKB, tn * BN, sh, full_bar(stage));
-              else tma_load_3d(a_dst + A_BYTES, &map_h, kb * BKB, tn * BN, sh, full_bar(stage));
+              tma_load_3d(a_dst + A_BYTES, &map_h, kb * BKB, tn * BN, sh, full_bar(stage));
               ++issued;
               if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             }
@@ -528,7 +523,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
       const long long j = (long long)tm * BM + row;
       const long long p0 = (long long)tn * BN;
       const bool row_ok = j < p.M;
-      double* crow = p.C + (row_ok ? j : 0) * p.ldc;
+      double* crow = p.C + (row_ok ? j : 0) * p.ldc;   // (read and written with keep_c only)
       const int ej = row_ok ? p.eexp[j] : 0;
       double dot = 0.0;
       for (int g = 0; g < p.ngroups && ok; ++g) {
@@ -643,9 +638,9 @@ bool gemm_tc_supported(long long d_in, long long d_out) {
 // (257 x 16384 1.1e-13 -> 3.5e-13).
 static bool half_product(long long d_in) { return d_in >= 3072; }
 
-size_t gemm_tc_h_bytes(long long d_in, int nh) {
-  return align_up((size_t)nh * d_in * tc_kpad(d_in)) + align_up(sizeof(int) * (size_t)d_in) +
-         (half_product(d_in) ? align_up((size_t)nh * d_in * i8::BN) + 2 * align_up(sizeof(int) * (size_t)d_in) : 0);   // diagonal blocks, D, row maxima
+size_t gemm_tc_h_bytes(long long d_in, int nh, TcUse use) {
+  return align_up((size_t)nh * d_in * tc_kpad(d_in)) +
+         (use != kTcProduct && half_product(d_in) ? 3 : 1) * align_up(sizeof(int) * (size_t)d_in);   // row exponents; row maxima, D
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -660,8 +655,7 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use,
   signed char* slices = (signed char*)hbuf;
   int* hexp = (int*)((char*)hbuf + align_up((size_t)nh * d_in * kp));
   if (half) {
-    signed char* diag = (signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
-    unsigned* rowmax = (unsigned*)(diag + align_up((size_t)nh * d_in * i8::BN));
+    unsigned* rowmax = (unsigned*)((char*)hexp + align_up(sizeof(int) * (size_t)d_in));
     int* feat = use == kTcSearch ? (int*)((char*)rowmax + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
     const int nb = (int)((d_in + i8::BN - 1) / i8::BN);
     const dim3 grid_m((unsigned)((d_in + 1023) / 1024), (unsigned)((d_in + 15) / 16)), grid_s(8, 1 + nb / 2, (unsigned)nb);
@@ -670,7 +664,7 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use,
     if (feat) { i8::feature_exp_kernel<<<(unsigned)((d_in + 255) / 256), 256, 0, st>>>(H, d_in, feat); count_launch(); }
     auto run = [&](auto max_kern, auto slice_kern) {
       { max_kern<<<grid_m, 256, 0, st>>>(H, d_in, feat, rowmax); count_launch(); }
-      { slice_kern<<<grid_s, 256, 0, st>>>(H, d_in, kp, feat, rowmax, nh, hexp, slices, diag); count_launch(); }
+      { slice_kern<<<grid_s, 256, 0, st>>>(H, d_in, kp, feat, rowmax, nh, hexp, slices); count_launch(); }
     };
     if (d_in % 4 == 0) run(i8::half_max_kernel<true>, i8::half_slice_kernel<true>);
     else run(i8::half_max_kernel<false>, i8::half_slice_kernel<false>);
@@ -716,8 +710,7 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& 
   const bool keep_c = use == kTcProduct, half = !keep_c && half_product(d_in);
   const signed char* hsl = (const signed char*)hbuf;
   const int* hexp = (const int*)((const char*)hbuf + align_up((size_t)nh * d_in * kp));
-  const signed char* dsl = (const signed char*)hexp + align_up(sizeof(int) * (size_t)d_in);
-  const int* feat = half && use == kTcSearch ? (const int*)(dsl + align_up((size_t)nh * d_in * BN) + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
+  const int* feat = half && use == kTcSearch ? (const int*)((const char*)hexp + 2 * align_up(sizeof(int) * (size_t)d_in)) : nullptr;
   signed char* esl = (signed char*)ebuf;
   int* eexp = (int*)((char*)ebuf + align_up((size_t)ne * d_out * kp));
   unsigned long long* colmax = (unsigned long long*)((char*)eexp + align_up(sizeof(int) * (size_t)d_out));
@@ -759,13 +752,10 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& 
   p.status = device_status_word();
   if (!p.status) return cudaErrorInvalidSymbol;
 
-  CUtensorMap map_e, map_h, map_d;
+  CUtensorMap map_e, map_h;
   e = encode_map3(&map_e, esl, kp, d_out, ne, BM);
   if (e != cudaSuccess) return e;
   e = encode_map3(&map_h, hsl, kp, d_in, nh, BN);
-  if (e != cudaSuccess) return e;
-  map_d = map_h;
-  if (half) e = encode_map3(&map_d, dsl, BN, d_in, nh, BN);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -773,7 +763,7 @@ cudaError_t gemm_tc_run(const void* hbuf, int nh, TcUse use, const ResidualSrc& 
   e = cudaFuncSetAttribute(gemm_i8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
   if (e != cudaSuccess) return e;
   const int ntiles = p.tiles_m * p.tiles_n;
-  { gemm_i8_kernel<<<ntiles < sms ? ntiles : sms, NUM_THREADS, SMEM_BYTES, st>>>(map_e, map_h, map_d, p); count_launch(); }
+  { gemm_i8_kernel<<<ntiles < sms ? ntiles : sms, NUM_THREADS, SMEM_BYTES, st>>>(map_e, map_h, p); count_launch(); }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (col_loss) {

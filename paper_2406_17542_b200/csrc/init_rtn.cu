@@ -421,12 +421,11 @@ cudaError_t launch_group_minmax(const Layer& ly, float* pmn, float* pmx, float* 
 //   OWC only : gammas [n_clip] f64, gam_col [d_out] f64, table [n_clip, d_out] f64,
 //              E [d_in, d_out] f64, loss partials (FAST) or the product H E (VERIFY)
 struct InitWs {
-  size_t pmn, pmx, mn, mx, gammas, gam_col, table, E, part, C, hbuf, ebuf, screen, mask, idx, cnt, loss_c, cj, ck, total;
+  size_t pmn, pmx, mn, mx, gammas, gam_col, table, E, part, hbuf, ebuf, screen, mask, idx, cnt, loss_c, cj, ck, total;
   bool screened;    // cheap losses first, exact ones for the near-tied strengths only
   int sbatch;       // strengths per screening product (several on small layers, where a product per strength is launch-bound)
-  long long wcap;   // columns that E, C and the slice buffers hold
+  long long wcap;   // columns that E and the slice buffers hold
   bool tc;          // losses on the int8 tensor cores
-  long long ldc;
 };
 static InitWs init_ws_layout(long long d_in, long long d_out, long long g, int n_clip, cdq_mode mode) {
   InitWs w{};
@@ -452,10 +451,8 @@ static InitWs init_ws_layout(long long d_in, long long d_out, long long g, int n
     w.wcap = d_out + 128 > (long long)w.sbatch * d_out ? d_out + 128 : (long long)w.sbatch * d_out;
     w.E = take(sizeof(double) * d_in * w.wcap);
     w.part = take(sizeof(double) * (mode == CDQ_MODE_FAST ? gemm_partials_elems(d_in, d_out) : (size_t)d_in * d_out));
-    w.ldc = (d_in + 3) / 4 * 4;
     if (w.tc) {
-      w.C = take(sizeof(double) * w.wcap * w.ldc);
-      w.hbuf = take(gemm_tc_h_bytes(d_in, kTcLossNH));
+      w.hbuf = take(gemm_tc_h_bytes(d_in, kTcLossNH, kTcSearch));
       w.ebuf = take(gemm_tc_e_bytes(d_in, w.wcap, kTcLossNE));
       if (w.screened) {
         w.screen = take(sizeof(double) * n_clip * d_out);
@@ -538,7 +535,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.g = g; src.d_out = d_out;
         if (gb > 1) { src.n_cols = width; src.k0 = k0; src.gammas = gammas; }   // column c: layer column c % d_out
         e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, width, screen_slices(ly.bits), screen_slices(ly.bits) + 1, 1.0,
-                        (double*)(base + L.C), L.ldc, screen + (long long)k0 * d_out, base + L.ebuf, st);
+                        nullptr, 0, screen + (long long)k0 * d_out, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
       }
       { owc_candidates_kernel<<<bx, 128, 0, st>>>(screen, n_clip, d_out, mask, table); count_launch(); }
@@ -553,7 +550,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
       const int total = offs.off[n_clip], padded = (total + 127) / 128 * 128;
       if (total <= 0) return cudaErrorUnknown;   // every column has at least its best strength as a candidate
       { owc_concat_kernel<<<(unsigned)((padded + 255) / 256), 256, 0, st>>>(idx, d_out, offs, n_clip, padded, cj, ck); count_launch(); }
-      const int cap = (int)(L.wcap / 128 * 128);   // columns per product: what E, C and the slice buffers hold
+      const int cap = (int)(L.wcap / 128 * 128);   // columns per product: what E and the slice buffers hold
       for (int b0 = 0; b0 < padded; b0 += cap) {
         const int width = padded - b0 < cap ? padded - b0 : cap;
         ResidualSrc src{};
@@ -561,7 +558,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
         src.mn = mn; src.mx = mx; src.L = ly.L; src.use_gamma = 1;
         src.g = g; src.d_out = d_out; src.col_idx = cj + b0; src.n_cols = width;
         src.col_gamma = ck + b0; src.gammas = gammas;
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, width, kTcLossNE, kTcLossSmax, 1.0, nullptr, 0,
                         loss_c, base + L.ebuf, st);
         if (e != cudaSuccess) return e;
         { owc_scatter_kernel<<<(unsigned)((width + 255) / 256), 256, 0, st>>>(loss_c, cj + b0, ck + b0, width, d_out, table); count_launch(); }
@@ -573,7 +570,7 @@ cudaError_t launch_init_rtn(const Layer& ly, const cdq_grid_desc& grid, float* s
       src.mn = mn; src.mx = mx; src.gamma = hg[k]; src.L = ly.L; src.use_gamma = 1;
       src.g = g; src.d_out = d_out;
       if (L.tc) {
-        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, (double*)(base + L.C), L.ldc,
+        e = gemm_tc_run(base + L.hbuf, kTcLossNH, kTcSearch, src, E, d_in, d_out, kTcLossNE, kTcLossSmax, 1.0, nullptr, 0,
                         table + (long long)k * d_out, base + L.ebuf, st);
       } else {
         e = launch_residual_f64(src, d_in, E, st);

@@ -669,7 +669,7 @@ static OwcWs owc_ws_layout(long long d_in, long long d_out, long long g, int nk,
   if (w.tc) {
     w.E = take(sizeof(double) * d_in * d_out);
     w.G = take(sizeof(double) * d_out * w.ldg);
-    w.hbuf = take(gemm_tc_h_bytes(d_in, kTcGradNH));
+    w.hbuf = take(gemm_tc_h_bytes(d_in, kTcGradNH, kTcProduct));
     w.ebuf = take(gemm_tc_e_bytes(d_in, d_out, kTcGradNE));
   }
   w.total = off;

@@ -86,6 +86,22 @@ def test_small_groups_keep_the_tables_of_the_general_owc_cd_kernel(lib):
         assert ws(d_in, d_out, g, nk) - ws(d_in, d_out, g, 2) < tables(d_in, d_out, nk) / 2
 
 
+def test_workspaces_hold_what_their_call_uses(lib):
+    """Losses take no matrix of products beside the residual, and descents none of the slices that only losses use: E and G in fp64, codes, and
+    one byte per digit of H (rows of d_in rounded up to 128) and of the residual, with one percent for what goes by rows or columns."""
+    for d_in, d_out, g, clips in [(4096, 4096, 128, 20), (3072, 130, 0, 4), (14336, 592, 0, 2), (18432, 1184, 128, 20), (19000, 140, 0, 8)]:
+        kp = (d_in + 127) // 128 * 128
+        need = lambda which, n_clip=1: B.workspace_bytes(which, 0, d_in, d_out, B.Grid(3, g, n_clip, 0.5, 1.0))
+        E, small = 8 * d_in * d_out, 16 * (d_in // 128 + 3) * d_out + 64 * (d_in + d_out) + 8192
+        loss = E + 6 * d_in * kp + 5 * d_out * kp + small
+        assert need(B.CALL_LAYER_LOSS) <= 1.01 * loss
+        assert need(B.CALL_CD_SOLVE) <= 1.01 * (loss + 9 * d_out * ((d_in + 3) // 4 * 4))
+        assert need(B.CALL_LAYER_LOSS) <= need(B.CALL_CD_SOLVE)
+        width = max(d_out + 128, d_out * max(1, min(clips, 2 ** 30 // E) if clips >= 4 else 1))   # columns of one product of the search
+        assert need(B.CALL_INIT_RTN, clips) - need(B.CALL_INIT_RTN) <= 1.01 * (
+            8 * d_in * width + 4 * d_in * kp + 4 * width * kp + 16 * (d_in // 128 + 3) * width + 40 * clips * d_out + small)
+
+
 def test_bad_arguments_are_rejected_before_any_launch(lib):
     gd = B.Grid(bits=3).c()
     dummy = ctypes.c_void_p(256)  # never dereferenced: validation fails first
