@@ -49,7 +49,7 @@ constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + (size_t)STAGES * STAGE_
 struct Params {
   long long n, d_in;
   int tiles_m, ntiles, splits, kblocks;
-  float* partials;   // [splits][ntiles][BM*BN]
+  float* partials;   // [splits][ntiles][BM*BN] (see partials_bytes)
   const int2* tiles; // [ntiles] (tm, tn) in the order the tiles are handed out
   float* H;          // without K splits: where the epilogue adds the tiles ...
   int accumulate;    // ... to what is there
@@ -315,22 +315,22 @@ hessian_tc_kernel(const __grid_constant__ CUtensorMap tmap, Params p) {
           }
         } else {
 #pragma unroll 1
-        for (int c = half; c < BN / 32; c += 2) {
-          uint32_t r[32];
-          tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), r);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          for (int c = half; c < BN / 32; c += 2) {
+            uint32_t r[32];
+            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), r);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            float4 x = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
-                                   __uint_as_float(r[4 * v + 3]));
-            float4* dst = reinterpret_cast<float4*>(out + c * 32 + v * 4);
-            if (!first) {
-              const float4 y = *dst;
-              x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+            for (int v = 0; v < 8; ++v) {
+              float4 x = make_float4(__uint_as_float(r[4 * v]), __uint_as_float(r[4 * v + 1]), __uint_as_float(r[4 * v + 2]),
+                                     __uint_as_float(r[4 * v + 3]));
+              float4* dst = reinterpret_cast<float4*>(out + c * 32 + v * 4);
+              if (!first) {
+                const float4 y = *dst;
+                x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w;
+              }
+              *dst = x;
             }
-            *dst = x;
           }
-        }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -439,6 +439,10 @@ static Plan make_plan(long long n, long long d_in) {
   pl.splits = splits;
   return pl;
 }
+// Partial tiles in the workspace: one per split; without splits only what the epilogue sums the chunks of more than KCHUNK K blocks in.
+static size_t partials_bytes(const Plan& pl) {
+  return pl.splits == 1 && pl.kblocks <= KCHUNK ? 0 : align_up((size_t)pl.splits * pl.ntiles * TILE_ELEMS * sizeof(float));
+}
 
 }  // namespace tc
 
@@ -450,7 +454,7 @@ bool hessian_tc_supported(long long n, long long d_in, long long ldx, const void
 size_t hessian_tc_workspace(long long n, long long d_in) {
   if (d_in < 256 || n < 256) return 0;
   const tc::Plan pl = tc::make_plan(n, d_in);
-  return align_up((size_t)pl.splits * pl.ntiles * tc::TILE_ELEMS * sizeof(float)) + align_up((size_t)pl.ntiles * sizeof(int2));
+  return tc::partials_bytes(pl) + align_up((size_t)pl.ntiles * sizeof(int2));
 }
 
 cudaError_t launch_hessian_tc(const void* X, long long n, long long d_in, long long ldx, int accumulate, float* H,
@@ -484,7 +488,7 @@ cudaError_t launch_hessian_tc(const void* X, long long n, long long d_in, long l
   Params p{};
   p.n = n; p.d_in = d_in; p.tiles_m = pl.tiles_m; p.ntiles = pl.ntiles; p.splits = pl.splits; p.kblocks = pl.kblocks;
   p.partials = (float*)ws;
-  int2* tiles = (int2*)((char*)ws + align_up((size_t)pl.splits * pl.ntiles * TILE_ELEMS * sizeof(float)));
+  int2* tiles = (int2*)((char*)ws + partials_bytes(pl));
   p.tiles = tiles;
   { hessian_tile_order_kernel<<<(pl.tiles_m + BAND - 1) / BAND, 128, 0, st>>>(pl.tiles_m, tiles); count_launch(); }
   p.status = device_status_word();

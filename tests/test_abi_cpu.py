@@ -102,6 +102,13 @@ def test_workspaces_hold_what_their_call_uses(lib):
             8 * d_in * width + 4 * d_in * kp + 4 * width * kp + 16 * (d_in // 128 + 3) * width + 40 * clips * d_out + small)
 
 
+def test_hessians_without_k_splits_take_no_partial_tiles(lib):
+    need = lambda n, d_in: B.workspace_bytes(B.CALL_HESSIAN, n, d_in, 0, None)
+    for n, d_in in [(4096, 8192), (1000, 4100), (16384, 18432)]:
+        assert need(n, d_in) <= 8 * (d_in // 128 + 2) ** 2
+    assert need(16448, 18432) >= 4 * 18432 * 18432 // 2    # more rows than one accumulator takes: the chunks of a tile are summed there
+
+
 def test_bad_arguments_are_rejected_before_any_launch(lib):
     gd = B.Grid(bits=3).c()
     dummy = ctypes.c_void_p(256)  # never dereferenced: validation fails first
