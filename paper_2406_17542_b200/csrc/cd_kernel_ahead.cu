@@ -39,7 +39,9 @@ constexpr unsigned kAbortKey = 0u;    // a copy did not land
 constexpr unsigned kFullKey = 1u;     // drop the move in flight and score everything (a warp has no idle lane left)
 constexpr unsigned kCrowdKey = 2u;    // the move in flight stands, but score everything after it (same reason)
 constexpr unsigned kNever = 0x7F000000u;   // a threshold that no gradient reaches
-constexpr int kHand = 8;             // coordinates a warp hands over to its idle lanes at a time
+// Coordinates a warp hands over to its idle lanes at a time.  (16: no faster on any row, 16384 x 296 columns 17.7 ms against 17.5, the others
+// within 0.5 %; and with 8 the table of H_ii fits beside 8 x 448 chunk slots.)
+constexpr int kHand = 8;
 constexpr float kGap0 = 0.3f, kGapMin = 1.f / 256, kGapMax = 0.5f, kGapGrow = 1.25f;
 
 // A coordinate that a lane is to watch, handed over by the thread that owns its chunk.
@@ -639,14 +641,17 @@ cudaError_t launch_cd_ahead(const CdParams& p, cudaStream_t st) {
   const long long ch = p.d_in >> 2;
   auto team = [&](long long chunks, int nch) { return (int)((chunks + nch - 1) / nch + 31) / 32 * 32; };
   // 384 threads as long as the row fits them: three warps per scheduler hide more latency than the two of 256 threads with up to
-  // 14 chunks each (14336 x 1184 columns 236 -> 226 ms, 11008 x 296 47.4 -> 43.3), and at 168 registers nothing spills; rows of 13825 to 14336 entries
-  // fill 8 x 448 slots, with room for the table of H_ii beside them; rows of
+  // 14 chunks each (14336 x 1184 columns 236 -> 226 ms, 11008 x 296 47.4 -> 43.3), and at 168 registers little spills (52 bytes at most, 12 x
+  // 384 per channel).  fp32 rows of 13825 to 14336 entries per channel fill 8 x 448 slots, with room for the table of H_ii beside them
+  // (13828 x 592 columns 60.1 ms against 61.1 for 10 x 384, 14336 x 592 62.6 / 62.2, x 1184 120.3 / 120.5); in groups, and as bf16 rows, 10 x 384 is
+  // the quicker one (a quarter of a pass, 8 x 448 / 10 x 384: 13952 in groups of 64 x 296 14.8 / 14.5 ms, 14336 in groups of 128 x 296 15.1 / 14.8, of
+  // 4 x 148 7.95 / 7.39, bf16 14336 x 296 15.8 / 14.6 and in groups of 128 17.5 / 16.6).  Rows of
   // 15361 to 16384 entries fill 8 x 512 slots (72 ms against 75 for 11 x 384 on 16384 x 296; 9 x 512 spills: 18432 x 592 226 ms
   // against 210 for 12 x 384).
   if (ch <= 2304) return launch_mode<6, 384, 1>(p, team(ch, 6), st);
   if (ch <= 3072) return launch_mode<8, 384, 1>(p, team(ch, 8), st);
   if (ch <= 3456) return launch_mode<9, 384, 1>(p, team(ch, 9), st);
-  if (ch <= 3584) return launch_mode<8, 448, 1>(p, team(ch, 8), st);
+  if (ch <= 3584 && p.ng == 1 && !p.H16) return launch_cfg<8, 448, 1, false, false>(p, team(ch, 8), st);
   if (ch <= 3840) return launch_mode<10, 384, 1>(p, team(ch, 10), st);
   if (ch <= 4096) return launch_mode<8, 512, 1>(p, team(ch, 8), st);
   if (ch <= 4224) return launch_mode<11, 384, 1>(p, team(ch, 11), st);
