@@ -82,6 +82,15 @@ __device__ __forceinline__ void pick_chunk(int k, const double (&g)[4 * NCH], co
 #undef CDQ_PICK
 }
 
+// Whether the table of H_ii fits beside the rows, the thresholds and the handovers of so many chunk slots is known when the kernel is compiled,
+// but to say it there changes what the compiler spills, for better or worse.  A quarter of a pass, said at run time / here (ms): 18432 x 296 per
+// channel 22.2 / 21.95, bf16 12288 x 296 in groups of 128 12.1 / 11.85, 14336 16.65 / 16.45; 14336 x 592 per channel 26.2 / 26.5, 17408 x 296 in
+// groups of 128 21.0 / 22.0, bf16 11264 x 296 9.96 / 10.1, 16384 x 148 in groups of 128 11.1 / 11.4, 15360 x 296 per channel 14.5 / 14.6.
+enum Table { kTableNever, kTableAlways, kTableIfFits };
+__host__ __device__ constexpr Table hd_table(int slots, bool grouped, bool row16) {
+  return row16 && grouped && slots <= 3840 ? kTableAlways : !row16 && !grouped && slots > 4224 ? kTableNever : kTableIfFits;
+}
+
 // NCH chunk slots per thread; the team covers ceil(d_in / 4) <= NT * NCH chunks.
 // ROW16: the rows come from a bf16 copy of H (half the bytes per move); the row's own diagonal element is
 // replaced by the exact H_ii, so the iteration is the descent on H with its off-diagonal entries rounded to bf16.
@@ -112,10 +121,15 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
   // team can go on, and from memory they come behind the row that is on its way into the SM (18432 in groups of 128 x 296 96.1 -> 93.3 ms,
   // 9004 in groups of 4 x 296 16.4 -> 15.5, 13312 in groups of 128 x 296 46.1 -> 45.4, 14336 x 592 111.9 -> 110.3).
   unsigned char* more = reinterpret_cast<unsigned char*>(reinterpret_cast<Handover*>(thr_s + NCH * NT) + kHand * nwarps);
-  const bool hd_here = (p.tables & 1) != 0, ag_here = GROUPED && (p.tables & 2) != 0;
+  constexpr Table kHd = hd_table(NCH * MAXNT, GROUPED, ROW16);
+  const bool hd_here = kHd == kTableAlways || (kHd == kTableIfFits && (p.tables & 1) != 0), ag_here = GROUPED && (p.tables & 2) != 0;
   float* hd_s = reinterpret_cast<float*>(more);
   float* ag_s = hd_s + (hd_here ? 4 * NCH * NT : 0);
   const float* hd_t = hd_here ? hd_s : p.hdiag;
+  auto hd_of = [&](int i) -> float { return kHd == kTableNever ? __ldg(p.hdiag + i) : hd_t[i]; };   // H_ii
+  auto hd4_of = [&](int cs) -> float4 {                                                            // those of a chunk
+    return kHd == kTableNever ? __ldg(reinterpret_cast<const float4*>(p.hdiag) + cs) : reinterpret_cast<const float4*>(hd_t)[cs];
+  };
   auto group_of = [&](unsigned i) -> unsigned { return p.g == 1 ? i : __umulhi(i, p.gmagic); };
 
   // slots past the end of the row stay zero: no copy ever writes there
@@ -244,7 +258,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
       float a = 1.f;
       if (GROUPED) a = scale_j[(long long)group_of((unsigned)istar) * scale_step];
       c2 = 2.0 * ((double)a * (double)((int)(w & 511u) - 256));
-      if constexpr (ROW16) cur_h = hd_t[istar];
+      if constexpr (ROW16) cur_h = hd_of(istar);
     };
     // Hands the coordinates of the two words over to idle lanes of the warp; true in the lanes that got one.
     // room: whether there were enough.
@@ -284,7 +298,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
               wid = hand[mine].id;
               wq = __uint_as_float(kMagicBits | hand[mine].q);
               wi = 4 * ((int)((wid >> 11) & 1023u) + NT * (int)(wid >> 21)) + (int)((wid >> 9) & 3u);
-              wh = hd_t[wi];
+              wh = hd_of(wi);
               if (GROUPED) wa = scale_j[(long long)group_of((unsigned)wi) * scale_step];
               fresh = true;
             }
@@ -316,7 +330,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
 #pragma unroll 1
       for (int k = 0; k < NCH; ++k) {
         const int cs = tid + NT * k;
-        const float4 hd = reinterpret_cast<const float4*>(hd_t)[cs];
+        const float4 hd = hd4_of(cs);
         const float4 hs = __ldg(reinterpret_cast<const float4*>(p.hs) + cs);
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
@@ -345,7 +359,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
 #pragma unroll 1
       for (int k = 0; k < NCH; ++k) {
         const int cs = tid + NT * k;
-        const float4 hd = reinterpret_cast<const float4*>(hd_t)[cs];
+        const float4 hd = hd4_of(cs);
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
           a = cs < nchs ? scale_j[(long long)group_of(4u * (unsigned)cs) * scale_step] : 0.f;
@@ -608,7 +622,8 @@ cudaError_t launch_cfg(CdParams p, int nt, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const size_t room = (size_t)optin - fa.sharedSizeBytes, hd = (size_t)NCH * nt * 16, ag = GROUPED ? ((size_t)p.ng * 4 + 15) / 16 * 16 : 0;
     p.tables = 0;
-    if (smem + hd <= room) { p.tables |= 1; smem += hd; }
+    constexpr Table kHd = hd_table(NCH * MAXNT, GROUPED, ROW16);
+    if (kHd == kTableAlways || (kHd == kTableIfFits && smem + hd <= room)) { p.tables |= 1; smem += hd; }
     if (GROUPED && smem + ag <= room) { p.tables |= 2; smem += ag; }
   }
   if (smem > 32 * 1024) {   // the 48 KB that need no opt-in include the kernel's static shared memory
