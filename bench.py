@@ -43,7 +43,7 @@ L2_BYTES = 126e6
 # capture divided by the moves of that capture), keyed by (kernel, d_in); a kernel and shape without a
 # capture of the kernel as it stands reports traffic null.  Each entry names the summary it comes from.
 NCU_TRAFFIC_PER_MOVE: dict = {
-    ("cd_ahead_kernel", 14336): (49490.0, "profiles/cd_ahead_kernel_C3_592cols.md"),
+    ("cd_ahead_kernel", 14336): (49334.0, "profiles/cd_ahead_kernel_C3_592cols.md"),
 }
 
 

@@ -148,8 +148,8 @@ cdq_status cdq_hessian_add_lambda(float* H, long long d_in, float lambda_rel, vo
  *   gamma_out  [d_out] fp32 out, chosen clipping strength; may be NULL.
  * FAST, layers of at least 256 x 128: the column losses are products on the int8 tensor cores.  All
  * strengths are first screened with three slice-pair products (six on grids of more than 4 bits); a strength
- * within 1 % of a column's smallest screened loss stays a candidate and gets the thirteen-pair loss (~1e-8
- * relative); the argmin is taken over the candidates.  The candidate counts go through the host: one synchronisation of `stream`.
+ * within 1 % of a column's smallest screened loss stays a candidate and gets the thirteen-pair loss (good to 2e-7
+ * relative, from 3072 inputs on to 1e-8); the argmin is taken over the candidates.  The candidate counts go through the host: one synchronisation of `stream`.
  * The codes are those of a rounding decision in fp64, in both modes (an fp32 quotient decides where it is clear of
  * the middle between two levels).
  */

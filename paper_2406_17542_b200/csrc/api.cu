@@ -95,9 +95,9 @@ SolveWs solve_ws_layout(long long d_in, long long d_out, cdq_mode mode, bool wit
   w.ldg = (d_in + 3) / 4 * 4;
   w.d_pad = cd_fast_pad(d_in);
   // On small layers the int8 product's 27 slice pairs are one long chain on a few SMs, and the slices come on top.  Loss of given
-  // codes, int8 against fp64 product (device time in us): 2.7e8 multiplications 229 / 98 (256 x 4096), 258 / 131 (1024 x 256), 280 / 161
-  // (1448 x 128); 5.4e8 237 / 139 (256 x 8192), 266 / 181 (1024 x 512), 312 / 215 (2048 x 128); 8.4e8 244 / 280 (724 x 1600); 1.07e9
-  // 250 / 224 (256 x 16384), 294 / 293 (1448 x 512), 330 / 307 (2048 x 256); 2.1e9 263 / 367 (512 x 8192), 300 / 519 (1448 x 1024).
+  // codes, int8 against fp64 product (us): 2.7e8 multiplications 122 / 89 (256 x 4096), 159 / 122 (1024 x 256), 196 / 157
+  // (1448 x 128); 5.4e8 126 / 128 (256 x 8192), 161 / 170 (1024 x 512), 224 / 198 (2048 x 128); 8.4e8 149 / 272 (724 x 1600); 1.07e9
+  // 139 / 209 (256 x 16384), 198 / 281 (1448 x 512), 231 / 292 (2048 x 256); 2.1e9 154 / 356 (512 x 8192), 203 / 507 (1448 x 1024).
   w.tc = mode == CDQ_MODE_FAST && gemm_tc_supported(d_in, d_out) && d_in * d_in * d_out >= 800000000ll;
   // the loss of a descended solution is a sum with heavy cancellation (the descent tunes e against the
   // large entries of H): it takes the same slice depth as the gradient; the shallower setting serves

@@ -507,7 +507,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_e, const __grid_constant_
       }
     }
   } else {
-    // ---------------- epilogue: TMEM -> fp64 running sum in C ----------------
+    // ---------------- epilogue: TMEM -> fp64 running sum in C, or column dots alone ----------------
     // Two warps per TMEM lane quarter; they take the 16-column chunks of the tile in turn.  Where only the dots are wanted, every group
     // gives its own, 128^-s E . acc, and there is no running sum
     // (16 bytes per entry and group; loss of 4096 x 4096 codes 1290 -> 1001 us, 1350 x 677 291 -> 202, clipping search 4.3 -> 4.1 ms).
@@ -632,10 +632,11 @@ bool gemm_tc_supported(long long d_in, long long d_out) {
   return d_in >= 256 && d_out >= 128 && d_in <= 26000 && d_out < (1ll << 30);
 }
 
-// Losses by half of the product.  Short sums are bound by the slices and the epilogue: loss of given codes, whole / half (us, both with a
-// running sum): 257 x 16384 388 / 406, 512 x 8192 273 / 276, 1350 x 677 291 / 283, 2048 x 2048 364 / 329, 3072 x 2048 775 / 657, 3072 x 130
-// 407 / 371, 4096 x 4096 1803 / 1290, 5376 x 300 640 / 499, 8192 x 1024 1719 / 1185; and with a few blocks only, it costs precision
-// (257 x 16384 1.1e-13 -> 3.5e-13).
+// Losses by half of the product.  Short sums are bound by the slices and the epilogue: loss of given codes, whole / half (us): 257 x 16384
+// 219 / 248, 512 x 8192 156 / 174, 1024 x 1024 167 / 167, 1350 x 677 195 / 189, 2048 x 2048 263 / 228, 2560 x 1024 297 / 239, 3072 x 130 314 /
+// 247, 3072 x 2048 585 / 416, 4096 x 4096 1477 / 965, 5376 x 300 573 / 393, 8192 x 1024 1541 / 965.  It would be the faster one from some 1350
+// rows on, but with fewer blocks the errors of given codes are up to 17 % larger (rms: 1024 x 1024 in groups 8.9e-13 -> 1.04e-12, 2048 x 512 in
+// groups 1.02e-12 -> 1.06e-12; from 2560 x 512 on no larger, 4.5e-13 -> 4.2e-13).
 static bool half_product(long long d_in) { return d_in >= 3072; }
 
 size_t gemm_tc_h_bytes(long long d_in, int nh, TcUse use) {

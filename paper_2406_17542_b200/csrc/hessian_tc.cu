@@ -118,8 +118,9 @@ __global__ void hessian_tile_order_kernel(int tiles_m, int2* __restrict__ tiles)
   }
 }
 
-// DIRECT: no K splits, the epilogue writes H (8 batches of 4096 x 8192: the pass over the partial tiles took 0.1 of 0.38 ms per batch,
-// 2.69 -> 2.27 ms in all; 4096 x 8192 4 batches 0.39 -> 0.32;
+// DIRECT: no K splits, the epilogue writes H (8 batches of 4096 rows x 8192 features: the pass over the partial tiles took 0.1 of 0.38 ms per
+// batch, kernels 2.69 -> 2.27 ms in all, whole calls 2.97 -> 2.58; one batch of 4096 x 4096 85 -> 71 us.  One batch of 4096 x 8192 alone: 259 us, 277
+// added to H, 1.09 PFLOP/s executed, tensor pipe 64 % of the active cycles, L1 and shared memory 72 % busy with the operand tiles;
 // streaming loads and stores of H no faster, with four epilogue warps 5352 features x 2048 rows 0.69 -> 0.78 ms).
 template <bool DIRECT>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -428,7 +429,9 @@ static Plan make_plan(long long n, long long d_in) {
   pl.kblocks = (int)((n + BK - 1) / BK);
   // K-splits: the units (tile x split) run in waves of one per SM; pick the split count whose waves cost
   // least -- ceil(units / SMs) waves of kblocks / splits K blocks each, plus a fixed cost per unit
-  // (pipeline fill, the epilogue that nothing overlaps) of about 16 K blocks
+  // (pipeline fill, the epilogue that nothing overlaps) of about 16 K blocks.  Rows x features, as planned here / with one split (us):
+  // 65536 x 2048 220 / 382, 16384 x 3072 163 / 204, 16384 x 14336 2460 / 2800.  The formula does not count the reduction pass that only splits
+  // pay; where it splits for a few percent the two are within 3 % (4096 x 3072 71 / 70, 8192 x 4608 194 / 189).
   int splits = 1;
   long long best = -1;
   for (int s = 1; s <= 16 && s <= pl.kblocks; ++s) {

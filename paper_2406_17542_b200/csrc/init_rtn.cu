@@ -101,7 +101,7 @@ __global__ void scale_zero_kernel(const float* __restrict__ mn, const float* __r
 }
 
 // Codes of kCodeRows rows of one group by V columns per thread (see rtn_code).  Bound by instructions (14336 x 16384 bf16 weights in
-// groups of 128: 231 us, 3.1 instructions per clock and SM, ALU pipe 51 %, 3.0 TB/s): these weights
+// groups of 256: 208 us, 22 instructions per weight, issue slots 70 % busy, 3.3 TB/s): as many weights
 // took 1180 us with an fp64 division and one byte per thread.
 constexpr int kCodeRows = 16;
 template <int V, bool BF16>
@@ -136,8 +136,9 @@ __global__ void __launch_bounds__(128) rtn_codes_kernel(const void* __restrict__
 
 // Grid and codes of one group of at most 8 WARPS rows for 128 columns, without a clipping search: the weights are read once and stay in
 // registers, eight rows of four columns per thread, while the block's warps put their minima and maxima together.  14336 x 16384
-// weights in groups of 128, against three passes: bf16 336 -> 265 us (2.7 TB/s), fp32 399 -> 271 (4.3); bound by instructions and by the
-// divisions that a block waits for.
+// weights in groups of 128, against three passes: bf16 336 -> 265 us (2.7 TB/s), fp32 399 -> 271 (4.3).  Bound by instructions and by what a
+// block's warps wait for together (bf16: 27 instructions per weight, issue slots 67 % busy, 26 warps per SM; the first loads and the barrier around
+// the divisions are the first stalls).  At 64 registers fp32 weights spill 124 bytes per thread, bf16 20 to 24.
 template <int WARPS, bool BF16>
 __global__ void __launch_bounds__(32 * WARPS, 1024 / (32 * WARPS)) group_codes_kernel(const void* __restrict__ W, long long d_out, long long ldw, long long g, int L,
                                                           float* __restrict__ scale, float* __restrict__ zero,
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1024 / (32 * WARPS)) group_codes_k
 // Residual E[i][c] = (a q + b) - w in fp64, either from stored codes or, for the OWC search, from min/max and a clipping
 // strength (codes formed on the fly, never stored).  With colmax it also leaves the largest |E| 2^row_exp of every column there (as
 // ordered bit patterns, zeroed by the caller), which the slicing of the int8 product needs.  8 bytes written
-// per entry; bound by the latency of its loads (4096 x 4096 bf16 weights in groups: 46 us, 16 warps per SM at 86 registers, 2.8 TB/s).
+// per entry; bound by the latency of its loads (4096 x 4096 bf16 weights in groups: 43 us, 13 warps per SM at 97 registers, 3.0 TB/s).
 // (One entry per thread with an fp64 division, and the maxima by a pass of their own over E: 1.0 ms for eight
 // strengths of a 4096 x 4096 layer, 0.16 ms of them the maxima.)
 template <int V, bool BF16>
