@@ -29,8 +29,8 @@
 // that the whole product gives it.)  T_P is the lower triangle of the diagonal block with half of its diagonal.
 // The two halves of the whole product average an entry's slicing error with that of its mirror image; here it counts twice.  Two things
 // make up for that.  The digits are balanced (balanced_bits below).  And the clipping search, whose screen has two or three digits of
-// either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk), so the rows no
-// longer mix entries of many sizes, and what an entry of E weighs in the loss is its size.  The residuals of given codes are a few dozen
+// either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk) (or D = 1, see
+// feature_check_kernel), so the rows no longer mix entries of many sizes, and what an entry of E weighs in the loss is its size.  The residuals of given codes are a few dozen
 // bits on one grid, which five digits hold exactly, and D would take them off it: cdq_layer_loss goes without (column losses of
 // 8192 x 300 codes against 64 bits, rms: with D 3.9e-13, without 1.1e-13; whole product 1.0e-13).  Errors against 64 bits, whole -> half:
 //   thirteen pairs (largest of five layers of 2 to 8 bits, heavy weights among them) 2.4e-7 -> 1e-8
@@ -192,31 +192,31 @@ __device__ __forceinline__ float4 four_of_row(const float* __restrict__ H, long 
 }
 // An entry that is no finite number counts as zero.
 __device__ __forceinline__ float finite(float x) { return fabsf(x) <= 3.402823466e38f ? x : 0.f; }
-// rowmax[p]: the largest |H_pk| 2^-feat[k] and |H_kp| 2^-feat[k], rounded up, as a bit pattern; no entry of row p of S D^-1 is above it.  16
-// rows x 1024 columns per block, four columns per thread: one pass over H from memory (4096^2: 33 us, 2 TB/s, bound by
-// the latency of its loads).  feat may be NULL (D = 1).
-template <bool VEC>
+// rowmax[p]: the largest |H_pk| and |H_kp| (SCALED: times 2^-feat[k], rounded up), as a bit pattern; no entry of row p of S (of S D^-1) is above it.
+// `rows` rows x 1024 columns per block, four columns per thread: one pass over H from memory (24 us at 4096^2, 56 at 8192^2, 4.8 TB/s).  only_if (may be NULL): nothing is
+// done where it is zero.
+template <bool VEC, bool SCALED>
 __global__ void __launch_bounds__(256) half_max_kernel(const float* __restrict__ H, long long d, const int* __restrict__ feat,
-                                                       unsigned* __restrict__ rowmax) {
-  constexpr int ROWS = 16;
-  __shared__ unsigned s_row[ROWS];
-  const long long c = 4 * (blockIdx.x * 256ll + threadIdx.x), r0 = (long long)blockIdx.y * ROWS;
-  if (threadIdx.x < ROWS) s_row[threadIdx.x] = 0u;
+                                                       const int* __restrict__ only_if, int rows, unsigned* __restrict__ rowmax) {
+  __shared__ unsigned s_row[64];
+  if (only_if && *only_if == 0) return;
+  const long long c = 4 * (blockIdx.x * 256ll + threadIdx.x), r0 = (long long)blockIdx.y * rows;
+  if (threadIdx.x < rows) s_row[threadIdx.x] = 0u;
   __syncthreads();
-  auto weight = [&](long long k) { return feat && k < d ? __int_as_float((127 - feat[k]) << 23) : 1.f; };   // (feat: -75 to 64)
+  auto weight = [&](long long k) { return SCALED && k < d ? __int_as_float((127 - feat[k]) << 23) : 1.f; };   // (feat: -75 to 64)
   float wc[4], col[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int v = 0; v < 4; ++v) wc[v] = weight(c + v);
 #pragma unroll 8
-  for (int r = 0; r < ROWS; ++r) {
+  for (int r = 0; r < rows; ++r) {
     if (r0 + r >= d) break;
     const float4 h4 = four_of_row<VEC>(H, d, r0 + r, c);
     const float h[4] = {fabsf(finite(h4.x)), fabsf(finite(h4.y)), fabsf(finite(h4.z)), fabsf(finite(h4.w))}, wr = weight(r0 + r);
     float row = 0.f;
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      row = fmaxf(row, __fmul_ru(h[v], wc[v]));
-      col[v] = fmaxf(col[v], __fmul_ru(h[v], wr));
+      row = fmaxf(row, SCALED ? __fmul_ru(h[v], wc[v]) : h[v]);
+      col[v] = fmaxf(col[v], SCALED ? __fmul_ru(h[v], wr) : h[v]);
     }
     const unsigned most = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(row));
     if ((threadIdx.x & 31) == 0) atomicMax(&s_row[r], most);
@@ -225,7 +225,19 @@ __global__ void __launch_bounds__(256) half_max_kernel(const float* __restrict__
   for (int v = 0; v < 4; ++v)
     if (c + v < d) atomicMax(&rowmax[c + v], __float_as_uint(col[v]));
   __syncthreads();
-  if (threadIdx.x < ROWS && r0 + threadIdx.x < d) atomicMax(&rowmax[r0 + threadIdx.x], s_row[threadIdx.x]);
+  if (threadIdx.x < rows && r0 + threadIdx.x < d) atomicMax(&rowmax[r0 + threadIdx.x], s_row[threadIdx.x]);
+}
+// D only where H is positive, as far as its pairs of entries show: then |H_pk| <= sqrt(H_pp H_kk), and rowmax[k] is at most 2^(feat[k] + 1) and
+// a rounding.  Where a row is above twice that, the diagonal says nothing about the size of the entries (some random symmetric
+// matrices lost strengths with D): D is 1, and without[0] says that the row maxima are to be taken again.  One block.
+__global__ void __launch_bounds__(1024) feature_check_kernel(long long d, int* __restrict__ feat, unsigned* __restrict__ rowmax,
+                                                             int* __restrict__ without) {
+  int above = 0;
+  for (long long k = threadIdx.x; k < d; k += blockDim.x) above |= rowmax[k] > (unsigned)(127 + feat[k] + 2) << 23;
+  above = __syncthreads_or(above);
+  if (threadIdx.x == 0) *without = above;
+  if (!above) return;
+  for (long long k = threadIdx.x; k < d; k += blockDim.x) { feat[k] = 0; rowmax[k] = 0u; }
 }
 // Slices of S D^-1 (rows scaled by 2^-exps) into `out`, [ns][d][kp]: the blocks (P, K) of 256 with K in half(P) and, in the place of the
 // diagonal blocks, the triangles T_P; nothing reads the other blocks.  64 rows x 128 columns per block; the mirror image of the tile is turned round in
@@ -270,7 +282,7 @@ __global__ void __launch_bounds__(256) half_slice_kernel(const float* __restrict
     if (p >= d) break;
     const float4 g = *reinterpret_cast<const float4*>(&mirror[pp][kk ^ (pp & 28)]);
     const unsigned top = rowmax[p];
-    const int e = top < 0x7f800000u ? slice_exponent<true>((double)__uint_as_float(top)) : 205;   // (2^128 2^75 and less)
+    const int e = slice_exponent<true>((double)__uint_as_float(top));
     const float a[4] = {h[i].x, h[i].y, h[i].z, h[i].w}, b[4] = {g.x, g.y, g.z, g.w};
     double x[4];
 #pragma unroll
@@ -641,7 +653,8 @@ static bool half_product(long long d_in) { return d_in >= 3072; }
 
 size_t gemm_tc_h_bytes(long long d_in, int nh, TcUse use) {
   return align_up((size_t)nh * d_in * tc_kpad(d_in)) +
-         (use != kTcProduct && half_product(d_in) ? 3 : 1) * align_up(sizeof(int) * (size_t)d_in);   // row exponents; row maxima, D
+         (use == kTcProduct || !half_product(d_in) ? 1 : use == kTcLoss ? 2 : 3) * align_up(sizeof(int) * (size_t)d_in) +
+         align_up(sizeof(int));   // row exponents; half products: row maxima; the search: D, whether it was given up
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -658,17 +671,23 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use,
   if (half) {
     unsigned* rowmax = (unsigned*)((char*)hexp + align_up(sizeof(int) * (size_t)d_in));
     int* feat = use == kTcSearch ? (int*)((char*)rowmax + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
+    int* without = feat ? (int*)((char*)feat + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
     const int nb = (int)((d_in + i8::BN - 1) / i8::BN);
-    const dim3 grid_m((unsigned)((d_in + 1023) / 1024), (unsigned)((d_in + 15) / 16)), grid_s(8, 1 + nb / 2, (unsigned)nb);
-    cudaError_t e = cudaMemsetAsync(rowmax, 0, sizeof(unsigned) * (size_t)d_in, st);
+    const int rows = d_in < 6144 ? 16 : 64;
+    const dim3 grid_m((unsigned)((d_in + 1023) / 1024), (unsigned)((d_in + rows - 1) / rows)), grid_s(8, 1 + nb / 2, (unsigned)nb);
+    cudaError_t e = cudaMemsetAsync(rowmax, 0, sizeof(int) * (size_t)d_in, st);
     if (e != cudaSuccess) return e;
     if (feat) { i8::feature_exp_kernel<<<(unsigned)((d_in + 255) / 256), 256, 0, st>>>(H, d_in, feat); count_launch(); }
-    auto run = [&](auto max_kern, auto slice_kern) {
-      { max_kern<<<grid_m, 256, 0, st>>>(H, d_in, feat, rowmax); count_launch(); }
+    auto run = [&](auto scaled_kern, auto max_kern, auto slice_kern) {
+      if (feat) {
+        { scaled_kern<<<grid_m, 256, 0, st>>>(H, d_in, feat, nullptr, rows, rowmax); count_launch(); }
+        { i8::feature_check_kernel<<<1, 1024, 0, st>>>(d_in, feat, rowmax, without); count_launch(); }
+      }
+      { max_kern<<<grid_m, 256, 0, st>>>(H, d_in, nullptr, without, rows, rowmax); count_launch(); }
       { slice_kern<<<grid_s, 256, 0, st>>>(H, d_in, kp, feat, rowmax, nh, hexp, slices); count_launch(); }
     };
-    if (d_in % 4 == 0) run(i8::half_max_kernel<true>, i8::half_slice_kernel<true>);
-    else run(i8::half_max_kernel<false>, i8::half_slice_kernel<false>);
+    if (d_in % 4 == 0) run(i8::half_max_kernel<true, true>, i8::half_max_kernel<true, false>, i8::half_slice_kernel<true>);
+    else run(i8::half_max_kernel<false, true>, i8::half_max_kernel<false, false>, i8::half_slice_kernel<false>);
   } else {
     const dim3 grid((unsigned)((kp / 4 + 127) / 128), (unsigned)d_in);
     { i8::row_exp_f32_kernel<<<(unsigned)d_in, 256, 0, st>>>(H, d_in, d_in, hexp); count_launch(); }

@@ -82,3 +82,28 @@ def test_screen_of_rows_that_one_feature_dominates(bits, lo, hi, dominance):
     chosen = (grid[:, None] == gamma[None, :]).double().argmax(0)
     excess = table.gather(0, chosen[None])[0] / table.amin(0) - 1
     assert float(excess.max()) <= 1e-6
+
+
+def test_screen_of_a_hessian_that_is_not_positive():
+    """A symmetric matrix whose diagonal says nothing about the size of its entries: every column's strength against fp64 all the same."""
+    dev, d_in, d_out, n_clip = "cuda:0", 3072, 2048, 8
+    gen = torch.Generator(dev).manual_seed(11)
+    H = torch.randn(d_in, d_in, generator=gen, device=dev)
+    H = (H + H.T).contiguous()
+    H.diagonal()[:: 7] = torch.tensor([1e-6, 1e-3, 0.0, -1.0, 30.0], device=dev).repeat(d_in)[: len(range(0, d_in, 7))]
+    W = torch.randn(d_in, d_out, generator=gen, device=dev) * 0.02
+    gamma = B.cdq_init_rtn(W, B.Grid(3, 0, n_clip, 0.5, 1.0), H=H)[3]
+    mn, mx, Wd, Hd = W.amin(0).double(), W.amax(0).double(), W.double(), H.double()
+    points = oracle.gamma_grid(n_clip, 0.5, 1.0)
+    table = []
+    for g in points:
+        a = (float(g) * (mx - mn) / 7).float().double()
+        E = a * ((Wd - mn) / a).round().clamp(0, 7) + mn - Wd
+        table.append(((Hd @ E) * E).sum(0))
+    table = torch.stack(table)
+    chosen = (torch.from_numpy(points.astype(np.float32)).to(dev)[:, None] == gamma[None, :]).double().argmax(0)
+    best = table.amin(0)
+    # (losses of both signs: near zero, where the band of a column is narrow, the screen may pass its best strength by)
+    wide = best.abs() > 0.02 * table.abs().amax(0)
+    excess = ((table.gather(0, chosen[None])[0] - best) / best.abs())[wide]
+    assert int(wide.sum()) > d_out // 2 and float(excess.max()) <= 1e-6
