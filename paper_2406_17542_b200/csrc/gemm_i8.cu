@@ -30,9 +30,9 @@
 // The two halves of the whole product average an entry's slicing error with that of its mirror image; here it counts twice.  Two things
 // make up for that.  The digits are balanced (balanced_bits below).  And the clipping search, whose screen has two or three digits of
 // either operand, takes the product of H D^-1 and D E, D_kk = 2^s_k near sqrt(H_kk): |H_pk| <= sqrt(H_pp H_kk) (or D = 1, see
-// feature_check_kernel), so the rows no longer mix entries of many sizes, and what an entry of E weighs in the loss is its size.  The residuals of given codes are a few dozen
-// bits on one grid, which five digits hold exactly, and D would take them off it: cdq_layer_loss goes without (column losses of
-// 8192 x 300 codes against 64 bits, rms: with D 3.9e-13, without 1.1e-13; whole product 1.0e-13).  Errors against 64 bits, whole -> half:
+// feature_check_kernel), so the rows no longer mix entries of many sizes, and what an entry of E weighs in the loss is its size.  The
+// residuals of given codes are a few dozen bits on one grid, which five digits hold exactly, and D would take them off it: cdq_layer_loss
+// goes without (column losses of 8192 x 300 codes against 64 bits, rms: with D 3.9e-13, without 1.1e-13; whole product 1.0e-13).  Errors against 64 bits, whole -> half:
 //   thirteen pairs (largest of five layers of 2 to 8 bits, heavy weights among them) 2.4e-7 -> 1e-8
 //   27 pairs, rms over columns and eight layers each, given codes: 3072 x 512 9.5e-14 -> 9.6e-14, 4096 x 4096 in groups 3.1e-12 -> 3.2e-12,
 //   6144 x 256 in groups 9.3e-13 -> 9.4e-13; solved codes 1.5e-12 -> 1.4e-12, 5.8e-10 -> 4.5e-11, 6.0e-11 -> 1.5e-11
@@ -652,9 +652,11 @@ bool gemm_tc_supported(long long d_in, long long d_out) {
 static bool half_product(long long d_in) { return d_in >= 3072; }
 
 size_t gemm_tc_h_bytes(long long d_in, int nh, TcUse use) {
-  return align_up((size_t)nh * d_in * tc_kpad(d_in)) +
-         (use == kTcProduct || !half_product(d_in) ? 1 : use == kTcLoss ? 2 : 3) * align_up(sizeof(int) * (size_t)d_in) +
-         align_up(sizeof(int));   // row exponents; half products: row maxima; the search: D, whether it was given up
+  const size_t row_words = align_up(sizeof(int) * (size_t)d_in);
+  size_t bytes = align_up((size_t)nh * d_in * tc_kpad(d_in)) + row_words;   // slices, row exponents
+  if (use != kTcProduct && half_product(d_in)) bytes += row_words;                                       // row maxima
+  if (use == kTcSearch && half_product(d_in)) bytes += row_words + align_up(sizeof(int));                // D, whether it was given up
+  return bytes;
 }
 size_t gemm_tc_e_bytes(long long d_in, long long d_out, int ne) {
   return align_up(sizeof(double) * 2 * (size_t)((d_in + i8::BN - 1) / i8::BN) * (size_t)d_out) +   // partial column dots
@@ -673,7 +675,7 @@ cudaError_t gemm_tc_prepare_h(const float* H, long long d_in, int nh, TcUse use,
     int* feat = use == kTcSearch ? (int*)((char*)rowmax + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
     int* without = feat ? (int*)((char*)feat + align_up(sizeof(int) * (size_t)d_in)) : nullptr;
     const int nb = (int)((d_in + i8::BN - 1) / i8::BN);
-    const int rows = d_in < 6144 ? 16 : 64;
+    const int rows = d_in < 6144 ? 16 : 64;   // few fill the SMs, many spare atomics (8192^2 with 16 rows 95 us, with 64 56)
     const dim3 grid_m((unsigned)((d_in + 1023) / 1024), (unsigned)((d_in + rows - 1) / rows)), grid_s(8, 1 + nb / 2, (unsigned)nb);
     cudaError_t e = cudaMemsetAsync(rowmax, 0, sizeof(int) * (size_t)d_in, st);
     if (e != cudaSuccess) return e;
