@@ -85,10 +85,12 @@ __device__ __forceinline__ void pick_chunk(int k, const double (&g)[4 * NCH], co
 // Whether the table of H_ii fits beside the rows, the thresholds and the handovers of so many chunk slots is known when the kernel is compiled,
 // but to say it there changes what the compiler spills, for better or worse.  A quarter of a pass, said at run time / here (ms): 18432 x 296 per
 // channel 22.2 / 21.95, bf16 12288 x 296 in groups of 128 12.1 / 11.85, 14336 16.65 / 16.45; 14336 x 592 per channel 26.2 / 26.5, 17408 x 296 in
-// groups of 128 21.0 / 22.0, bf16 11264 x 296 9.96 / 10.1, 16384 x 148 in groups of 128 11.1 / 11.4, 15360 x 296 per channel 14.5 / 14.6.
+// groups of 128 21.0 / 22.0, bf16 11264 x 296 9.96 / 10.1, 15360 x 296 per channel 14.5 / 14.6.  Bf16 rows of 15361 to 16384 entries in groups
+// are better off without either table (16384 x 296 in groups of 128 22.2 / 21.9).
 enum Table { kTableNever, kTableAlways, kTableIfFits };
 __host__ __device__ constexpr Table hd_table(int slots, bool grouped, bool row16) {
-  return row16 && grouped && slots <= 3840 ? kTableAlways : !row16 && !grouped && slots > 4224 ? kTableNever : kTableIfFits;
+  if (row16 && grouped) return slots <= 3840 ? kTableAlways : slots <= 4096 ? kTableNever : kTableIfFits;
+  return !row16 && !grouped && slots > 4224 ? kTableNever : kTableIfFits;
 }
 
 // NCH chunk slots per thread; the team covers ceil(d_in / 4) <= NT * NCH chunks.
@@ -122,7 +124,8 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
   // 9004 in groups of 4 x 296 16.4 -> 15.5, 13312 in groups of 128 x 296 46.1 -> 45.4, 14336 x 592 111.9 -> 110.3).
   unsigned char* more = reinterpret_cast<unsigned char*>(reinterpret_cast<Handover*>(thr_s + NCH * NT) + kHand * nwarps);
   constexpr Table kHd = hd_table(NCH * MAXNT, GROUPED, ROW16);
-  const bool hd_here = kHd == kTableAlways || (kHd == kTableIfFits && (p.tables & 1) != 0), ag_here = GROUPED && (p.tables & 2) != 0;
+  constexpr bool kAg = GROUPED && !(ROW16 && kHd == kTableNever);   // (the group scales go with it)
+  const bool hd_here = kHd == kTableAlways || (kHd == kTableIfFits && (p.tables & 1) != 0), ag_here = kAg && (p.tables & 2) != 0;
   float* hd_s = reinterpret_cast<float*>(more);
   float* ag_s = hd_s + (hd_here ? 4 * NCH * NT : 0);
   const float* hd_t = hd_here ? hd_s : p.hdiag;
@@ -170,6 +173,9 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
     }
     const float* scale_j = ag_here ? ag_s : p.scale + j;   // GROUPED: scale of group t at scale_j[t * scale_step]
     const long long scale_step = ag_here ? 1 : p.d_out;
+    auto scale_of = [&](unsigned group) -> float {
+      return kAg ? scale_j[(long long)group * scale_step] : __ldg(p.scale + j + (long long)group * p.d_out);
+    };
     if (ag_here) {
       for (int t = tid; t < (int)p.ng; t += NT) ag_s[t] = p.scale[(long long)t * p.d_out + j];
       __syncthreads();
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
     // The step of move w, and what else its sweep needs (loads: they overlap with the copy).
     auto load_step = [&](unsigned w, int istar) {
       float a = 1.f;
-      if (GROUPED) a = scale_j[(long long)group_of((unsigned)istar) * scale_step];
+      if (GROUPED) a = scale_of(group_of((unsigned)istar));
       c2 = 2.0 * ((double)a * (double)((int)(w & 511u) - 256));
       if constexpr (ROW16) cur_h = hd_of(istar);
     };
@@ -299,7 +305,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
               wq = __uint_as_float(kMagicBits | hand[mine].q);
               wi = 4 * ((int)((wid >> 11) & 1023u) + NT * (int)(wid >> 21)) + (int)((wid >> 9) & 3u);
               wh = hd_of(wi);
-              if (GROUPED) wa = scale_j[(long long)group_of((unsigned)wi) * scale_step];
+              if (GROUPED) wa = scale_of(group_of((unsigned)wi));
               fresh = true;
             }
             who &= ~__ballot_sync(0xFFFFFFFFu, give);
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         const float4 hs = __ldg(reinterpret_cast<const float4*>(p.hs) + cs);
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
-          a = cs < nchs ? scale_j[(long long)group_of(4u * (unsigned)cs) * scale_step] : 0.f;
+          a = cs < nchs ? scale_of(group_of(4u * (unsigned)cs)) : 0.f;
           ia = a > 0.f ? 1.0f / a : 0.f;
         }
         double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -362,7 +368,7 @@ __global__ void __launch_bounds__(MAXNT, MINB) cd_ahead_kernel(CdParams p) {
         const float4 hd = hd4_of(cs);
         float a = 1.f, ia = 1.f;
         if (GROUPED) {
-          a = cs < nchs ? scale_j[(long long)group_of(4u * (unsigned)cs) * scale_step] : 0.f;
+          a = cs < nchs ? scale_of(group_of(4u * (unsigned)cs)) : 0.f;
           ia = a > 0.f ? 1.0f / a : 0.f;
         }
         double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -624,7 +630,7 @@ cudaError_t launch_cfg(CdParams p, int nt, cudaStream_t st) {
     p.tables = 0;
     constexpr Table kHd = hd_table(NCH * MAXNT, GROUPED, ROW16);
     if (kHd == kTableAlways || (kHd == kTableIfFits && smem + hd <= room)) { p.tables |= 1; smem += hd; }
-    if (GROUPED && smem + ag <= room) { p.tables |= 2; smem += ag; }
+    if (GROUPED && !(ROW16 && kHd == kTableNever) && smem + ag <= room) { p.tables |= 2; smem += ag; }
   }
   if (smem > 32 * 1024) {   // the 48 KB that need no opt-in include the kernel's static shared memory
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
